@@ -178,14 +178,15 @@ __global__ void __launch_bounds__(kPairThreads) k_pairs_f32(PairArgs a) {
   }
 }
 
-// FP64 path: every pair in FP64, sigma_t read from the padded FP64 lattice.
+// FP64 path with the march: every pair in FP64, sigma_t read from the padded
+// FP64 lattice.
 struct PairArgs64 {
   const double *sig;
   const double *src;
   double *partial;
   long N;
-  int n, P, tiles, splits, chunk, S, closed;
-  double h, sigma_c, wcoef;
+  int n, P, tiles, splits, chunk, S;
+  double h, wcoef;
 };
 
 template <int DIM>
@@ -235,23 +236,97 @@ __global__ void __launch_bounds__(kPairThreads) k_pairs_f64(PairArgs64 a) {
       double r2 = 0.0;
       for (int d = 0; d < DIM; ++d) r2 += (uk[d] - uj[d]) * (uk[d] - uj[d]);
       double r = sqrt(r2);
-      double tau;
-      if (a.closed) {
-        tau = a.sigma_c * a.h * r;
-      } else {
-        double acc = 0.0, p[3];
-        for (int i = 0; i < a.S; ++i) {
-          double t = (i + 0.5) / a.S;
-          for (int d = 0; d < DIM; ++d) p[d] = uj[d] + t * (uk[d] - uj[d]);
-          acc += sample64<DIM>(a.sig, a.P, p);
-        }
-        tau = a.h * r * acc / a.S;
+      double acc = 0.0, p[3];
+      for (int i = 0; i < a.S; ++i) {
+        double t = (i + 0.5) / a.S;
+        for (int d = 0; d < DIM; ++d) p[d] = uj[d] + t * (uk[d] - uj[d]);
+        acc += sample64<DIM>(a.sig, a.P, p);
       }
+      const double tau = a.h * r * acc / a.S;
       double ker = DIM == 3 ? 1.0 / r2 : 1.0 / r;
       sum += a.wcoef * exp(-tau) * ker * a.src[k];
     }
     a.partial[(long)split * a.N + j] = sum;
   }
+}
+
+// ---- FP64 pairs with the closed-form tau (constant sigma_t)
+//
+// The entry of a pair depends on |D| alone there, D = k - j, so the n^dim
+// values E(|dx|, |dy|, |dz|) = (h / |S^{d-1}|) e^{-sigma_c h r} / r^{d-1} (in
+// cells; E(0) = 0) are computed once per handle and an apply is one load and
+// one multiply-add per pair.  What bounds it then is the FP64 pipe (2
+// multiply-adds per clock and SM on this chip: 0.44 ms for the 2.7e8 pairs of
+// 128^2); the table (131 KB at 128^2) stays in L1.  A thread owns kClosedRows
+// targets stacked along y on one x, with independent sums, and runs over the
+// source rows of its split; lanes run along x (flattened over the row blocks,
+// so no lane idles on odd n), which makes the table loads of a warp
+// consecutive and the sources uniform.  Evaluating sqrt, exp and a divide per
+// pair (k_pairs_f64) took 19.3 ms per apply at 128^2 and 181 us at 32^2;
+// with the table 0.45 ms and 10 us.
+constexpr int kClosedThreads = 128;
+constexpr int kClosedRows = 4;
+
+__global__ void k_closed_table(int dim, int n, double h, double sigma_c, double wcoef, double *__restrict__ E) {
+  const long N = dim == 2 ? (long)n * n : (long)n * n * n;
+  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < N; i += (long)gridDim.x * blockDim.x) {
+    const double dx = (double)(i % n), dy = (double)((i / n) % n);
+    const double dz = dim == 3 ? (double)(i / ((long)n * n)) : 0.0;
+    double r2 = 0.0;
+    r2 += dx * dx;
+    r2 += dy * dy;
+    if (dim == 3) r2 += dz * dz;
+    const double r = sqrt(r2);
+    const double tau = sigma_c * h * r;
+    const double ker = dim == 3 ? 1.0 / r2 : 1.0 / r;
+    E[i] = i == 0 ? 0.0 : wcoef * exp(-tau) * ker;
+  }
+}
+
+// blockIdx.x: targets (x fastest, then blocks of kClosedRows y, then z),
+// blockIdx.y: split = source rows [split chunk, (split + 1) chunk) of n cells
+template <int DIM>
+__global__ void __launch_bounds__(kClosedThreads) k_pairs_f64_closed(int n, long N, int chunk,
+                                                                     const double *__restrict__ E,
+                                                                     const double *__restrict__ src,
+                                                                     double *__restrict__ partial) {
+  const int nyb = (n + kClosedRows - 1) / kClosedRows;
+  const long t = blockIdx.x * (long)kClosedThreads + threadIdx.x;
+  const long total = (long)n * nyb * (DIM == 3 ? n : 1);
+  if (t >= total) return;
+  const int jx = (int)(t % n);
+  const long rest = t / n;
+  const int jy = (int)(rest % nyb) * kClosedRows, jz = DIM == 3 ? (int)(rest / nyb) : 0;
+  const long rows = N / n;
+  const long row0 = (long)blockIdx.y * chunk, row1 = min(rows, row0 + chunk);
+  double acc[kClosedRows];
+#pragma unroll
+  for (int q = 0; q < kClosedRows; ++q) acc[q] = 0.0;
+  for (long row = row0; row < row1; ++row) {
+    const int ky = DIM == 3 ? (int)(row % n) : (int)row;
+    const int az = DIM == 3 ? abs((int)(row / n) - jz) : 0;
+    const double *base[kClosedRows];
+    bool self[kClosedRows];  // the target's own row: its own cell is skipped, not multiplied by E(0)
+#pragma unroll
+    for (int q = 0; q < kClosedRows; ++q) {
+      const int ay = abs(ky - min(jy + q, n - 1));  // rows past the grid repeat the last one
+      base[q] = E + ((long)az * n + ay) * n;
+      self[q] = az == 0 && ay == 0;
+    }
+    const double *s = src + row * n;
+#pragma unroll 4
+    for (int kx = 0; kx < n; ++kx) {
+      const double sk = __ldg(s + kx);
+      const int ax = abs(kx - jx);
+#pragma unroll
+      for (int q = 0; q < kClosedRows; ++q)
+        if (!(self[q] && ax == 0)) acc[q] = fma(__ldg(base[q] + ax), sk, acc[q]);
+    }
+  }
+  const long j = ((long)jz * n + jy) * n + jx;
+#pragma unroll
+  for (int q = 0; q < kClosedRows; ++q)
+    if (jy + q < n) partial[(long)blockIdx.y * N + j + (long)q * n] = acc[q];
 }
 
 __global__ void k_source_prep_f32(long N, int op, const double *__restrict__ ss,
@@ -393,6 +468,20 @@ vie_status plan_pairs(const Medium &m, int steps, int tau_closed, int precision,
   size_t lattice = m.dim == 2 ? (size_t)m.P * m.P : (size_t)m.P * m.P * m.P;
   size_t stage = sizeof(float4) * kPairThreads;
   int bps = 1;
+  if (precision == VIE_PREC_FP64 && tau_closed) {
+    // splits of whole source rows: about eight CTAs per SM, which evens out
+    // the SMs' shares to a few percent and keeps the partial sums short
+    const long rows = m.N / m.n;
+    const long total = (long)m.n * ((m.n + kClosedRows - 1) / kClosedRows) * (m.dim == 3 ? m.n : 1);
+    p.tiles = (int)((total + kClosedThreads - 1) / kClosedThreads);
+    const long want = (8L * prop.multiProcessorCount + p.tiles - 1) / p.tiles;
+    const long splits = std::max(1L, std::min(want, rows));
+    p.chunk = (int)((rows + splits - 1) / splits);
+    p.splits = (int)((rows + p.chunk - 1) / p.chunk);
+    p.grid = p.tiles * p.splits;
+    *plan = p;
+    return VIE_OK;
+  }
   if (precision == VIE_PREC_FP64) {
     p.smem_sigma = 0;
     p.smem_bytes = 0;
@@ -426,6 +515,17 @@ vie_status plan_pairs(const Medium &m, int steps, int tau_closed, int precision,
 vie_status launch_pairs(const Medium &m, const PairPlan &plan, int steps, int tau_closed,
                         int precision, const void *src, double *partial, cudaStream_t st) {
   const double h = 1.0 / m.n;
+  if (precision == VIE_PREC_FP64 && tau_closed) {
+    const dim3 grid((unsigned)plan.tiles, (unsigned)plan.splits);
+    if (m.dim == 2)
+      k_pairs_f64_closed<2><<<grid, kClosedThreads, 0, st>>>(m.n, m.N, plan.chunk, m.closed, (const double *)src,
+                                                             partial);
+    else
+      k_pairs_f64_closed<3><<<grid, kClosedThreads, 0, st>>>(m.n, m.N, plan.chunk, m.closed, (const double *)src,
+                                                             partial);
+    VIE_CHECK_LAUNCH("k_pairs_f64_closed");
+    return VIE_OK;
+  }
   if (precision == VIE_PREC_FP64) {
     PairArgs64 a;
     a.sig = m.sig64;
@@ -438,9 +538,7 @@ vie_status launch_pairs(const Medium &m, const PairPlan &plan, int steps, int ta
     a.splits = plan.splits;
     a.chunk = plan.chunk;
     a.S = steps;
-    a.closed = tau_closed;
     a.h = h;
-    a.sigma_c = m.sigma_c;
     a.wcoef = m.dim == 2 ? h / (2.0 * kPi) : h / (4.0 * kPi);
     if (m.dim == 2)
       k_pairs_f64<2><<<plan.grid, kPairThreads, 0, st>>>(a);
@@ -517,6 +615,15 @@ vie_status launch_pad_sigma(int dim, int n, const double *sig, float *out32, dou
   long total = dim == 2 ? P * P : P * P * P;
   k_pad_sigma<<<grid_for(total, 256), 256, 0, st>>>(dim, n, sig, out32, out64);
   VIE_CHECK_LAUNCH("k_pad_sigma");
+  return VIE_OK;
+}
+
+vie_status launch_closed_table(int dim, int n, double sigma_c, double *table, cudaStream_t st) {
+  const double h = 1.0 / n;
+  const long N = dim == 2 ? (long)n * n : (long)n * n * n;
+  k_closed_table<<<grid_for(N, 256), 256, 0, st>>>(dim, n, h, sigma_c,
+                                                   dim == 2 ? h / (2.0 * kPi) : h / (4.0 * kPi), table);
+  VIE_CHECK_LAUNCH("k_closed_table");
   return VIE_OK;
 }
 

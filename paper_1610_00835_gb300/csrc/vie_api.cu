@@ -162,6 +162,7 @@ struct vie_handle {
   float *sig32 = nullptr;                     // padded FP32 lattice
   double *sig64 = nullptr;                    // padded FP64 lattice
   double *diag = nullptr;                     // self-cell d_j [N]
+  double *closed = nullptr;                   // FP64 closed-form entries by |D| [N]
   Medium med{};
   PairPlan plan{};
   SymPlan sym{};                              // symmetric kernel, when usable
@@ -251,6 +252,7 @@ void free_all(vie_handle *h) {
   dfree(h->sig32);
   dfree(h->sig64);
   dfree(h->diag);
+  dfree(h->closed);
   if (h->src) vie_free(h->src);
   h->src = nullptr;
   if (h->pairs) vie_free(h->pairs);
@@ -936,6 +938,11 @@ vie_status vie_create(vie_handle **out, const vie_grid *g, const double *sigma_t
   h->med.sig32 = h->sig32;
   h->med.sig64 = h->sig64;
   h->med.sigma_c = sigma_t[0];
+  if (opts.precision == VIE_PREC_FP64 && opts.tau_mode == VIE_TAU_CLOSED) {
+    TRY(dalloc(&h->closed, N));
+    TRY(launch_closed_table(g->dim, g->n, sigma_t[0], h->closed, st));
+    h->med.closed = h->closed;
+  }
   TRY(plan_pairs(h->med, opts.steps, opts.tau_mode == VIE_TAU_CLOSED, opts.precision,
                  opts.device, &h->plan));
   {

@@ -106,6 +106,7 @@ struct Medium {
   const float *sig32; // padded FP32 sigma_t, P^dim, pad = copy of the edge
   const double *sig64;// padded FP64 sigma_t
   double sigma_c;     // constant sigma_t (closed-form tau)
+  const double *closed;  // FP64 with the closed-form tau: entry of every |D| [N]; else null
 };
 
 // Launch plan of the FP32 pair kernel for one medium.
@@ -133,6 +134,8 @@ vie_status launch_pad_sigma(int dim, int n, const double *sig, float *out32, dou
                             cudaStream_t st);
 vie_status launch_selfcell(int dim, int n, const double *sigma_t, double *diag,
                            cudaStream_t st);
+// entries of a homogeneous medium by |D| (FP64 [N], x fastest; 0 at D = 0)
+vie_status launch_closed_table(int dim, int n, double sigma_c, double *table, cudaStream_t st);
 
 // ---- symmetric pair kernel (k_pairs_sym.cu): FP32 tiles, S = 64, lattice
 // in shared memory.  partial must hold [T][N] doubles.
