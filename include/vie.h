@@ -455,8 +455,8 @@ vie_status vie_fft_precondition(vie_handle *h, const double *v, double *z, void 
  *   z = v + D^{-1}(sigma_s v),
  * D^{-1} one geometric-multigrid V-cycle from zero (levels n, n/2, ... while
  * even and above 8; red-black Gauss-Seidel 2 + 2; mean restriction; bilinear
- * prolongation; 200 sweeps on the coarsest grid), FP64, replayed from a CUDA
- * graph.  It works where the diffusion approximation holds and the cells are
+ * prolongation; 200 sweeps on the coarsest grid), FP64, one launch per level
+ * and direction.  It works where the diffusion approximation holds and the cells are
  * optically thin (sigma_t h well below 1); on thick cells the correction can
  * overshoot and the stall fallback takes over.  It replaces any other
  * preconditioner set on the handle.  2D handles; sigma_t > 0 in every cell.

@@ -18,10 +18,27 @@
 // above 8 (coarse mu and mu_s the means of the 2 x 2 children, the operator
 // rediscretised); red-black Gauss-Seidel, 2 sweeps before and after the
 // correction; restriction = mean of the children's residuals; bilinear
-// prolongation in the cell centres; 200 red-black sweeps on the coarsest grid
-// in one CTA.  FP64 (the grids are small).  The V-cycle runs on fixed
-// buffers, so it is captured once into a CUDA graph; an application is the
-// source kernel, the graph and the finishing kernel.
+// prolongation in the cell centres; 200 red-black sweeps on the coarsest
+// grid.  FP64 (the grids are small).
+//
+// One launch per level and direction.  A CTA owns a kTile x kTile tile of the
+// level and keeps it with a halo in shared memory, so that its four colour
+// half-sweeps (and the residual, or the interpolated correction) need no data
+// from other CTAs: every half-sweep updates a region one cell smaller on each
+// side, cells in the halos being recomputed by their neighbours' CTAs with the
+// same arithmetic.  What bounds a level is launch latency and the SM's narrow
+// FP64 pipe (tile 16: 2.2 times the cells in the first half-sweep, but 64 CTAs
+// at 128^2; tile 32 leaves 16 CTAs with three times the work each).  A launch
+// per colour (50 in a graph) took 2.3 us each, 100 us per V-cycle at 128^2.
+//
+// The coarsest grid's sweeps from zero are a fixed linear map f -> u.  Up to
+// kMapCells cells it is set up as a matrix (the sweeps applied to the unit
+// vectors, once per medium) and applied as one product: 200 sweeps in one CTA
+// took 160 us of each V-cycle at 128^2 (an 8 x 8 grid).  Larger coarsest grids
+// (odd sizes of 27 and more) run the sweeps on tiles, kCoarseSweeps / 4
+// launches of four.
+// Measured at 128^2 (five levels): 40 us per V-cycle in 9 launches; 265 us
+// in 50 before.
 #include <math.h>
 
 #include <algorithm>
@@ -33,8 +50,10 @@ namespace vie {
 
 namespace {
 
-constexpr int kPre = 2, kPost = 2, kCoarseSweeps = 200;
+constexpr int kCoarseSweeps = 200;
 constexpr int kT = 256;
+constexpr int kTile = 16;        // tile side of the smoothing kernels (even: colours and children align)
+constexpr int kMapCells = 625;   // largest coarsest grid (25 x 25) kept as a matrix: 3.1 MB, set up in < 1 ms
 
 __device__ __forceinline__ double neighbour_sum(const double *__restrict__ c, const double *__restrict__ u, int n,
                                                long N, int ix, int iy, long j) {
@@ -46,68 +65,184 @@ __device__ __forceinline__ double neighbour_sum(const double *__restrict__ c, co
   return s;
 }
 
-// one colour of a red-black Gauss-Seidel sweep (red: ix + iy even); plane 5
-// of c holds 1 / diag
-__global__ void k_dp_rbgs(int n, const double *__restrict__ c, const double *__restrict__ f, double *__restrict__ u,
-                          int colour) {
+// A CTA's tile with a halo of M cells: local cell (lx, ly) of the S x S
+// region is cell (x0 + lx, y0 + ly) of the level.
+template <int M>
+struct Tile {
+  static constexpr int S = kTile + 2 * M;
+  int n, x0, y0;
+  __device__ __forceinline__ Tile(int n_) : n(n_), x0((int)blockIdx.x * kTile - M), y0((int)blockIdx.y * kTile - M) {}
+  __device__ __forceinline__ bool inside(int x, int y) const { return x >= 0 && x < n && y >= 0 && y < n; }
+  // the coupled neighbours of local cell l, in neighbour_sum's order
+  __device__ __forceinline__ double sum(const double *__restrict__ c, const double *U, int x, int y, int l) const {
+    const long N = (long)n * n, j = (long)y * n + x;
+    double s = 0.0;
+    if (x > 0) s += c[N + j] * U[l - 1];
+    if (x < n - 1) s += c[2 * N + j] * U[l + 1];
+    if (y > 0) s += c[3 * N + j] * U[l - S];
+    if (y < n - 1) s += c[4 * N + j] * U[l + S];
+    return s;
+  }
+  // one colour of a red-black Gauss-Seidel sweep (red: x + y even) on the
+  // cells at least `m` from the region's edge; plane 5 of c holds 1 / diag
+  __device__ __forceinline__ void half_sweep(const double *__restrict__ c, const double *F, double *U, int colour,
+                                             int m) const {
+    const int w = S - 2 * m, half = (w + 1) / 2;
+    for (int i = threadIdx.x; i < w * half; i += kT) {
+      const int ly = m + i / half, first = (x0 + m + y0 + ly + colour) & 1;
+      const int lx = m + 2 * (i % half) + first;
+      const int x = x0 + lx, y = y0 + ly;
+      if (lx >= S - m || !inside(x, y)) continue;
+      const int l = ly * S + lx;
+      U[l] = (F[l] + sum(c, U, x, y, l)) * c[5L * n * n + (long)y * n + x];
+    }
+    __syncthreads();
+  }
+};
+
+// Down: two sweeps from zero, u, and f_coarse = mean over the 2 x 2 children
+// of the residual f - D u.  Finest level: f = ss v (f null).
+__global__ void __launch_bounds__(kT) k_dp_down(int n, const double *__restrict__ c, const double *__restrict__ f,
+                                                const double *__restrict__ ss, const double *__restrict__ v,
+                                                double *__restrict__ u, double *__restrict__ fc) {
+  using T = Tile<4>;
+  __shared__ double F[T::S * T::S], U[T::S * T::S], R[kTile * kTile];
+  const T t(n);
   const long N = (long)n * n;
-  for (long j = blockIdx.x * (long)blockDim.x + threadIdx.x; j < N; j += (long)gridDim.x * blockDim.x) {
-    const int ix = (int)(j % n), iy = (int)(j / n);
-    if (((ix + iy) & 1) != colour) continue;
-    u[j] = (f[j] + neighbour_sum(c, u, n, N, ix, iy, j)) * c[5 * N + j];
+  for (int l = threadIdx.x; l < T::S * T::S; l += kT) {
+    const int x = t.x0 + l % T::S, y = t.y0 + l / T::S;
+    double fl = 0.0, ul = 0.0;
+    if (t.inside(x, y)) {
+      const long j = (long)y * n + x;
+      fl = f ? f[j] : ss[j] * v[j];
+      if (((x + y) & 1) == 0) ul = fl * c[5 * N + j];  // the first red half-sweep: all neighbours still zero
+    }
+    F[l] = fl;
+    U[l] = ul;
+  }
+  __syncthreads();
+  t.half_sweep(c, F, U, 1, 1);
+  t.half_sweep(c, F, U, 0, 2);
+  t.half_sweep(c, F, U, 1, 3);
+  static_assert(kTile * kTile == kT, "one thread per cell of the tile");
+  {
+    const int lx = 4 + threadIdx.x % kTile, ly = 4 + threadIdx.x / kTile, l = ly * T::S + lx;
+    const int x = t.x0 + lx, y = t.y0 + ly;
+    double r = 0.0;
+    if (t.inside(x, y)) {
+      const long j = (long)y * n + x;
+      u[j] = U[l];
+      r = F[l] - (c[j] * U[l] - t.sum(c, U, x, y, l));
+    }
+    R[threadIdx.x] = r;
+  }
+  __syncthreads();
+  constexpr int H = kTile / 2;
+  if (threadIdx.x < H * H) {
+    const int a = threadIdx.x % H, b = threadIdx.x / H, nc = n / 2;
+    const int I = (int)blockIdx.x * H + a, J = (int)blockIdx.y * H + b;
+    const double *q = R + 2 * b * kTile + 2 * a;
+    if (I < nc && J < nc) fc[(long)J * nc + I] = 0.25 * (q[0] + q[1] + q[kTile] + q[kTile + 1]);
   }
 }
 
-// f_coarse = mean over the 2 x 2 children of the fine residual f - D u
-__global__ void k_dp_restrict(int n, const double *__restrict__ c, const double *__restrict__ f,
-                              const double *__restrict__ u, double *__restrict__ fc) {
+// Up: u plus the bilinear interpolation of the coarse correction e (a
+// neighbour outside the coarse grid replaced by the coarse cell itself), then
+// two sweeps, into w.  Finest level: f = ss v (f null) and w = v + the result.
+__global__ void __launch_bounds__(kT) k_dp_up(int n, const double *__restrict__ c, const double *__restrict__ f,
+                                              const double *__restrict__ ss, const double *__restrict__ v,
+                                              const double *__restrict__ u, const double *__restrict__ e,
+                                              double *__restrict__ w) {
+  using T = Tile<4>;
+  __shared__ double F[T::S * T::S], U[T::S * T::S];
+  const T t(n);
   const int nc = n / 2;
-  const long N = (long)n * n, Nc = (long)nc * nc;
-  for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < Nc; t += (long)gridDim.x * blockDim.x) {
-    const int I = (int)(t % nc), J = (int)(t / nc);
-    double acc = 0.0;
-    for (int b = 0; b < 2; ++b)
-      for (int a = 0; a < 2; ++a) {
-        const int ix = 2 * I + a, iy = 2 * J + b;
-        const long j = (long)iy * n + ix;
-        acc += f[j] - (c[j] * u[j] - neighbour_sum(c, u, n, N, ix, iy, j));
-      }
-    fc[t] = 0.25 * acc;
+  for (int l = threadIdx.x; l < T::S * T::S; l += kT) {
+    const int x = t.x0 + l % T::S, y = t.y0 + l / T::S;
+    double fl = 0.0, ul = 0.0;
+    if (t.inside(x, y)) {
+      const long j = (long)y * n + x;
+      fl = f ? f[j] : ss[j] * v[j];
+      const int I = x >> 1, J = y >> 1;
+      const int I2 = (x & 1) ? min(I + 1, nc - 1) : max(I - 1, 0);
+      const int J2 = (y & 1) ? min(J + 1, nc - 1) : max(J - 1, 0);
+      ul = u[j] + (9.0 * e[(long)J * nc + I] + 3.0 * e[(long)J * nc + I2] + 3.0 * e[(long)J2 * nc + I] +
+                   e[(long)J2 * nc + I2]) / 16.0;
+    }
+    F[l] = fl;
+    U[l] = ul;
+  }
+  __syncthreads();
+  t.half_sweep(c, F, U, 0, 1);
+  t.half_sweep(c, F, U, 1, 2);
+  t.half_sweep(c, F, U, 0, 3);
+  t.half_sweep(c, F, U, 1, 4);
+  const int lx = 4 + threadIdx.x % kTile, ly = 4 + threadIdx.x / kTile;
+  const int x = t.x0 + lx, y = t.y0 + ly;
+  if (t.inside(x, y)) {
+    const long j = (long)y * n + x;
+    const double r = U[ly * T::S + lx];
+    w[j] = f ? r : v[j] + r;
   }
 }
 
-// u_fine += bilinear interpolation of the coarse correction (a neighbour
-// outside the coarse grid replaced by the coarse cell itself)
-__global__ void k_dp_prolong(int nc, const double *__restrict__ e, double *__restrict__ u) {
-  const int n = 2 * nc;
-  const long N = (long)n * n;
-  for (long j = blockIdx.x * (long)blockDim.x + threadIdx.x; j < N; j += (long)gridDim.x * blockDim.x) {
-    const int fx = (int)(j % n), fy = (int)(j / n);
-    const int I = fx >> 1, J = fy >> 1;
-    const int I2 = (fx & 1) ? min(I + 1, nc - 1) : max(I - 1, 0);
-    const int J2 = (fy & 1) ? min(J + 1, nc - 1) : max(J - 1, 0);
-    u[j] += (9.0 * e[(long)J * nc + I] + 3.0 * e[(long)J * nc + I2] + 3.0 * e[(long)J2 * nc + I] +
-             e[(long)J2 * nc + I2]) / 16.0;
+// Four sweeps on a large coarsest grid: u (null: zero) -> w.
+__global__ void __launch_bounds__(kT) k_dp_sweeps(int n, const double *__restrict__ c, const double *__restrict__ f,
+                                                  const double *__restrict__ u, double *__restrict__ w) {
+  using T = Tile<8>;
+  __shared__ double F[T::S * T::S], U[T::S * T::S];
+  const T t(n);
+  for (int l = threadIdx.x; l < T::S * T::S; l += kT) {
+    const int x = t.x0 + l % T::S, y = t.y0 + l / T::S;
+    const bool in = t.inside(x, y);
+    const long j = (long)y * n + x;
+    F[l] = in ? f[j] : 0.0;
+    U[l] = in && u ? u[j] : 0.0;
   }
+  __syncthreads();
+  for (int s = 0; s < 8; ++s) t.half_sweep(c, F, U, s & 1, s + 1);
+  const int lx = 8 + threadIdx.x % kTile, ly = 8 + threadIdx.x / kTile;
+  const int x = t.x0 + lx, y = t.y0 + ly;
+  if (t.inside(x, y)) w[(long)y * n + x] = U[ly * T::S + lx];
 }
 
-__global__ void k_dp_zero(long N, double *__restrict__ u) {
-  for (long j = blockIdx.x * (long)blockDim.x + threadIdx.x; j < N; j += (long)gridDim.x * blockDim.x) u[j] = 0.0;
-}
-
-// the coarsest grid: zero guess, kCoarseSweeps red-black sweeps, one CTA
-__global__ void k_dp_coarse(int n, const double *__restrict__ c, const double *__restrict__ f, double *__restrict__ u) {
-  const long N = (long)n * n;
+// The coarsest grid's map, column by column: CTA k runs kCoarseSweeps
+// red-black sweeps from zero on the unit vector of cell k into G[k][.].
+__global__ void k_dp_coarse_map(int n, const double *__restrict__ c, double *__restrict__ G) {
+  const long N = (long)n * n, k = blockIdx.x;
+  double *u = G + k * N;
   for (long j = threadIdx.x; j < N; j += blockDim.x) u[j] = 0.0;
   __syncthreads();
   for (int s = 0; s < kCoarseSweeps; ++s)
     for (int colour = 0; colour < 2; ++colour) {
       for (long j = threadIdx.x; j < N; j += blockDim.x) {
         const int ix = (int)(j % n), iy = (int)(j / n);
-        if (((ix + iy) & 1) == colour) u[j] = (f[j] + neighbour_sum(c, u, n, N, ix, iy, j)) * c[5 * N + j];
+        if (((ix + iy) & 1) == colour)
+          u[j] = ((j == k ? 1.0 : 0.0) + neighbour_sum(c, u, n, N, ix, iy, j)) * c[5 * N + j];
       }
       __syncthreads();
     }
+}
+
+// u = sum_k f_k G[k][.]: a CTA takes 32 cells, its 8 warps every 8th k, and
+// warp 0 adds the warps' sums in order.  f = ss v and u = v + the result where
+// the coarsest grid is the only one (f null).
+__global__ void __launch_bounds__(kT) k_dp_coarse(int N, const double *__restrict__ G, const double *__restrict__ f,
+                                                  const double *__restrict__ ss, const double *__restrict__ v,
+                                                  double *__restrict__ u) {
+  __shared__ double part[kT];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, j = blockIdx.x * 32 + lane;
+  double s = 0.0;
+  if (j < N) {
+#pragma unroll 4
+    for (int k = warp; k < N; k += kT / 32) s += (f ? f[k] : ss[k] * v[k]) * G[(long)k * N + j];
+  }
+  part[threadIdx.x] = s;
+  __syncthreads();
+  if (warp == 0 && j < N) {
+    for (int q = 1; q < kT / 32; ++q) s += part[q * 32 + lane];
+    u[j] = f ? s : v[j] + s;
+  }
 }
 
 __global__ void k_dp_source(long N, const double *__restrict__ ss, const double *__restrict__ v,
@@ -151,40 +286,6 @@ void level_coefficients(int n, const std::vector<double> &mu, const std::vector<
     }
 }
 
-// the V-cycle on the level buffers (kernels only; captured into the graph)
-cudaError_t enqueue_vcycle(const DiffPre &dp, cudaStream_t st, int *kernels) {
-  const DiffLevel *lv = dp.lv;
-  const int L = dp.L;
-  int k = 0;
-  for (int l = 0; l + 1 < L; ++l) {
-    const long N = (long)lv[l].n * lv[l].n;
-    k_dp_zero<<<blocks_for(N), kT, 0, st>>>(N, lv[l].u);
-    ++k;
-    for (int s = 0; s < kPre; ++s)
-      for (int colour = 0; colour < 2; ++colour, ++k)
-        k_dp_rbgs<<<blocks_for(N), kT, 0, st>>>(lv[l].n, lv[l].c, lv[l].f, lv[l].u, colour);
-    k_dp_restrict<<<blocks_for(N / 4), kT, 0, st>>>(lv[l].n, lv[l].c, lv[l].f, lv[l].u, lv[l + 1].f);
-    ++k;
-  }
-  {
-    // one CTA just large enough for the coarsest grid: its barriers stay cheap
-    const long Nc = (long)lv[L - 1].n * lv[L - 1].n;
-    const int threads = (int)std::min(1024L, std::max(32L, (Nc + 31) / 32 * 32));
-    k_dp_coarse<<<1, threads, 0, st>>>(lv[L - 1].n, lv[L - 1].c, lv[L - 1].f, lv[L - 1].u);
-  }
-  ++k;
-  for (int l = L - 2; l >= 0; --l) {
-    const long N = (long)lv[l].n * lv[l].n;
-    k_dp_prolong<<<blocks_for(N), kT, 0, st>>>(lv[l + 1].n, lv[l + 1].u, lv[l].u);
-    ++k;
-    for (int s = 0; s < kPost; ++s)
-      for (int colour = 0; colour < 2; ++colour, ++k)
-        k_dp_rbgs<<<blocks_for(N), kT, 0, st>>>(lv[l].n, lv[l].c, lv[l].f, lv[l].u, colour);
-  }
-  *kernels = k;
-  return cudaGetLastError();
-}
-
 }  // namespace
 
 vie_status diffusion_prepare(DiffPre *dp, int n, const double *sigma_t, const double *sigma_s,
@@ -209,6 +310,7 @@ vie_status diffusion_prepare(DiffPre *dp, int n, const double *sigma_t, const do
     VIE_CUDA(vie_malloc((void **)&L.c, sizeof(double) * 6 * M));
     VIE_CUDA(vie_malloc((void **)&L.f, sizeof(double) * M));
     VIE_CUDA(vie_malloc((void **)&L.u, sizeof(double) * M));
+    VIE_CUDA(vie_malloc((void **)&L.w, sizeof(double) * M));
     VIE_CUDA(cudaMemcpyAsync(L.c, c.data(), sizeof(double) * 6 * M, cudaMemcpyHostToDevice, st));
     VIE_CUDA(cudaStreamSynchronize(st));
     if (ln % 2 || ln <= 8 || dp->L == kDiffMaxLevels) break;
@@ -226,45 +328,67 @@ vie_status diffusion_prepare(DiffPre *dp, int n, const double *sigma_t, const do
   }
   dp->ss = sigma_s_dev;
   dp->n = n;
-  // the V-cycle as a graph on a private capture stream
-  VIE_CUDA(cudaStreamCreateWithFlags(&dp->cap, cudaStreamNonBlocking));
-  VIE_CUDA(cudaStreamBeginCapture(dp->cap, cudaStreamCaptureModeThreadLocal));
-  int kernels = 0;
-  const cudaError_t ek = enqueue_vcycle(*dp, dp->cap, &kernels);
-  cudaGraph_t graph = nullptr;
-  const cudaError_t ec = cudaStreamEndCapture(dp->cap, &graph);
-  if (ek != cudaSuccess || ec != cudaSuccess) {
-    if (graph) cudaGraphDestroy(graph);
-    return cuda_fail(ek != cudaSuccess ? ek : ec, "diffusion V-cycle capture");
+  const DiffLevel &C = dp->lv[dp->L - 1];
+  const int Nc = C.n * C.n;
+  if (Nc <= kMapCells) {
+    VIE_CUDA(vie_malloc((void **)&dp->map, sizeof(double) * (size_t)Nc * Nc));
+    k_dp_coarse_map<<<Nc, (Nc + 31) / 32 * 32, 0, st>>>(C.n, C.c, dp->map);
+    VIE_CHECK_LAUNCH("k_dp_coarse_map");
   }
-  dp->graph = graph;
-  VIE_CUDA(cudaGraphInstantiate(&dp->exec, graph, 0));
-  dp->graph_kernels = kernels;
   dp->on = 1;
   return VIE_OK;
 }
 
 void diffusion_release(DiffPre *dp) {
-  if (dp->exec) cudaGraphExecDestroy(dp->exec);
-  if (dp->graph) cudaGraphDestroy(dp->graph);
-  if (dp->cap) cudaStreamDestroy(dp->cap);
+  if (dp->map) vie_free(dp->map);
   for (int l = 0; l < dp->L; ++l) {
     if (dp->lv[l].c) vie_free(dp->lv[l].c);
     if (dp->lv[l].f) vie_free(dp->lv[l].f);
     if (dp->lv[l].u) vie_free(dp->lv[l].u);
+    if (dp->lv[l].w) vie_free(dp->lv[l].w);
   }
   *dp = DiffPre{};
 }
 
 vie_status diffusion_precondition(const DiffPre &dp, const double *v, double *z, cudaStream_t st) {
   const DiffLevel *lv = dp.lv;
-  const long N = (long)dp.n * dp.n;
-  k_dp_source<<<blocks_for(N), kT, 0, st>>>(N, dp.ss, v, lv[0].f);
-  VIE_CHECK_LAUNCH("k_dp_source");
-  VIE_CUDA(cudaGraphLaunch(dp.exec, st));
-  for (int i = 0; i < dp.graph_kernels; ++i) count_launch();
-  k_dp_finish<<<blocks_for(N), kT, 0, st>>>(N, v, lv[0].u, z);
-  VIE_CHECK_LAUNCH("k_dp_finish");
+  const int L = dp.L;
+  auto tiles = [](int n) { return dim3((unsigned)((n + kTile - 1) / kTile), (unsigned)((n + kTile - 1) / kTile)); };
+  for (int l = 0; l + 1 < L; ++l) {
+    k_dp_down<<<tiles(lv[l].n), kT, 0, st>>>(lv[l].n, lv[l].c, l ? lv[l].f : nullptr, dp.ss, v, lv[l].u,
+                                             lv[l + 1].f);
+    VIE_CHECK_LAUNCH("k_dp_down");
+  }
+  const DiffLevel &C = lv[L - 1];
+  const int Nc = C.n * C.n;
+  const double *e = C.u;  // the level's result, read by the level above
+  if (dp.map) {
+    k_dp_coarse<<<(Nc + 31) / 32, kT, 0, st>>>(Nc, dp.map, L > 1 ? C.f : nullptr, dp.ss, v, L > 1 ? C.u : z);
+    VIE_CHECK_LAUNCH("k_dp_coarse");
+    if (L == 1) return VIE_OK;
+  } else {
+    if (L == 1) {
+      k_dp_source<<<blocks_for(Nc), kT, 0, st>>>(Nc, dp.ss, v, C.f);
+      VIE_CHECK_LAUNCH("k_dp_source");
+    }
+    for (int s = 0; s < kCoarseSweeps; s += 4) {
+      double *out = (s / 4) % 2 ? C.w : C.u;
+      k_dp_sweeps<<<tiles(C.n), kT, 0, st>>>(C.n, C.c, C.f, s ? e : nullptr, out);
+      VIE_CHECK_LAUNCH("k_dp_sweeps");
+      e = out;
+    }
+    if (L == 1) {
+      k_dp_finish<<<blocks_for(Nc), kT, 0, st>>>(Nc, v, e, z);
+      VIE_CHECK_LAUNCH("k_dp_finish");
+      return VIE_OK;
+    }
+  }
+  for (int l = L - 2; l >= 0; --l) {
+    double *out = l ? lv[l].w : z;
+    k_dp_up<<<tiles(lv[l].n), kT, 0, st>>>(lv[l].n, lv[l].c, l ? lv[l].f : nullptr, dp.ss, v, lv[l].u, e, out);
+    VIE_CHECK_LAUNCH("k_dp_up");
+    e = out;
+  }
   return VIE_OK;
 }
 

@@ -279,15 +279,14 @@ struct DiffLevel {
   int n = 0;
   double *c = nullptr;  // [6][n * n]: diagonal, the west, east, south, north couplings, 1 / diagonal
   double *f = nullptr;  // right-hand side of this level
-  double *u = nullptr;  // its V-cycle iterate (level 0: the correction D^{-1}(sigma_s r))
+  double *u = nullptr;  // its iterate after the first smoothing
+  double *w = nullptr;  // its result (level 0 writes the caller's z instead)
 };
 struct DiffPre {
-  int on = 0, n = 0, L = 0, graph_kernels = 0;
+  int on = 0, n = 0, L = 0;
   const double *ss = nullptr;  // sigma_s on the device (the handle's)
   DiffLevel lv[kDiffMaxLevels];
-  cudaStream_t cap = nullptr;
-  cudaGraph_t graph = nullptr;
-  cudaGraphExec_t exec = nullptr;
+  double *map = nullptr;  // the coarsest grid's sweeps as a matrix [cell k of f][cell of u]; null: too large
 };
 // sigma_t, sigma_s: host FP64 [n * n] (sigma_t > 0); sigma_s_dev stays the caller's
 vie_status diffusion_prepare(DiffPre *dp, int n, const double *sigma_t, const double *sigma_s,
