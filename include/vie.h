@@ -266,8 +266,7 @@ typedef struct {
  * each.  Each solve keeps its own restart cycles, residual estimate, stall
  * fallback and FP64 true residual, and leaves the lockstep when it
  * converges (its report counts its own steps).
- * The call synchronises the stream once per Arnoldi step (residual test; one
- * copy of all nrhs estimates).  Returns NOT_CONVERGED (U and rep valid) when
+ * The host waits for every Arnoldi step (residual test).  Returns NOT_CONVERGED (U and rep valid) when
  * maxit is reached (for any source). */
 vie_status vie_solve_gmres(vie_handle *h, const double *f, double *U,
                            const vie_gmres_opts *o, vie_report *rep, void *stream);

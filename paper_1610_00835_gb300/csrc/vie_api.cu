@@ -180,9 +180,11 @@ struct vie_handle {
   // GMRES workspace
   int gm_m = 0;
   double *V = nullptr, *phi = nullptr, *r = nullptr, *w = nullptr, *H = nullptr;
-  double *cs = nullptr, *sn = nullptr, *gv = nullptr, *yv = nullptr, *hcol = nullptr;
-  double *htmp = nullptr, *part = nullptr, *scal = nullptr;
+  double *cs = nullptr, *sn = nullptr, *gv = nullptr, *part = nullptr, *scal = nullptr;
   double *h_pinned = nullptr;                 // host-pinned scalars / gv seed
+  double *slots = nullptr;                    // host-pinned result of the last Arnoldi step (KBatch::slots)
+  unsigned *bar = nullptr;                    // grid barrier of the Arnoldi step (zero between launches)
+  unsigned long long step_seq = 0;            // sequence number of the last Arnoldi step launched
   // apply timing
   bool opts_disable_sym = false;              // force the general kernel (tests)
   // assembled operator
@@ -195,7 +197,7 @@ struct vie_handle {
   DBuf<float> g32;                            // FP32 copy of a right-hand side
   DBuf<unsigned char> gemm_ws;                // split-K partials + BF16 G
   int *dev_err = nullptr;                     // device error word of the products
-  int *ticket = nullptr;                      // block ticket of the fused dot kernels (0 between launches)
+  int *ticket = nullptr;                      // block ticket of the norms (0 between launches)
   bool sig_s_positive = false;                // phi = K (f / sigma_s) is available
   UnetImpl *precond = nullptr;                // learned right preconditioner
   double precond_inv_ref = 0.2;
@@ -223,11 +225,10 @@ void free_gmres(vie_handle *h) {
   dfree(h->cs);
   dfree(h->sn);
   dfree(h->gv);
-  dfree(h->yv);
-  dfree(h->hcol);
-  dfree(h->htmp);
   dfree(h->part);
   dfree(h->scal);
+  if (h->slots) vie_free_host(h->slots);
+  h->slots = nullptr;
   if (h->h_pinned) vie_free_host(h->h_pinned);
   h->h_pinned = nullptr;
   h->gm_m = 0;
@@ -235,14 +236,15 @@ void free_gmres(vie_handle *h) {
 
 void free_multi(MultiGmres &g) {
   KBatch &b = g.kb;
-  for (double **p : {&g.V, &g.Z, &g.phi, &g.r, &g.w, &b.H, &b.cs, &b.sn, &b.gv, &b.yv, &b.hcol, &b.htmp, &b.part,
-                     &b.scal, &b.bnorm})
+  for (double **p : {&g.V, &g.Z, &g.phi, &g.r, &g.w, &b.H, &b.cs, &b.sn, &b.gv, &b.hcol, &b.htmp, &b.part, &b.scal,
+                     &b.inv_bnorm})
     dfree(*p);
   for (int **p : {&b.ticket, &b.act, &g.kk}) dfree(*p);
   dfree(g.net_x);
   if (g.h_scal) vie_free_host(g.h_scal);
   if (g.h_gv) vie_free_host(g.h_gv);
   if (g.h_act) vie_free_host(g.h_act);
+  if (b.slots) vie_free_host(b.slots);
   g = MultiGmres{};
 }
 
@@ -275,6 +277,7 @@ void free_all(vie_handle *h) {
   h->gemm_ws.release();
   dfree(h->dev_err);
   dfree(h->ticket);
+  dfree(h->bar);
   sym_release(&h->sym);
   disp_release(&h->disp);
   fft_release(&h->fft);
@@ -305,16 +308,19 @@ vie_status ensure_gmres(vie_handle *h, int m) {
   if ((s = dalloc(&h->cs, m)) != VIE_OK) return s;
   if ((s = dalloc(&h->sn, m)) != VIE_OK) return s;
   if ((s = dalloc(&h->gv, m + 1)) != VIE_OK) return s;
-  if ((s = dalloc(&h->yv, m)) != VIE_OK) return s;
-  if ((s = dalloc(&h->hcol, m + 1)) != VIE_OK) return s;
-  if ((s = dalloc(&h->htmp, m + 1)) != VIE_OK) return s;
-  if ((s = dalloc(&h->part, (size_t)blocks * (m + 1))) != VIE_OK) return s;
+  if ((s = dalloc(&h->part, (size_t)2 * blocks * (m + 1))) != VIE_OK) return s;
   if ((s = dalloc(&h->scal, 8)) != VIE_OK) return s;
   if (!h->ticket) {
     if ((s = dalloc(&h->ticket, 1)) != VIE_OK) return s;
     VIE_CUDA(cudaMemset(h->ticket, 0, sizeof(int)));
   }
+  if (!h->bar) {
+    if ((s = dalloc(&h->bar, 2)) != VIE_OK) return s;
+    VIE_CUDA(cudaMemset(h->bar, 0, 2 * sizeof(unsigned)));
+  }
   VIE_CUDA(vie_malloc_host((void **)&h->h_pinned, sizeof(double) * (m + 1 + 8)));
+  VIE_CUDA(vie_malloc_host((void **)&h->slots, sizeof(double) * 4));
+  memset(h->slots, 0, sizeof(double) * 4);  // the buffer may come from an earlier solver
   h->gm_m = m;
   return VIE_OK;
 }
@@ -454,12 +460,27 @@ vie_status apply_dev(vie_handle *h, int op, const double *g, double *y, cudaStre
   return VIE_OK;
 }
 
-// ||x||^2 into dev scalar *out (part: dot partials buffer).
-vie_status norm2_dev(vie_handle *h, const double *x, double *out, cudaStream_t st) {
-  const int blocks = dot_blocks(h->N);
-  vie_status s = launch_dots(x, 1, h->N, x, h->N, h->part, blocks, st);
-  if (s != VIE_OK) return s;
-  return launch_dots_finish(h->part, blocks, 1, out, 0, st);
+// the single solve's arrays for GMRES(m), as the Krylov kernels take them
+KBatch single_batch(const vie_handle *h, int m) {
+  KBatch b{};
+  b.H = h->H;
+  b.cs = h->cs;
+  b.sn = h->sn;
+  b.gv = h->gv;
+  b.part = h->part;
+  b.scal = h->scal;
+  b.slots = h->slots;
+  b.ticket = h->ticket;
+  b.N = h->N;
+  b.m = m;
+  b.R = 1;
+  b.blocks = dot_blocks(h->N);
+  return b;
+}
+
+// ||x||^2 into h->scal[slot]
+vie_status norm2_dev(vie_handle *h, int m, const double *x, int slot, cudaStream_t st) {
+  return launch_bnorm2(single_batch(h, m), x, h->N, slot, st);
 }
 
 // Device error words of the handle's tensor-core kernels (the product's and
@@ -494,10 +515,44 @@ vie_status read_scalar(vie_handle *h, const double *dev, double *val, cudaStream
   return take_errors(h, st);
 }
 
-bool all_finite(const double *a, long n) {
-  for (long i = 0; i < n; ++i)
-    if (!isfinite(a[i])) return false;
-  return true;
+// Wait for the Arnoldi step `seq` of every right-hand side with act[r] != 0
+// (act null: one): the kernel writes each slot's sequence number last.  The
+// host polls pinned memory; the stream is asked now and then, so that a failed
+// launch ends the wait.
+vie_status wait_slots(vie_handle *h, const double *slots, int R, const int *act, unsigned long long seq,
+                      cudaStream_t st) {
+  bool gave_up = false;
+  int e0 = 0, e1 = 0;
+  for (int r = 0; r < R; ++r) {
+    if (act && !act[r]) continue;
+    const unsigned long long *q = reinterpret_cast<const unsigned long long *>(slots + 4 * r + 3);
+    for (long spin = 1; __atomic_load_n(q, __ATOMIC_ACQUIRE) != seq; ++spin) {
+      if (spin % 4096) continue;
+      const cudaError_t e = cudaStreamQuery(st);
+      if (e == cudaErrorNotReady) continue;
+      if (e != cudaSuccess) return cuda_fail(e, "vie_solve_gmres: Arnoldi step");
+      if (__atomic_load_n(q, __ATOMIC_ACQUIRE) == seq) break;
+      set_error("vie_solve_gmres: the Arnoldi step ended without a result");
+      return VIE_ERR_CUDA;
+    }
+    const int *he = reinterpret_cast<const int *>(slots + 4 * r + 1);
+    e0 |= he[0];
+    e1 |= he[1];
+    gave_up = gave_up || he[2] != 0;
+  }
+  if (e0 || e1) {
+    vie_status s = queue_errors(h, st);
+    if (s != VIE_OK) return s;
+    VIE_CUDA(cudaStreamSynchronize(st));
+    return take_errors(h, st);
+  }
+  if (gave_up) {
+    VIE_CUDA(cudaStreamSynchronize(st));
+    VIE_CUDA(cudaMemset(h->bar, 0, 2 * sizeof(unsigned)));
+    set_error("vie_solve_gmres: a bounded device wait of the Arnoldi step ran out");
+    return VIE_ERR_TIMEOUT;
+  }
+  return VIE_OK;
 }
 
 vie_status ensure_multi(vie_handle *h, int R, int m, bool need_z, bool need_net) {
@@ -517,12 +572,11 @@ vie_status ensure_multi(vie_handle *h, int R, int m, bool need_z, bool need_net)
   if ((s = dalloc(&b.cs, (size_t)R * m)) != VIE_OK) return s;
   if ((s = dalloc(&b.sn, (size_t)R * m)) != VIE_OK) return s;
   if ((s = dalloc(&b.gv, (size_t)R * (m + 1))) != VIE_OK) return s;
-  if ((s = dalloc(&b.yv, (size_t)R * m)) != VIE_OK) return s;
   if ((s = dalloc(&b.hcol, (size_t)R * (m + 1))) != VIE_OK) return s;
   if ((s = dalloc(&b.htmp, (size_t)R * (m + 1))) != VIE_OK) return s;
-  if ((s = dalloc(&b.part, (size_t)R * blocks * (m + 1))) != VIE_OK) return s;
+  if ((s = dalloc(&b.part, (size_t)2 * R * blocks * (m + 1))) != VIE_OK) return s;
   if ((s = dalloc(&b.scal, (size_t)R * 8)) != VIE_OK) return s;
-  if ((s = dalloc(&b.bnorm, (size_t)R)) != VIE_OK) return s;
+  if ((s = dalloc(&b.inv_bnorm, (size_t)R)) != VIE_OK) return s;
   if ((s = dalloc(&b.ticket, (size_t)R)) != VIE_OK) return s;
   if ((s = dalloc(&b.act, (size_t)R)) != VIE_OK) return s;
   if ((s = dalloc(&g.kk, (size_t)R)) != VIE_OK) return s;
@@ -531,6 +585,8 @@ vie_status ensure_multi(vie_handle *h, int R, int m, bool need_z, bool need_net)
   VIE_CUDA(vie_malloc_host((void **)&g.h_scal, sizeof(double) * 8 * R));
   VIE_CUDA(vie_malloc_host((void **)&g.h_gv, sizeof(double) * (size_t)R * (m + 1)));
   VIE_CUDA(vie_malloc_host((void **)&g.h_act, sizeof(int) * 2 * R));
+  VIE_CUDA(vie_malloc_host((void **)&b.slots, sizeof(double) * 4 * R));
+  memset(b.slots, 0, sizeof(double) * 4 * R);
   g.R = R;
   g.m = m;
   g.has_z = need_z;
@@ -658,26 +714,28 @@ vie_status solve_multi(vie_handle *h, const double *fdev, double *x, int R, cons
       conv[r] = 1;
     }
   }
-  VIE_CUDA(cudaMemcpyAsync(b.bnorm, bnorm.data(), sizeof(double) * R, cudaMemcpyHostToDevice, st));
+  std::vector<double> inv_bnorm(R);
+  for (int r = 0; r < R; ++r) inv_bnorm[r] = bnorm[r] > 0.0 ? 1.0 / bnorm[r] : 0.0;
+  VIE_CUDA(cudaMemcpyAsync(b.inv_bnorm, inv_bnorm.data(), sizeof(double) * R, cudaMemcpyHostToDevice, st));
   bool x_is_zero = opt.zero_x0 != 0;
   for (;;) {
     for (int r = 0; r < R; ++r) act[r] = !conv[r] && !done[r];
     if (std::none_of(act.begin(), act.end(), [](int a) { return a != 0; })) break;
     if ((s = upload_act(h, act, st)) != VIE_OK) return s;
-    // true residuals r = phi - (I - K) x
-    if (x_is_zero) {
-      VIE_CUDA(cudaMemcpyAsync(g.r, g.phi, sizeof(double) * R * N, cudaMemcpyDeviceToDevice, st));
-    } else {
+    // true residuals r = phi - (I - K) x; phi itself (its norms are known) at x = 0
+    const double *res = x_is_zero ? g.phi : g.r;
+    const int res_slot = x_is_zero ? 0 : 1;
+    if (!x_is_zero) {
       if ((s = apply_multi(h, VIE_OP_I_MINUS_K, x, N, g.w, N, R, act.data(), st, timed)) != VIE_OK) return s;
       for (int r = 0; r < R; ++r) napply[r] += act[r];
       if ((s = launch_baxpby(b, 1.0, g.phi, N, -1.0, g.w, N, g.r, N, st)) != VIE_OK) return s;
+      if ((s = launch_bnorm2(b, g.r, N, 1, st)) != VIE_OK) return s;
+      if ((s = read_multi_scal(h, R, st)) != VIE_OK) return s;
     }
     x_is_zero = false;
-    if ((s = launch_bnorm2(b, g.r, N, 1, st)) != VIE_OK) return s;
-    if ((s = read_multi_scal(h, R, st)) != VIE_OK) return s;
     for (int r = 0; r < R; ++r) {
       if (!act[r]) continue;
-      const double rn2 = g.h_scal[8 * r + 1];
+      const double rn2 = g.h_scal[8 * r + res_slot];
       if (!isfinite(rn2)) {
         set_error("vie_solve_gmres: non-finite residual");
         return VIE_ERR_NONFINITE;
@@ -690,11 +748,11 @@ vie_status solve_multi(vie_handle *h, const double *fdev, double *x, int R, cons
     if (std::none_of(act.begin(), act.end(), [](int a) { return a != 0; })) break;
     if ((s = upload_act(h, act, st)) != VIE_OK) return s;
     // V_r0 = r_r / beta_r, gv_r = beta_r e_1
-    if ((s = launch_bscale(b, g.r, N, 1, 1, g.V, ldv, st)) != VIE_OK) return s;
+    if ((s = launch_bscale(b, res, N, res_slot, g.V, ldv, st)) != VIE_OK) return s;
     for (int r = 0; r < R; ++r) {
       double *gv = g.h_gv + (size_t)r * (m + 1);
       for (int i = 0; i <= m; ++i) gv[i] = 0.0;
-      gv[0] = act[r] ? sqrt(g.h_scal[8 * r + 1]) : 0.0;
+      gv[0] = act[r] ? sqrt(g.h_scal[8 * r + res_slot]) : 0.0;
     }
     VIE_CUDA(cudaMemcpyAsync(b.gv, g.h_gv, sizeof(double) * R * (m + 1), cudaMemcpyHostToDevice, st));
     const std::vector<int> cycle = act;  // the solves that take part in this cycle
@@ -748,13 +806,21 @@ vie_status solve_multi(vie_handle *h, const double *fdev, double *x, int R, cons
         return s;
       for (int r = 0; r < R; ++r) napply[r] += act[r];
       // CGS2 (two passes of h = V^T w, w -= V h), the norm and the Givens step
-      if ((s = launch_bdots(b, g.V, ldv, k + 1, vk1, ldv, b.hcol, nullptr, st)) != VIE_OK) return s;
-      if ((s = launch_borth_update(b, g.V, ldv, k + 1, b.hcol, vk1, ldv, st)) != VIE_OK) return s;
-      if ((s = launch_bdots(b, g.V, ldv, k + 1, vk1, ldv, b.htmp, b.hcol, st)) != VIE_OK) return s;
-      if ((s = launch_borth_update(b, g.V, ldv, k + 1, b.htmp, vk1, ldv, st)) != VIE_OK) return s;
-      if ((s = launch_bnorm2_givens(b, vk1, ldv, k, st)) != VIE_OK) return s;
-      if ((s = launch_bscale(b, vk1, ldv, 2, 1, vk1, ldv, st)) != VIE_OK) return s;
-      if ((s = read_multi_scal(h, R, st)) != VIE_OK) return s;
+      if (arnoldi_fused(b)) {
+        const int *err1 = h->precond ? unet_error_word(h->precond) : nullptr;
+        if ((s = launch_arnoldi(b, g.V, ldv, k, 0.0, h->dev_err, err1, ++h->step_seq, nullptr, st)) != VIE_OK)
+          return s;
+        if ((s = wait_slots(h, b.slots, R, act.data(), h->step_seq, st)) != VIE_OK) return s;
+        for (int r = 0; r < R; ++r) g.h_scal[8 * r + 3] = b.slots[4 * r];
+      } else {
+        if ((s = launch_bdots(b, g.V, ldv, k + 1, vk1, ldv, b.hcol, nullptr, st)) != VIE_OK) return s;
+        if ((s = launch_borth_update(b, g.V, ldv, k + 1, b.hcol, vk1, ldv, st)) != VIE_OK) return s;
+        if ((s = launch_bdots(b, g.V, ldv, k + 1, vk1, ldv, b.htmp, b.hcol, st)) != VIE_OK) return s;
+        if ((s = launch_borth_update(b, g.V, ldv, k + 1, b.htmp, vk1, ldv, st)) != VIE_OK) return s;
+        if ((s = launch_bnorm2_givens(b, vk1, ldv, k, st)) != VIE_OK) return s;
+        if ((s = launch_bscale(b, vk1, ldv, 2, vk1, ldv, st)) != VIE_OK) return s;
+        if ((s = read_multi_scal(h, R, st)) != VIE_OK) return s;
+      }
       if (timed && (s = harvest_events(h)) != VIE_OK) return s;
       bool changed = false;
       for (int r = 0; r < R; ++r) {
@@ -787,7 +853,7 @@ vie_status solve_multi(vie_handle *h, const double *fdev, double *x, int R, cons
     for (int r = 0; r < R; ++r) upd[r] = cycle[r] && kk[r] > 0;
     if ((s = upload_act(h, upd, st)) != VIE_OK) return s;
     VIE_CUDA(cudaMemcpyAsync(g.kk, kk.data(), sizeof(int) * R, cudaMemcpyHostToDevice, st));
-    if ((s = launch_bupdate(b, flexible ? g.Z : g.V, flexible ? ldz : ldv, g.kk, x, N, st)) != VIE_OK) return s;
+    if ((s = launch_update(b, flexible ? g.Z : g.V, flexible ? ldz : ldv, -1, g.kk, x, N, st)) != VIE_OK) return s;
     // the cycle's host vectors must outlive the copies above
     VIE_CUDA(cudaStreamSynchronize(st));
     for (int r = 0; r < R; ++r) {
@@ -1486,8 +1552,9 @@ vie_status vie_solve_gmres(vie_handle *h, const double *f, double *U, const vie_
   } else if ((s = apply_dev(h, VIE_OP_A_RAW, fdev, h->phi, st, timed)) != VIE_OK) {
     return s;
   }
+  const KBatch kb = single_batch(h, m);
   double bn2 = 0.0;
-  if ((s = norm2_dev(h, h->phi, h->scal, st)) != VIE_OK) return s;
+  if ((s = norm2_dev(h, m, h->phi, 0, st)) != VIE_OK) return s;
   if ((s = read_scalar(h, h->scal, &bn2, st)) != VIE_OK) return s;
   if (!isfinite(bn2)) {
     set_error("vie_solve_gmres: non-finite right-hand side");
@@ -1502,20 +1569,19 @@ vie_status vie_solve_gmres(vie_handle *h, const double *f, double *U, const vie_
     VIE_CUDA(cudaMemsetAsync(x, 0, sizeof(double) * N, st));
     converged = true;
   }
-  const int blocks = dot_blocks(N);
   bool x_is_zero = opt.zero_x0 != 0;
   while (!converged) {
-    // true residual r = phi - (I - K) x
-    if (x_is_zero) {
-      VIE_CUDA(cudaMemcpyAsync(h->r, h->phi, sizeof(double) * N, cudaMemcpyDeviceToDevice, st));
-    } else {
+    // true residual r = phi - (I - K) x; phi itself (its norm is known) at x = 0
+    const double *res = x_is_zero ? h->phi : h->r;
+    const int res_slot = x_is_zero ? 0 : 1;
+    double rn2 = bn2;
+    if (!x_is_zero) {
       if ((s = apply_dev(h, VIE_OP_I_MINUS_K, x, h->w, st, timed)) != VIE_OK) return s;
       if ((s = launch_axpby(1.0, h->phi, -1.0, h->w, h->r, N, st)) != VIE_OK) return s;
+      if ((s = norm2_dev(h, m, h->r, 1, st)) != VIE_OK) return s;
+      if ((s = read_scalar(h, h->scal + 1, &rn2, st)) != VIE_OK) return s;
     }
     x_is_zero = false;
-    double rn2 = 0.0;
-    if ((s = norm2_dev(h, h->r, h->scal + 1, st)) != VIE_OK) return s;
-    if ((s = read_scalar(h, h->scal + 1, &rn2, st)) != VIE_OK) return s;
     if (!isfinite(rn2)) {
       set_error("vie_solve_gmres: non-finite residual");
       return VIE_ERR_NONFINITE;
@@ -1528,7 +1594,7 @@ vie_status vie_solve_gmres(vie_handle *h, const double *f, double *U, const vie_
     }
     if (R.iters >= opt.maxit) break;
     // V_0 = r / beta, gv = beta e_1
-    if ((s = launch_scale(h->r, h->scal + 1, 1, h->V, N, st)) != VIE_OK) return s;
+    if ((s = launch_scale(res, h->scal + res_slot, h->V, N, st)) != VIE_OK) return s;
     for (int i = 0; i <= m; ++i) h->h_pinned[i] = 0.0;
     h->h_pinned[0] = beta;
     VIE_CUDA(cudaMemcpyAsync(h->gv, h->h_pinned, sizeof(double) * (m + 1), cudaMemcpyHostToDevice, st));
@@ -1549,7 +1615,7 @@ vie_status vie_solve_gmres(vie_handle *h, const double *f, double *U, const vie_
         } else if (h->precond && h->precond_on_diff) {
           // the diffusion preconditioner, then the network's correction of it
           if ((s = diffusion_precondition(h->diff, vk, zk, st)) != VIE_OK) return s;
-          if ((s = norm2_dev(h, vk, h->scal + 4, st)) != VIE_OK) return s;
+          if ((s = norm2_dev(h, m, vk, 4, st)) != VIE_OK) return s;
           if ((s = unet_precondition(h->precond, h->sig_t, h->sig_s, h->precond_inv_ref, vk, h->scal + 4,
                                      h->n, h->net_x, zk, zk, st)) != VIE_OK)
             return s;
@@ -1557,7 +1623,7 @@ vie_status vie_solve_gmres(vie_handle *h, const double *f, double *U, const vie_
           // the diffusion preconditioner (Section 4.4, Eq. EQ:DA)
           if ((s = diffusion_precondition(h->diff, vk, zk, st)) != VIE_OK) return s;
         } else {
-          if ((s = norm2_dev(h, vk, h->scal + 4, st)) != VIE_OK) return s;
+          if ((s = norm2_dev(h, m, vk, 4, st)) != VIE_OK) return s;
           if ((s = unet_precondition(h->precond, h->sig_t, h->sig_s, h->precond_inv_ref, vk, h->scal + 4,
                                      h->n, h->net_x, nullptr, zk, st)) != VIE_OK)
             return s;
@@ -1566,22 +1632,12 @@ vie_status vie_solve_gmres(vie_handle *h, const double *f, double *U, const vie_
         ++R.precond_iters;
       }
       if ((s = apply_dev(h, VIE_OP_I_MINUS_K, op_in, vk1, st, timed)) != VIE_OK) return s;
-      // CGS2: two passes of h = V^T w, w -= V h; hcol accumulates both.
-      // (each dot pass is one launch: its last block sums the block partials)
-      if ((s = launch_dots_last(h->V, k + 1, N, vk1, N, h->part, blocks, h->ticket, h->hcol, nullptr, st)) !=
-          VIE_OK)
+      // CGS2 (two passes of h = V^T w, w -= V h), the norm, the Givens step and the scaling
+      const int *err1 = h->precond ? unet_error_word(h->precond) : nullptr;
+      if ((s = launch_arnoldi(kb, h->V, 0, k, 1.0 / bnorm, h->dev_err, err1, ++h->step_seq, h->bar, st)) != VIE_OK)
         return s;
-      if ((s = launch_orth_update(h->V, k + 1, N, h->hcol, vk1, N, st)) != VIE_OK) return s;
-      if ((s = launch_dots_last(h->V, k + 1, N, vk1, N, h->part, blocks, h->ticket, h->htmp, h->hcol, st)) !=
-          VIE_OK)
-        return s;
-      if ((s = launch_orth_update(h->V, k + 1, N, h->htmp, vk1, N, st)) != VIE_OK) return s;
-      if ((s = launch_norm2_givens(vk1, N, h->part, blocks, h->ticket, h->scal + 2, h->H, m, k, h->hcol, h->cs,
-                                   h->sn, h->gv, bnorm, h->scal + 3, st)) != VIE_OK)
-        return s;
-      if ((s = launch_scale(vk1, h->scal + 2, 1, vk1, N, st)) != VIE_OK) return s;
-      double est = 0.0;
-      if ((s = read_scalar(h, h->scal + 3, &est, st)) != VIE_OK) return s;
+      if ((s = wait_slots(h, h->slots, 1, nullptr, h->step_seq, st)) != VIE_OK) return s;
+      const double est = h->slots[0];
       if (timed && (s = harvest_events(h)) != VIE_OK) return s;
       ++k;
       ++R.iters;
@@ -1605,8 +1661,7 @@ vie_status vie_solve_gmres(vie_handle *h, const double *f, double *U, const vie_
       est_prev = est;
     }
     if (k > 0) {
-      if ((s = launch_backsolve(h->H, m, k, h->gv, h->yv, st)) != VIE_OK) return s;
-      if ((s = launch_lincomb_add(flexible ? h->Z : h->V, k, N, h->yv, x, N, st)) != VIE_OK) return s;
+      if ((s = launch_update(kb, flexible ? h->Z : h->V, 0, k, nullptr, x, N, st)) != VIE_OK) return s;
     }
     if (stall) R.fell_back = 1;
     ++R.restarts;

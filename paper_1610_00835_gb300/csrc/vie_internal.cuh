@@ -315,15 +315,17 @@ void fmm_release(FmmPlan *fp);
 // y = A s (op A_RAW, K_SIGMA_S: s already multiplied by sigma_s) or g - A s (I_MINUS_K)
 vie_status fmm_apply(const FmmPlan &fp, int op, const float *s, const double *g, double *y, cudaStream_t st);
 
-// ---- R GMRES solves in lockstep (k_krylov.cu).  Per right-hand side r:
-// basis vector i at V + r ldv_r + i N, Hessenberg H + r (m + 1) m
-// (column-major), rotations cs/sn + r m, residual vector gv + r (m + 1), the
-// triangular solution yv + r m, the dot columns hcol/htmp + r (m + 1), dot
-// partials part + r blocks (m + 1), block ticket ticket[r] (0 between
-// launches), scalars scal + 8 r (slot 2: ||w||^2, 3: the Givens residual
-// estimate), bnorm[r] = ||phi_r||, act[r] != 0 while r takes part.
+// ---- R GMRES solves in lockstep (k_krylov.cu; R = 1: the single solve).  Per
+// right-hand side r: basis vector i at V + r ldv_r + i N, Hessenberg
+// H + r (m + 1) m (column-major), rotations cs/sn + r m, residual vector
+// gv + r (m + 1), the dot columns hcol/htmp + r (m + 1), dot partials
+// part + r 2 blocks (m + 1), block ticket ticket[r] (0 between launches),
+// scalars scal + 8 r (slot 2: ||w||^2, 3: the Givens residual estimate),
+// inv_bnorm[r] = 1 / ||phi_r||, act[r] != 0 while r takes part (null: all), slots + 4 r
+// (pinned host memory): {estimate, two error words, 1 if a wait gave up,
+// sequence number} of r's last Arnoldi step.
 struct KBatch {
-  double *H, *cs, *sn, *gv, *yv, *hcol, *htmp, *part, *scal, *bnorm;
+  double *H, *cs, *sn, *gv, *hcol, *htmp, *part, *scal, *inv_bnorm, *slots;
   int *ticket, *act;
   long N;
   int m, R, blocks;
@@ -334,12 +336,19 @@ vie_status launch_bnorm2_givens(const KBatch &b, const double *w, long ldw_r, in
 vie_status launch_bnorm2(const KBatch &b, const double *w, long ldw_r, int slot, cudaStream_t st);
 vie_status launch_borth_update(const KBatch &b, const double *V, long ldv_r, int nv, const double *h, double *w,
                                long ldw_r, cudaStream_t st);
-vie_status launch_bscale(const KBatch &b, const double *x, long ldx_r, int slot, int use_sqrt, double *y,
-                         long ldy_r, cudaStream_t st);
+vie_status launch_bscale(const KBatch &b, const double *x, long ldx_r, int slot, double *y, long ldy_r,
+                         cudaStream_t st);
 vie_status launch_baxpby(const KBatch &b, double a, const double *x, long ldx_r, double c, const double *y,
                          long ldy_r, double *z, long ldz_r, cudaStream_t st);
-vie_status launch_bupdate(const KBatch &b, const double *B, long ldb_r, const int *kk, double *x, long ldx_r,
-                          cudaStream_t st);
+// one launch for the whole Arnoldi step (arnoldi_fused), or the separate ones
+// above; bar: two zeroed device words; err0, err1: device error words to
+// report or null
+bool arnoldi_fused(const KBatch &b);
+vie_status launch_arnoldi(const KBatch &b, double *V, long ldv_r, int k, double inv_bnorm1, const int *err0,
+                          const int *err1, unsigned long long seq, unsigned *bar, cudaStream_t st);
+// the triangular solve and x_r += sum_{v < k} y_v B_r[v] (k_all >= 0, else kk[r])
+vie_status launch_update(const KBatch &b, const double *B, long ldb_r, int k_all, const int *kk, double *x,
+                         long ldx_r, cudaStream_t st);
 
 // ---- assembled operator (k_assemble.cu, k_gemm_tc.cu)
 long assembled_ldk(long N);
@@ -382,29 +391,10 @@ vie_status unet_precondition(UnetImpl *u, const double *sigma_t, const double *s
 
 // ---- Krylov kernels (k_krylov.cu)
 int dot_blocks(long N);
-vie_status launch_dots(const double *V, int nv, long ldv, const double *w, long N, double *part,
-                       int blocks, cudaStream_t st);
-vie_status launch_dots_finish(const double *part, int blocks, int nv, double *out, int accumulate,
-                              cudaStream_t st);
-vie_status launch_orth_update(const double *V, int nv, long ldv, const double *h, double *w,
-                              long N, cudaStream_t st);
-vie_status launch_dots_last(const double *V, int nv, long ldv, const double *w, long N, double *part,
-                            int blocks, int *ticket, double *out1, double *out2, cudaStream_t st);
-vie_status launch_norm2_givens(const double *w, long N, double *part, int blocks, int *ticket, double *norm2,
-                               double *H, int m, int k, const double *hcol, double *cs, double *sn, double *gv,
-                               double bnorm, double *est, cudaStream_t st);
-vie_status launch_scale(const double *x, const double *norm2, int use_sqrt, double *y, long N,
-                        cudaStream_t st);
+// y = x / sqrt(*norm2)
+vie_status launch_scale(const double *x, const double *norm2, double *y, long N, cudaStream_t st);
 vie_status launch_axpby(double a, const double *x, double b, const double *y, double *z, long N,
                         cudaStream_t st);
-vie_status launch_givens(double *H, int m, int k, const double *hcol, const double *hk1sq,
-                         double *cs, double *sn, double *gv, double bnorm, double *est,
-                         cudaStream_t st);
-vie_status launch_backsolve(const double *H, int m, int k, const double *gv, double *y,
-                            cudaStream_t st);
-vie_status launch_lincomb_add(const double *V, int nv, long ldv, const double *y, double *x,
-                              long N, cudaStream_t st);
-
 // ---- sweep kernels (k_sweep.cu)
 vie_status launch_make_q(int dim, int n, const double *sigma_s, const double *U, const double *f,
                          float *qpad, cudaStream_t st);
