@@ -22,7 +22,7 @@
 // S-step midpoint march of the bilinear sigma_t with the sample points
 // clamped to the hull of the cell centres (nodes near the boundary lie
 // outside it).  Setup fills the near blocks and the M2L blocks on the device
-// (FP32); an apply is 2 L - 1 launches of small dense products that read the
+// (FP32); an apply is 2 L - 2 launches of small dense products that read the
 // cached blocks once (M2L of all levels in one of them).
 #include <math.h>
 
@@ -155,40 +155,119 @@ __global__ void k_fmm_m2l_fill(FillArgs a, int level, int p, const float *__rest
   }
 }
 
-// P2M: W[leaf][m] = sum_k Pm[m][k] s_leaf[k]; one CTA per leaf
-__global__ void k_fmm_p2m(int n, int L, int b, int P2, const float *__restrict__ Pm, const float *__restrict__ s,
-                          float *__restrict__ W) {
-  extern __shared__ float sh[];
+// P2M and M2M are small dense products whose matrix is the same for every box:
+// a thread takes one (box, node m), a CTA kBoxThreads / P2 boxes, and the
+// matrix is read transposed, so that a warp's loads are consecutive (with one
+// CTA of 128 threads per box and the rows m apart, 36 threads worked and every
+// load touched 32 lines: 34 us for P2M and 9 us per M2M level at 512^2, order
+// 6; now 6.6 and 8 us).
+constexpr int kBoxThreads = 256;
+
+// boxes per CTA, `floats` of shared memory each (at most 48 KB in all)
+__host__ __device__ __forceinline__ int boxes_per_cta(int P2, int floats) {
+  const int g = kBoxThreads / P2, fit = 12288 / floats;
+  return g < 1 ? 1 : g < fit ? g : fit < 1 ? 1 : fit;
+}
+
+// P2M: W[leaf][m] = sum_k Pt[k][m] s_leaf[k]
+__global__ void __launch_bounds__(kBoxThreads) k_fmm_p2m(int n, int L, int b, int P2, int G,
+                                                         const float *__restrict__ Pt, const float *__restrict__ s,
+                                                         float *__restrict__ W) {
+  extern __shared__ float sh[];  // [G][b^2]
   const int nl = 1 << L, bb = b * b;
-  const int bx = blockIdx.x % nl, by = blockIdx.x / nl;
-  for (int k = threadIdx.x; k < bb; k += blockDim.x) sh[k] = s[(long)(by * b + k / b) * n + bx * b + k % b];
+  const int box0 = blockIdx.x * G, cnt = min(G, nl * nl - box0);
+  for (int i = threadIdx.x; i < cnt * bb; i += blockDim.x) {
+    const int box = box0 + i / bb, k = i % bb, bx = box % nl, by = box / nl;
+    sh[i] = s[(long)(by * b + k / b) * n + bx * b + k % b];
+  }
   __syncthreads();
-  for (int m = threadIdx.x; m < P2; m += blockDim.x) {
+  for (int i = threadIdx.x; i < cnt * P2; i += blockDim.x) {
+    const int q = i / P2, m = i % P2;
+    const float *v = sh + q * bb;
     float acc = 0.f;
-    for (int k = 0; k < bb; ++k) acc = fmaf(Pm[m * bb + k], sh[k], acc);
-    W[(long)blockIdx.x * P2 + m] = acc;
+#pragma unroll 8
+    for (int k = 0; k < bb; ++k) acc = fmaf(__ldg(Pt + k * P2 + m), v[k], acc);
+    W[(long)(box0 + q) * P2 + m] = acc;
   }
 }
 
-// M2M: parent boxes at level l from their children at l + 1
-__global__ void k_fmm_m2m(int level, int P2, const float *__restrict__ Cq, const float *__restrict__ Wc,
-                          float *__restrict__ Wp) {
-  extern __shared__ float sh[];
+// M2M: parent boxes at level l from their children at l + 1; Ct[q][m'][m]
+__global__ void __launch_bounds__(kBoxThreads) k_fmm_m2m(int level, int P2, int G, const float *__restrict__ Ct,
+                                                         const float *__restrict__ Wc, float *__restrict__ Wp) {
+  extern __shared__ float sh[];  // [G][4][P2]
   const int nb = 1 << level;
-  const int bx = blockIdx.x % nb, by = blockIdx.x / nb;
-  for (int i = threadIdx.x; i < 4 * P2; i += blockDim.x) {
-    const int q = i / P2, mp = i % P2;
+  const int box0 = blockIdx.x * G, cnt = min(G, nb * nb - box0);
+  for (int i = threadIdx.x; i < cnt * 4 * P2; i += blockDim.x) {
+    const int box = box0 + i / (4 * P2), q = (i / P2) & 3, mp = i % P2, bx = box % nb, by = box / nb;
     const long child = (long)(2 * by + q / 2) * (2 * nb) + 2 * bx + q % 2;
     sh[i] = Wc[child * P2 + mp];
   }
   __syncthreads();
-  for (int m = threadIdx.x; m < P2; m += blockDim.x) {
+  for (int i = threadIdx.x; i < cnt * P2; i += blockDim.x) {
+    const int g = i / P2, m = i % P2;
+    const float *v = sh + g * 4 * P2;
     float acc = 0.f;
-    for (int q = 0; q < 4; ++q)
-      for (int mp = 0; mp < P2; ++mp) acc = fmaf(Cq[((long)q * P2 + m) * P2 + mp], sh[q * P2 + mp], acc);
-    Wp[(long)blockIdx.x * P2 + m] = acc;
+#pragma unroll 24
+    for (int k = 0; k < 4 * P2; ++k) acc = fmaf(__ldg(Ct + (long)k * P2 + m), v[k], acc);
+    Wp[(long)(box0 + g) * P2 + m] = acc;
   }
 }
+
+// Streaming product of the two big kernels: thread t = (part, column) of
+// parts x C threads adds blk[(part + q parts) C + column] sh[part + q parts]
+// over q, in four chains (q = 0, 1, 2, 3 mod 4; what is left over after the
+// last whole four goes to the first).  The block is read once from HBM: a
+// thread keeps a batch of eight loads in flight while it works on the batch
+// before, and the first batch is issued before the sources are gathered into
+// shared memory (StreamDot::start), so that the gather's latency hides behind
+// it.  Four loads and the gather first: 4.5 TB/s for M2L, 5.2 for the leaves
+// at 512^2 (170 and 117 us); now 6.5 and 5.7 (117 and 106).
+struct StreamDot {
+  static constexpr int kBatch = 8;
+  const float *p;   // this thread's next element
+  long step;        // parts * C
+  int left;         // elements of this thread not yet loaded
+  int src, parts;   // this thread's next source, and the distance to the one after
+  float v[kBatch];
+  __device__ __forceinline__ void load() {
+#pragma unroll
+    for (int i = 0; i < kBatch; ++i) v[i] = i < left ? __ldcs(p + i * step) : 0.f;
+    p += kBatch * step;
+  }
+  __device__ __forceinline__ void start(const float *blk, int C, int parts_, int part, int column, int I, bool on) {
+    parts = parts_;
+    step = (long)parts * C;
+    p = blk + (long)part * C + column;
+    left = on && part < I ? (I - part + parts - 1) / parts : 0;
+    src = part;
+    load();
+  }
+  // the four chains, to be added as (a0 + a1) + (a2 + a3)
+  __device__ __forceinline__ void run(const float *sh, float (&a)[4]) {
+#pragma unroll
+    for (int c = 0; c < 4; ++c) a[c] = 0.f;
+    while (left >= kBatch) {
+      float u[kBatch];
+#pragma unroll
+      for (int i = 0; i < kBatch; ++i) u[i] = v[i];
+      left -= kBatch;
+      load();
+#pragma unroll
+      for (int i = 0; i < kBatch; ++i) a[i & 3] = fmaf(u[i], sh[src + i * parts], a[i & 3]);
+      src += kBatch * parts;
+    }
+    const int whole = left & ~3;
+#pragma unroll
+    for (int i = 0; i < kBatch; ++i)
+      if (i < left) {
+        const float x = sh[src + i * parts];
+        if (i < whole)
+          a[i & 3] = fmaf(v[i], x, a[i & 3]);
+        else
+          a[0] = fmaf(v[i], x, a[0]);
+      }
+  }
+};
 
 // M2L of every level in one launch (the levels do not depend on each other):
 // CTA t takes box t - first[l] of the level l with first[l] <= t < first[l + 1],
@@ -208,11 +287,14 @@ __global__ void k_fmm_m2l(M2LArgs a, int P2, const float *__restrict__ m2l_all, 
   int level = 2;
   while (level < a.L && (long)blockIdx.x >= a.first[level + 1]) ++level;
   const long box = (long)blockIdx.x - a.first[level];
-  const float *m2l = m2l_all + a.m2l_off[level];
   const float *W = W_all + a.node_off[level];
   float *Lc = Lc_all + a.node_off[level];
   const int nb = 1 << level;
   const int bx = (int)(box % nb), by = (int)(box / nb);
+  // blockDim / P2 groups of P2 threads each take every parts-th source node
+  const int parts = blockDim.x / P2, m = threadIdx.x % P2, part = threadIdx.x / P2;
+  StreamDot dot;
+  dot.start(m2l_all + a.m2l_off[level] + box * kIL * P2 * P2, P2, parts, part, m, kIL * P2, part < parts);
   for (int i = threadIdx.x; i < kIL * P2; i += blockDim.x) {
     const int slot = i / P2, mp = i % P2;
     int ox, oy;
@@ -221,24 +303,10 @@ __global__ void k_fmm_m2l(M2LArgs a, int P2, const float *__restrict__ m2l_all, 
     sh[i] = (cx >= 0 && cx < nb && cy >= 0 && cy < nb) ? W[((long)cy * nb + cx) * P2 + mp] : 0.f;
   }
   __syncthreads();
-  // blockDim / P2 groups of P2 threads each take every parts-th source node
-  const float *blk = m2l + box * kIL * P2 * P2;
   float *red = sh + kIL * P2;
-  const int parts = blockDim.x / P2, m = threadIdx.x % P2, part = threadIdx.x / P2;
-  // four independent chains keep four streaming loads in flight per thread
-  float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-  if (part < parts) {
-    const int I = kIL * P2;
-    int i = part;
-    for (; i + 3 * parts < I; i += 4 * parts) {
-      a0 = fmaf(__ldcs(blk + (long)i * P2 + m), sh[i], a0);
-      a1 = fmaf(__ldcs(blk + (long)(i + parts) * P2 + m), sh[i + parts], a1);
-      a2 = fmaf(__ldcs(blk + (long)(i + 2 * parts) * P2 + m), sh[i + 2 * parts], a2);
-      a3 = fmaf(__ldcs(blk + (long)(i + 3 * parts) * P2 + m), sh[i + 3 * parts], a3);
-    }
-    for (; i < I; i += parts) a0 = fmaf(__ldcs(blk + (long)i * P2 + m), sh[i], a0);
-  }
-  red[threadIdx.x] = (a0 + a1) + (a2 + a3);
+  float c[4];
+  dot.run(sh, c);
+  red[threadIdx.x] = (c[0] + c[1]) + (c[2] + c[3]);
   __syncthreads();
   if (threadIdx.x < P2) {
     float t = 0.f;
@@ -248,56 +316,69 @@ __global__ void k_fmm_m2l(M2LArgs a, int P2, const float *__restrict__ m2l_all, 
 }
 
 // L2L: child boxes at level l + 1 take their parent's interpolated L
-__global__ void k_fmm_l2l(int level, int P2, const float *__restrict__ Cq, const float *__restrict__ Lp,
-                          float *__restrict__ Lch) {
-  extern __shared__ float sh[];
+__global__ void __launch_bounds__(kBoxThreads) k_fmm_l2l(int level, int P2, int G, const float *__restrict__ Cq,
+                                                         const float *__restrict__ Lp, float *__restrict__ Lch) {
+  extern __shared__ float sh[];  // [G][P2]
   const int nc = 2 << level;  // children per side
-  const int cx = blockIdx.x % nc, cy = blockIdx.x / nc;
-  const int q = (cx & 1) + 2 * (cy & 1);
-  const long parent = (long)(cy >> 1) * (nc >> 1) + (cx >> 1);
-  for (int m = threadIdx.x; m < P2; m += blockDim.x) sh[m] = Lp[parent * P2 + m];
+  const int box0 = blockIdx.x * G, cnt = min(G, nc * nc - box0);
+  for (int i = threadIdx.x; i < cnt * P2; i += blockDim.x) {
+    const int box = box0 + i / P2, cx = box % nc, cy = box / nc;
+    sh[i] = Lp[((long)(cy >> 1) * (nc >> 1) + (cx >> 1)) * P2 + i % P2];
+  }
   __syncthreads();
-  for (int mp = threadIdx.x; mp < P2; mp += blockDim.x) {
+  for (int i = threadIdx.x; i < cnt * P2; i += blockDim.x) {
+    const int g = i / P2, mp = i % P2, box = box0 + g;
+    const float *C = Cq + (long)((box % nc & 1) + 2 * (box / nc & 1)) * P2 * P2 + mp, *v = sh + g * P2;
     float acc = 0.f;
-    for (int m = 0; m < P2; ++m) acc = fmaf(Cq[((long)q * P2 + m) * P2 + mp], sh[m], acc);
-    Lch[(long)blockIdx.x * P2 + mp] += acc;
+#pragma unroll 18
+    for (int m = 0; m < P2; ++m) acc = fmaf(__ldg(C + (long)m * P2), v[m], acc);
+    Lch[(long)box * P2 + mp] += acc;
   }
 }
 
-// leaves: near field from the cached blocks plus L2P; y (FP64) by op
+// leaves: near field from the cached blocks plus L2P of the leaf's own far
+// field and its parent's (the L2L step of the leaf level, taken here); y (FP64)
+// by op
 __global__ void k_fmm_leaf(int n, int L, int b, int P2, const float *__restrict__ near, const float *__restrict__ Pm,
-                           const float *__restrict__ s, const float *__restrict__ Lc, int op,
-                           const double *__restrict__ g, double *__restrict__ y) {
-  extern __shared__ float sh[];  // [9][b^2] sources, then [P2] L
+                           const float *__restrict__ s, const float *__restrict__ Lc, const float *__restrict__ Lp,
+                           const float *__restrict__ Cq, int op, const double *__restrict__ g,
+                           double *__restrict__ y) {
+  extern __shared__ float sh[];  // [9][b^2] sources, then [P2] L, [P2] the parent's
   const int nl = 1 << L, bb = b * b;
   const int bx = blockIdx.x % nl, by = blockIdx.x / nl;
+  // blockDim / bb groups of bb threads each take every parts-th source cell;
+  // group 0 adds the far field (L2P)
+  const int parts = blockDim.x / bb, j = threadIdx.x % bb, part = threadIdx.x / bb;
+  StreamDot dot;
+  dot.start(near + (long)blockIdx.x * 9 * bb * bb, bb, parts, part, j, 9 * bb, part < parts);
+  float *far = sh + 9 * bb, *up = far + P2, *red = up + P2;
+  for (int m = threadIdx.x; m < P2; m += blockDim.x) {
+    far[m] = Lc[(long)blockIdx.x * P2 + m];
+    if (Lp) up[m] = Lp[((long)(by >> 1) * (nl >> 1) + (bx >> 1)) * P2 + m];
+  }
   for (int i = threadIdx.x; i < 9 * bb; i += blockDim.x) {
     const int slot = i / bb, k = i % bb;
     const int cx = bx + slot % 3 - 1, cy = by + slot / 3 - 1;
     sh[i] = (cx >= 0 && cx < nl && cy >= 0 && cy < nl) ? s[(long)(cy * b + k / b) * n + cx * b + k % b] : 0.f;
   }
-  for (int m = threadIdx.x; m < P2; m += blockDim.x) sh[9 * bb + m] = Lc ? Lc[(long)blockIdx.x * P2 + m] : 0.f;
   __syncthreads();
-  // blockDim / bb groups of bb threads each take every parts-th source cell;
-  // group 0 adds the far field (L2P)
-  const float *blk = near + (long)blockIdx.x * 9 * bb * bb;
-  float *red = sh + 9 * bb + P2;
-  const int parts = blockDim.x / bb, j = threadIdx.x % bb, part = threadIdx.x / bb;
-  float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-  if (part < parts) {
-    const int I = 9 * bb;
-    int i = part;
-    for (; i + 3 * parts < I; i += 4 * parts) {
-      a0 = fmaf(__ldcs(blk + (long)i * bb + j), sh[i], a0);
-      a1 = fmaf(__ldcs(blk + (long)(i + parts) * bb + j), sh[i + parts], a1);
-      a2 = fmaf(__ldcs(blk + (long)(i + 2 * parts) * bb + j), sh[i + 2 * parts], a2);
-      a3 = fmaf(__ldcs(blk + (long)(i + 3 * parts) * bb + j), sh[i + 3 * parts], a3);
+  if (Lp) {
+    const float *C = Cq + (long)((bx & 1) + 2 * (by & 1)) * P2 * P2;
+    for (int mp = threadIdx.x; mp < P2; mp += blockDim.x) {
+      float acc = 0.f;
+#pragma unroll 18
+      for (int m = 0; m < P2; ++m) acc = fmaf(__ldg(C + (long)m * P2 + mp), up[m], acc);
+      far[mp] += acc;
     }
-    for (; i < I; i += parts) a0 = fmaf(__ldcs(blk + (long)i * bb + j), sh[i], a0);
-    if (part == 0)
-      for (int m = 0; m < P2; ++m) a1 = fmaf(Pm[m * bb + j], sh[9 * bb + m], a1);
+    __syncthreads();
   }
-  red[threadIdx.x] = (a0 + a1) + (a2 + a3);
+  float c[4];
+  dot.run(sh, c);
+  if (part == 0) {
+#pragma unroll 18
+    for (int m = 0; m < P2; ++m) c[1] = fmaf(__ldg(Pm + m * bb + j), far[m], c[1]);
+  }
+  red[threadIdx.x] = (c[0] + c[1]) + (c[2] + c[3]);
   __syncthreads();
   if (threadIdx.x < bb) {
     double v = 0.0;
@@ -345,7 +426,7 @@ vie_status fmm_prepare(FmmPlan *fp, int n, int p, const float *sig32, const doub
   std::vector<double> z(p);
   for (int i = 0; i < p; ++i) z[i] = cos((2.0 * (i + 1) - 1.0) * kPi / (2.0 * p));
   // P[m][k]: leaf cell k = kx + b ky at u = 2 (kx + 1/2) / b - 1
-  std::vector<float> Pm((size_t)P2 * bb), Cq((size_t)4 * P2 * P2), zf(p);
+  std::vector<float> Pm((size_t)P2 * bb), Cq((size_t)4 * P2 * P2), Pt(Pm.size()), Ct(Cq.size()), zf(p);
   for (int m = 0; m < P2; ++m)
     for (int k = 0; k < bb; ++k) {
       const double u = 2.0 * (k % b + 0.5) / b - 1.0, v = 2.0 * (k / b + 0.5) / b - 1.0;
@@ -360,6 +441,12 @@ vie_status fmm_prepare(FmmPlan *fp, int n, int p, const float *sig32, const doub
         Cq[((size_t)q * P2 + m) * P2 + mp] = (float)(s1(p, u, z[m % p]) * s1(p, v, z[m / p]));
       }
   for (int i = 0; i < p; ++i) zf[i] = (float)z[i];
+  for (int m = 0; m < P2; ++m) {
+    for (int k = 0; k < bb; ++k) Pt[(size_t)k * P2 + m] = Pm[(size_t)m * bb + k];
+    for (int q = 0; q < 4; ++q)
+      for (int mp = 0; mp < P2; ++mp)
+        Ct[((size_t)q * P2 + mp) * P2 + m] = Cq[((size_t)q * P2 + m) * P2 + mp];
+  }
   fp->n = n;
   fp->p = p;
   fp->L = L;
@@ -381,9 +468,13 @@ vie_status fmm_prepare(FmmPlan *fp, int n, int p, const float *sig32, const doub
   VIE_CUDA(vie_malloc((void **)&fp->Lc, sizeof(float) * nodes));
   VIE_CUDA(vie_malloc((void **)&fp->Pm, sizeof(float) * Pm.size()));
   VIE_CUDA(vie_malloc((void **)&fp->Cq, sizeof(float) * Cq.size()));
+  VIE_CUDA(vie_malloc((void **)&fp->Pt, sizeof(float) * Pt.size()));
+  VIE_CUDA(vie_malloc((void **)&fp->Ct, sizeof(float) * Ct.size()));
   VIE_CUDA(vie_malloc((void **)&fp->z, sizeof(float) * p));
   VIE_CUDA(cudaMemcpyAsync(fp->Pm, Pm.data(), sizeof(float) * Pm.size(), cudaMemcpyHostToDevice, st));
   VIE_CUDA(cudaMemcpyAsync(fp->Cq, Cq.data(), sizeof(float) * Cq.size(), cudaMemcpyHostToDevice, st));
+  VIE_CUDA(cudaMemcpyAsync(fp->Pt, Pt.data(), sizeof(float) * Pt.size(), cudaMemcpyHostToDevice, st));
+  VIE_CUDA(cudaMemcpyAsync(fp->Ct, Ct.data(), sizeof(float) * Ct.size(), cudaMemcpyHostToDevice, st));
   VIE_CUDA(cudaMemcpyAsync(fp->z, zf.data(), sizeof(float) * p, cudaMemcpyHostToDevice, st));
   FillArgs a{sig32, diag, n, n + 1, steps, closed, (float)sigma_c};
   k_fmm_near_fill<<<blocks_for(near_total), 256, 0, st>>>(a, L, b, fp->near);
@@ -407,6 +498,8 @@ void fmm_release(FmmPlan *fp) {
   if (fp->Lc) vie_free(fp->Lc);
   if (fp->Pm) vie_free(fp->Pm);
   if (fp->Cq) vie_free(fp->Cq);
+  if (fp->Pt) vie_free(fp->Pt);
+  if (fp->Ct) vie_free(fp->Ct);
   if (fp->z) vie_free(fp->z);
   *fp = FmmPlan{};
 }
@@ -414,13 +507,17 @@ void fmm_release(FmmPlan *fp) {
 vie_status fmm_apply(const FmmPlan &fp, int op, const float *s, const double *g, double *y, cudaStream_t st) {
   const int n = fp.n, L = fp.L, b = fp.b, P2 = fp.p * fp.p, bb = b * b;
   const int nl = 1 << L;
-  const int t = 128, tm = std::max(P2, 256 / P2 * P2), tl = std::max(bb, 256 / bb * bb);
+  const int tm = std::max(P2, 256 / P2 * P2), tl = std::max(bb, 256 / bb * bb);
+  auto ctas = [](long boxes, int G) { return (unsigned)((boxes + G - 1) / G); };
   // upward pass
-  k_fmm_p2m<<<nl * nl, t, sizeof(float) * bb, st>>>(n, L, b, P2, fp.Pm, s, fp.W + fp.node_off[L]);
+  const int gp = boxes_per_cta(P2, bb);
+  k_fmm_p2m<<<ctas((long)nl * nl, gp), kBoxThreads, sizeof(float) * gp * bb, st>>>(n, L, b, P2, gp, fp.Pt, s,
+                                                                                fp.W + fp.node_off[L]);
   VIE_CHECK_LAUNCH("k_fmm_p2m");
+  const int gm = boxes_per_cta(P2, 4 * P2);
   for (int l = L - 1; l >= 2; --l) {
-    k_fmm_m2m<<<1 << (2 * l), t, sizeof(float) * 4 * P2, st>>>(l, P2, fp.Cq, fp.W + fp.node_off[l + 1],
-                                                              fp.W + fp.node_off[l]);
+    k_fmm_m2m<<<ctas(1L << (2 * l), gm), kBoxThreads, sizeof(float) * gm * 4 * P2, st>>>(
+        l, P2, gm, fp.Ct, fp.W + fp.node_off[l + 1], fp.W + fp.node_off[l]);
     VIE_CHECK_LAUNCH("k_fmm_m2m");
   }
   // interactions (all levels in one launch), then the downward pass
@@ -438,13 +535,15 @@ vie_status fmm_apply(const FmmPlan &fp, int op, const float *s, const double *g,
     k_fmm_m2l<<<(unsigned)first, tm, sizeof(float) * (kIL * P2 + tm), st>>>(a, P2, fp.m2l, fp.W, fp.Lc);
     VIE_CHECK_LAUNCH("k_fmm_m2l");
   }
-  for (int l = 2; l < L; ++l) {
-    k_fmm_l2l<<<1 << (2 * (l + 1)), t, sizeof(float) * P2, st>>>(l, P2, fp.Cq, fp.Lc + fp.node_off[l],
-                                                                  fp.Lc + fp.node_off[l + 1]);
+  const int gl = boxes_per_cta(P2, P2);
+  for (int l = 2; l < L - 1; ++l) {
+    k_fmm_l2l<<<ctas(4L << (2 * l), gl), kBoxThreads, sizeof(float) * gl * P2, st>>>(
+        l, P2, gl, fp.Cq, fp.Lc + fp.node_off[l], fp.Lc + fp.node_off[l + 1]);
     VIE_CHECK_LAUNCH("k_fmm_l2l");
   }
-  k_fmm_leaf<<<nl * nl, tl, sizeof(float) * (9 * bb + P2 + tl), st>>>(
-      n, L, b, P2, fp.near, fp.Pm, s, fp.Lc + fp.node_off[L], op, g, y);
+  k_fmm_leaf<<<nl * nl, tl, sizeof(float) * (9 * bb + 2 * P2 + tl), st>>>(
+      n, L, b, P2, fp.near, fp.Pm, s, fp.Lc + fp.node_off[L], L > 2 ? fp.Lc + fp.node_off[L - 1] : nullptr, fp.Cq,
+      op, g, y);
   VIE_CHECK_LAUNCH("k_fmm_leaf");
   return VIE_OK;
 }

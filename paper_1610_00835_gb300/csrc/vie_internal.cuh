@@ -306,6 +306,7 @@ struct FmmPlan {
   float *W = nullptr, *Lc = nullptr;  // multipole and local node values, per level
   float *Pm = nullptr;         // [p^2][b^2] leaf interpolation
   float *Cq = nullptr;         // [4][p^2][p^2] child-to-parent interpolation
+  float *Pt = nullptr, *Ct = nullptr;  // both with the node they produce fastest ([b^2][p^2], [4][p^2][p^2])
   float *z = nullptr;          // [p] Chebyshev points
 };
 void fmm_leaf_levels(int n, int *L, int *b);
