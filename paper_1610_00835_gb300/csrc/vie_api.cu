@@ -176,7 +176,7 @@ struct vie_handle {
   double *partial = nullptr;                  // [plan.splits][N]
   DBuf<double> stage_a, stage_b, stage_c;     // host-pointer staging
   DBuf<float> stage_f1, stage_f2;
-  float *qpad = nullptr;                      // sweep source lattice
+  float2 *qpad = nullptr;                     // sweep lattice (sigma_t, Q)
   // GMRES workspace
   int gm_m = 0;
   double *V = nullptr, *phi = nullptr, *r = nullptr, *w = nullptr, *H = nullptr;
@@ -1721,12 +1721,9 @@ vie_status ert_sweep(vie_handle *h, const double *U, const double *f, const floa
     if ((s = h->stage_f2.reserve((size_t)M * N)) != VIE_OK) return s;
     Pd = h->stage_f2.ptr;
   }
-  if (!h->qpad) {
-    const long lattice = h->dim == 2 ? (long)h->P * h->P : (long)h->P * h->P * h->P;
-    if ((s = dalloc(&h->qpad, lattice)) != VIE_OK) return s;
-  }
-  if ((s = launch_make_q(h->dim, h->n, h->sig_s, Ud, fd, h->qpad, st)) != VIE_OK) return s;
-  if ((s = launch_sweep(h->dim, h->n, h->sig32, h->qpad, dd, M, Pd, st)) != VIE_OK) return s;
+  if (!h->qpad && (s = dalloc(&h->qpad, sweep_lattice_points(h->dim, h->n))) != VIE_OK) return s;
+  if ((s = launch_make_q(h->dim, h->n, h->sig_t, h->sig_s, Ud, fd, h->qpad, st)) != VIE_OK) return s;
+  if ((s = launch_sweep(h->dim, h->n, h->qpad, dd, M, Pd, st)) != VIE_OK) return s;
   if (!pd) {
     VIE_CUDA(cudaMemcpyAsync(Phi, Pd, sizeof(float) * M * N, cudaMemcpyDeviceToHost, st));
     VIE_CUDA(cudaStreamSynchronize(st));

@@ -397,9 +397,10 @@ vie_status launch_scale(const double *x, const double *norm2, double *y, long N,
 vie_status launch_axpby(double a, const double *x, double b, const double *y, double *z, long N,
                         cudaStream_t st);
 // ---- sweep kernels (k_sweep.cu)
-vie_status launch_make_q(int dim, int n, const double *sigma_s, const double *U, const double *f,
-                         float *qpad, cudaStream_t st);
-vie_status launch_sweep(int dim, int n, const float *sigpad, const float *qpad, const float *dirs,
-                        int M, float *Phi, cudaStream_t st);
+// lat: (sigma_t, Q) with a ghost layer, sweep_lattice_points pairs
+size_t sweep_lattice_points(int dim, int n);
+vie_status launch_make_q(int dim, int n, const double *sigma_t, const double *sigma_s, const double *U,
+                         const double *f, float2 *lat, cudaStream_t st);
+vie_status launch_sweep(int dim, int n, const float2 *lat, const float *dirs, int M, float *Phi, cudaStream_t st);
 
 }  // namespace vie
