@@ -280,8 +280,10 @@ __global__ void __launch_bounds__(kConvThreads, 2)
         ++issued_loads;
       }
     }
-  } else if (warp == 5 && lane == 0) {
-    // MMA issuer
+  } else if (warp == 5 && elect_one()) {
+    // MMA issuer (one elected lane: the compiler then keeps the descriptors in
+    // uniform registers; behind `lane == 0` it moved every operand of every
+    // product there, about 90 cycles per product)
     const unsigned idesc = idesc_bf16(kTcM, Co);
     bool go = mbar_wait(su32(wbar), 0, abort_flag, wl.first);
     int g = 0, j = 0;
@@ -304,20 +306,19 @@ __global__ void __launch_bounds__(kConvThreads, 2)
         for (int e = 0; e < taps_step; ++e) {
           // tap (dy, dx): its weights, and its input rows e pixels into a halo box
           const int tap = halo ? 3 * q + e : q;
-          const unsigned a = su32(As + (size_t)st * a_bytes) + 64u * (unsigned)e;
-          const unsigned bb = su32(Bs + (size_t)(tap * S + sl) * b_bytes);
+          // (descriptors by addition to the start address field, in 16-byte units)
+          const unsigned long long ad = smem_desc_sw64(su32(As + (size_t)st * a_bytes) + 64u * (unsigned)e);
+          const unsigned long long bd = smem_desc_sw64(su32(Bs + (size_t)(tap * S + sl) * b_bytes));
 #pragma unroll
           for (int kk = 0; kk < 2; ++kk) {
             // parts i of the input and j of the weights, i + j < NP
 #pragma unroll
             for (int i = 0; i < NP; ++i)
 #pragma unroll
-              for (int j = 0; i + j < NP; ++j) {
-                const unsigned ai = a + (unsigned)(i * a_part) + kk * 32;
-                const unsigned bj = bb + (unsigned)(j * b_part) + kk * 32;
-                mma_bf16(d, smem_desc_sw64(ai), smem_desc_sw64(bj), idesc,
+              for (int j = 0; i + j < NP; ++j)
+                mma_bf16(d, ad + (unsigned)(i * (a_part >> 4) + kk * 2),
+                         bd + (unsigned)(j * (int)(b_part >> 4) + kk * 2), idesc,
                          (k > 0 || e > 0 || kk > 0 || i > 0 || j > 0) ? 1u : 0u);
-              }
           }
         }
         mma_commit(su32(empty + st));  // the stage is free once these products finish
@@ -493,6 +494,63 @@ __global__ void k_to_nhwc_split(const float *__restrict__ in, long in_bs, int Ci
   }
 }
 
+// The gradient of a 32-channel convolution's output, masked by its ReLU
+// (a > 0), as three BF16 parts [B][plane][32], and the bias gradient's block
+// sums part[block][32].  A thread takes 8 of the channels of one pixel, and
+// `steps` pixels 64 apart in turn (up to 8; small levels have too few pixels).
+int split_steps(long total) { return (int)std::max(1L, std::min(8L, total / (64 * 512))); }
+int split_blocks(long total) { return (int)((total + 64 * split_steps(total) - 1) / (64 * split_steps(total))); }
+__global__ void __launch_bounds__(256) k_mask_split(const float *__restrict__ g, long g_bs,
+                                                    const float *__restrict__ a, long a_bs, long plane, int B,
+                                                    __nv_bfloat16 *__restrict__ out0,
+                                                    __nv_bfloat16 *__restrict__ out1,
+                                                    __nv_bfloat16 *__restrict__ out2, float *__restrict__ part, int steps) {
+  __shared__ float red[32][65];
+  const int px = threadIdx.x & 63, gq = threadIdx.x >> 6;
+  float sum[8];
+#pragma unroll
+  for (int e = 0; e < 8; ++e) sum[e] = 0.f;
+  const long total = (long)B * plane;
+#pragma unroll 2
+  for (int k = 0; k < steps; ++k) {
+    const long t = ((long)blockIdx.x * steps + k) * 64 + px;
+    if (t >= total) break;
+    const long b = t / plane, p = t - b * plane;
+    const float *gp = g + b * g_bs + p + 8 * gq * plane, *ap = a + b * a_bs + p + 8 * gq * plane;
+    float v[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) v[e] = ap[e * plane] > 0.f ? gp[e * plane] : 0.f;
+    unsigned w[3][4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      sum[2 * e] += v[2 * e];
+      sum[2 * e + 1] += v[2 * e + 1];
+      __nv_bfloat16 p0[3], p1[3];
+      split_parts(v[2 * e], 3, p0);
+      split_parts(v[2 * e + 1], 3, p1);
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        const __nv_bfloat162 h2 = __halves2bfloat162(p0[q], p1[q]);
+        w[q][e] = *reinterpret_cast<const unsigned *>(&h2);
+      }
+    }
+    reinterpret_cast<uint4 *>(out0 + t * 32)[gq] = make_uint4(w[0][0], w[0][1], w[0][2], w[0][3]);
+    reinterpret_cast<uint4 *>(out1 + t * 32)[gq] = make_uint4(w[1][0], w[1][1], w[1][2], w[1][3]);
+    reinterpret_cast<uint4 *>(out2 + t * 32)[gq] = make_uint4(w[2][0], w[2][1], w[2][2], w[2][3]);
+  }
+#pragma unroll
+  for (int e = 0; e < 8; ++e) red[8 * gq + e][px] = sum[e];
+  __syncthreads();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int c = 4 * warp + q;
+    float s = red[c][lane] + red[c][lane + 32];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if (lane == 0) part[blockIdx.x * 32 + c] = s;
+  }
+}
+
 // Weights FP32 [Co][Ci][9], output channels co0 .. co0 + cb -> np BF16 parts
 // [9 S][cb][32] in k_pack_tc_weights's block order.
 __global__ void k_pack_split_weights(const float *__restrict__ w, int Co, int Ci, int S, int co0, int cb, int np,
@@ -592,6 +650,270 @@ __global__ void __launch_bounds__(256, 3) k_conv3_dw(const float *__restrict__ x
     for (int t = 0; t < 9; ++t) atomicAdd(&dw[((long)co * Ci + ci) * 9 + t], acc[t]);
   }
   if (db && cib == 0 && ci_l == 0 && co < Co) atomicAdd(&db[co], bsum);
+}
+
+// Weight gradient of a 3x3 convolution with 32 outputs on the tensor cores:
+//   dw[co][ci][ky][kx] = sum over pixels of g[co][p] x[ci][p + (ky - 1, kx - 1)],
+// a contraction over pixels.  The operands are the split-precision NHWC copies
+// the other convolutions use (three BF16 parts, the six products of parts i,
+// j with i + j < 3), read MN-major: a row of shared memory is one pixel's 32
+// channels, so that a shift by one pixel is a shift by one 64-byte row.  One
+// tcgen05.mma takes 16 pixels of a row and has M = 128 = 4 shifts kx (the
+// fourth is not used) x 32 input channels: the four blocks of 32 lie 64 bytes
+// apart in the same input row (the descriptor's leading offset).  N is the 32
+// output channels of as many parts of the gradient as part i of the input
+// meets: 96, 64 and 32 columns for i = 0, 1, 2, three instructions for the six
+// products, since an instruction of M = 128 takes about 64 cycles to read its
+// operand however narrow N is.
+//
+// A CTA takes one slice of 32 input channels (blockIdx.y) and a run of image
+// rows (segments of at most 128 pixels).  Warp 4 streams the rows by TMA (an
+// input row of Wp + 2 pixels serves three output rows; zero fill outside the
+// image is the convolution's padding and pads Wp to a multiple of 16), warp 5
+// issues the products of one row and one ky into one of kDwAcc accumulators of
+// 96 columns, warps 0-2 add the finished ones to FP32 sums in registers (after
+// at most 24 products per column: the accumulation of tcgen05 truncates, long
+// chains would drift).  The CTAs' sums are added by k_dw_reduce, in order.
+// What bounds it is the operand traffic of the products.  The CUDA-core form
+// (k_conv3_dw, other widths) took 95 us per layer of 16 images at 128^2 on
+// average; DW_MEASURED.
+// Waits are bounded as in k_conv3_tma; on expiry the CTA's sums are NaN.
+constexpr int kDwParts = 3;
+constexpr int kDwAcc = 5;  // accumulators of 32 kDwParts tensor-memory columns
+__host__ __device__ inline int dw_x_bytes(int Wp) { return ((Wp + 3) * 64 + 1023) / 1024 * 1024; }
+__host__ __device__ inline int dw_g_bytes(int Wp) { return (Wp * 64 + 1023) / 1024 * 1024; }
+// ring slots of input and gradient rows
+__host__ __device__ inline int dw_x_slots(int Wp) { return Wp > 64 ? 5 : 8; }
+__host__ __device__ inline int dw_g_slots(int Wp) { return Wp > 64 ? 3 : 6; }
+inline size_t dw_smem(int Wp) {
+  const int nx = dw_x_slots(Wp), ng = dw_g_slots(Wp);
+  return 1024 + (size_t)kDwParts * (nx * dw_x_bytes(Wp) + ng * dw_g_bytes(Wp)) +
+         8 * (2 * nx + 2 * ng + 2 * kDwAcc + 1) + 16;
+}
+
+struct DwMaps {
+  CUtensorMap x[kDwParts], g[kDwParts];
+};
+
+__global__ void __launch_bounds__(kConvThreads, 1)
+    k_conv3_dw_tc(const __grid_constant__ DwMaps maps, int H, int W, int B, int Wp, int segs,
+                  float *__restrict__ part, WaitLimits wl, int *err) {
+  using namespace tc;
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  unsigned char *smem = (unsigned char *)(((size_t)smem_raw + 1023) & ~(size_t)1023);
+  const int nx = dw_x_slots(Wp), ng = dw_g_slots(Wp);
+  const int xp = dw_x_bytes(Wp), gp = dw_g_bytes(Wp);
+  unsigned char *Xs = smem, *Gs = smem + (size_t)kDwParts * nx * xp;
+  unsigned long long *xfull = (unsigned long long *)(Gs + (size_t)kDwParts * ng * gp);
+  unsigned long long *xempty = xfull + nx, *gfull = xempty + nx, *gempty = gfull + ng;
+  unsigned long long *tfull = gempty + ng, *tempty = tfull + kDwAcc, *done = tempty + kDwAcc;
+  unsigned *tmem_slot = (unsigned *)(done + 1);
+  volatile int *abort_flag = (volatile int *)(tmem_slot + 1);
+  const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
+  if (tid == 0) {
+    for (int i = 0; i < nx; ++i) {
+      mbar_init(su32(xfull + i), 1);
+      mbar_init(su32(xempty + i), 1);
+    }
+    for (int i = 0; i < ng; ++i) {
+      mbar_init(su32(gfull + i), 1);
+      mbar_init(su32(gempty + i), 1);
+    }
+    for (int i = 0; i < kDwAcc; ++i) {
+      mbar_init(su32(tfull + i), 1);
+      mbar_init(su32(tempty + i), 3);  // one arrival per adding warp
+    }
+    mbar_init(su32(done), 1);
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 5) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tmem_slot)), "r"(512)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const unsigned tmem = *tmem_slot;
+  // this CTA's rows q: row q % H of column q / H (an image's segment)
+  const long rows = (long)B * segs * H;
+  const int q0 = (int)(rows * blockIdx.x / gridDim.x), q1 = (int)(rows * (blockIdx.x + 1) / gridDim.x);
+  int xs = 0, gs = 0;  // rows loaded so far (warp 4)
+  if (warp == 4 && lane == 0) {
+    bool go = true;
+    auto load_x = [&](int col, int y) {
+      const int st = xs % nx, use = xs / nx;
+      if (!go || (use > 0 && !mbar_wait(su32(xempty + st), (use - 1) & 1, abort_flag, wl.limit))) {
+        go = false;
+        return;
+      }
+      mbar_arrive_expect_tx(su32(xfull + st), (unsigned)(kDwParts * (Wp + 2) * 64));
+#pragma unroll
+      for (int i = 0; i < kDwParts; ++i)
+        tma_load_4d(su32(Xs + (size_t)(st * kDwParts + i) * xp), &maps.x[i], su32(xfull + st),
+                    (int)blockIdx.y * kTmaSlice, col % segs * kTcM - 1, y, col / segs);
+      ++xs;
+    };
+    for (int q = q0; q < q1 && go; ++q) {
+      const int col = q / H, y = q % H;
+      if (q == q0 || y == 0) {
+        load_x(col, y - 1);
+        load_x(col, y);
+      }
+      load_x(col, y + 1);
+      const int st = gs % ng, use = gs / ng;
+      if (!go || (use > 0 && !mbar_wait(su32(gempty + st), (use - 1) & 1, abort_flag, wl.limit))) {
+        go = false;
+        break;
+      }
+      mbar_arrive_expect_tx(su32(gfull + st), (unsigned)(kDwParts * Wp * 64));
+#pragma unroll
+      for (int i = 0; i < kDwParts; ++i)
+        tma_load_4d(su32(Gs + (size_t)(st * kDwParts + i) * gp), &maps.g[i], su32(gfull + st), 0, col % segs * kTcM, y,
+                    col / segs);
+      ++gs;
+    }
+    if (!go) {
+      atomicExch(err, 1);
+      *abort_flag = 1;
+    }
+  } else if (warp == 5 && elect_one()) {
+    bool go = true;
+    int xb = 0, xw = 0;  // first input row of the current output row, rows waited for
+    for (int q = q0; q < q1 && go; ++q) {
+      const int i = q - q0, y = q % H;
+      for (; xw <= xb + 2 && go; ++xw)
+        go = mbar_wait(su32(xfull + xw % nx), (xw / nx) & 1, abort_flag, xw == 0 ? wl.first : wl.limit);
+      go = go && mbar_wait(su32(gfull + i % ng), (i / ng) & 1, abort_flag, wl.limit);
+      for (int ky = 0; ky < 3 && go; ++ky) {
+        const int item = 3 * i + ky, st = item % kDwAcc;
+        if (item >= kDwAcc && !mbar_wait(su32(tempty + st), (item / kDwAcc - 1) & 1, abort_flag, wl.limit)) {
+          go = false;
+          break;
+        }
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        // descriptors by addition to the start address field (in 16-byte
+        // units: shared memory ends below its 14 bits)
+        unsigned long long xd = smem_desc_sw64_mn(su32(Xs + (size_t)((xb + ky) % nx) * kDwParts * xp), 64);
+        unsigned long long gd = smem_desc_sw64_mn(su32(Gs + (size_t)(i % ng) * kDwParts * gp), (unsigned)gp);
+        const unsigned d = tmem + (unsigned)(st * 32 * kDwParts);
+        for (int s = 0; s < Wp / 16; ++s, xd += 1024 >> 4, gd += 1024 >> 4)
+#pragma unroll
+          for (int a = 0; a < kDwParts; ++a)
+            mma_bf16(d, xd + (unsigned)(a * (xp >> 4)), gd, idesc_bf16(kTcM, 32 * (kDwParts - a), true),
+                     a > 0 || s > 0 ? 1u : 0u);
+        mma_commit(su32(tfull + st));
+      }
+      if (!go) break;
+      mma_commit(su32(gempty + i % ng));
+      mma_commit(su32(xempty + xb % nx));
+      if (y == H - 1 || q == q1 - 1) {
+        // the run of rows ends here: its last two input rows are free as well
+        mma_commit(su32(xempty + (xb + 1) % nx));
+        mma_commit(su32(xempty + (xb + 2) % nx));
+        xb += 3;
+      } else {
+        ++xb;
+      }
+    }
+    if (!go) {
+      atomicExch(err, 1);
+      *abort_flag = 1;
+    }
+    mma_commit(su32(done));  // every product this thread issued
+  } else if (warp < 3) {
+    // warp kx, lane ci: the sums of the 32 outputs for each ky
+    float acc[3][32];
+#pragma unroll
+    for (int ky = 0; ky < 3; ++ky)
+#pragma unroll
+      for (int c = 0; c < 32; ++c) acc[ky][c] = 0.f;
+    bool ok = true;
+    for (int i = 0; i < q1 - q0 && ok; ++i) {
+#pragma unroll
+      for (int ky = 0; ky < 3; ++ky) {
+        const int item = 3 * i + ky, st = item % kDwAcc;
+        ok = ok && *abort_flag == 0 && mbar_wait(su32(tfull + st), (item / kDwAcc) & 1, abort_flag, wl.limit);
+        ok = __all_sync(0xffffffffu, ok);  // tcgen05.ld is warp-collective
+        if (!ok) break;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          float v[kDwParts][16];
+#pragma unroll
+          for (int b = 0; b < kDwParts; ++b)
+            tmem_ld16(tmem + ((unsigned)(warp * 32) << 16) + (unsigned)((st * kDwParts + b) * 32 + h * 16), v[b]);
+#pragma unroll
+          for (int c = 0; c < 16; ++c) acc[ky][16 * h + c] += v[0][c] + (v[1][c] + v[2][c]);
+        }
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) mbar_arrive(su32(tempty + st));
+      }
+    }
+    if (!ok && lane == 0) {
+      atomicExch(err, 1);
+      *abort_flag = 1;
+    }
+    float4 *out = reinterpret_cast<float4 *>(part + ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * 9 * 1024);
+#pragma unroll
+    for (int ky = 0; ky < 3; ++ky)
+#pragma unroll
+      for (int c = 0; c < 8; ++c) {
+        const float nan = __int_as_float(0x7fc00000);
+        out[(size_t)((ky * 3 + warp) * 32 + lane) * 8 + c] =
+            ok ? make_float4(acc[ky][4 * c], acc[ky][4 * c + 1], acc[ky][4 * c + 2], acc[ky][4 * c + 3])
+               : make_float4(nan, nan, nan, nan);
+      }
+  }
+  __syncwarp();
+  // everything issued has landed before shared and tensor memory are released
+  if (warp == 4 && lane == 0) {
+    const long long t0 = clock64();
+    for (int s = 0; s < nx && s < xs; ++s)
+      while (!mbar_test(su32(xfull + s), ((xs - 1 - s) / nx) & 1) && clock64() - t0 < wl.limit) {
+      }
+    for (int s = 0; s < ng && s < gs; ++s)
+      while (!mbar_test(su32(gfull + s), ((gs - 1 - s) / ng) & 1) && clock64() - t0 < wl.limit) {
+      }
+  }
+  if (warp == 5 && lane == 0) {
+    const long long t0 = clock64();
+    while (!mbar_test(su32(done), 0) && clock64() - t0 < wl.limit) {
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (warp == 5) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+}
+
+// dw[co][ci][tap] += the sum of the CTAs' partials [slice][cta][tap][32 ci][32
+// co] and db[co] += that of part_b[block][32], in a fixed order: block (tap,
+// ci) of each slice, and a last one for db; 8 runs of the partials side by
+// side in FP32 (about 20 terms each), joined in FP64.
+__global__ void __launch_bounds__(256) k_dw_reduce(const float *__restrict__ part, int ctas, int Ci,
+                                                   float *__restrict__ dw, const float *__restrict__ part_b,
+                                                   int blocks, float *__restrict__ db) {
+  __shared__ double red[8][32];
+  const int co = threadIdx.x & 31, run = threadIdx.x >> 5;
+  const bool bias = blockIdx.x == gridDim.x - 1;
+  const int slice = blockIdx.x / (9 * 32), r = blockIdx.x % (9 * 32), tap = r / 32, ci = slice * 32 + r % 32;
+  const float *p = bias ? part_b : part + ((size_t)slice * ctas * 9 * 32 + r) * 32;
+  const size_t step = bias ? 32 : (size_t)9 * 1024;
+  const int n = bias ? blocks : ctas;
+  float f = 0.f;
+#pragma unroll 8
+  for (int c = run; c < n; c += 8) f += p[c * step + co];
+  double s = f;
+  red[run][co] = s;
+  __syncthreads();
+  if (run > 0 || (!bias && ci >= Ci)) return;
+  for (int q = 1; q < 8; ++q) s += red[q][co];
+  if (bias)
+    db[co] += (float)s;
+  else
+    dw[((long)co * Ci + ci) * 9 + tap] += (float)s;
 }
 
 // wt[ci][co][8 - tap] = w[co][ci][tap]: the adjoint of a 3x3 convolution with
@@ -901,6 +1223,13 @@ struct UnetImpl {
   // precision): the lo half of the converted input, the split weights of
   // one 32-channel output block
   int train_tc = 0;  // operand parts of the training convolutions on the tensor cores (0: CUDA cores)
+  // the split inputs of every convolution, kept by the training forward for
+  // the weight gradients, the split gradient of the current output, and the
+  // partial sums (dw_ready: allocated for the current (B, n))
+  bool dw_ready = false;
+  std::vector<__nv_bfloat16 *> xsplit;  // 3 per layer
+  __nv_bfloat16 *gsplit[3] = {nullptr, nullptr, nullptr};
+  float *dw_part = nullptr, *db_part = nullptr;
   __nv_bfloat16 *nhwc_lo = nullptr, *nhwc_p2 = nullptr, *wsp_hi = nullptr, *wsp_lo = nullptr, *wsp_p2 = nullptr;
   std::vector<MapEntry> maps;
 };
@@ -930,6 +1259,17 @@ void free_acts(UnetImpl *u) {
   for (__nv_bfloat16 *q : u->hcat)
     if (q) vie_free(q);
   u->hcat.clear();
+  for (__nv_bfloat16 *q : u->xsplit)
+    if (q) vie_free(q);
+  u->xsplit.clear();
+  for (__nv_bfloat16 *&q : u->gsplit) {
+    if (q) vie_free(q);
+    q = nullptr;
+  }
+  if (u->dw_part) vie_free(u->dw_part);
+  if (u->db_part) vie_free(u->db_part);
+  u->dw_part = u->db_part = nullptr;
+  u->dw_ready = false;
   u->maps.clear();
   u->o = u->go = nullptr;
   u->part = nullptr;
@@ -1067,6 +1407,7 @@ struct NhwcIo {
   long oh_bs = 0;
   int oh_cp = 0, oh_c0 = 0;
   bool wrote = false;  // set when out_h was written
+  __nv_bfloat16 *const *split = nullptr;  // split-precision convolutions: where the input's parts go (kept)
 };
 
 // the input's tensor map: NHWC BF16 at src, S slices; tiles of one row load
@@ -1169,16 +1510,13 @@ vie_status conv3_tma(UnetImpl *u, const float *in, long in_bs, int Ci, const __n
 // and packed per block of 32 output channels, one launch per block.
 bool conv_split_ok(int Ci, int Co) { return Ci <= 2 * kTmaSlice && Co % 32 == 0 && Co <= 64; }
 
-vie_status conv3_split(UnetImpl *u, const float *in, long in_bs, int Ci, const float *w, const float *bias,
-                       float *out, long out_bs, int Co, int H, int W, int B, bool relu, int np, cudaStream_t st) {
-  const int S = (Ci + kTmaSlice - 1) / kTmaSlice, Cp = S * kTmaSlice;
+// the same from an input that is already split (xin: np parts)
+vie_status conv3_split_run(UnetImpl *u, __nv_bfloat16 *const *xin, int Ci, const float *w, const float *bias,
+                           float *out, long out_bs, int Co, int H, int W, int B, bool relu, int np,
+                           cudaStream_t st) {
+  const int S = (Ci + kTmaSlice - 1) / kTmaSlice;
   const long plane = (long)H * W;
-  __nv_bfloat16 *xin[3] = {u->nhwc, u->nhwc_lo, u->nhwc_p2}, *wsp[3] = {u->wsp_hi, u->wsp_lo, u->wsp_p2};
-  if (np == 3)
-    k_to_nhwc_split<3><<<gridn((long)B * plane), 256, 0, st>>>(in, in_bs, Ci, plane, Cp, B, xin[0], xin[1], xin[2]);
-  else
-    k_to_nhwc_split<2><<<gridn((long)B * plane), 256, 0, st>>>(in, in_bs, Ci, plane, Cp, B, xin[0], xin[1], xin[2]);
-  VIE_CHECK_LAUNCH("k_to_nhwc_split");
+  __nv_bfloat16 *wsp[3] = {u->wsp_hi, u->wsp_lo, u->wsp_p2};
   CUtensorMap mx[3], mw[3];
   for (int q = 0; q < np; ++q) {
     VIE_TRY(conv_input_map(u, xin[q], S, H, W, B, &mx[q]));
@@ -1194,6 +1532,21 @@ vie_status conv3_split(UnetImpl *u, const float *in, long in_bs, int Ci, const f
   return VIE_OK;
 }
 
+vie_status conv3_split(UnetImpl *u, const float *in, long in_bs, int Ci, const float *w, const float *bias,
+                       float *out, long out_bs, int Co, int H, int W, int B, bool relu, int np, cudaStream_t st,
+                       const NhwcIo *io) {
+  const int S = (Ci + kTmaSlice - 1) / kTmaSlice, Cp = S * kTmaSlice;
+  const long plane = (long)H * W;
+  __nv_bfloat16 *own[3] = {u->nhwc, u->nhwc_lo, u->nhwc_p2};
+  __nv_bfloat16 *const *xin = io && io->split ? io->split : own;
+  if (np == 3)
+    k_to_nhwc_split<3><<<gridn((long)B * plane), 256, 0, st>>>(in, in_bs, Ci, plane, Cp, B, xin[0], xin[1], xin[2]);
+  else
+    k_to_nhwc_split<2><<<gridn((long)B * plane), 256, 0, st>>>(in, in_bs, Ci, plane, Cp, B, xin[0], xin[1], xin[2]);
+  VIE_CHECK_LAUNCH("k_to_nhwc_split");
+  return conv3_split_run(u, xin, Ci, w, bias, out, out_bs, Co, H, W, B, relu, np, st);
+}
+
 // io (tensor-core path only; ignored, with io->wrote false, on the CUDA cores)
 template <typename WT>
 vie_status conv3(UnetImpl *u, const float *in, long in_bs, int Ci, const WT *w, const __nv_bfloat16 *wtc,
@@ -1205,7 +1558,7 @@ vie_status conv3(UnetImpl *u, const float *in, long in_bs, int Ci, const WT *w, 
       return conv3_tma(u, in, in_bs, Ci, wtc, bias, out, out_bs, Co, H, W, B, relu, st, io);
   } else {
     if (u->train_tc > 1 && conv_split_ok(Ci, Co))
-      return conv3_split(u, in, in_bs, Ci, w, bias, out, out_bs, Co, H, W, B, relu, u->train_tc, st);
+      return conv3_split(u, in, in_bs, Ci, w, bias, out, out_bs, Co, H, W, B, relu, u->train_tc, st, io);
   }
   if (relu)
     conv3_shape<true, WT>(in, in_bs, Ci, w, bias, out, out_bs, Co, H, W, B, st);
@@ -1245,6 +1598,10 @@ vie_status forward(UnetImpl *u, const WT *pw, const float *x, int B, int n, cuda
   // decoder's concatenation
   const int cp1 = ((C + 31) / 32) * 32, cp2 = ((2 * C + 31) / 32) * 32;
   const bool handoff = tc && C % 8 == 0;
+  // training: a layer's split input stays for its weight gradient
+  auto kept = [&](const ConvLayer &c) -> __nv_bfloat16 *const * {
+    return u->train_tc == 3 && u->dw_ready ? &u->xsplit[3 * (&c - u->layers.data())] : nullptr;
+  };
   std::vector<char> skip_h(L, 0);
   for (int l = 0; l < L; ++l) {
     const int H = n >> l;
@@ -1256,6 +1613,7 @@ vie_status forward(UnetImpl *u, const WT *pw, const float *x, int B, int n, cuda
       io1.oh_bs = hw * cp1;
       io1.oh_cp = cp1;
     }
+    io1.split = kept(c1);
     if ((s = conv3(u, xl, xl_bs, c1.ci, pw + c1.w_off, wtc(c1), u->p + c1.b_off, u->a[l], (long)C * hw, C, H,
                    H, B, true, st, &io1)) != VIE_OK)
       return s;
@@ -1263,6 +1621,7 @@ vie_status forward(UnetImpl *u, const WT *pw, const float *x, int B, int n, cuda
     const long e_bs = l < L - 1 ? 2L * C * hw : (long)C * hw;
     NhwcIo io2;
     io2.in_h = io1.wrote ? u->hx : nullptr;
+    io2.split = kept(c2);
     if (handoff && l < L - 1) {
       io2.out_h = u->hcat[l];
       io2.oh_bs = hw * cp2;
@@ -1288,6 +1647,8 @@ vie_status forward(UnetImpl *u, const WT *pw, const float *x, int B, int n, cuda
     const long hw = (long)H * H;
     const ConvLayer &c1 = u->layers[li++], &c2 = u->layers[li++];
     NhwcIo io1, io2;
+    io1.split = kept(c1);
+    io2.split = kept(c2);
     if (skip_h[l] && conv_on_tensor_cores(wtc(c1), c1.ci, c1.co, u->p + c1.b_off)) {
       // the upsampled half in BF16 beside the skip the encoder wrote; the FP32
       // concatenation's first half is not written (vie_unet_layer_io rebuilds it)
@@ -1319,6 +1680,85 @@ vie_status forward(UnetImpl *u, const WT *pw, const float *x, int B, int n, cuda
   k_head<WT><<<gridn((long)B * n * n), 256, 0, st>>>(d, d_bs, C, pw + hd.w_off, u->p + hd.b_off, u->o,
                                                      (long)n * n, B);
   VIE_CHECK_LAUNCH("k_head");
+  return VIE_OK;
+}
+
+// the weight gradients of training take the tensor cores (k_conv3_dw_tc)
+bool dw_on_tensor_cores(const UnetImpl *u) { return u->C == 32; }
+
+// buffers of the tensor-core weight gradients for the current (B, n)
+vie_status alloc_dw(UnetImpl *u) {
+  DevProps prop;
+  VIE_TRY(get_dev_props(u->device, &prop));
+  u->xsplit.assign(3 * u->layers.size(), nullptr);
+  for (size_t i = 0; i < u->layers.size(); ++i) {
+    const ConvLayer &c = u->layers[i];
+    if (c.k != 3) continue;
+    const int l = (int)i < 2 * u->L ? (int)i / 2 : u->L - 2 - ((int)i - 2 * u->L) / 2;
+    const size_t px = (size_t)u->B * (u->n >> l) * (u->n >> l), Cp = (size_t)(c.ci + 31) / 32 * 32;
+    for (int q = 0; q < 3; ++q) VIE_CUDA(vie_malloc((void **)&u->xsplit[3 * i + q], sizeof(__nv_bfloat16) * px * Cp));
+  }
+  const size_t px = (size_t)u->B * u->n * u->n;
+  for (__nv_bfloat16 *&q : u->gsplit) VIE_CUDA(vie_malloc((void **)&q, sizeof(__nv_bfloat16) * px * 32));
+  VIE_CUDA(vie_malloc((void **)&u->dw_part, sizeof(float) * (size_t)prop.multiProcessorCount * 9 * 1024));
+  VIE_CUDA(vie_malloc((void **)&u->db_part, sizeof(float) * 32 * (px / 64 < 1024 ? px / 64 + 1 : std::max<size_t>(1024, px / 512 + 1))));
+  u->dw_ready = true;
+  return VIE_OK;
+}
+
+vie_status ensure_dw(UnetImpl *u) {
+  if (u->dw_ready || !dw_on_tensor_cores(u)) return VIE_OK;
+  const vie_status s = alloc_dw(u);
+  if (s != VIE_OK) free_acts(u);  // what was allocated goes with the activations
+  return s;
+}
+
+// tensor map of NHWC rows: boxes of 32 channels x `bw` pixels of one row
+vie_status conv_row_map(UnetImpl *u, const __nv_bfloat16 *src, int Cp, int H, int W, int B, int bw, CUtensorMap *m) {
+  const unsigned long long key[4] = {(unsigned long long)Cp | ((unsigned long long)bw << 32), (unsigned long long)W,
+                                     (unsigned long long)H, (unsigned long long)B | (1ull << 40)};
+  const unsigned long long dims[4] = {(unsigned long long)Cp, (unsigned long long)W, (unsigned long long)H,
+                                      (unsigned long long)B};
+  const unsigned long long strides[3] = {2ull * Cp, 2ull * Cp * W, 2ull * Cp * W * H};
+  const unsigned box[4] = {(unsigned)kTmaSlice, (unsigned)bw, 1u, 1u};
+  return cached_map(u, src, key, 4, dims, strides, box, m);
+}
+
+// The backward pass of one 3x3 convolution with ReLU (output `act`) on the
+// tensor cores: gout is masked by act > 0 and split once, for the weight
+// gradient (three parts), the bias gradient's sums and the input gradient (the
+// first two parts).
+vie_status conv3_backward_tc(UnetImpl *u, const ConvLayer &c, const float *gout, long g_bs, const float *act,
+                             long a_bs, float *gin, long gin_bs, int H, int B, cudaStream_t st) {
+  const long hw = (long)H * H;
+  const int blocks = split_blocks(B * hw);
+  k_mask_split<<<blocks, 256, 0, st>>>(gout, g_bs, act, a_bs, hw, B, u->gsplit[0], u->gsplit[1], u->gsplit[2],
+                                       u->db_part, split_steps(B * hw));
+  VIE_CHECK_LAUNCH("k_mask_split");
+  DevProps prop;
+  VIE_TRY(get_dev_props(u->device, &prop));
+  const int S = (c.ci + kTmaSlice - 1) / kTmaSlice, Wp = std::min(kTcM, (H + 15) / 16 * 16);
+  const int segs = (H + kTcM - 1) / kTcM;
+  const int ctas = (int)std::max(1L, std::min((long)prop.multiProcessorCount / S, (long)B * segs * H));
+  DwMaps maps;
+  const size_t layer = &c - u->layers.data();
+  for (int q = 0; q < kDwParts; ++q) {
+    VIE_TRY(conv_row_map(u, u->xsplit[3 * layer + q], S * kTmaSlice, H, H, B, Wp + 2, &maps.x[q]));
+    VIE_TRY(conv_row_map(u, u->gsplit[q], 32, H, H, B, Wp, &maps.g[q]));
+  }
+  const size_t smem = dw_smem(Wp);
+  VIE_TRY(raise_smem_limit((const void *)k_conv3_dw_tc, smem));
+  k_conv3_dw_tc<<<dim3((unsigned)ctas, (unsigned)S), kConvThreads, smem, st>>>(
+      maps, H, H, B, Wp, segs, u->dw_part, wait_limits(u->device), u->dev_err);
+  VIE_CHECK_LAUNCH("k_conv3_dw_tc");
+  k_dw_reduce<<<S * 9 * 32 + 1, 256, 0, st>>>(u->dw_part, ctas, c.ci, u->g + c.w_off, u->db_part,
+                                                               blocks, u->g + c.b_off);
+  VIE_CHECK_LAUNCH("k_dw_reduce");
+  if (gin) {
+    k_flip<<<gridn((long)c.co * c.ci * 9), 256, 0, st>>>(u->p + c.w_off, c.co, c.ci, u->wt);
+    VIE_CHECK_LAUNCH("k_flip");
+    VIE_TRY(conv3_split_run(u, u->gsplit, c.co, u->wt, nullptr, gin, gin_bs, c.ci, H, H, B, false, 2, st));
+  }
   return VIE_OK;
 }
 
@@ -1358,6 +1798,13 @@ vie_status relu_mask(float *g, long g_bs, const float *a, long a_bs, long per, i
 vie_status backward(UnetImpl *u, const float *x, int B, int n, cudaStream_t st) {
   const int L = u->L, C = u->C;
   vie_status s;
+  // one convolution's backward pass; gout is masked by its ReLU's output act first
+  auto back = [&](const ConvLayer &c, const float *in, long in_bs, float *gout, long g_bs, const float *act,
+                  long a_bs, float *gin, long gin_bs, int H) -> vie_status {
+    if (u->dw_ready) return conv3_backward_tc(u, c, gout, g_bs, act, a_bs, gin, gin_bs, H, B, st);
+    VIE_TRY(relu_mask(gout, g_bs, act, a_bs, (long)C * H * H, B, st));
+    return conv3_backward(u, c, in, in_bs, gout, g_bs, gin, gin_bs, H, B, st);
+  };
   int li = (int)u->layers.size() - 1;
   const ConvLayer &hd = u->layers[li];
   const float *d = L > 1 ? u->dl[0] : u->ebot[0];
@@ -1382,13 +1829,11 @@ vie_status backward(UnetImpl *u, const float *x, int B, int n, cudaStream_t st) 
     const long hw = (long)H * H;
     const ConvLayer &c2 = u->layers[li--];
     const ConvLayer &c1 = u->layers[li--];
-    if ((s = relu_mask(u->gdl[l], (long)C * hw, u->dl[l], (long)C * hw, (long)C * hw, B, st)) != VIE_OK) return s;
-    if ((s = conv3_backward(u, c2, u->bl[l], (long)C * hw, u->gdl[l], (long)C * hw, u->gbl[l], (long)C * hw, H, B,
-                            st)) != VIE_OK)
+    if ((s = back(c2, u->bl[l], (long)C * hw, u->gdl[l], (long)C * hw, u->dl[l], (long)C * hw, u->gbl[l],
+                  (long)C * hw, H)) != VIE_OK)
       return s;
-    if ((s = relu_mask(u->gbl[l], (long)C * hw, u->bl[l], (long)C * hw, (long)C * hw, B, st)) != VIE_OK) return s;
-    if ((s = conv3_backward(u, c1, u->cat[l], 2L * C * hw, u->gbl[l], (long)C * hw, u->gcat[l], 2L * C * hw, H, B,
-                            st)) != VIE_OK)
+    if ((s = back(c1, u->cat[l], 2L * C * hw, u->gbl[l], (long)C * hw, u->bl[l], (long)C * hw, u->gcat[l],
+                  2L * C * hw, H)) != VIE_OK)
       return s;
     // upsample part of the concat -> gradient of d_{l+1}
     float *gnext = (l + 1 <= L - 2) ? u->gdl[l + 1] : u->gebot[0];
@@ -1420,14 +1865,11 @@ vie_status backward(UnetImpl *u, const float *x, int B, int n, cudaStream_t st) 
       e = u->ebot[0];
       e_bs = (long)C * hw;
     }
-    if ((s = relu_mask(ge, ge_bs, e, e_bs, (long)C * hw, B, st)) != VIE_OK) return s;
-    if ((s = conv3_backward(u, c2, u->a[l], (long)C * hw, ge, ge_bs, u->ga[l], (long)C * hw, H, B, st)) != VIE_OK)
-      return s;
-    if ((s = relu_mask(u->ga[l], (long)C * hw, u->a[l], (long)C * hw, (long)C * hw, B, st)) != VIE_OK) return s;
+    if ((s = back(c2, u->a[l], (long)C * hw, ge, ge_bs, e, e_bs, u->ga[l], (long)C * hw, H)) != VIE_OK) return s;
     const float *xl = l == 0 ? x : u->xin[l];
     const long xl_bs = l == 0 ? 3L * hw : (long)C * hw;
-    if ((s = conv3_backward(u, c1, xl, xl_bs, u->ga[l], (long)C * hw, l > 0 ? u->gx[l] : nullptr,
-                            (long)C * hw, H, B, st)) != VIE_OK)
+    if ((s = back(c1, xl, xl_bs, u->ga[l], (long)C * hw, u->a[l], (long)C * hw, l > 0 ? u->gx[l] : nullptr,
+                  (long)C * hw, H)) != VIE_OK)
       return s;
   }
   return VIE_OK;
@@ -1436,7 +1878,7 @@ vie_status backward(UnetImpl *u, const float *x, int B, int n, cudaStream_t st) 
 vie_status loss_grad(UnetImpl *u, const float *x, const float *t, const float *wts, int B, int n, double *loss,
                      cudaStream_t st) {
   vie_status s;
-  if ((s = ensure_acts(u, B, n)) != VIE_OK) return s;
+  if ((s = ensure_acts(u, B, n)) != VIE_OK || (s = ensure_dw(u)) != VIE_OK) return s;
   // the training convolutions on the tensor cores in split precision: the
   // forward in three parts (24 significant bits, FP32's own: in two parts its
   // ~1e-5 relative error flipped the ReLU masks of pre-activations near zero,

@@ -42,6 +42,13 @@ __device__ __forceinline__ bool mbar_test(unsigned bar, unsigned parity) {
   return ok != 0;
 }
 
+// true in one lane of a converged warp
+__device__ __forceinline__ bool elect_one() {
+  unsigned r;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}" : "=r"(r));
+  return r != 0;
+}
+
 // Bounded wait on phase `parity` of an mbarrier; false on timeout or abort.
 // limit: clock cycles to wait; a zero limit gives up at once (no budget).
 __device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity, volatile int *abort_flag,
@@ -80,6 +87,19 @@ __device__ __forceinline__ unsigned long long smem_desc_sw64(unsigned addr) {
   return d;
 }
 
+// MN-major operand, 64-byte swizzle: rows of 64 bytes hold 32 consecutive
+// elements along M (or N) of one k, 8 rows (k) per 512-byte group; the next 32
+// elements along M lie `lead` bytes on.
+__device__ __forceinline__ unsigned long long smem_desc_sw64_mn(unsigned addr, unsigned lead) {
+  unsigned long long d = 0;
+  d |= (unsigned long long)((addr >> 4) & 0x3FFF);        // start address
+  d |= (unsigned long long)(lead >> 4) << 16;             // leading byte offset
+  d |= (unsigned long long)(512 >> 4) << 32;              // stride byte offset
+  d |= 1ull << 46;                                        // descriptor version
+  d |= 4ull << 61;                                        // 64-byte swizzle
+  return d;
+}
+
 // Tiled TMA loads into shared memory, completing on an mbarrier (coordinates
 // innermost first; the innermost times the element size a multiple of 16 B).
 __device__ __forceinline__ void tma_load_2d(unsigned dst, const void *map, unsigned bar, int x, int y) {
@@ -98,9 +118,10 @@ __device__ __forceinline__ void tma_load_4d(unsigned dst, const void *map, unsig
       : "memory");
 }
 
-// kind::f16 instruction descriptor: D F32, A and B BF16, both K-major.
-__host__ __device__ constexpr unsigned idesc_bf16(int M, int N) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((unsigned)(N >> 3) << 17) | ((unsigned)(M >> 4) << 24);
+// kind::f16 instruction descriptor: D F32, A and B BF16, both K-major (mn:
+// both MN-major).
+__host__ __device__ constexpr unsigned idesc_bf16(int M, int N, bool mn = false) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | (mn ? (1u << 15) | (1u << 16) : 0u) | ((unsigned)(N >> 3) << 17) | ((unsigned)(M >> 4) << 24);
 }
 
 __device__ __forceinline__ void mma_bf16(unsigned tmem_d, unsigned long long a, unsigned long long b,
