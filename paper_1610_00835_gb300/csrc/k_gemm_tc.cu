@@ -311,8 +311,9 @@ __global__ void __launch_bounds__(128, 1)
       tma_load_2d(su32(st + 2 * a_bytes + 2 * b_bytes), &map_glo, full, kx, 0);
       ++issued_loads;
     }
-  } else if (warp == 1 && lane == 0) {
-    // MMA issuer
+  } else if (warp == 1 && elect_one()) {
+    // MMA issuer (one elected lane: the compiler then keeps the descriptors in
+    // uniform registers)
     for (int i = 0; i < nkb; ++i) {
       const int s = i % STAGES, use = i / STAGES;
       if (!mbar_wait(su32(bars + s), use & 1, abort_flag, i == 0 ? a.wl.first : a.wl.limit)) {
@@ -322,9 +323,9 @@ __global__ void __launch_bounds__(128, 1)
       }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       unsigned char *st = stages + s * stage_bytes;
-      const unsigned a_hi = su32(st), a_lo = su32(st + a_bytes);
-      const unsigned b_hi = su32(st + 2 * a_bytes), b_mid = su32(st + 2 * a_bytes + b_bytes);
-      const unsigned b_lo = su32(st + 2 * a_bytes + 2 * b_bytes);
+      const unsigned long long a_hi = smem_desc_sw128(su32(st)), a_lo = smem_desc_sw128(su32(st + a_bytes));
+      const unsigned long long b_hi = smem_desc_sw128(su32(st + 2 * a_bytes));
+      const unsigned long long b_mid = smem_desc_sw128(su32(st + 2 * a_bytes + b_bytes));
       // accumulator columns: main_q at q * rpad (q < n_main); after them the
       // cross block of 2 rpad columns, [Khi Gmid + Klo Ghi | Khi Glo + Klo Gmid]
       const int q = i % a.n_main;
@@ -332,14 +333,14 @@ __global__ void __launch_bounds__(128, 1)
       const unsigned d_cross = tmem + (unsigned)(a.n_main * a.rpad);
 #pragma unroll
       for (int kk = 0; kk < BK / UMMA_K; ++kk) {
-        const unsigned off = kk * UMMA_K * 2;  // bytes along the swizzled row
+        const unsigned off = kk * UMMA_K * 2 / 16;  // along the swizzled row, in the descriptor's 16-byte units
         const unsigned first_main = (i < a.n_main && kk == 0) ? 0u : 1u;
         const unsigned first_cross = (i == 0 && kk == 0) ? 0u : 1u;
-        mma_bf16(d_main, smem_desc_sw128(a_hi + off), smem_desc_sw128(b_hi + off), idesc, first_main);
+        mma_bf16(d_main, a_hi + off, b_hi + off, idesc, first_main);
         // the G slices sit back to back, so [Gmid; Glo] and [Ghi; Gmid] are
         // operands of 2 rpad rows: one instruction each for Khi and Klo
-        mma_bf16(d_cross, smem_desc_sw128(a_hi + off), smem_desc_sw128(b_mid + off), idesc2, first_cross);
-        mma_bf16(d_cross, smem_desc_sw128(a_lo + off), smem_desc_sw128(b_hi + off), idesc2, 1u);
+        mma_bf16(d_cross, a_hi + off, b_mid + off, idesc2, first_cross);
+        mma_bf16(d_cross, a_lo + off, b_hi + off, idesc2, 1u);
       }
       mma_commit(su32(bars + STAGES + s));  // frees the stage once these MMAs finish
       ++issued_mma;
