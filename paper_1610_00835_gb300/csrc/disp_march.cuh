@@ -225,5 +225,10 @@ __device__ __forceinline__ void red_add(unsigned long long *p, unsigned long lon
   asm volatile("red.global.add.u64 [%0], %1;" ::"l"(p), "l"(v));
 }
 
+// the same at a 32-bit byte offset
+__device__ __forceinline__ void red_add(char *base, unsigned off, unsigned long long v) {
+  asm volatile("red.global.add.u64 [%0], %1;" ::"l"(base + off), "l"(v));
+}
+
 }  // namespace dmarch
 }  // namespace vie

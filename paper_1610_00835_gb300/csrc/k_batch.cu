@@ -383,9 +383,8 @@ vie_status enqueue_one(vie_batch *b, int op, const double *g, double *y, cudaStr
     if (b->use_disp[i]) {
       const DispPlan &dp = b->disp[i];
       const double h = 1.0 / G.n;
-      if ((s = disp_source(dp, G.N, op, b->sig_s + off, g + off, b->src + off, st)) != VIE_OK) return s;
-      if ((s = disp_launch(dp, G.n, (float)(h / kS * 1.4426950408889634), (float)(h / (2.0 * kPi)), b->src + off,
-                           st)) != VIE_OK)
+      if ((s = disp_source(dp, G.N, op, b->sig_s + off, g + off, st)) != VIE_OK) return s;
+      if ((s = disp_launch(dp, G.n, (float)(h / kS * 1.4426950408889634), (float)(h / (2.0 * kPi)), st)) != VIE_OK)
         return s;
       if ((s = disp_reduce(dp, G.N, op, b->diag + off, b->sig_s + off, g + off, y + off, st)) != VIE_OK) return s;
       k += 3;

@@ -99,8 +99,7 @@ struct DispArgs {
   const float *lat;            // [n + R][ldp] sigma_t on the cell lattice, edge repeated
   const float *lat_t;          // global-lattice kernels: the same lattice with y fastest
   const float4 *stencil;       // chunk records of every W_D
-  const float *src;            // s_k, FP32 [N]
-  const float *src_t;          // s transposed: s at (x, y) is src_t[x n + y]
+  const float *src;            // s, FP32 [2 N]: s at (x, y) in [y n + x] and in [N + x n + y]
   const float *wtab;           // M-ii: h / (2 pi) times the cell integral of 1/|z| per D
                                // of the half plane (disp_index order); null for M-iii
   unsigned *smax;              // bits of max |s_k| (set by the source kernel)
@@ -232,12 +231,22 @@ __device__ __forceinline__ void disp_body(const DispArgs &a) {
     const int wx = xhi - xlo;
     // sums of targets on consecutive x (runs along y) go to yacc with x
     // fastest, those on consecutive y (runs along x) to its second half with
-    // y fastest, so a warp's atomics cover contiguous words; s and its
-    // transpose follow the same layouts.  Stacked targets are n apart in both.
-    const float *sv = along_y ? a.src : a.src_t;
-    unsigned long long *ya = along_y ? a.yacc : a.yacc + N;
-    const long j0 = along_y ? (long)y * n + x : (long)x * n + y;
-    const long dk = along_y ? (long)dy * n + dx : (long)dx * n + dy;
+    // y fastest, so a warp's atomics cover contiguous words; s is kept in both
+    // layouts the same way.  Stacked targets are n apart in both.  The epilogue
+    // is a quarter of all instructions, so its addresses are 32-bit offsets
+    // from the kernel's pointers (one addition each; 64-bit pointers that
+    // depended on the run axis took three times as many instructions).
+    const unsigned jb = (along_y ? (unsigned)(y * n + x) : (unsigned)N + (unsigned)(x * n + y)) * 4u;
+    const unsigned kb = jb + 4u * (unsigned)(along_y ? dy * n + dx : dx * n + dy);
+    const unsigned n4 = 4u * (unsigned)n;
+    const char *sb = reinterpret_cast<const char *>(a.src);
+    char *yb = reinterpret_cast<char *>(a.yacc);
+    // stacked targets of this lane
+    const int cnt = lvalid ? min(R, along_y ? yhi - y : xhi - x) : 0;
+    // stored weights of this lane's targets: row-major in D's rectangle
+    float *wp = nullptr;
+    const int wstep = along_y ? wx : 1;
+    if constexpr (MODE != kApply) wp = a.wbuf + woff + (long)(y - ylo) * wx + (x - xlo);
     if constexpr (MODE == kStream) {
       // four targets at a time: their global loads are issued before their atomics
 #pragma unroll
@@ -246,42 +255,41 @@ __device__ __forceinline__ void disp_body(const DispArgs &a) {
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           const int q = q0 + i;
-          const int xq = along_y ? x : x + q, yq = along_y ? y + q : y;
           wv[i] = sjv[i] = skv[i] = 0.f;
-          if (lvalid && (along_y ? yq < yhi : xq < xhi)) {
-            const long wi = woff + (long)(yq - ylo) * wx + (xq - xlo);
-            wv[i] = __ldcs(a.wbuf + wi);
-            sjv[i] = __ldg(sv + j0 + (long)q * n);
-            skv[i] = __ldg(sv + j0 + (long)q * n + dk);
+          if (q < cnt) {
+            wv[i] = __ldcs(wp + (long)q * wstep);
+            sjv[i] = __ldg(reinterpret_cast<const float *>(sb + (jb + (unsigned)q * n4)));
+            skv[i] = __ldg(reinterpret_cast<const float *>(sb + (kb + (unsigned)q * n4)));
           }
         }
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           const int q = q0 + i;
-          const int xq = along_y ? x : x + q, yq = along_y ? y + q : y;
-          if (lvalid && (along_y ? yq < yhi : xq < xhi)) {
+          if (q < cnt) {
             const float w = wv[i] * scale;
-            const long j = j0 + (long)q * n;
-            red_add(ya + j, (unsigned long long)__float2ll_rn(w * skv[i]));
-            red_add(ya + j + dk, (unsigned long long)__float2ll_rn(w * sjv[i]));
+            red_add(yb, 2u * (jb + (unsigned)q * n4), (unsigned long long)__float2ll_rn(w * skv[i]));
+            red_add(yb, 2u * (kb + (unsigned)q * n4), (unsigned long long)__float2ll_rn(w * sjv[i]));
           }
         }
       }
+    } else if constexpr (MODE == kStore) {
+#pragma unroll
+      for (int q = 0; q < R; ++q)
+        if (q < cnt) wp[(long)q * wstep] = wk * exp2f(tscale * acc[q]);
     } else {
+      // the scale is a power of two: applied to wk it changes no bit of a
+      // product (weights below 2^-126, where it could, add nothing in fixed
+      // point)
+      const float wks = wk * scale;
 #pragma unroll
       for (int q = 0; q < R; ++q) {
-        const int xq = along_y ? x : x + q, yq = along_y ? y + q : y;
-        if (lvalid && (along_y ? yq < yhi : xq < xhi)) {
-          const float wq = wk * exp2f(tscale * acc[q]);
-          if constexpr (MODE == kStore) {
-            a.wbuf[woff + (long)(yq - ylo) * wx + (xq - xlo)] = wq;
-          } else {
-            const long j = j0 + (long)q * n;
-            const float sj = __ldg(sv + j), sk = __ldg(sv + j + dk);
-            const float w = wq * scale;
-            red_add(ya + j, (unsigned long long)__float2ll_rn(w * sk));
-            red_add(ya + j + dk, (unsigned long long)__float2ll_rn(w * sj));
-          }
+        if (q < cnt) {
+          const unsigned oj = jb + (unsigned)q * n4, ok = kb + (unsigned)q * n4;
+          const float sj = __ldg(reinterpret_cast<const float *>(sb + oj));
+          const float sk = __ldg(reinterpret_cast<const float *>(sb + ok));
+          const float w = wks * exp2f(tscale * acc[q]);
+          red_add(yb, 2u * oj, (unsigned long long)__float2ll_rn(w * sk));
+          red_add(yb, 2u * ok, (unsigned long long)__float2ll_rn(w * sj));
         }
       }
     }
@@ -1047,7 +1055,7 @@ vie_status disp_prepare(DispPlan *dp, int n, const float *sig_padded, int device
   VIE_CUDA(vie_malloc((void **)&dp->smax, sizeof(unsigned)));
   VIE_CUDA(cudaMemset(dp->smax, 0, sizeof(unsigned)));
   VIE_CUDA(vie_malloc((void **)&dp->scale, sizeof(double)));
-  VIE_CUDA(vie_malloc((void **)&dp->src_t, sizeof(float) * (size_t)n * n));
+  VIE_CUDA(vie_malloc((void **)&dp->src2, sizeof(float) * 2 * (size_t)n * n));
   VIE_CUDA(vie_malloc((void **)&dp->ss32, sizeof(float) * (size_t)n * n));
   VIE_CUDA(vie_malloc((void **)&dp->yacc, sizeof(unsigned long long) * 2 * (size_t)n * n));
   VIE_CUDA(cudaMemset(dp->yacc, 0, sizeof(unsigned long long) * 2 * (size_t)n * n));
@@ -1078,7 +1086,7 @@ void disp_release(DispPlan *dp) {
   if (dp->lattice_t) vie_free(dp->lattice_t);
   if (dp->smax) vie_free(dp->smax);
   if (dp->scale) vie_free(dp->scale);
-  if (dp->src_t) vie_free(dp->src_t);
+  if (dp->src2) vie_free(dp->src2);
   if (dp->ss32) vie_free(dp->ss32);
   if (dp->yacc) vie_free(dp->yacc);
   if (dp->wtab) vie_free((void *)dp->wtab);
@@ -1086,7 +1094,7 @@ void disp_release(DispPlan *dp) {
   dp->yacc = nullptr;
   dp->ss32 = nullptr;
   dp->geometry = nullptr;
-  dp->src_t = nullptr;
+  dp->src2 = nullptr;
   dp->smax = nullptr;
   dp->scale = nullptr;
   dp->units = nullptr;
@@ -1099,10 +1107,9 @@ void disp_release(DispPlan *dp) {
   dp->usable = 0;
 }
 
-vie_status disp_source(const DispPlan &dp, long N, int op, const double *sigma_s, const double *g,
-                       float *src, cudaStream_t st) {
+vie_status disp_source(const DispPlan &dp, long N, int op, const double *sigma_s, const double *g, cudaStream_t st) {
   const int blocks = (int)std::min((N + 255) / 256, 1024L);
-  k_disp_source<<<blocks, 256, 0, st>>>(N, dp.n, op, sigma_s, g, src, dp.src_t, dp.smax);
+  k_disp_source<<<blocks, 256, 0, st>>>(N, dp.n, op, sigma_s, g, dp.src2, dp.src2 + N, dp.smax);
   VIE_CHECK_LAUNCH("k_disp_source");
   return VIE_OK;
 }
@@ -1181,13 +1188,12 @@ vie_status disp_reduce(const DispPlan &dp, long N, int op, const double *diag, c
 
 namespace {
 
-DispArgs disp_args(const DispPlan &dp, int n, float tau_scale2, float wcoef, const float *src, float *wbuf) {
+DispArgs disp_args(const DispPlan &dp, int n, float tau_scale2, float wcoef, float *wbuf) {
   DispArgs a;
   a.lat = (const float *)dp.lattice;
   a.lat_t = (const float *)dp.lattice_t;
   a.stencil = (const float4 *)dp.stencil;
-  a.src = src;
-  a.src_t = dp.src_t;
+  a.src = dp.src2;
   a.smax = dp.smax;
   a.scale_out = dp.scale;
   a.rbound = dp.rbound;
@@ -1208,9 +1214,8 @@ DispArgs disp_args(const DispPlan &dp, int n, float tau_scale2, float wcoef, con
 
 }  // namespace
 
-vie_status disp_launch(const DispPlan &dp, int n, float tau_scale2, float wcoef, const float *src,
-                       cudaStream_t st) {
-  DispArgs a = disp_args(dp, n, tau_scale2, wcoef, src, nullptr);
+vie_status disp_launch(const DispPlan &dp, int n, float tau_scale2, float wcoef, cudaStream_t st) {
+  DispArgs a = disp_args(dp, n, tau_scale2, wcoef, nullptr);
   void *args[] = {&a};
   VIE_CUDA(cudaLaunchKernel(dp.kernel, dim3(dp.grid), dim3(kThreads), args, dp.smem, st));
   count_launch();
@@ -1218,15 +1223,15 @@ vie_status disp_launch(const DispPlan &dp, int n, float tau_scale2, float wcoef,
 }
 
 vie_status disp_store(const DispPlan &dp, int n, float tau_scale2, float wcoef, float *wbuf, cudaStream_t st) {
-  DispArgs a = disp_args(dp, n, tau_scale2, wcoef, nullptr, wbuf);
+  DispArgs a = disp_args(dp, n, tau_scale2, wcoef, wbuf);
   void *args[] = {&a};
   VIE_CUDA(cudaLaunchKernel(dp.kernel_store, dim3(dp.grid_store), dim3(kThreads), args, dp.smem_store, st));
   count_launch();
   return VIE_OK;
 }
 
-vie_status disp_stream(const DispPlan &dp, int n, const float *wbuf, const float *src, cudaStream_t st) {
-  DispArgs a = disp_args(dp, n, 0.f, 0.f, src, const_cast<float *>(wbuf));
+vie_status disp_stream(const DispPlan &dp, int n, const float *wbuf, cudaStream_t st) {
+  DispArgs a = disp_args(dp, n, 0.f, 0.f, const_cast<float *>(wbuf));
   void *args[] = {&a};
   VIE_CUDA(cudaLaunchKernel(dp.kernel_stream, dim3(dp.grid_stream), dim3(kThreads), args, dp.smem_stream, st));
   count_launch();

@@ -425,7 +425,7 @@ vie_status apply_dev(vie_handle *h, int op, const double *g, double *y, cudaStre
     return VIE_OK;
   }
   vie_status s = h->use_kernel == VIE_KERNEL_DISPLACEMENT
-                     ? disp_source(h->disp, h->N, op, h->sig_s, g, (float *)h->src, st)
+                     ? disp_source(h->disp, h->N, op, h->sig_s, g, st)
                      : launch_source_prep(h->N, op, h->sig_s, g, prec, h->src, st);
   if (s != VIE_OK) return s;
   if (timed) VIE_CUDA(cudaEventRecord(ev->e[1], st));
@@ -435,9 +435,9 @@ vie_status apply_dev(vie_handle *h, int op, const double *g, double *y, cudaStre
   const float wcoef = (float)(h->dim == 2 ? hh / (2.0 * kPi) : hh / (4.0 * kPi));
   if (h->use_kernel == VIE_KERNEL_DISPLACEMENT) {
     if (h->asm_mode == VIE_OPERATOR_PAIRS32) {
-      s = disp_stream(h->disp, h->n, (const float *)h->kmat, (const float *)h->src, st);
+      s = disp_stream(h->disp, h->n, (const float *)h->kmat, st);
     } else {
-      s = disp_launch(h->disp, h->n, tau_scale2, wcoef, (const float *)h->src, st);
+      s = disp_launch(h->disp, h->n, tau_scale2, wcoef, st);
     }
   } else if (h->use_kernel == VIE_KERNEL_SYMMETRIC) {
     s = sym_launch(h->sym, h->dim, h->n, h->N, tau_scale2, wcoef, (const float *)h->src,

@@ -170,7 +170,7 @@ struct DispPlan {
   long n_units = 0, lat_elems = 0;
   int ldp = 0, grid = 0, n = 0;
   size_t smem = 0;
-  float *src_t = nullptr;     // s transposed (FP32 [N])
+  float *src2 = nullptr;      // s and its transpose (FP32 [2 N])
   float *ss32 = nullptr;      // sigma_s in FP32 (for the expansion into K)
   void *yacc = nullptr;       // int64 [2 N]: fixed-point sums (x fastest, then y fastest), zero between applies
   void *geometry = nullptr;   // shared stencils and units of this n (owned by a cache)
@@ -235,8 +235,7 @@ vie_status symv3_apply(const DispPlan3 &dp, int op, const double *sigma_s, const
 
 size_t disp_smem_bytes(int n, int R);  // shared lattice bytes at stack depth R
 bool disp_expand_fits(int n, int device);  // k_expand_pairs has room for the grid (n <= 169)
-vie_status disp_source(const DispPlan &dp, long N, int op, const double *sigma_s, const double *g,
-                       float *src, cudaStream_t st);
+vie_status disp_source(const DispPlan &dp, long N, int op, const double *sigma_s, const double *g, cudaStream_t st);
 vie_status disp_reduce(const DispPlan &dp, long N, int op, const double *diag, const double *sigma_s,
                        const double *g, double *y, cudaStream_t st);
 vie_status disp_prepare(DispPlan *dp, int n, const float *sig_padded, int device, cudaStream_t st);
@@ -244,8 +243,7 @@ vie_status disp_prepare(DispPlan *dp, int n, const float *sig_padded, int device
 // diagonal value A_jj (the same for every cell); widens rbound to its row sums
 vie_status disp_mii_prepare(DispPlan *dp, int n, double *diag_value, cudaStream_t st);
 void disp_release(DispPlan *dp);
-vie_status disp_launch(const DispPlan &dp, int n, float tau_scale2, float wcoef, const float *src,
-                       cudaStream_t st);
+vie_status disp_launch(const DispPlan &dp, int n, float tau_scale2, float wcoef, cudaStream_t st);
 vie_status disp_store(const DispPlan &dp, int n, float tau_scale2, float wcoef, float *wbuf, cudaStream_t st);
 int symv_max_n();  // largest grid the symmetric-block product takes (160)
 size_t symv_block_floats(int n);
@@ -254,7 +252,7 @@ vie_status symv_apply(int n, int op, const double *sigma_s, const double *g, con
                       float *partial, double *y, int device, cudaStream_t st);
 vie_status disp_expand(const DispPlan &dp, int n, const float *wbuf, const double *sigma_s, const double *diag,
                        long ldk, float *k32, void *khi, void *klo, int device, cudaStream_t st);
-vie_status disp_stream(const DispPlan &dp, int n, const float *wbuf, const float *src, cudaStream_t st);
+vie_status disp_stream(const DispPlan &dp, int n, const float *wbuf, cudaStream_t st);
 
 // integral of 1/|z| over the unit square centred at (t1, t2), FP64 (the
 // closed form of Remark REM: NEW KERNEL; k_pairs_disp.cu)
