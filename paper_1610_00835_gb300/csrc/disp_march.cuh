@@ -157,31 +157,88 @@ __device__ __forceinline__ const float4 *chunks2_smem(const float4 *__restrict__
   return rec;
 }
 
+// Two tiles of targets of one displacement: a chunk's record is loaded once
+// for both.
 template <int LC, int ST, int R>
-__device__ __forceinline__ const float4 *chunks2_global(const float4 *__restrict__ rec, int cnt,
-                                                        const float *__restrict__ base, Acc2<R> &s) {
+__device__ __forceinline__ const float4 *chunks2_smem_pair(const float4 *__restrict__ rec, int cnt, unsigned base_a,
+                                                           unsigned base_b, int st, Acc2<R> &sa, Acc2<R> &sb) {
   constexpr int RS = (LC + 4) / 4;
 #pragma unroll 1
   for (int c = 0; c < cnt; ++c, rec += RS) {
     int off;
     float w[LC];
     load_chunk<LC>(rec, off, w);
-    const float *p = base + off;
-    float v[LC + R - 1];
-#pragma unroll
-    for (int m = 0; m < LC + R - 1; ++m) v[m] = __ldg(p + ST * m);
-    taps2<LC, R>(w, v, s);
+    float v[LC + R - 1], u[LC + R - 1];
+    LoadRun<ST, 0, LC + R - 1>::go(base_a + 4u * (unsigned)off, st, v);
+    LoadRun<ST, 0, LC + R - 1>::go(base_b + 4u * (unsigned)off, st, u);
+    taps2<LC, R>(w, v, sa);
+    taps2<LC, R>(w, u, sb);
   }
   return rec;
 }
 
-// acc[q] = sum over the chunks of one unit of w(c) sigma[target q + c], the
+template <int LC, int ST, int R>
+__device__ __forceinline__ const float4 *chunks2_global_pair(const float4 *__restrict__ rec, int cnt,
+                                                             const float *__restrict__ base_a,
+                                                             const float *__restrict__ base_b, Acc2<R> &sa,
+                                                             Acc2<R> &sb) {
+  constexpr int RS = (LC + 4) / 4;
+#pragma unroll 1
+  for (int c = 0; c < cnt; ++c, rec += RS) {
+    int off;
+    float w[LC];
+    load_chunk<LC>(rec, off, w);
+    const float *p = base_a + off, *q = base_b + off;
+    float v[LC + R - 1], u[LC + R - 1];
+#pragma unroll
+    for (int m = 0; m < LC + R - 1; ++m) v[m] = __ldg(p + ST * m);
+#pragma unroll
+    for (int m = 0; m < LC + R - 1; ++m) u[m] = __ldg(q + ST * m);
+    taps2<LC, R>(w, v, sa);
+    taps2<LC, R>(w, u, sb);
+  }
+  return rec;
+}
+
+template <int ST, int R>
+__device__ __forceinline__ void march_runs_pair(const float4 *__restrict__ rec, unsigned base_a, unsigned base_b,
+                                                int st, Acc2<R> &sa, Acc2<R> &sb) {
+  const float4 hdr = __ldg(rec);
+  ++rec;
+  int c;
+  if ((c = chunk_count<1>(hdr)) > 0) rec = chunks2_smem_pair<1, ST, R>(rec, c, base_a, base_b, st, sa, sb);
+  if ((c = chunk_count<2>(hdr)) > 0) rec = chunks2_smem_pair<2, ST, R>(rec, c, base_a, base_b, st, sa, sb);
+  if ((c = chunk_count<3>(hdr)) > 0) rec = chunks2_smem_pair<3, ST, R>(rec, c, base_a, base_b, st, sa, sb);
+  if ((c = chunk_count<4>(hdr)) > 0) rec = chunks2_smem_pair<4, ST, R>(rec, c, base_a, base_b, st, sa, sb);
+  if ((c = chunk_count<5>(hdr)) > 0) rec = chunks2_smem_pair<5, ST, R>(rec, c, base_a, base_b, st, sa, sb);
+  if ((c = chunk_count<6>(hdr)) > 0) rec = chunks2_smem_pair<6, ST, R>(rec, c, base_a, base_b, st, sa, sb);
+  if ((c = chunk_count<7>(hdr)) > 0) rec = chunks2_smem_pair<7, ST, R>(rec, c, base_a, base_b, st, sa, sb);
+  if ((c = chunk_count<8>(hdr)) > 0) rec = chunks2_smem_pair<8, ST, R>(rec, c, base_a, base_b, st, sa, sb);
+}
+
+// The same with the lattice in global memory (read through L1): the chunk's
+// cells and stacked targets lie ST elements apart from base + offset.
+template <int ST, int R>
+__device__ __forceinline__ void march_runs_global_pair(const float4 *__restrict__ rec,
+                                                       const float *__restrict__ base_a,
+                                                       const float *__restrict__ base_b, Acc2<R> &sa, Acc2<R> &sb) {
+  const float4 hdr = __ldg(rec);
+  ++rec;
+  int c;
+  if ((c = chunk_count<1>(hdr)) > 0) rec = chunks2_global_pair<1, ST, R>(rec, c, base_a, base_b, sa, sb);
+  if ((c = chunk_count<2>(hdr)) > 0) rec = chunks2_global_pair<2, ST, R>(rec, c, base_a, base_b, sa, sb);
+  if ((c = chunk_count<3>(hdr)) > 0) rec = chunks2_global_pair<3, ST, R>(rec, c, base_a, base_b, sa, sb);
+  if ((c = chunk_count<4>(hdr)) > 0) rec = chunks2_global_pair<4, ST, R>(rec, c, base_a, base_b, sa, sb);
+  if ((c = chunk_count<5>(hdr)) > 0) rec = chunks2_global_pair<5, ST, R>(rec, c, base_a, base_b, sa, sb);
+  if ((c = chunk_count<6>(hdr)) > 0) rec = chunks2_global_pair<6, ST, R>(rec, c, base_a, base_b, sa, sb);
+  if ((c = chunk_count<7>(hdr)) > 0) rec = chunks2_global_pair<7, ST, R>(rec, c, base_a, base_b, sa, sb);
+  if ((c = chunk_count<8>(hdr)) > 0) rec = chunks2_global_pair<8, ST, R>(rec, c, base_a, base_b, sa, sb);
+}
+
+// s += the chunks of one unit: s.sum() then gives sum_c w(c) sigma[target q + c], the
 // lattice in shared memory (base: the first stacked target's byte address).
 template <int ST, int R>
-__device__ __forceinline__ void march_runs(const float4 *__restrict__ rec, unsigned base, int st,
-                                           float (&acc)[R]) {
-  Acc2<R> s;
-  s.zero();
+__device__ __forceinline__ void march_runs(const float4 *__restrict__ rec, unsigned base, int st, Acc2<R> &s) {
   const float4 hdr = __ldg(rec);
   ++rec;
   int c;
@@ -193,28 +250,6 @@ __device__ __forceinline__ void march_runs(const float4 *__restrict__ rec, unsig
   if ((c = chunk_count<6>(hdr)) > 0) rec = chunks2_smem<6, ST, R>(rec, c, base, st, s);
   if ((c = chunk_count<7>(hdr)) > 0) rec = chunks2_smem<7, ST, R>(rec, c, base, st, s);
   if ((c = chunk_count<8>(hdr)) > 0) rec = chunks2_smem<8, ST, R>(rec, c, base, st, s);
-  s.sum(acc);
-}
-
-// The same with the lattice in global memory (read through L1): the chunk's
-// cells and stacked targets lie ST elements apart from base + offset.
-template <int ST, int R>
-__device__ __forceinline__ void march_runs_global(const float4 *__restrict__ rec, const float *__restrict__ base,
-                                                  float (&acc)[R]) {
-  Acc2<R> s;
-  s.zero();
-  const float4 hdr = __ldg(rec);
-  ++rec;
-  int c;
-  if ((c = chunk_count<1>(hdr)) > 0) rec = chunks2_global<1, ST, R>(rec, c, base, s);
-  if ((c = chunk_count<2>(hdr)) > 0) rec = chunks2_global<2, ST, R>(rec, c, base, s);
-  if ((c = chunk_count<3>(hdr)) > 0) rec = chunks2_global<3, ST, R>(rec, c, base, s);
-  if ((c = chunk_count<4>(hdr)) > 0) rec = chunks2_global<4, ST, R>(rec, c, base, s);
-  if ((c = chunk_count<5>(hdr)) > 0) rec = chunks2_global<5, ST, R>(rec, c, base, s);
-  if ((c = chunk_count<6>(hdr)) > 0) rec = chunks2_global<6, ST, R>(rec, c, base, s);
-  if ((c = chunk_count<7>(hdr)) > 0) rec = chunks2_global<7, ST, R>(rec, c, base, s);
-  if ((c = chunk_count<8>(hdr)) > 0) rec = chunks2_global<8, ST, R>(rec, c, base, s);
-  s.sum(acc);
 }
 
 // Integer add whose old value nobody reads: the reduction form, with no

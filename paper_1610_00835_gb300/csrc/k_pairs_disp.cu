@@ -25,13 +25,15 @@
 // R Lc multiply-adds, issued as packed FP32 pairs (fma.rn.f32x2, two
 // stacked targets per instruction) in code unrolled for each Lc.  Lanes sit
 // on consecutive x (runs along y) or consecutive y with an odd row pitch
-// (runs along x), so every load is free of bank conflicts.
+// (runs along x), so every load is free of bank conflicts.  What bounds the
+// kernel is the L1 data pipe (lattice loads, record broadcasts) and issue.
 //
 // Work units are (D, block of the targets j with j + D inside the grid) for D
 // in a half plane (dy > 0, or dy = 0 and dx > 0): A_jk = A_kj, so each
 // unordered pair is marched once and feeds y_j (weight s_{j+D}) and y_{j+D}
-// (weight s_j).  Units are sorted by estimated cost, largest first, and warps
-// take them four at a time from a global counter.  Every term w s is rounded
+// (weight s_j).  Units are sorted by estimated cost, largest first (grids of 96
+// and more: by run axis before that), and warps take up to four at a time from
+// a global counter.  Every term w s is rounded
 // once to a multiple of 1/scale (64-bit fixed point, scale the power of two
 // at or below 2^62 / (max|s| R), R a bound on every row sum of A) and added
 // with an integer reduction (red.add, no value returned) into a global int64
@@ -70,8 +72,10 @@ namespace {
 using march::kS;
 
 using dmarch::kMaxChunk;
+using dmarch::Acc2;
 using dmarch::march_runs;
-using dmarch::march_runs_global;
+using dmarch::march_runs_global_pair;
+using dmarch::march_runs_pair;
 // R, the targets stacked along the run axis in one thread: 12 on grids of
 // 96 and more, 8 below (measured per apply: 8 / 12 took 0.100 / 0.107 ms at
 // 64^2, 0.550 / 0.519 at 100^2, 1.41 / 1.38 at 128^2, 42.9 / 38.3 at 256^2;
@@ -81,10 +85,30 @@ using dmarch::march_runs_global;
 // reach past the rectangle of targets (chunks carry no padding).
 using dmarch::red_add;
 constexpr int kThreads = 1024;
+// Tiles per unit, and threads per CTA of the marching kernels.  On grids of 96
+// and more a warp takes two tiles of one displacement and loads every record
+// once for both: a record load returns 16 bytes to each of 32 lanes, four
+// data-pipe wavefronts, 28 % of a single tile's.  The accumulators of two tiles
+// take 96 registers, so 640 threads; the code of the march doubles, which the
+// instruction cache only bears because units are sorted by run axis (warps run
+// one axis' loops at a time; unsorted 1977 us at 128^2) and the epilogue is one
+// loop over the tiles.  Measured per apply with one and two tiles: 424 / 419 us
+// at 97^2, 1282 / 1254 at 128^2 (512 threads 1374, 768 1263), 3470 / 3378 at
+// 160^2, 10075 / 9916 at 200^2.  Small grids have too few units per warp.
+__host__ __device__ constexpr int disp_tiles(int n) { return n >= 96 ? 2 : 1; }
+__host__ __device__ constexpr int disp_threads(int T) { return T == 2 ? 640 : kThreads; }
 __host__ __device__ constexpr int disp_depth(int n) { return n >= 96 ? 12 : 8; }
 // lattice pitch: room for R - 1 stacked targets past the grid, odd so that
 // 32 consecutive rows of one column fall in 32 different banks
 __host__ __device__ constexpr int disp_pitch(int n, int R) { return (n + R) | 1; }
+// Shared lattices take the next of these pitches, each compiled in: loads at
+// immediate offsets (a run-time stride adds an instruction per load).
+constexpr int kPitch8[] = {41, 57, 73, 89, 105}, kPitch12[] = {109, 141, 173, 205, 239};
+inline int shared_pitch(int n, int R) {
+  for (int p : (R == 8 ? kPitch8 : kPitch12))
+    if (disp_pitch(n, R) <= p) return p;
+  return disp_pitch(n, R);  // past the last: a run-time stride
+}
 // Lane groups of a ragged lane block sit s blocks apart along the stack, s R
 // rows of an odd pitch: s R = 16 (mod 32) for pairs and 8 or 24 for quads,
 // so the groups load from disjoint banks.
@@ -107,13 +131,14 @@ struct DispArgs {
   double rbound;               // bound on sum_k A_jk for every j
   unsigned long long *yacc;    // [2 N] int64 sums (x fastest, then y fastest), zero between applies
   const int4 *units;           // {the D's record header (float4 index), dx | dy << 16,
-                               //  lane block | stack block << 16,
-                               //  runs along y | lane groups << 1 | record float4s << 12}
+                               //  tile | second tile << 16 (tile_code; bit 15: there is one),
+                               //  runs along y | record float4s << 12}
   int *counter;                // [2]
   float *wbuf;                 // stored weights (store: written, stream: read)
   const long long *doff;       // first stored weight of each D of the half plane
   long n_units;
   int n, ldp;
+  int grab;                    // units a warp takes from the counter at a time
   long lat_elems;
   float tau_scale2, wcoef;
 };
@@ -130,15 +155,131 @@ __device__ __forceinline__ int disp_index(int dx, int dy, int n) {
   return dy == 0 ? dx - 1 : (n - 1) + (dy - 1) * (2 * n - 1) + (dx + n - 1);
 }
 
+// A tile: 32 lanes (32-lane block lb, in 1 << lg groups) x R stacked targets
+// from row row0 of D's rectangle.
+__host__ __device__ constexpr int tile_code(int lb, int row0, int lg) { return lb | (row0 << 4) | (lg << 13); }
+
+struct TileAt {
+  int x, y;     // the first stacked target of this lane (clamped into the rectangle)
+  bool valid;   // this lane has targets here
+};
+
+// the rectangle of targets of D
+struct Rect {
+  int xlo, xhi, ylo, yhi;
+  __device__ __forceinline__ Rect(int dx, int dy, int n)
+      : xlo(dx < 0 ? -dx : 0), xhi(dx > 0 ? n - dx : n), ylo(dy < 0 ? -dy : 0), yhi(dy > 0 ? n - dy : n) {}
+};
+
+template <int R>
+__device__ __forceinline__ TileAt tile_at(int code, const Rect &b, bool along_y, int lane) {
+  const int lb = code & 15, row0 = (code >> 4) & 511, lg = (code >> 13) & 3;
+  // lane groups: 1, 2 or 4 groups of 32 >> lg lanes, group g on the block
+  // starting R s g rows after row0 (s = group_stride); a group past the
+  // last block is masked off
+  const int gw = 32 >> lg, g = lane >> (5 - lg), lig = lane & (gw - 1);
+  const int stack = along_y ? b.yhi - b.ylo : b.xhi - b.xlo;
+  TileAt t;
+  int row = row0 + R * group_stride(R, lg) * g;
+  t.valid = row < stack;
+  if (!t.valid) row = row0;
+  // lane coordinate (clamped to the rectangle) and the first stacked target
+  if (along_y) {
+    const int xr = b.xlo + 32 * lb + lig;
+    t.valid = t.valid && xr < b.xhi;
+    t.x = xr < b.xhi ? xr : b.xhi - 1;
+    t.y = b.ylo + row;
+  } else {
+    const int yr = b.ylo + 32 * lb + lig;
+    t.valid = t.valid && yr < b.yhi;
+    t.y = yr < b.yhi ? yr : b.yhi - 1;
+    t.x = b.xlo + row;
+  }
+  return t;
+}
+
+// what becomes of a tile's pairs (acc: their tau sums; not read when streaming)
+template <int MODE, int R>
+__device__ __forceinline__ void tile_pairs(const DispArgs &a, const float (&acc)[R], const TileAt &t, const Rect &b,
+                                           int dx, int dy, bool along_y, float scale, float tscale, float wk,
+                                           long woff) {
+  const int wx = b.xhi - b.xlo, x = t.x, y = t.y, n = a.n;
+  const long N = (long)n * n;
+  // sums of targets on consecutive x (runs along y) go to yacc with x
+  // fastest, those on consecutive y (runs along x) to its second half with
+  // y fastest, so a warp's atomics cover contiguous words; s is kept in both
+  // layouts the same way.  Stacked targets are n apart in both.  The epilogue
+  // is a quarter of all instructions, so its addresses are 32-bit offsets
+  // from the kernel's pointers (one addition each; 64-bit pointers that
+  // depended on the run axis took three times as many instructions).
+  const unsigned jb = (along_y ? (unsigned)(y * n + x) : (unsigned)N + (unsigned)(x * n + y)) * 4u;
+  const unsigned kb = jb + 4u * (unsigned)(along_y ? dy * n + dx : dx * n + dy);
+  const unsigned n4 = 4u * (unsigned)n;
+  const char *sb = reinterpret_cast<const char *>(a.src);
+  char *yb = reinterpret_cast<char *>(a.yacc);
+  // stacked targets of this lane
+  const int cnt = t.valid ? min(R, along_y ? b.yhi - y : b.xhi - x) : 0;
+  // stored weights of this lane's targets: row-major in D's rectangle
+  float *wp = nullptr;
+  const int wstep = along_y ? wx : 1;
+  if constexpr (MODE != kApply) wp = a.wbuf + woff + (long)(y - b.ylo) * wx + (x - b.xlo);
+  if constexpr (MODE == kStream) {
+    // four targets at a time: their global loads are issued before their atomics
+#pragma unroll
+    for (int q0 = 0; q0 < R; q0 += 4) {
+      float wv[4], sjv[4], skv[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int q = q0 + i;
+        wv[i] = sjv[i] = skv[i] = 0.f;
+        if (q < cnt) {
+          wv[i] = __ldcs(wp + (long)q * wstep);
+          sjv[i] = __ldg(reinterpret_cast<const float *>(sb + (jb + (unsigned)q * n4)));
+          skv[i] = __ldg(reinterpret_cast<const float *>(sb + (kb + (unsigned)q * n4)));
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int q = q0 + i;
+        if (q < cnt) {
+          const float w = wv[i] * scale;
+          red_add(yb, 2u * (jb + (unsigned)q * n4), (unsigned long long)__float2ll_rn(w * skv[i]));
+          red_add(yb, 2u * (kb + (unsigned)q * n4), (unsigned long long)__float2ll_rn(w * sjv[i]));
+        }
+      }
+    }
+  } else if constexpr (MODE == kStore) {
+#pragma unroll
+    for (int q = 0; q < R; ++q)
+      if (q < cnt) wp[(long)q * wstep] = wk * exp2f(tscale * acc[q]);
+  } else {
+    // the scale is a power of two: applied to wk it changes no bit of a
+    // product (weights below 2^-126, where it could, add nothing in fixed
+    // point)
+    const float wks = wk * scale;
+#pragma unroll
+    for (int q = 0; q < R; ++q) {
+      if (q < cnt) {
+        const unsigned oj = jb + (unsigned)q * n4, ok = kb + (unsigned)q * n4;
+        const float sj = __ldg(reinterpret_cast<const float *>(sb + oj));
+        const float sk = __ldg(reinterpret_cast<const float *>(sb + ok));
+        const float w = wks * exp2f(tscale * acc[q]);
+        red_add(yb, 2u * oj, (unsigned long long)__float2ll_rn(w * sk));
+        red_add(yb, 2u * ok, (unsigned long long)__float2ll_rn(w * sj));
+      }
+    }
+  }
+}
+
 // GLAT: the lattice stays in global memory (read through L1).  Units whose
 // runs go along y read lat from (x, y) on, the others lat_t from (y, x) on:
 // in both the run axis has stride LDP and the lanes are consecutive elements,
 // and the records of the runs along x carry their offsets in lat_t's layout.
-template <int LDP, int MODE, bool GLAT, int R>
+// T: tiles per unit (1, or 2 that share every record load).
+template <int LDP, int MODE, bool GLAT, int R, int T>
 __device__ __forceinline__ void disp_body(const DispArgs &a) {
   extern __shared__ float4 smem4[];
   const int n = a.n;
-  const long N = (long)n * n;
   // shared memory: the lattice (none when streaming)
   float *lat = reinterpret_cast<float *>(smem4);
   const int tid = threadIdx.x, lane = tid & 31;
@@ -146,76 +287,68 @@ __device__ __forceinline__ void disp_body(const DispArgs &a) {
     const float4 *g4 = reinterpret_cast<const float4 *>(a.lat);
     float4 *l4 = reinterpret_cast<float4 *>(lat);
     const long n4 = a.lat_elems / 4;
-    for (long i = tid; i < n4; i += kThreads) l4[i] = g4[i];
-    for (long i = n4 * 4 + tid; i < a.lat_elems; i += kThreads) lat[i] = a.lat[i];
+    for (long i = tid; i < n4; i += blockDim.x) l4[i] = g4[i];
+    for (long i = n4 * 4 + tid; i < a.lat_elems; i += blockDim.x) lat[i] = a.lat[i];
+  }
+  // power-of-two scale: 2^k <= 2^62 / (max|s| R), so w * scale is exact; one
+  // thread's FP64 division (by every thread it held the narrow pipe for 3 us)
+  __shared__ double scale_s;
+  if (MODE != kStore && tid == 0) {
+    const float smax = __uint_as_float(*a.smax);
+    scale_s = smax > 0.f ? ldexp(1.0, ilogb(4.611686018427387904e18 / ((double)smax * a.rbound))) : 1.0;
   }
   __syncthreads();
-  // power-of-two scale: 2^k <= 2^62 / (max|s| R), so w * scale is exact
-  double scale_d = 1.0;
-  if constexpr (MODE != kStore) {
-    const float smax = __uint_as_float(*a.smax);
-    if (smax > 0.f) scale_d = ldexp(1.0, ilogb(4.611686018427387904e18 / ((double)smax * a.rbound)));
-  }
-  const float scale = (float)scale_d;
+  const float scale = MODE != kStore ? (float)scale_s : 1.f;
   const int ldp = LDP > 0 ? LDP : a.ldp;
   const unsigned lat_base = (unsigned)__cvta_generic_to_shared(lat);
   long u0 = 0, u_end = 0;
   for (;;) {
     if (u0 >= u_end) {
       long got = 0;
-      if (lane == 0) got = atomicAdd(a.counter, 4);
+      if (lane == 0) got = atomicAdd(a.counter, a.grab);
       got = __shfl_sync(0xffffffffu, got, 0);
       if (got >= a.n_units) break;
       u0 = got;
-      u_end = min(got + 4, a.n_units);
+      u_end = min(got + a.grab, a.n_units);
     }
     const int4 un = a.units[u0++];
-    {
     const int dx = (short)(un.y & 0xffff), dy = un.y >> 16;
-    const int lb = un.z & 0xffff, row0 = un.z >> 16;
-    const int xlo = dx < 0 ? -dx : 0, xhi = dx > 0 ? n - dx : n;
-    const int ylo = dy < 0 ? -dy : 0, yhi = dy > 0 ? n - dy : n;
     const bool along_y = (un.w & 1) != 0;
-    const int lg = (un.w >> 1) & 3, nrec = un.w >> 12;
-    // lane groups: 1, 2 or 4 groups of 32 >> lg lanes, group g on the block
-    // starting R s g rows after row0 (s = group_stride); a group past the
-    // last block is masked off
-    const int gw = 32 >> lg, g = lane >> (5 - lg), lig = lane & (gw - 1);
-    const int stack = along_y ? yhi - ylo : xhi - xlo;
-    int row = row0 + R * group_stride(R, lg) * g;
-    bool lvalid = row < stack;
-    if (!lvalid) row = row0;
-    // lane coordinate (clamped to the rectangle) and the first stacked target
-    int x, y;
-    if (along_y) {
-      const int xr = xlo + 32 * lb + lig;
-      lvalid = lvalid && xr < xhi;
-      x = xr < xhi ? xr : xhi - 1;
-      y = ylo + row;
-    } else {
-      const int yr = ylo + 32 * lb + lig;
-      lvalid = lvalid && yr < yhi;
-      y = yr < yhi ? yr : yhi - 1;
-      x = xlo + row;
-    }
-    float acc[R];
-#pragma unroll
-    for (int q = 0; q < R; ++q) acc[q] = 0.f;
+    const int nrec = un.w >> 12;
+    const Rect rect(dx, dy, n);
+    Acc2<R> sa, sb;
+    const TileAt ta = tile_at<R>(un.z, rect, along_y, lane);
     if constexpr (MODE != kStream) {
-      const unsigned base = lat_base + 4u * (unsigned)(x + ldp * y);
+      // a unit of one tile (T = 2) marches it twice
+      const TileAt tb = T == 2 ? tile_at<R>(un.z & 0x8000 ? un.z >> 16 : un.z, rect, along_y, lane) : ta;
       {
         // bring this D's chunk records into L1 (one 128-byte line per lane)
         const char *r0 = reinterpret_cast<const char *>(a.stencil + un.x);
         const int lines = (int)(((reinterpret_cast<size_t>(r0) & 127) + 16L * nrec + 127) >> 7);
         for (int l = lane; l < lines; l += 32) asm volatile("prefetch.global.L1 [%0];" ::"l"(r0 + 128L * l));
       }
+      sa.zero();
+      sb.zero();
+      const float4 *rec = a.stencil + un.x;
       if constexpr (GLAT) {
-        const float *gb = along_y ? a.lat + (x + (long)LDP * y) : a.lat_t + (y + (long)LDP * x);
-        march_runs_global<LDP, R>(a.stencil + un.x, gb, acc);
-      } else if (along_y) {
-        march_runs<LDP, R>(a.stencil + un.x, base, ldp, acc);
+        const float *lt = along_y ? a.lat : a.lat_t;
+        const long oa = along_y ? ta.x + (long)LDP * ta.y : ta.y + (long)LDP * ta.x;
+        const long ob = along_y ? tb.x + (long)LDP * tb.y : tb.y + (long)LDP * tb.x;
+        march_runs_global_pair<LDP, R>(rec, lt + oa, lt + ob, sa, sb);
       } else {
-        march_runs<1, R>(a.stencil + un.x, base, 1, acc);
+        const unsigned ba = lat_base + 4u * (unsigned)(ta.x + ldp * ta.y);
+        const unsigned bb = lat_base + 4u * (unsigned)(tb.x + ldp * tb.y);
+        if constexpr (T == 2) {
+          if (along_y)
+            march_runs_pair<LDP, R>(rec, ba, bb, ldp, sa, sb);
+          else
+            march_runs_pair<1, R>(rec, ba, bb, 1, sa, sb);
+        } else {
+          if (along_y)
+            march_runs<LDP, R>(rec, ba, ldp, sa);
+          else
+            march_runs<1, R>(rec, ba, 1, sa);
+        }
       }
     }
     const float r2 = (float)(dx * dx + dy * dy);
@@ -228,78 +361,27 @@ __device__ __forceinline__ void disp_body(const DispArgs &a) {
     // write 128 contiguous bytes; lanes along y each write their R targets)
     long woff = 0;
     if constexpr (MODE != kApply) woff = a.doff[disp_index(dx, dy, n)];
-    const int wx = xhi - xlo;
-    // sums of targets on consecutive x (runs along y) go to yacc with x
-    // fastest, those on consecutive y (runs along x) to its second half with
-    // y fastest, so a warp's atomics cover contiguous words; s is kept in both
-    // layouts the same way.  Stacked targets are n apart in both.  The epilogue
-    // is a quarter of all instructions, so its addresses are 32-bit offsets
-    // from the kernel's pointers (one addition each; 64-bit pointers that
-    // depended on the run axis took three times as many instructions).
-    const unsigned jb = (along_y ? (unsigned)(y * n + x) : (unsigned)N + (unsigned)(x * n + y)) * 4u;
-    const unsigned kb = jb + 4u * (unsigned)(along_y ? dy * n + dx : dx * n + dy);
-    const unsigned n4 = 4u * (unsigned)n;
-    const char *sb = reinterpret_cast<const char *>(a.src);
-    char *yb = reinterpret_cast<char *>(a.yacc);
-    // stacked targets of this lane
-    const int cnt = lvalid ? min(R, along_y ? yhi - y : xhi - x) : 0;
-    // stored weights of this lane's targets: row-major in D's rectangle
-    float *wp = nullptr;
-    const int wstep = along_y ? wx : 1;
-    if constexpr (MODE != kApply) wp = a.wbuf + woff + (long)(y - ylo) * wx + (x - xlo);
-    if constexpr (MODE == kStream) {
-      // four targets at a time: their global loads are issued before their atomics
-#pragma unroll
-      for (int q0 = 0; q0 < R; q0 += 4) {
-        float wv[4], sjv[4], skv[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int q = q0 + i;
-          wv[i] = sjv[i] = skv[i] = 0.f;
-          if (q < cnt) {
-            wv[i] = __ldcs(wp + (long)q * wstep);
-            sjv[i] = __ldg(reinterpret_cast<const float *>(sb + (jb + (unsigned)q * n4)));
-            skv[i] = __ldg(reinterpret_cast<const float *>(sb + (kb + (unsigned)q * n4)));
-          }
-        }
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int q = q0 + i;
-          if (q < cnt) {
-            const float w = wv[i] * scale;
-            red_add(yb, 2u * (jb + (unsigned)q * n4), (unsigned long long)__float2ll_rn(w * skv[i]));
-            red_add(yb, 2u * (kb + (unsigned)q * n4), (unsigned long long)__float2ll_rn(w * sjv[i]));
-          }
-        }
-      }
-    } else if constexpr (MODE == kStore) {
-#pragma unroll
-      for (int q = 0; q < R; ++q)
-        if (q < cnt) wp[(long)q * wstep] = wk * exp2f(tscale * acc[q]);
+    if constexpr (T == 1) {
+      float acc[R];
+      if constexpr (MODE != kStream) sa.sum(acc);
+      tile_pairs<MODE, R>(a, acc, ta, rect, dx, dy, along_y, scale, tscale, wk, woff);
     } else {
-      // the scale is a power of two: applied to wk it changes no bit of a
-      // product (weights below 2^-126, where it could, add nothing in fixed
-      // point)
-      const float wks = wk * scale;
-#pragma unroll
-      for (int q = 0; q < R; ++q) {
-        if (q < cnt) {
-          const unsigned oj = jb + (unsigned)q * n4, ok = kb + (unsigned)q * n4;
-          const float sj = __ldg(reinterpret_cast<const float *>(sb + oj));
-          const float sk = __ldg(reinterpret_cast<const float *>(sb + ok));
-          const float w = wks * exp2f(tscale * acc[q]);
-          red_add(yb, 2u * oj, (unsigned long long)__float2ll_rn(w * sk));
-          red_add(yb, 2u * ok, (unsigned long long)__float2ll_rn(w * sj));
-        }
+      // one copy of the epilogue's code for both tiles
+#pragma unroll 1
+      for (int z = un.z;; z >>= 16, sa = sb) {
+        float acc[R];
+        if constexpr (MODE != kStream) sa.sum(acc);
+        tile_pairs<MODE, R>(a, acc, tile_at<R>(z, rect, along_y, lane), rect, dx, dy, along_y, scale, tscale, wk,
+                            woff);
+        if (!(z & 0x8000)) break;
       }
-    }
     }
   }
   // every warp of this CTA is past its last unit before the CTA counts as done
   // (the last CTA resets the unit counter for the next launch)
   __syncthreads();
   if constexpr (MODE != kStore) {
-    if (blockIdx.x == 0 && tid == 0) *a.scale_out = scale_d;
+    if (blockIdx.x == 0 && tid == 0) *a.scale_out = scale_s;
   }
   if (tid == 0) {
     __threadfence();
@@ -312,29 +394,29 @@ __device__ __forceinline__ void disp_body(const DispArgs &a) {
   }
 }
 
-template <int LDP, int R>
-__global__ void __launch_bounds__(kThreads, 1) k_pairs_disp(DispArgs a) {
-  disp_body<LDP, kApply, false, R>(a);
+template <int LDP, int R, int T>
+__global__ void __launch_bounds__(disp_threads(T), 1) k_pairs_disp(DispArgs a) {
+  disp_body<LDP, kApply, false, R, T>(a);
 }
 
-template <int LDP, int R>
-__global__ void __launch_bounds__(kThreads, 1) k_store_disp(DispArgs a) {
-  disp_body<LDP, kStore, false, R>(a);
+template <int LDP, int R, int T>
+__global__ void __launch_bounds__(disp_threads(T), 1) k_store_disp(DispArgs a) {
+  disp_body<LDP, kStore, false, R, T>(a);
 }
 
-template <int R>
+template <int R, int T>
 __global__ void __launch_bounds__(kThreads, 1) k_stream_disp(DispArgs a) {
-  disp_body<1, kStream, false, R>(a);
+  disp_body<1, kStream, false, R, T>(a);
 }
 
-template <int R>
-__global__ void __launch_bounds__(kThreads, 1) k_pairs_disp_global(DispArgs a) {
-  disp_body<disp_pitch(kGlobalMaxN, R), kApply, true, R>(a);
+template <int R, int T>
+__global__ void __launch_bounds__(disp_threads(T), 1) k_pairs_disp_global(DispArgs a) {
+  disp_body<disp_pitch(kGlobalMaxN, R), kApply, true, R, T>(a);
 }
 
-template <int R>
-__global__ void __launch_bounds__(kThreads, 1) k_store_disp_global(DispArgs a) {
-  disp_body<disp_pitch(kGlobalMaxN, R), kStore, true, R>(a);
+template <int R, int T>
+__global__ void __launch_bounds__(disp_threads(T), 1) k_store_disp_global(DispArgs a) {
+  disp_body<disp_pitch(kGlobalMaxN, R), kStore, true, R, T>(a);
 }
 
 
@@ -624,18 +706,19 @@ __global__ void k_disp_source(long N, int n, int op, const double *__restrict__ 
 
 typedef void (*DispKernel)(DispArgs);
 
-// compile-time lattice pitches of the 64^2 and 128^2 grids (stack depths
-// disp_depth(64) = 8 and disp_depth(128) = 12)
-constexpr int kLdp64 = disp_pitch(64, disp_depth(64)), kLdp128 = disp_pitch(128, disp_depth(128));
-
-// the shared-lattice apply (store) kernel of lattice pitch ldp, depth R
-DispKernel pick_disp(int ldp, int R, bool store) {
-  if (R == 8) {
-    if (ldp == kLdp64) return store ? k_store_disp<kLdp64, 8> : k_pairs_disp<kLdp64, 8>;
-    return store ? k_store_disp<0, 8> : k_pairs_disp<0, 8>;
+// the shared-lattice apply (store) kernel of lattice pitch ldp, depth R, T tiles per unit
+template <int R, int T, int I = 0>
+DispKernel pick_pitch(int ldp, bool store) {
+  if constexpr (I < 5) {
+    constexpr int P = R == 8 ? kPitch8[I] : kPitch12[I];
+    if (ldp == P) return store ? k_store_disp<P, R, T> : k_pairs_disp<P, R, T>;
+    return pick_pitch<R, T, I + 1>(ldp, store);
   }
-  if (ldp == kLdp128) return store ? k_store_disp<kLdp128, 12> : k_pairs_disp<kLdp128, 12>;
-  return store ? k_store_disp<0, 12> : k_pairs_disp<0, 12>;
+  return store ? k_store_disp<0, R, T> : k_pairs_disp<0, R, T>;
+}
+DispKernel pick_disp(int ldp, int R, int T, bool store) {
+  if (R == 8) return T == 1 ? pick_pitch<8, 1>(ldp, store) : store ? k_store_disp<0, 8, 2> : k_pairs_disp<0, 8, 2>;
+  return pick_pitch<12, 2>(ldp, store);
 }
 
 
@@ -731,7 +814,7 @@ bool disp_expand_fits(int n, int device) {
 
 size_t disp_smem_bytes(int n, int R) {
   const long rows = n + R;
-  return sizeof(float) * (size_t)rows * disp_pitch(n, R) + 16;
+  return sizeof(float) * (size_t)rows * shared_pitch(n, R) + 16;
 }
 
 namespace {
@@ -778,6 +861,7 @@ void geometry_trim() {
 // global: the lattice-in-global-memory layout (runs along x address lat_t)
 vie_status geometry_build(int n, int ldp, bool global, int R, Geometry *geo) {
   // stencils and work units, the run axis of each D chosen by estimated cost
+  const int T = disp_tiles(n);
   struct U {
     int4 u;
     long cost;
@@ -805,7 +889,7 @@ vie_status geometry_build(int n, int ldp, bool global, int R, Geometry *geo) {
     std::vector<float> &rec = o.rec;
     double &taps = o.taps;
     std::vector<Cell> cy_cells, cx_cells;
-    std::vector<int> cy_runs, cx_runs;
+    std::vector<int> cy_runs, cx_runs, tiles;
     for (int dx = -(n - 1); dx < n; ++dx) {
       if (dy == 0 && dx <= 0) continue;
       const int wx = n - std::abs(dx), wy = n - dy;
@@ -850,9 +934,9 @@ vie_status geometry_build(int n, int ldp, bool global, int R, Geometry *geo) {
       const int nfb = (stack + R - 1) / R, full = lanes / 32, rem = lanes % 32;
       const int w = (along_y ? 1 : 0) | ((int)(pl.recs + 1) << 12);
       const int dxy = (dx & 0xffff) | (dy << 16);
+      tiles.clear();
       for (int sb = 0; sb < nfb; ++sb)
-        for (int lb = 0; lb < full; ++lb)
-          units.push_back({make_int4(off, dxy, lb | ((R * sb) << 16), w), pl.cost});
+        for (int lb = 0; lb < full; ++lb) tiles.push_back(tile_code(lb, R * sb, 0));
       if (rem > 0) {
         // the ragged last lane block: 2 or 4 blocks share a warp when it
         // is at most 16 or 8 lanes wide (blocks sb, sb + s, ...; s =
@@ -862,7 +946,12 @@ vie_status geometry_build(int n, int ldp, bool global, int R, Geometry *geo) {
         const int span = lg == 0 ? 1 : G * sstride;
         for (int base = 0; base < nfb; base += span)
           for (int j = 0; j < (lg == 0 ? 1 : sstride) && base + j < nfb; ++j)
-            units.push_back({make_int4(off, dxy, full | ((R * (base + j)) << 16), w | (lg << 1)), pl.cost});
+            tiles.push_back(tile_code(full, R * (base + j), lg));
+      }
+      for (size_t i = 0; i < tiles.size(); i += T) {
+        const bool two = T == 2 && i + 1 < tiles.size();
+        const int z = tiles[i] | (two ? 0x8000 | (tiles[i + 1] << 16) : 0);
+        units.push_back({make_int4(off, dxy, z, w), two ? 2 * pl.cost : pl.cost});
       }
     }
   };
@@ -895,7 +984,10 @@ vie_status geometry_build(int n, int ldp, bool global, int R, Geometry *geo) {
     std::vector<float>().swap(o.rec);
   }
   for (int i = 0; i < 32; ++i) rec.push_back(0.f);  // the L1 prefetch may reach 127 bytes past a stencil
-  std::stable_sort(units.begin(), units.end(), [](const U &p, const U &q) { return p.cost > q.cost; });
+  std::stable_sort(units.begin(), units.end(), [T](const U &p, const U &q) {
+    if (T == 2 && (p.u.w & 1) != (q.u.w & 1)) return (p.u.w & 1) > (q.u.w & 1);
+    return p.cost > q.cost;
+  });
   std::vector<int4> uv(units.size());
   for (size_t i = 0; i < units.size(); ++i) uv[i] = units[i].u;
   VIE_CUDA(vie_malloc((void **)&geo->units, sizeof(int4) * uv.size()));
@@ -1004,11 +1096,12 @@ vie_status disp_prepare(DispPlan *dp, int n, const float *sig_padded, int device
   if (disp_smem_bytes(n, R) > optin && disp_smem_bytes(n, 8) <= optin) R = 8;
   const bool global = disp_smem_bytes(n, R) > optin;
   if (global && n > kGlobalMaxN) return VIE_OK;
-  const int ldp = disp_pitch(global ? kGlobalMaxN : n, R), rows = global ? ldp : n + R;
+  const int ldp = global ? disp_pitch(kGlobalMaxN, R) : shared_pitch(n, R), rows = global ? ldp : n + R;
   const size_t smem = global ? 16 : disp_smem_bytes(n, R);
-  DispKernel k = global ? (R == 8 ? k_pairs_disp_global<8> : k_pairs_disp_global<12>) : pick_disp(ldp, R, false);
-  DispKernel ks = global ? (R == 8 ? k_store_disp_global<8> : k_store_disp_global<12>) : pick_disp(ldp, R, true);
-  DispKernel kst = R == 8 ? k_stream_disp<8> : k_stream_disp<12>;
+  const int T = disp_tiles(n);
+  DispKernel k = global ? k_pairs_disp_global<12, 2> : pick_disp(ldp, R, T, false);
+  DispKernel ks = global ? k_store_disp_global<12, 2> : pick_disp(ldp, R, T, true);
+  DispKernel kst = R == 12 ? k_stream_disp<12, 2> : T == 2 ? k_stream_disp<8, 2> : k_stream_disp<8, 1>;
   VIE_TRY(raise_smem_limit((const void *)k, (size_t)((int)smem)));
   if (global) {
     // all of the SM's unified memory it can get as L1 (a per-kernel preference)
@@ -1016,7 +1109,7 @@ vie_status disp_prepare(DispPlan *dp, int n, const float *sig_padded, int device
     VIE_CUDA(cudaFuncSetAttribute((const void *)ks, cudaFuncAttributePreferredSharedMemoryCarveout, 0));
   }
   int bps = 0;
-  VIE_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k, kThreads, smem));
+  VIE_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k, disp_threads(T), smem));
   if (bps < 1) return VIE_OK;
   // the store and stream kernels of the displacement-major operator
   const long N = (long)n * n;
@@ -1025,7 +1118,7 @@ vie_status disp_prepare(DispPlan *dp, int n, const float *sig_padded, int device
   VIE_TRY(raise_smem_limit((const void *)ks, (size_t)((int)smem_store)));
   VIE_TRY(raise_smem_limit((const void *)kst, (size_t)((int)smem_stream)));
   int bps_store = 0, bps_stream = 0;
-  VIE_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps_store, ks, kThreads, smem_store));
+  VIE_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps_store, ks, disp_threads(T), smem_store));
   VIE_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps_stream, kst, kThreads, smem_stream));
   if (bps_store < 1 || bps_stream < 1) return VIE_OK;
   Geometry *geo = nullptr;
@@ -1200,6 +1293,11 @@ DispArgs disp_args(const DispPlan &dp, int n, float tau_scale2, float wcoef, flo
   a.yacc = (unsigned long long *)dp.yacc;
   a.units = (const int4 *)dp.units;
   a.counter = dp.counter;
+  // units a warp takes at a time: up to 4, fewer where a grid has few for each
+  // warp (measured per apply at 47^2: 44.8 us with 1, 59.3 with 4; at 110^2
+  // 719 and 675)
+  const long warps = (long)dp.grid * disp_threads(disp_tiles(n)) / 32;
+  a.grab = (int)std::max(1L, std::min(4L, dp.n_units / (2 * warps)));
   a.wbuf = wbuf;
   a.doff = dp.doff;
   a.wtab = dp.wtab;
@@ -1217,7 +1315,7 @@ DispArgs disp_args(const DispPlan &dp, int n, float tau_scale2, float wcoef, flo
 vie_status disp_launch(const DispPlan &dp, int n, float tau_scale2, float wcoef, cudaStream_t st) {
   DispArgs a = disp_args(dp, n, tau_scale2, wcoef, nullptr);
   void *args[] = {&a};
-  VIE_CUDA(cudaLaunchKernel(dp.kernel, dim3(dp.grid), dim3(kThreads), args, dp.smem, st));
+  VIE_CUDA(cudaLaunchKernel(dp.kernel, dim3(dp.grid), dim3(disp_threads(disp_tiles(n))), args, dp.smem, st));
   count_launch();
   return VIE_OK;
 }
@@ -1225,7 +1323,7 @@ vie_status disp_launch(const DispPlan &dp, int n, float tau_scale2, float wcoef,
 vie_status disp_store(const DispPlan &dp, int n, float tau_scale2, float wcoef, float *wbuf, cudaStream_t st) {
   DispArgs a = disp_args(dp, n, tau_scale2, wcoef, wbuf);
   void *args[] = {&a};
-  VIE_CUDA(cudaLaunchKernel(dp.kernel_store, dim3(dp.grid_store), dim3(kThreads), args, dp.smem_store, st));
+  VIE_CUDA(cudaLaunchKernel(dp.kernel_store, dim3(dp.grid_store), dim3(disp_threads(disp_tiles(n))), args, dp.smem_store, st));
   count_launch();
   return VIE_OK;
 }

@@ -147,15 +147,16 @@ __global__ void __launch_bounds__(kThreads3, 1) k_pairs_disp3(Disp3Args a) {
       const int lines = (int)(((reinterpret_cast<size_t>(r0) & 127) + 16L * nrec + 127) >> 7);
       for (int l = lane; l < lines; l += 32) asm volatile("prefetch.global.L1 [%0];" ::"l"(r0 + 128L * l));
     }
-    float acc[kR];
-#pragma unroll
-    for (int q = 0; q < kR; ++q) acc[q] = 0.f;
+    dmarch::Acc2<kR> sums;
+    sums.zero();
     if (orient == 0)
-      march_runs<PLANE, kR>(a.stencil + un.x, base, plane, acc);
+      march_runs<PLANE, kR>(a.stencil + un.x, base, plane, sums);
     else if (orient == 1)
-      march_runs<LDP, kR>(a.stencil + un.x, base, ldp, acc);
+      march_runs<LDP, kR>(a.stencil + un.x, base, ldp, sums);
     else
-      march_runs<1, kR>(a.stencil + un.x, base, 1, acc);
+      march_runs<1, kR>(a.stencil + un.x, base, 1, sums);
+    float acc[kR];
+    sums.sum(acc);
     const float r2 = (float)(dx * dx + dy * dy + dz * dz);
     const float inv_r = rsqrtf(r2);
     const float tscale = -a.tau_scale2 * r2 * inv_r;  // -(h/S) log2(e) r
