@@ -308,94 +308,152 @@ __device__ __forceinline__ ExpItem exp_decode(int t, int n, const int *__restric
   return it;
 }
 
-// row i of this warp holds dx = -(n - 1) + warp + i kExpWarps (lane = xj - xlo)
-__device__ __forceinline__ bool exp_row(const ExpItem &it, int n, int warp, int i, int lane, int &dx, int &xlo,
-                                        int &wx) {
-  dx = -(n - 1) + warp + i * kExpWarps;
-  xlo = dx < 0 ? -dx : 0;
-  wx = n - (dx < 0 ? -dx : dx);
-  return dx < n && !(it.same && dx <= 0) && lane < wx;
-}
+// The expansion takes the items by pairs of planes (zj, zk = zj + dz): item u is
+// (yj, yk) of its pair, yk fastest, so that the CTAs at work at one time write
+// neighbouring segments of a few planes' rows, and the stored weights of a
+// pair lie in a few contiguous KB per D.  (For dz = 0 the items yk < yj are
+// empty.)  A CTA steps from item to item by additions.
+struct ExpStep {
+  int zj, dz, yj, yk;
+  __device__ __forceinline__ void start(int u, int n) {
+    int pair = u / (n * n);
+    const int r = u - pair * n * n;
+    yj = r / n;
+    yk = r - yj * n;
+    for (dz = 0; dz < n && pair >= n - dz; ++dz) pair -= n - dz;
+    zj = pair;
+  }
+  // by by = (gridDim / n, gridDim % n); past the last item dz reaches n
+  __device__ __forceinline__ void advance(int by_j, int by_k, int n) {
+    yj += by_j;
+    yk += by_k;
+    if (yk >= n) {
+      yk -= n;
+      ++yj;
+    }
+    while (yj >= n) {
+      yj -= n;
+      if (++zj >= n - dz) {
+        ++dz;
+        zj = 0;
+      }
+    }
+  }
+  __device__ __forceinline__ bool empty() const { return dz == 0 && yk < yj; }
+  __device__ __forceinline__ bool same() const { return dz == 0 && yk == yj; }
+};
 
-// this warp's stored rows of item it into v, and the lane's sigma_s on both lines
-__device__ __forceinline__ void exp_load(const ExpItem &it, int n, int warp, int lane, const float *__restrict__ w,
-                                         const long long *__restrict__ doff, const float *__restrict__ ss,
-                                         float (&v)[kExpRows], float &ssj, float &ssk) {
-  const int m2 = 2 * n - 1;
+// What a thread's rows have in common over all items: row i of its warp is dx =
+// -(n - 1) + warp + i kExpWarps, lane = xj - xlo.
+struct ExpRows {
+  short wx[kExpRows];  // targets of the row (0: no such row)
+  int pre[kExpRows];   // targets of the rows before it
+  short at[kExpRows];  // its place in T
+  __device__ __forceinline__ ExpRows(int n, int warp, int lane, int p) {
+#pragma unroll
+    for (int i = 0; i < kExpRows; ++i) {
+      const int row = warp + i * kExpWarps, dx = row - (n - 1);
+      wx[i] = (short)(row < 2 * n - 1 ? n - abs(dx) : 0);
+      pre[i] = dx <= 0 ? row * (row + 1) / 2 : n * n - (2 * n - 1 - row) * (2 * n - row) / 2;
+      at[i] = (short)(row * p + max(-dx, 0) + lane);
+    }
+  }
+};
+
+// this warp's stored rows of an item into v, and the lane's sigma_s on both
+// lines; the rows of one (dy, dz) lie one after the other, so one offset is
+// looked up per item
+__device__ __forceinline__ void exp_load(const ExpStep &it, const ExpRows &rows, int n, int warp, int lane,
+                                         const float *__restrict__ w, const long long *__restrict__ doff,
+                                         const float *__restrict__ ss, float (&v)[kExpRows], float &ssj, float &ssk) {
+  const int m2 = 2 * n - 1, dy = it.yk - it.yj;
+  const int wyl = n - abs(dy), line = it.zj * wyl + it.yj - (dy < 0 ? -dy : 0), area = wyl * (n - it.dz);
+  const bool same = it.same();
+  const long long *dp = doff + ((it.dz + n - 1) * m2 + dy + n - 1) * m2;
+  // (the one-line displacement stores dx > 0 only, from row n on)
+  const float *base = w + (same ? (n > 1 ? dp[n] : 0) - (long long)area * (n * (n + 1) / 2) : it.empty() ? 0 : dp[0]);
+  const int first = it.empty() ? m2 : same ? n : 0;  // first stored row
 #pragma unroll
   for (int i = 0; i < kExpRows; ++i) {
-    int dx, xlo, wx;
     v[i] = 0.f;
-    if (exp_row(it, n, warp, i, lane, dx, xlo, wx))
-      v[i] = __ldcs(w + doff[((long)(it.dz + n - 1) * m2 + (it.dy + n - 1)) * m2 + (dx + n - 1)] +
-                    ((long)it.zj * it.wyl + (it.yj - it.ylo)) * wx + lane);
+    if (warp + i * kExpWarps >= first && lane < rows.wx[i])
+      v[i] = __ldcs(base + (area * rows.pre[i] + line * rows.wx[i] + lane));
   }
-  ssj = lane < n ? __ldg(ss + it.jrow + lane) : 0.f;  // n <= 32: one column per lane
-  ssk = lane < n ? __ldg(ss + it.krow + lane) : 0.f;
+  const int c = min(lane, n - 1);  // n <= 32: one column per lane
+  ssj = __ldg(ss + n * (it.yj + n * it.zj) + c);
+  ssk = __ldg(ss + n * (it.yk + n * (it.zj + it.dz)) + c);
 }
 
 // Software-pipelined: while a CTA writes the K entries of one item, the row
-// loads of its next item are in flight.
+// loads of its next item are in flight.  What bounds it is instruction issue
+// and the loads' latency before HBM (2.15 GB read, 4.3 written at 32^3): a row
+// takes a handful of instructions, its addresses by addition (with a binary
+// search and 64-bit products per row: 4450 instructions a warp and item,
+// 3.3 ms; EXP3_MEASURED).
 template <int OUT>
 __global__ void __launch_bounds__(kExpThreads, 4) k_expand_pairs3(int n, const float *__restrict__ w,
                                                            const long long *__restrict__ doff,
-                                                           const int *__restrict__ ioff, const int *__restrict__ iqd,
-                                                           int nq, const float *__restrict__ ss,
+                                                           const int *__restrict__ ioff,
+                                                           const float *__restrict__ ss,
                                                            const double *__restrict__ diag,
                                                            const double *__restrict__ ss64, long ldk, float *k32,
                                                            unsigned short *khi, unsigned short *klo) {
   extern __shared__ float T[];  // [2n - 1][p]
   const int p = n + 2;           // strides p and 1 - p: at most one is even (2-way conflicts)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;  // blockDim.x = kExpThreads
-  const int items = ioff[nq];
-  int t = blockIdx.x;
-  if (t >= items) return;
-  ExpItem cur = exp_decode(t, n, ioff, iqd, nq);
+  const int by_j = gridDim.x / n, by_k = gridDim.x % n;
+  ExpStep cur;
+  cur.start(blockIdx.x, n);
+  if (cur.dz >= n) return;
+  const ExpRows rows(n, warp, lane, p);
   float v[kExpRows], ssj_n, ssk_n;
-  exp_load(cur, n, warp, lane, w, doff, ss, v, ssj_n, ssk_n);
-  for (; t < items; t += gridDim.x) {
+  exp_load(cur, rows, n, warp, lane, w, doff, ss, v, ssj_n, ssk_n);
+  for (;;) {
 #pragma unroll
-    for (int i = 0; i < kExpRows; ++i) {
-      int dx, xlo, wx;
-      if (exp_row(cur, n, warp, i, lane, dx, xlo, wx)) T[(dx + n - 1) * p + xlo + lane] = v[i];
-    }
+    for (int i = 0; i < kExpRows; ++i)
+      if (lane < rows.wx[i]) T[rows.at[i]] = v[i];  // (rows not stored hold 0, not read)
     const float ssj_l = ssj_n, ssk_l = ssk_n;
     __syncthreads();
-    ExpItem nxt = cur;
-    const int tn = t + gridDim.x;
-    if (tn < items) {
-      nxt = exp_decode(tn, n, ioff, iqd, nq);
-      exp_load(nxt, n, warp, lane, w, doff, ss, v, ssj_n, ssk_n);
-    }
-    const long jrow = cur.jrow, krow = cur.krow;
-    if constexpr (OUT == kExpSym) {
+    ExpStep nxt = cur;
+    nxt.advance(by_j, by_k, n);
+    const bool more = nxt.dz < n;
+    if (more) exp_load(nxt, rows, n, warp, lane, w, doff, ss, v, ssj_n, ssk_n);
+    const long jrow = n * (cur.yj + n * cur.zj), krow = n * (cur.yk + n * (cur.zj + cur.dz));
+    const bool same = cur.same();
+    if (cur.empty()) {
+    } else if constexpr (OUT == kExpSym) {
       // block t: A_jk for j on line (yj, zj) (row xj), k on line (yk, zk)
       // (column xk); no sigma_s; the one-line blocks whole, with d_j
-      float *blk = k32 + (long)t * n * n;
+      const int dy = cur.yk - cur.yj, q = cur.dz == 0 ? dy : n + (cur.dz - 1) * (2 * n - 1) + dy + n - 1;
+      const long t = ioff[q] + (long)cur.zj * (n - abs(dy)) + cur.yj - (dy < 0 ? -dy : 0);
+      float *blk = k32 + t * n * n;
       for (int xj = warp; xj < n; xj += kExpWarps) {
         const int xk = lane;
         if (xk < n) {
           const int dx = xk - xj;
           float tv;
-          if (!cur.same || dx > 0)
+          if (!same || dx > 0)
             tv = T[(dx + n - 1) * p + xj];
           else if (dx < 0)
             tv = T[(-dx + n - 1) * p + xk];  // A_jk = A_kj, stored under (-dx, 0, 0) for target xk
           else
             tv = (float)diag[jrow + xj];
-          blk[(long)xj * n + xk] = tv;
+          blk[xj * n + xk] = tv;
         }
       }
-    } else if (!cur.same) {
-      for (int xj = warp; xj < n; xj += kExpWarps) {
-        const float *tb = T + (n - 1 - xj) * p + xj;  // T[(xk - xj + n - 1) p + xj]
-        const long rb = (jrow + xj) * ldk + krow;
-        if (lane < n) put_k<OUT>(rb + lane, tb[lane * p] * ssk_l, k32, khi, klo);
-      }
-      for (int xk = warp; xk < n; xk += kExpWarps) {
-        const float *tb = T + (xk + n - 1) * p;  // T[(xk - xj + n - 1) p + xj]
-        const long rb = (krow + xk) * ldk + jrow;
-        if (lane < n) put_k<OUT>(rb + lane, tb[lane * (1 - p)] * ssj_l, k32, khi, klo);
+    } else if (!same) {
+      if (lane < n) {
+        const float *tb = T + (n - 1 - warp + lane) * p + warp;  // T[(xk - xj + n - 1) p + xj], xk = lane
+        const long step = kExpWarps * ldk;
+        long at = (jrow + warp) * ldk + krow + lane;
+#pragma unroll
+        for (int i = 0; i < kMaxN3 / kExpWarps; ++i, tb += kExpWarps * (1 - p), at += step)
+          if (warp + i * kExpWarps < n) put_k<OUT>(at, *tb * ssk_l, k32, khi, klo);
+        tb = T + (warp + n - 1 - lane) * p + lane;  // the same seen from k, xj = lane
+        at = (krow + warp) * ldk + jrow + lane;
+#pragma unroll
+        for (int i = 0; i < kMaxN3 / kExpWarps; ++i, tb += kExpWarps * p, at += step)
+          if (warp + i * kExpWarps < n) put_k<OUT>(at, *tb * ssj_l, k32, khi, klo);
       }
     } else {
       for (int r = warp; r < n; r += kExpWarps) {
@@ -411,6 +469,7 @@ __global__ void __launch_bounds__(kExpThreads, 4) k_expand_pairs3(int n, const f
         put_k<OUT>(j * ldk + j, (float)(diag[j] * ss64[j]), k32, khi, klo);
       }
     }
+    if (!more) return;
     __syncthreads();
     cur = nxt;
   }
@@ -1040,13 +1099,13 @@ vie_status disp3_assemble(DispPlan3 *dp, float tau_scale2, float wcoef, const do
     if (s == VIE_OK) {
       const int grid = 4 * prop.multiProcessorCount;
       if (ldk == 0)
-        k_expand_pairs3<kExpSym><<<grid, kExpThreads, smem, st>>>(n, pairs, dp->doff, dp->ioff, dp->iqd, dp->nq, ss32,
+        k_expand_pairs3<kExpSym><<<grid, kExpThreads, smem, st>>>(n, pairs, dp->doff, dp->ioff, ss32,
                                                                  diag, sigma_s, 0, k32, nullptr, nullptr);
       else if (k32)
-        k_expand_pairs3<kExpF32><<<grid, kExpThreads, smem, st>>>(n, pairs, dp->doff, dp->ioff, dp->iqd, dp->nq, ss32, diag,
+        k_expand_pairs3<kExpF32><<<grid, kExpThreads, smem, st>>>(n, pairs, dp->doff, dp->ioff, ss32, diag,
                                                           sigma_s, ldk, k32, nullptr, nullptr);
       else
-        k_expand_pairs3<kExpBF16><<<grid, kExpThreads, smem, st>>>(n, pairs, dp->doff, dp->ioff, dp->iqd, dp->nq, ss32,
+        k_expand_pairs3<kExpBF16><<<grid, kExpThreads, smem, st>>>(n, pairs, dp->doff, dp->ioff, ss32,
                                                            diag, sigma_s, ldk, nullptr, (unsigned short *)khi,
                                                            (unsigned short *)klo);
       ce = cudaGetLastError();
