@@ -441,99 +441,115 @@ __device__ __forceinline__ void put_entry(long idx, float v, float *k32, unsigne
 // K_jk = A_jk sigma_s,k (j != k) and K_jj = d_j sigma_s,j, row-major N x ldk
 // (FP32, or BF16 hi + lo with lo = bf16(v - hi)), from the stored pair
 // weights, each read once.  An item is (dy, target row yj): the stored rows
-// "D = (dx, dy), targets (., yj)" of every dx go to shared memory
-// (T[dx + n - 1][xj]), then
+// "D = (dx, dy), targets (., yj)" of every dx are copied into the diagonals of
+// an n x n tile T[xj][xk] (xk = xj + dx), then
 //   K[j][k]  = T sigma_s,k  for j = (xj, yj), k = (xk, yj + dy), and
 //   K[k][j]  = T sigma_s,j  for the same pairs seen from k,
 // each written as whole row segments of n columns.  Every ordered pair is
 // written once: by its own D when D is in the half plane, else from -D.  For
 // dy = 0 the row of j gets its columns k > j from the first part and k < j
 // from the second, and the diagonal K_jj = d_j sigma_s,j.
-
 //
 // kSymBlocks writes A itself (A_jk = A_kj, no sigma_s): block t = item (dy, yj),
 // n x n row-major at t n^2, row xj, column xk; only the first part (and for
 // dy = 0 the whole block with its diagonal d_j).
+//
+// What bounds it is HBM (at 128^2, blocks: 0.54 GB read, 0.54 written) as long
+// as copies of other items are in flight while one is written: the copies are
+// asynchronous, and the tile holds the n^2 entries and no more, so that three
+// CTAs share an SM up to n = 137.  (One CTA of 1024 threads per SM, with a tile
+// of 2n - 1 whole diagonals loaded through registers, took 491 us for those
+// blocks, this 296; for dense K at 169^2 2.06 ms and 1.74.)
+constexpr int kExpThreads2 = 512, kExpWarps2 = kExpThreads2 / 32;
+
+// Row pitch of the tile.  A copied diagonal takes steps of p + 1 floats, a
+// written row 1, the rows seen from k steps of p: blocks have whole rows only,
+// and p a multiple of 4 makes the diagonals free of bank conflicts and the rows
+// readable by 16 bytes; dense K reads columns too, and p = 1 mod 4 leaves
+// two-way conflicts in the diagonals alone.
+__host__ __device__ constexpr int expand_pitch(int n, int out) {
+  return out == kSymBlocks ? (n + 3) & ~3 : ((n + 2) & ~3) + 1;
+}
+
 template <int OUT>
-__global__ void __launch_bounds__(1024, 1) k_expand_pairs(int n, const float *__restrict__ w,
-                                                          const long long *__restrict__ doff,
-                                                          const float *__restrict__ ss,
-                                                          const double *__restrict__ diag,
-                                                          const double *__restrict__ ss64, long ldk, float *k32,
-                                                          unsigned short *khi, unsigned short *klo) {
-  extern __shared__ float T[];  // [2n - 1][p]
-  const int p = n + 2;           // strides p and 1 - p: at most one is even (2-way conflicts)
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, warps = blockDim.x >> 5;
+__global__ void __launch_bounds__(kExpThreads2, 3) k_expand_pairs(int n, const float *__restrict__ w,
+                                                                 const long long *__restrict__ doff,
+                                                                 const float *__restrict__ ss,
+                                                                 const double *__restrict__ diag,
+                                                                 const double *__restrict__ ss64, long ldk, float *k32,
+                                                                 unsigned short *khi, unsigned short *klo) {
+  extern __shared__ __align__(16) float T[];  // [n][p]
+  const int p = expand_pitch(n, OUT);
+  const unsigned ts = (unsigned)__cvta_generic_to_shared(T);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int items = n * (n + 1) / 2;
   // item t -> (dy, yj), rows of dy holding n - dy items; advanced by gridDim.x per step
   int dy = 0, yj = blockIdx.x;
-  while (dy < n && yj >= n - dy) {
-    yj -= n - dy;
-    ++dy;
-  }
   for (int t = blockIdx.x; t < items; t += gridDim.x) {
-    if (t != (int)blockIdx.x) {
-      yj += gridDim.x;
-      while (dy < n && yj >= n - dy) {
-        yj -= n - dy;
-        ++dy;
-      }
+    while (dy < n && yj >= n - dy) {
+      yj -= n - dy;
+      ++dy;
     }
-    const int yk = yj + dy;
-    for (int dx = -(n - 1) + warp; dx < n; dx += warps) {
-      if (dy == 0 && dx <= 0) continue;
-      const int xlo = dx < 0 ? -dx : 0, wx = n - (dx < 0 ? -dx : dx);
-      const float *row = w + doff[disp_index(dx, dy, n)] + (long)yj * wx;
-      float *trow = T + (dx + n - 1) * p + xlo;
-      for (int x = lane; x < wx; x += 32) trow[x] = __ldcs(row + x);
+    // copy the diagonals dx = -(n - 1) + r, r = warp + i kExpWarps2: lane i looks up the i-th offset
+    const int mine = warp + lane * kExpWarps2, first = dy == 0 ? n : 0;
+    const long long off = mine >= first && mine < 2 * n - 1 ? doff[disp_index(mine - (n - 1), dy, n)] : 0;
+    for (int r = warp, i = 0; r < 2 * n - 1; r += kExpWarps2, ++i) {
+      const long long ro = __shfl_sync(0xffffffffu, off, i);
+      if (r < first) continue;
+      const int dx = r - (n - 1), xlo = max(-dx, 0), wx = n - abs(dx);
+      const float *row = w + ro + yj * wx;
+      unsigned dst = ts + 4u * (xlo * (p + 1) + dx + lane * (p + 1));
+      for (int x = lane; x < wx; x += 32, dst += 128u * (p + 1))
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(row + x) : "memory");
     }
+    asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
-    const long jrow = (long)n * yj, krow = (long)n * yk;
+    const long jrow = (long)n * yj, krow = (long)n * (yj + dy);
     const float *ssj = ss + jrow, *ssk = ss + krow;
     if constexpr (OUT == kSymBlocks) {
       float *blk = k32 + (long)t * n * n;
-      for (int xj = warp; xj < n; xj += warps) {
-        float *out = blk + (long)xj * n;
-        for (int xk = lane; xk < n; xk += 32) {
-          const int dx = xk - xj;
-          float v;
-          if (dy > 0 || dx > 0)
-            v = T[(dx + n - 1) * p + xj];
-          else if (dx < 0)
-            v = T[(-dx + n - 1) * p + xk];  // A_jk = A_kj, stored under (-dx, 0) for target xk
-          else
-            v = (float)diag[jrow + xj];
-          out[xk] = v;
-        }
+      if (dy > 0 && p == n) {  // the tile as it lies
+        for (int q = threadIdx.x; q < n * n / 4; q += kExpThreads2) ((float4 *)blk)[q] = ((const float4 *)T)[q];
+      } else {
+        for (int xj = warp; xj < n; xj += kExpWarps2)
+          for (int xk = lane; xk < n; xk += 32) {
+            float v;
+            if (dy > 0 || xk > xj)
+              v = T[xj * p + xk];
+            else if (xk < xj)
+              v = T[xk * p + xj];  // A_jk = A_kj
+            else
+              v = (float)diag[jrow + xj];
+            blk[xj * n + xk] = v;
+          }
       }
     } else if (dy > 0) {
       // every (xj, xk) is a pair of this item
-      for (int xj = warp; xj < n; xj += warps) {
-        const float *tb = T + (n - 1 - xj) * p + xj;  // T[(xk - xj + n - 1) p + xj]
+      for (int xj = warp; xj < n; xj += kExpWarps2) {
         const long rb = (jrow + xj) * ldk + krow;
-        for (int xk = lane; xk < n; xk += 32) put_entry<OUT>(rb + xk, tb[xk * p] * ssk[xk], k32, khi, klo);
+        for (int xk = lane; xk < n; xk += 32) put_entry<OUT>(rb + xk, T[xj * p + xk] * ssk[xk], k32, khi, klo);
       }
-      for (int xk = warp; xk < n; xk += warps) {
-        const float *tb = T + (xk + n - 1) * p;  // T[(xk - xj + n - 1) p + xj]
+      for (int xk = warp; xk < n; xk += kExpWarps2) {
         const long rb = (krow + xk) * ldk + jrow;
-        for (int xj = lane; xj < n; xj += 32) put_entry<OUT>(rb + xj, tb[xj * (1 - p)] * ssj[xj], k32, khi, klo);
+        for (int xj = lane; xj < n; xj += 32) put_entry<OUT>(rb + xj, T[xj * p + xk] * ssj[xj], k32, khi, klo);
       }
     } else {
       // one grid row: columns right of the diagonal from j, left of it from k
-      for (int r = warp; r < n; r += warps) {
+      for (int r = warp; r < n; r += kExpWarps2) {
         const long rb = (jrow + r) * ldk + jrow;
         for (int x = lane; x < n; x += 32) {
           if (x == r) continue;
-          const float v = x > r ? T[(x - r + n - 1) * p + r] : T[(r - x + n - 1) * p + x];
+          const float v = x > r ? T[r * p + x] : T[x * p + r];
           put_entry<OUT>(rb + x, v * ssj[x], k32, khi, klo);
         }
       }
-      for (int r = threadIdx.x; r < n; r += blockDim.x) {
+      for (int r = threadIdx.x; r < n; r += kExpThreads2) {
         const long j = jrow + r;
         put_entry<OUT>(j * ldk + j, (float)(diag[j] * ss64[j]), k32, khi, klo);
       }
     }
     __syncthreads();
+    yj += gridDim.x;
   }
 }
 
@@ -803,14 +819,10 @@ Plan chunk_plan(const std::vector<int> &starts, int R) {
 
 }  // namespace
 
-// the expansion's sheared tile: 2 n - 1 diagonals of n + 2 floats
-static size_t expand_smem_bytes(int n) { return sizeof(float) * (size_t)(2 * n - 1) * (n + 2); }
+// the largest grid of the expansion: larger ones are assembled by tile pairs
+constexpr int kExpandMaxN = 169;
 
-bool disp_expand_fits(int n, int device) {
-  int optin = 0;
-  if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device) != cudaSuccess) return false;
-  return expand_smem_bytes(n) <= (size_t)optin;
-}
+bool disp_expand_fits(int n) { return n <= kExpandMaxN; }
 
 size_t disp_smem_bytes(int n, int R) {
   const long rows = n + R;
@@ -1221,8 +1233,7 @@ vie_status disp_expand(const DispPlan &dp, int n, const float *wbuf, const doubl
   }
   DevProps prop;
   VIE_TRY(get_dev_props(device, &prop));
-  const size_t smem = expand_smem_bytes(n);
-  if (smem > (size_t)prop.sharedMemPerBlockOptin) {
+  if (!disp_expand_fits(n)) {
     set_error("vie_assemble: grid too large for the pair-weight expansion");
     return VIE_ERR_UNSUPPORTED;
   }
@@ -1230,18 +1241,21 @@ vie_status disp_expand(const DispPlan &dp, int n, const float *wbuf, const doubl
   const void *kx = out == kSymBlocks  ? (const void *)k_expand_pairs<kSymBlocks>
                    : out == kDenseF32 ? (const void *)k_expand_pairs<kDenseF32>
                                       : (const void *)k_expand_pairs<kDenseBF16>;
-  VIE_TRY(raise_smem_limit(kx, (size_t)((int)smem)));
+  const size_t smem = sizeof(float) * (size_t)n * expand_pitch(n, out);
+  VIE_TRY(raise_smem_limit(kx, smem));
   k_to_f32<<<(int)std::min((N + 255) / 256, 1024L), 256, 0, st>>>(N, sigma_s, dp.ss32);
   VIE_CHECK_LAUNCH("k_to_f32");
-  const int grid = prop.multiProcessorCount;
+  // as many CTAs as an SM's 228 KB hold (1 KB of each is the system's), three at most
+  const int per_sm = (int)std::min<size_t>(3, (228 << 10) / (smem + 1024));
+  const int grid = per_sm * prop.multiProcessorCount;
   if (out == kSymBlocks)
-    k_expand_pairs<kSymBlocks><<<grid, 1024, smem, st>>>(n, wbuf, dp.doff, dp.ss32, diag, sigma_s, 0, k32, nullptr,
+    k_expand_pairs<kSymBlocks><<<grid, kExpThreads2, smem, st>>>(n, wbuf, dp.doff, dp.ss32, diag, sigma_s, 0, k32, nullptr,
                                                          nullptr);
   else if (out == kDenseF32)
-    k_expand_pairs<kDenseF32><<<grid, 1024, smem, st>>>(n, wbuf, dp.doff, dp.ss32, diag, sigma_s, ldk, k32,
+    k_expand_pairs<kDenseF32><<<grid, kExpThreads2, smem, st>>>(n, wbuf, dp.doff, dp.ss32, diag, sigma_s, ldk, k32,
                                                         nullptr, nullptr);
   else
-    k_expand_pairs<kDenseBF16><<<grid, 1024, smem, st>>>(n, wbuf, dp.doff, dp.ss32, diag, sigma_s, ldk, nullptr,
+    k_expand_pairs<kDenseBF16><<<grid, kExpThreads2, smem, st>>>(n, wbuf, dp.doff, dp.ss32, diag, sigma_s, ldk, nullptr,
                                                          (unsigned short *)khi, (unsigned short *)klo);
   VIE_CHECK_LAUNCH("k_expand_pairs");
   return VIE_OK;

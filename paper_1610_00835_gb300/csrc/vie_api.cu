@@ -1224,7 +1224,7 @@ static vie_status assemble_impl(vie_handle *h, int mode, int order, void *stream
   }
   if (mode == VIE_OPERATOR_SYM32) {
     // A in the symmetric blocks of grid-row pairs: the pair weights, expanded
-    if (h->use_kernel != VIE_KERNEL_DISPLACEMENT || h->dim != 2 || !disp_expand_fits(h->n, h->device) ||
+    if (h->use_kernel != VIE_KERNEL_DISPLACEMENT || h->dim != 2 || !disp_expand_fits(h->n) ||
         h->n > symv_max_n()) {
       set_error("vie_assemble: VIE_OPERATOR_SYM32 needs the displacement kernel, its expansion and the "
                 "block product (2D, FP32 tiles, S = 64, n <= 160)");
@@ -1263,7 +1263,7 @@ static vie_status assemble_impl(vie_handle *h, int mode, int order, void *stream
   // dense K from the displacement kernel's pair weights where the expansion
   // has room for the grid, else from the tile-pair assembler (M-iii only)
   const bool disp2 =
-      h->use_kernel == VIE_KERNEL_DISPLACEMENT && h->dim == 2 && disp_expand_fits(h->n, h->device);
+      h->use_kernel == VIE_KERNEL_DISPLACEMENT && h->dim == 2 && disp_expand_fits(h->n);
   // 3D: the pair weights of the 3D displacement kernel, expanded along grid lines
   const bool disp3 = h->use_kernel == VIE_KERNEL_DISPLACEMENT && h->dim == 3 && h->disp3.usable &&
                      h->opts.disc == VIE_DISC_MIII;

@@ -234,7 +234,7 @@ vie_status symv3_apply(const DispPlan3 &dp, int op, const double *sigma_s, const
                        float *s, float *partial, double *y, int device, cudaStream_t st);
 
 size_t disp_smem_bytes(int n, int R);  // shared lattice bytes at stack depth R
-bool disp_expand_fits(int n, int device);  // k_expand_pairs has room for the grid (n <= 169)
+bool disp_expand_fits(int n);  // k_expand_pairs takes the grid (n <= 169)
 vie_status disp_source(const DispPlan &dp, long N, int op, const double *sigma_s, const double *g, cudaStream_t st);
 vie_status disp_reduce(const DispPlan &dp, long N, int op, const double *diag, const double *sigma_s,
                        const double *g, double *y, cudaStream_t st);
