@@ -12,15 +12,26 @@
 // same records and packed-pair march as in 2D, disp_march.cuh).  Three orientations,
 // chosen per D by estimated cost: runs along z with lanes on x (units fix a y),
 // runs along y with lanes on x (units fix a z), runs along x with lanes on y
-// (units fix a z).  A thread stacks kR targets along the run axis.  When the
-// lane extent of D is below 32, a warp holds 32 / gw lane groups of width gw
-// (gw the power of two at or above it) at third-axis coordinates gw apart:
-// with the odd pitches n + 1 and (n + 1)^2 the groups fall in distinct banks.
+// (units fix a z).  A thread stacks kR targets along the run axis.
 //
-// The lattice is the padded (n + 1)^3 sigma_t array, linear (x fastest), with
-// kPad3 zero planes appended: reads of discarded stacked targets only run
-// forward along the run axis, by at most kPad3 strides, so every read stays in
-// shared memory.  The weights of valid
+// What bounds the march is the shared-memory data path: per chunk of L cells and
+// tile L + kR - 1 lattice words a lane, and 4 wavefronts per record load (a
+// uniform 16-byte load fills 32 lanes' registers).  So a unit is two tiles of
+// 32 lanes that share every record load, and the tiles of a D are few: a tile's
+// lanes are 32 / gw groups of gw = 2^k consecutive lanes, at other third-axis
+// coordinates or stack blocks, and a lane extent that is no power of two is cut
+// into such widths (20 = 16 + 4) where that takes fewer tiles (cover_box
+// below): at 32^3 81 % of the lanes' products are of valid targets, where one
+// tile a unit and one group width per D gave 68 %.  Measured: the march of the
+// stored weights 6.44 -> 5.25 ms at 32^3 (the data path at about 80 %), an apply
+// 7.08 -> 5.97 ms, and 35.4 -> 4.92 at 31^3, where the even pitch n + 1 put the
+// lane groups into one bank.
+//
+// The lattice is the padded (n + 1)^3 sigma_t array, x fastest, with odd row
+// and plane pitches (17 for n <= 16, 33 above, and their squares), with which
+// the lane groups fall in distinct banks, and kPad3 zero planes appended: reads
+// of discarded stacked targets only run forward along the run axis, by at most
+// kPad3 strides, so every read stays in shared memory.  The weights of valid
 // targets only touch the (n + 1)^3 part.
 //
 // Only D in a half space is marched (A_jk = A_kj); each pair adds w s_k to y_j
@@ -29,6 +40,7 @@
 // reproducible.  Runs along x put their sums in a second array with y fastest,
 // so a warp's atomics always cover contiguous words.  k_disp3_reduce adds the
 // two sums of each target, converts once, adds the self cell and clears both.
+#include <limits.h>
 #include <math.h>
 
 #include <algorithm>
@@ -47,11 +59,13 @@ namespace {
 
 using dmarch::kMaxChunk;
 using dmarch::kR;
-using dmarch::march_runs;
-using dmarch::red_add;
+using dmarch::march_runs_pair;
 using march::kS;
 
-constexpr int kThreads3 = 1024;
+// two tiles per thread in 72 registers; 28 warps hide the record loads (apply at
+// 32^3: 8.16 ms with 512 threads, 7.00 with 640, 6.23 with 768, 5.96 with 896, 6.36 with 1024)
+constexpr int kThreads3 = 896;
+constexpr int kGrab3 = 2;       // units taken from the counter at a time
 constexpr int kPad3 = kR - 1;  // zero planes after the lattice
 constexpr int kMaxN3 = 32;                     // one lane block per unit
 
@@ -69,18 +83,52 @@ struct Disp3Args {
   const int4 *units;         // see geometry3_build
   int *counter;              // [2]
   long n_units;
-  int n, ldp, plane;
+  int n;
   long lat_elems;
   float tau_scale2, wcoef;
 };
+
+// A tile of a D's box of targets, in coordinates relative to the box: 32 lanes
+// in 2^lg groups of gw = 32 >> lg consecutive lanes from lane0 on, 2^lgs of
+// every 2^lg groups on different stack blocks (of kR targets), the others on
+// different third-axis coordinates, from third0 and block0 on.  The offsets
+// below keep the groups in distinct banks, for odd pitches: as multiples of gw
+// mod 32, third-axis steps give gw times 0, 1, ..; with 2 or 4 stack blocks these
+// give 8 times 0 .. 3 (16 for gw = 16, two blocks apart), and the third axis takes
+// the multiples of gw below 8, then those 16 further on.
+__host__ __device__ constexpr int tile3_code(int lane0, int third0, int block0, int lg, int lgs) {
+  return lane0 | (third0 << 5) | (block0 << 10) | (lg << 12) | (lgs << 15);
+}
+
+struct Tile3 {
+  int lane, stack, third;  // the first stacked target of this lane
+  bool valid;              // this lane has targets here (else the coordinates are some target's)
+};
+
+__host__ __device__ inline Tile3 tile3_at(int code, int lanes, int stack, int thirds, int lane) {
+  const int lg = (code >> 12) & 7, lgs = (code >> 15) & 3, gw = 32 >> lg;
+  const int g = lane >> (5 - lg), gs = g & ((1 << lgs) - 1), o = gw * (g >> lgs);
+  Tile3 t;
+  t.lane = (code & 31) + (lane & (gw - 1));
+  t.third = ((code >> 5) & 31) + (lgs == 0 ? o : (o & 7) + 2 * (o & 8));
+  t.stack = kR * (((code >> 10) & 3) + (lg == 1 ? 2 * gs : gs));
+  t.valid = t.lane < lanes && t.third < thirds && t.stack < stack;
+  if (!t.valid) {
+    t.lane = t.lane < lanes ? t.lane : lanes - 1;
+    t.third = (code >> 5) & 31;
+    t.stack = kR * ((code >> 10) & 3);
+  }
+  return t;
+}
 
 // STORE: instead of the apply's sums, write w = h^3 e^{-tau} / (4 pi r^2) of
 // every pair (j, j + D) to pairs: per D of the half space its box of targets,
 // x fastest, then y, then z.  A warp's stores are contiguous when its lanes
 // run along x; for runs along x (lanes on y) they are strided, but the units
 // of one D run back to back and L2 gathers its box before writing it out.
-template <int LDP, int PLANE, bool STORE>
+template <int LDP, bool STORE>
 __global__ void __launch_bounds__(kThreads3, 1) k_pairs_disp3(Disp3Args a) {
+  constexpr int PLANE = LDP * LDP;
   extern __shared__ float4 smem4[];
   float *lat = reinterpret_cast<float *>(smem4);
   const int tid = threadIdx.x, lane = tid & 31;
@@ -90,112 +138,115 @@ __global__ void __launch_bounds__(kThreads3, 1) k_pairs_disp3(Disp3Args a) {
     for (long i = tid; i < n4; i += kThreads3) smem4[i] = g4[i];
     for (long i = n4 * 4 + tid; i < a.lat_elems; i += kThreads3) lat[i] = a.lat[i];
   }
-  __syncthreads();
-  double scale_d = 1.0;
-  if constexpr (!STORE) {
+  // power-of-two scale 2^k <= 2^62 / (max|s| R), by one thread (FP64)
+  __shared__ double scale_s;
+  if (!STORE && tid == 0) {
     const float smax = __uint_as_float(*a.smax);
-    if (smax > 0.f) scale_d = ldexp(1.0, ilogb(4.611686018427387904e18 / ((double)smax * a.rbound)));
+    scale_s = smax > 0.f ? ldexp(1.0, ilogb(4.611686018427387904e18 / ((double)smax * a.rbound))) : 1.0;
   }
-  const float scale = (float)scale_d;
-  const int n = a.n;
-  const int ldp = LDP > 0 ? LDP : a.ldp, plane = PLANE > 0 ? PLANE : a.plane;
+  __syncthreads();
+  const float scale = STORE ? 1.f : (float)scale_s;
+  const int n = a.n, nn = n * n;
   const unsigned lat_base = (unsigned)__cvta_generic_to_shared(lat);
   long u0 = 0, u_end = 0;
   for (;;) {
     if (u0 >= u_end) {
       long got = 0;
-      if (lane == 0) got = atomicAdd(a.counter, 4);
+      if (lane == 0) got = atomicAdd(a.counter, kGrab3);
       got = __shfl_sync(0xffffffffu, got, 0);
       if (got >= a.n_units) break;
       u0 = got;
-      u_end = min(got + 4, a.n_units);
+      u_end = min(got + kGrab3, a.n_units);
     }
     const int4 un = a.units[u0++];
     const int dx = (signed char)(un.y & 0xff), dy = (signed char)((un.y >> 8) & 0xff);
     const int dz = (signed char)((un.y >> 16) & 0xff);
-    const int orient = (un.y >> 24) & 3, lg = (un.y >> 26) & 7;
-    const int sb = un.z & 0xff, c3 = (un.z >> 8) & 0xff;
-    const int nrec = un.w;
-    const int xlo = max(0, -dx), xhi = n - max(0, dx);
-    const int ylo = max(0, -dy), yhi = n - max(0, dy);
-    const int zlo = max(0, -dz), zhi = n - max(0, dz);
+    const int orient = (un.y >> 24) & 3;
+    const int nrec = un.w >> 17;
+    const int wx = n - abs(dx), wy = n - abs(dy), wz = n - dz;
+    const int xlo = max(0, -dx), ylo = max(0, -dy);  // (dz >= 0: z from 0 on)
     // lane, stack (run) and third axes of this orientation
-    const int llo = orient == 2 ? ylo : xlo, lhi = orient == 2 ? yhi : xhi;
-    const int slo = orient == 0 ? zlo : orient == 1 ? ylo : xlo;
-    const int shi = orient == 0 ? zhi : orient == 1 ? yhi : xhi;
-    const int thi = orient == 0 ? yhi : zhi;
-    const int gw = 32 >> lg, g = lane >> (5 - lg), lig = lane & (gw - 1);
-    int c = c3 + gw * g;
-    bool lvalid = c < thi;
-    if (!lvalid) c = c3;
-    int la = llo + lig;
-    lvalid = lvalid && la < lhi;
-    la = min(la, lhi - 1);
-    const int b0 = slo + kR * sb;
-    int x, y, z;
-    if (orient == 0) {
-      x = la; z = b0; y = c;
-    } else if (orient == 1) {
-      x = la; y = b0; z = c;
-    } else {
-      y = la; x = b0; z = c;
-    }
-    const unsigned base = lat_base + 4u * (unsigned)(x + ldp * y + plane * z);
+    const int lanes = orient == 2 ? wy : wx, stack = orient == 0 ? wz : orient == 1 ? wy : wx;
+    const int thirds = orient == 0 ? wy : wz;
+    const bool two = un.z < 0;
+    const Tile3 ta = tile3_at(un.z, lanes, stack, thirds, lane);
+    // (a unit of one tile marches it twice)
+    const Tile3 tb = tile3_at(two ? un.w : un.z, lanes, stack, thirds, lane);
     {
       // bring this D's chunk records into L1 (one 128-byte line per lane)
       const char *r0 = reinterpret_cast<const char *>(a.stencil + un.x);
       const int lines = (int)(((reinterpret_cast<size_t>(r0) & 127) + 16L * nrec + 127) >> 7);
       for (int l = lane; l < lines; l += 32) asm volatile("prefetch.global.L1 [%0];" ::"l"(r0 + 128L * l));
     }
-    dmarch::Acc2<kR> sums;
-    sums.zero();
+    dmarch::Acc2<kR> sa, sb;
+    sa.zero();
+    sb.zero();
+    const float4 *rec = a.stencil + un.x;
+    const unsigned box = lat_base + 4u * (unsigned)(xlo + LDP * ylo);
+    const int sl = orient == 2 ? LDP : 1, sq = orient == 0 ? PLANE : orient == 1 ? LDP : 1;
+    const int st = orient == 0 ? LDP : PLANE;
+    const unsigned ba = box + 4u * (unsigned)(ta.lane * sl + ta.stack * sq + ta.third * st);
+    const unsigned bb = box + 4u * (unsigned)(tb.lane * sl + tb.stack * sq + tb.third * st);
     if (orient == 0)
-      march_runs<PLANE, kR>(a.stencil + un.x, base, plane, sums);
+      march_runs_pair<PLANE, kR>(rec, ba, bb, PLANE, sa, sb);
     else if (orient == 1)
-      march_runs<LDP, kR>(a.stencil + un.x, base, ldp, sums);
+      march_runs_pair<LDP, kR>(rec, ba, bb, LDP, sa, sb);
     else
-      march_runs<1, kR>(a.stencil + un.x, base, 1, sums);
-    float acc[kR];
-    sums.sum(acc);
+      march_runs_pair<1, kR>(rec, ba, bb, 1, sa, sb);
     const float r2 = (float)(dx * dx + dy * dy + dz * dz);
     const float inv_r = rsqrtf(r2);
     const float tscale = -a.tau_scale2 * r2 * inv_r;  // -(h/S) log2(e) r
     const float wk = a.wcoef * inv_r * inv_r;
-    if constexpr (STORE) {
-      const int m2 = 2 * n - 1;
-      const long base = __ldg(a.doff + ((long)(dz + n - 1) * m2 + (dy + n - 1)) * m2 + (dx + n - 1));
-      const long wx = xhi - xlo, wy = yhi - ylo;
-      // the unit's first target in the box, and the stride of its stacked targets
-      const long o0 = base + ((long)(z - zlo) * wy + (y - ylo)) * wx + (x - xlo);
-      const long ostep = orient == 0 ? wx * wy : orient == 1 ? wx : 1;
+    // one copy of the epilogue's code for both tiles
+#pragma unroll 1
+    for (int code = un.z;; code = un.w, sa = sb) {
+      const Tile3 t = tile3_at(code, lanes, stack, thirds, lane);
+      float acc[kR];
+      sa.sum(acc);
+      const int cnt = t.valid ? min(kR, stack - t.stack) : 0;  // stacked targets of this lane
+      if constexpr (STORE) {
+        // the unit's first target in the stored box, and the stride of its stacked targets
+        const int m2 = 2 * n - 1, wxy = wx * wy;
+        float *out = a.pairs + __ldg(a.doff + ((dz + n - 1) * m2 + (dy + n - 1)) * m2 + (dx + n - 1));
+        unsigned o = orient == 0   ? t.lane + wx * t.third + wxy * t.stack
+                     : orient == 1 ? t.lane + wx * t.stack + wxy * t.third
+                                   : wx * t.lane + t.stack + wxy * t.third;
+        const unsigned ostep = orient == 0 ? wxy : orient == 1 ? wx : 1;
 #pragma unroll
-      for (int q = 0; q < kR; ++q)
-        if (lvalid && b0 + q < shi) __stcs(a.pairs + o0 + q * ostep, wk * exp2f(tscale * acc[q]));
-      continue;
-    }
-    // targets and partners in the layout whose fastest axis carries the lanes:
-    // x fastest (s, the first half of yacc) or, for runs along x, y fastest
-    // (s_t, the second half), so the atomics of a warp hit contiguous words
-    const long nn = (long)n * n;
-    const bool ty = orient == 2;
-    const float *sv = ty ? a.src_t : a.src;
-    unsigned long long *ya = ty ? a.yacc + nn * n : a.yacc;
-    const long j0 = ty ? ((long)z * n + x) * n + y : x + (long)n * (y + (long)n * z);
-    const long jstep = orient == 0 ? nn : n;
-    const long dk = ty ? dy + (long)n * (dx + (long)n * dz) : dx + (long)n * (dy + (long)n * dz);
+        for (int q = 0; q < kR; ++q, o += ostep)
+          if (q < cnt) __stcs(out + o, wk * exp2f(tscale * acc[q]));
+      } else {
+        // targets and partners in the layout whose fastest axis carries the lanes:
+        // x fastest (s, the first half of yacc) or, for runs along x, y fastest
+        // (s_t, the second half), so the atomics of a warp hit contiguous words;
+        // byte offsets of 32 bits, and the scale (a power of two) folded into
+        // the weight, as in 2D
+        const bool ty = orient == 2;
+        const char *sv = reinterpret_cast<const char *>(ty ? a.src_t : a.src);
+        char *ya = reinterpret_cast<char *>(ty ? a.yacc + nn * n : a.yacc);
+        const int jl = t.lane + (ty ? ylo : xlo), js = t.stack + (ty ? xlo : orient == 1 ? ylo : 0);
+        const int jt = t.third + (orient == 0 ? ylo : 0);
+        unsigned oj = 4u * (unsigned)(jl + (orient == 0 ? n * jt + nn * js : n * js + nn * jt));
+        const unsigned dk = 4u * (unsigned)((ty ? dy + n * dx : dx + n * dy) + nn * dz);
+        const unsigned step = 4u * (unsigned)(orient == 0 ? nn : n);
+        const float wks = wk * scale;
 #pragma unroll
-    for (int q = 0; q < kR; ++q) {
-      if (lvalid && b0 + q < shi) {
-        const long j = j0 + q * jstep, k = j + dk;
-        const float sj = __ldg(sv + j), sk = __ldg(sv + k);
-        const float w = wk * exp2f(tscale * acc[q]) * scale;
-        red_add(ya + j, (unsigned long long)__float2ll_rn(w * sk));
-        red_add(ya + k, (unsigned long long)__float2ll_rn(w * sj));
+        for (int q = 0; q < kR; ++q, oj += step) {
+          if (q < cnt) {
+            const unsigned ok = oj + dk;
+            const float sj = __ldg(reinterpret_cast<const float *>(sv + oj));
+            const float sk = __ldg(reinterpret_cast<const float *>(sv + ok));
+            const float w = wks * exp2f(tscale * acc[q]);
+            dmarch::red_add(ya, 2u * oj, (unsigned long long)__float2ll_rn(w * sk));
+            dmarch::red_add(ya, 2u * ok, (unsigned long long)__float2ll_rn(w * sj));
+          }
+        }
       }
+      if (!two || code == un.w) break;
     }
   }
   __syncthreads();
-  if (!STORE && blockIdx.x == 0 && tid == 0) *a.scale_out = scale_d;
+  if (!STORE && blockIdx.x == 0 && tid == 0) *a.scale_out = scale_s;
   if (tid == 0) {
     __threadfence();
     if (atomicAdd(a.counter + 1, 1) == (int)gridDim.x - 1) {
@@ -207,10 +258,15 @@ __global__ void __launch_bounds__(kThreads3, 1) k_pairs_disp3(Disp3Args a) {
   }
 }
 
-// the padded lattice (pitch n + 1, x fastest) followed by kPad3 zero planes
-__global__ void k_make_lattice3(long lat, long total, const float *__restrict__ pad, float *__restrict__ out) {
-  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < total; i += (long)gridDim.x * blockDim.x)
-    out[i] = i < lat ? pad[i] : 0.f;
+// row pitch of the lattice in shared memory (its square is the plane pitch)
+constexpr int disp3_pitch(int n) { return n <= 16 ? 17 : 33; }
+
+// the padded lattice (n + 1 values a row, x fastest) at pitch ldp, zero elsewhere
+__global__ void k_make_lattice3(int n, int ldp, long total, const float *__restrict__ pad, float *__restrict__ out) {
+  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < total; i += (long)gridDim.x * blockDim.x) {
+    const int x = (int)(i % ldp), y = (int)(i / ldp % ldp), z = (int)(i / (ldp * ldp));
+    out[i] = x <= n && y <= n && z <= n ? pad[x + (n + 1) * (y + (n + 1) * z)] : 0.f;
+  }
 }
 
 // s = sigma_s g (or g) in FP32, its copy with y fastest, and max |s|
@@ -604,8 +660,8 @@ __global__ void k_to_f32_3(long N, const double *__restrict__ x, float *__restri
 typedef void (*Disp3Kernel)(Disp3Args);
 
 Disp3Kernel pick_disp3(int n, bool store = false) {
-  if (store) return n == 32 ? k_pairs_disp3<33, 1089, true> : k_pairs_disp3<0, 0, true>;
-  return n == 32 ? k_pairs_disp3<33, 1089, false> : k_pairs_disp3<0, 0, false>;
+  if (disp3_pitch(n) == 17) return store ? k_pairs_disp3<17, true> : k_pairs_disp3<17, false>;
+  return store ? k_pairs_disp3<33, true> : k_pairs_disp3<33, false>;
 }
 
 // ---- geometry (host): stencils, chunk records and work units, per (device, n)
@@ -733,8 +789,52 @@ void geometry3_trim() {
 
 struct Unit3 {
   int4 u;
+  int orient;
   long cost;
 };
+
+// The fewest tiles that cover a box of lanes x thirds targets and nsb stack
+// blocks, lanes from lane0 on: groups of gw = 2^k lanes at or above the lane
+// extent, or those of the next lower 2^k and a cover of the rest.  For one gw
+// the groups of a tile lie at other thirds; with gw <= 8 also on 2 or 4 stack
+// blocks, with gw = 16 on two blocks two apart.
+void cover_box(int lane0, int lanes, int thirds, int nsb, std::vector<int> &codes) {
+  const auto one = [&](int gw, std::vector<int> &out) {
+    const int lg = 5 - __builtin_ctz(gw);
+    std::vector<int> best, alt;
+    for (int sb = 0; sb < nsb; ++sb)
+      for (int j = 0; j < std::min(gw, thirds); ++j) best.push_back(tile3_code(lane0, j, sb, lg, 0));
+    const auto keep = [&]() {
+      if (alt.size() < best.size()) best = alt;
+      alt.clear();
+    };
+    if (gw <= 8 && nsb > 1) {
+      for (int sb = 0; sb < nsb; sb += 4)
+        for (int m = 0; m < thirds; m += 8)
+          for (int j = m; j < std::min(m + gw, thirds); ++j) alt.push_back(tile3_code(lane0, j, sb, lg, 2));
+      keep();
+      for (int sb = 0; sb < nsb; sb += 2)
+        for (int m = 0; m < std::min(16, thirds); m += 8)
+          for (int j = m; j < std::min(m + gw, thirds); ++j) alt.push_back(tile3_code(lane0, j, sb, lg, 1));
+      keep();
+    }
+    if (gw == 16 && nsb > 2) {
+      for (int sb = 0; sb < 2; ++sb)
+        for (int j = 0; j < thirds; ++j) alt.push_back(tile3_code(lane0, j, sb, lg, 1));
+      keep();
+    }
+    out.insert(out.end(), best.begin(), best.end());
+  };
+  const int up = pow2ceil(lanes);
+  std::vector<int> whole, cut;
+  one(up, whole);
+  if (up > lanes) {
+    one(up / 2, cut);
+    cover_box(lane0 + up / 2, lanes - up / 2, thirds, nsb, cut);
+    if (cut.size() < whole.size()) whole = cut;
+  }
+  codes.insert(codes.end(), whole.begin(), whole.end());
+}
 
 // the records and units of the displacements with one dz (record offsets local
 // to this plane's record list)
@@ -745,7 +845,7 @@ struct Plane3 {
 };
 
 void build_plane3(int n, int dz, Plane3 &out) {
-  const int ldp = n + 1, plane = ldp * ldp;
+  const int ldp = disp3_pitch(n), plane = ldp * ldp;
   std::vector<double> box;
   std::vector<Run3> runs[3];
   std::vector<double> wts[3];
@@ -800,22 +900,22 @@ void build_plane3(int n, int dz, Plane3 &out) {
           for (int i = 0; i < lc; ++i) rec.push_back((float)wts[best][r.woff + c0 + i]);
           for (int i = lc + 1; i < 4 * ((lc + 4) / 4); ++i) rec.push_back(0.f);
         });
-      const int lanes = lanes_of[best], third = third_of[best];
-      const int gw = pow2ceil(lanes), lg = 5 - __builtin_ctz(gw);  // 32 / gw lane groups
-      const int tlo = best == 0 ? std::max(0, -dy) : 0;           // third axis y (orientation 0) or z
-      const int nsb = (stack_of[best] + kR - 1) / kR;
-      const int dxyz = (dx & 0xff) | ((dy & 0xff) << 8) | ((dz & 0xff) << 16) | (best << 24) | (lg << 26);
-      const int w = (int)pl.recs;  // the D's record float4s (header included)
-      for (int sb = 0; sb < nsb; ++sb)
-        for (int j = 0; j < gw && j < third; ++j)
-          units.push_back({make_int4(off, dxyz, sb | ((tlo + j) << 8), w), pl.cost});
+      const int dxyz = (dx & 0xff) | ((dy & 0xff) << 8) | ((dz & 0xff) << 16) | (best << 24);
+      std::vector<int> codes;
+      cover_box(0, lanes_of[best], third_of[best], (stack_of[best] + kR - 1) / kR, codes);
+      for (size_t c = 0; c < codes.size(); c += 2) {
+        const bool two = c + 1 < codes.size();
+        const int z = codes[c] | (two ? INT_MIN : 0), w = (two ? codes[c + 1] : 0) | ((int)pl.recs << 17);
+        units.push_back({make_int4(off, dxyz, z, w), best, pl.cost});
+      }
     }
 }
 
 // Units (int4): x = the D's record header (float4 index); y = dx | dy << 8 |
-// dz << 16 (8-bit two's complement) | orientation << 24 | log2(lane groups)
-// << 26; z = stack block | first third-axis coordinate << 8; w = the D's
-// record float4s.
+// dz << 16 (8-bit two's complement) | orientation << 24; z = the first tile's
+// code, the sign bit set if there is a second; w = the second's code | the D's
+// record float4s << 17.  They are sorted by orientation (one march's code at a
+// time in the instruction cache), then by falling cost.
 // The planes dz are built on host threads and joined in dz order.
 vie_status geometry3_build(int n, Geometry3 *geo) {
   std::vector<Plane3> planes(n);
@@ -841,7 +941,9 @@ vie_status geometry3_build(int n, Geometry3 *geo) {
     std::vector<float>().swap(planes[dz].rec);
   }
   for (int i = 0; i < 32; ++i) rec.push_back(0.f);  // the L1 prefetch may reach 127 bytes past a stencil
-  std::stable_sort(units.begin(), units.end(), [](const Unit3 &p, const Unit3 &q) { return p.cost > q.cost; });
+  std::stable_sort(units.begin(), units.end(), [](const Unit3 &p, const Unit3 &q) {
+    return p.orient != q.orient ? p.orient < q.orient : p.cost > q.cost;
+  });
   std::vector<int4> uv(units.size());
   for (size_t i = 0; i < units.size(); ++i) uv[i] = units[i].u;
   VIE_CUDA(vie_malloc((void **)&geo->units, sizeof(int4) * uv.size()));
@@ -884,10 +986,9 @@ void geometry3_release(Geometry3 *g) {
 
 }  // namespace
 
-size_t disp3_smem_bytes(int n) {
-  const long p = n + 1;
-  return sizeof(float) * (size_t)(p * p * (p + kPad3));
-}
+static long lattice3_elems(int n) { return (long)disp3_pitch(n) * disp3_pitch(n) * (n + 1 + kPad3); }
+
+size_t disp3_smem_bytes(int n) { return sizeof(float) * (size_t)lattice3_elems(n); }
 
 vie_status disp3_prepare(DispPlan3 *dp, int n, const float *sig_padded, int device, cudaStream_t st) {
   dp->usable = 0;
@@ -909,13 +1010,12 @@ vie_status disp3_prepare(DispPlan3 *dp, int n, const float *sig_padded, int devi
   dp->stencil = geo->stencil;
   dp->n_units = geo->n_units;
   dp->taps = geo->taps;
-  const long N = (long)n * n * n, p = n + 1;
-  const long lat = p * p * p, lat_elems = p * p * (p + kPad3);
+  const long N = (long)n * n * n, lat_elems = lattice3_elems(n);
   VIE_CUDA(vie_malloc((void **)&dp->counter, 2 * sizeof(int)));
   VIE_CUDA(cudaMemset(dp->counter, 0, 2 * sizeof(int)));
   VIE_CUDA(vie_malloc((void **)&dp->lattice, sizeof(float) * lat_elems));
-  k_make_lattice3<<<(int)std::min((lat_elems + 255) / 256, 4096L), 256, 0, st>>>(lat, lat_elems, sig_padded,
-                                                                                 (float *)dp->lattice);
+  k_make_lattice3<<<(int)std::min((lat_elems + 255) / 256, 4096L), 256, 0, st>>>(n, disp3_pitch(n), lat_elems,
+                                                                                 sig_padded, (float *)dp->lattice);
   VIE_CHECK_LAUNCH("k_make_lattice3");
   VIE_CUDA(vie_malloc((void **)&dp->smax, sizeof(unsigned)));
   VIE_CUDA(cudaMemset(dp->smax, 0, sizeof(unsigned)));
@@ -975,8 +1075,6 @@ vie_status disp3_apply(const DispPlan3 &dp, int op, const double *sigma_s, const
   a.counter = dp.counter;
   a.n_units = dp.n_units;
   a.n = n;
-  a.ldp = n + 1;
-  a.plane = (n + 1) * (n + 1);
   a.lat_elems = dp.lat_elems;
   a.tau_scale2 = tau_scale2;
   a.wcoef = wcoef;
@@ -1068,8 +1166,6 @@ vie_status disp3_assemble(DispPlan3 *dp, float tau_scale2, float wcoef, const do
     a.counter = dp->counter;
     a.n_units = dp->n_units;
     a.n = n;
-    a.ldp = n + 1;
-    a.plane = (n + 1) * (n + 1);
     a.lat_elems = dp->lat_elems;
     a.tau_scale2 = tau_scale2;
     a.wcoef = wcoef;
