@@ -183,6 +183,40 @@ size_t conv_tma_smem(int S, int Co, int Wb, int nst, int np = 1) {
          16;
 }
 
+// The split-precision operands of training: v = p0 + p1 [+ p2], p0 = bf16(v),
+// each later part the BF16 rounding of what the earlier ones leave (exact in
+// FP32): 16 significant bits for two parts, 24 (all of FP32's) for three.
+__device__ __forceinline__ void split_parts(float v, int np, __nv_bfloat16 (&part)[3]) {
+  float r = v;
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    part[q] = __float2bfloat16_rn(q < np ? r : 0.f);
+    r -= __bfloat162float(part[q]);
+  }
+}
+
+// 8 consecutive channels as NP BF16 parts, one 16-byte store each at element o
+template <int NP>
+__device__ __forceinline__ void store_parts(const float *v, __nv_bfloat16 *__restrict__ out0,
+                                            __nv_bfloat16 *__restrict__ out1, __nv_bfloat16 *__restrict__ out2,
+                                            long o) {
+  unsigned w[3][4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    __nv_bfloat16 p0[3], p1[3];
+    split_parts(v[2 * e], NP, p0);
+    split_parts(v[2 * e + 1], NP, p1);
+#pragma unroll
+    for (int q = 0; q < NP; ++q) {
+      const __nv_bfloat162 h2 = __halves2bfloat162(p0[q], p1[q]);
+      w[q][e] = *reinterpret_cast<const unsigned *>(&h2);
+    }
+  }
+  *reinterpret_cast<uint4 *>(out0 + o) = make_uint4(w[0][0], w[0][1], w[0][2], w[0][3]);
+  if (NP > 1) *reinterpret_cast<uint4 *>(out1 + o) = make_uint4(w[1][0], w[1][1], w[1][2], w[1][3]);
+  if (NP > 2) *reinterpret_cast<uint4 *>(out2 + o) = make_uint4(w[2][0], w[2][1], w[2][2], w[2][3]);
+}
+
 // NP > 1: the FP32 convolutions of training in split precision: input and
 // weights each as NP BF16 parts (v = p0 + p1 [+ p2], each part the BF16
 // rounding of what the earlier ones leave; map_x1 / map_w1, map_x2 / map_w2
@@ -197,7 +231,8 @@ __global__ void __launch_bounds__(kConvThreads, 2)
                 const __grid_constant__ CUtensorMap map_x2, const __grid_constant__ CUtensorMap map_w2,
                 const float *__restrict__ bias, float *__restrict__ out, long out_bs, int Co, int H, int W, int S,
                 int Wb, int R, int tiles_x, int tiles, int nst, WaitLimits wl, int *err,
-                __nv_bfloat16 *__restrict__ out_h, long oh_bs, int oh_cp, int oh_c0) {
+                __nv_bfloat16 *__restrict__ out_h, __nv_bfloat16 *__restrict__ out_h1,
+                __nv_bfloat16 *__restrict__ out_h2, long oh_bs, int oh_cp, int oh_c0) {
   using namespace tc;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char *smem = (unsigned char *)(((size_t)smem_raw + 1023) & ~(size_t)1023);
@@ -368,19 +403,14 @@ __global__ void __launch_bounds__(kConvThreads, 2)
         if (c < Co && pvalid) ob[(long)c * plane] = x;
       }
       if (out_h && pvalid) {
-        // the same values in BF16 for the next convolution's NHWC input:
-        // channels oh_c0 .. oh_c0 + Co of this pixel, 16 bytes at a time
-        uint4 *hp = reinterpret_cast<uint4 *>(out_h + img * oh_bs + ((long)py * W + px) * oh_cp + oh_c0);
+        // the same values in BF16 (NP = 3: in three parts) for the next
+        // convolution's NHWC input: channels oh_c0 .. oh_c0 + Co of this pixel,
+        // 16 bytes at a time
+        const long ho = img * oh_bs + ((long)py * W + px) * oh_cp + oh_c0;
 #pragma unroll
         for (int g8 = 0; g8 < 4; ++g8) {
           if (8 * g8 >= Co) break;
-          unsigned w4[4];
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const __nv_bfloat162 q2 = __floats2bfloat162_rn(v[8 * g8 + 2 * e], v[8 * g8 + 2 * e + 1]);
-            w4[e] = *reinterpret_cast<const unsigned *>(&q2);
-          }
-          hp[g8] = make_uint4(w4[0], w4[1], w4[2], w4[3]);
+          store_parts<NP == 3 ? 3 : 1>(v + 8 * g8, out_h, out_h1, out_h2, ho + 8 * g8);
         }
       }
     }
@@ -451,18 +481,6 @@ __global__ void k_pack_tc_weights(const float *__restrict__ w, int Co, int Ci, i
   }
 }
 
-// The split-precision operands of training: v = p0 + p1 [+ p2], p0 = bf16(v),
-// each later part the BF16 rounding of what the earlier ones leave (exact in
-// FP32): 16 significant bits for two parts, 24 (all of FP32's) for three.
-__device__ __forceinline__ void split_parts(float v, int np, __nv_bfloat16 (&part)[3]) {
-  float r = v;
-#pragma unroll
-  for (int q = 0; q < 3; ++q) {
-    part[q] = __float2bfloat16_rn(q < np ? r : 0.f);
-    r -= __bfloat162float(part[q]);
-  }
-}
-
 // Input: FP32 [B][Ci][plane] -> NP BF16 parts [B][plane][Cp] (out0, out1,
 // out2), one thread per (image, pixel) as in k_to_nhwc_bf16.
 template <int NP>
@@ -474,22 +492,10 @@ __global__ void k_to_nhwc_split(const float *__restrict__ in, long in_bs, int Ci
     const long b = t / plane, p = t - b * plane;
     const float *src = in + b * in_bs + p;
     for (int gq = 0; gq < Cp / 8; ++gq) {
-      unsigned w[3][4];
+      float v[8];
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const int c = gq * 8 + 2 * e;
-        __nv_bfloat16 p0[3], p1[3];
-        split_parts(c < Ci ? src[(long)c * plane] : 0.f, NP, p0);
-        split_parts(c + 1 < Ci ? src[(long)(c + 1) * plane] : 0.f, NP, p1);
-#pragma unroll
-        for (int q = 0; q < 3; ++q) {
-          const __nv_bfloat162 h2 = __halves2bfloat162(p0[q], p1[q]);
-          w[q][e] = *reinterpret_cast<const unsigned *>(&h2);
-        }
-      }
-      reinterpret_cast<uint4 *>(out0 + t * Cp)[gq] = make_uint4(w[0][0], w[0][1], w[0][2], w[0][3]);
-      if (NP > 1) reinterpret_cast<uint4 *>(out1 + t * Cp)[gq] = make_uint4(w[1][0], w[1][1], w[1][2], w[1][3]);
-      if (NP > 2) reinterpret_cast<uint4 *>(out2 + t * Cp)[gq] = make_uint4(w[2][0], w[2][1], w[2][2], w[2][3]);
+      for (int e = 0; e < 8; ++e) v[e] = gq * 8 + e < Ci ? src[(long)(gq * 8 + e) * plane] : 0.f;
+      store_parts<NP>(v, out0, out1, out2, t * Cp + 8 * gq);
     }
   }
 }
@@ -498,10 +504,18 @@ __global__ void k_to_nhwc_split(const float *__restrict__ in, long in_bs, int Ci
 // (a > 0), as three BF16 parts [B][plane][32], and the bias gradient's block
 // sums part[block][32].  A thread takes 8 of the channels of one pixel, and
 // `steps` pixels 64 apart in turn (up to 8; small levels have too few pixels).
+// Where the gradient comes from (FROM): g itself (kFromG); the 1x1 head, w_c times
+// the output's gradient g (kFromHead, g one plane); 2x2 upsampling, the sum over
+// the 4 pixels of the finer g (kFromUp); g plus a quarter of the pooled level's
+// gradient g2 (kFromPool).  (As kernels of their own these three passed the
+// gradient through memory once more, 65 us of 16 images' step at 128^2.)
+enum GradFrom { kFromG = 0, kFromHead = 1, kFromUp = 2, kFromPool = 3 };
 int split_steps(long total) { return (int)std::max(1L, std::min(8L, total / (64 * 512))); }
 int split_blocks(long total) { return (int)((total + 64 * split_steps(total) - 1) / (64 * split_steps(total))); }
+template <int FROM>
 __global__ void __launch_bounds__(256) k_mask_split(const float *__restrict__ g, long g_bs,
-                                                    const float *__restrict__ a, long a_bs, long plane, int B,
+                                                    const float *__restrict__ g2, long g2_bs,
+                                                    const float *__restrict__ a, long a_bs, int W, long plane, int B,
                                                     __nv_bfloat16 *__restrict__ out0,
                                                     __nv_bfloat16 *__restrict__ out1,
                                                     __nv_bfloat16 *__restrict__ out2, float *__restrict__ part, int steps) {
@@ -516,27 +530,38 @@ __global__ void __launch_bounds__(256) k_mask_split(const float *__restrict__ g,
     const long t = ((long)blockIdx.x * steps + k) * 64 + px;
     if (t >= total) break;
     const long b = t / plane, p = t - b * plane;
-    const float *gp = g + b * g_bs + p + 8 * gq * plane, *ap = a + b * a_bs + p + 8 * gq * plane;
+    const float *ap = a + b * a_bs + p + 8 * gq * plane;
     float v[8];
+    if constexpr (FROM == kFromHead) {
+      const float go = g[b * g_bs + p];
 #pragma unroll
-    for (int e = 0; e < 8; ++e) v[e] = ap[e * plane] > 0.f ? gp[e * plane] : 0.f;
-    unsigned w[3][4];
+      for (int e = 0; e < 8; ++e) v[e] = g2[8 * gq + e] * go;
+    } else if constexpr (FROM == kFromUp) {
+      const int y = (int)p / W, x = (int)p - y * W;
+      const float *gp = g + b * g_bs + 32 * gq * plane + 4L * y * W + 2 * x;
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      sum[2 * e] += v[2 * e];
-      sum[2 * e + 1] += v[2 * e + 1];
-      __nv_bfloat16 p0[3], p1[3];
-      split_parts(v[2 * e], 3, p0);
-      split_parts(v[2 * e + 1], 3, p1);
+      for (int e = 0; e < 8; ++e) {
+        const float2 r0 = *reinterpret_cast<const float2 *>(gp + 4 * e * plane);
+        const float2 r1 = *reinterpret_cast<const float2 *>(gp + 4 * e * plane + 2 * W);
+        v[e] = r0.x + r0.y + r1.x + r1.y;
+      }
+    } else {
+      const float *gp = g + b * g_bs + p + 8 * gq * plane;
 #pragma unroll
-      for (int q = 0; q < 3; ++q) {
-        const __nv_bfloat162 h2 = __halves2bfloat162(p0[q], p1[q]);
-        w[q][e] = *reinterpret_cast<const unsigned *>(&h2);
+      for (int e = 0; e < 8; ++e) v[e] = gp[e * plane];
+      if constexpr (FROM == kFromPool) {
+        const int y = (int)p / W, x = (int)p - y * W;
+        const float *cp = g2 + b * g2_bs + 2 * gq * plane + (long)(y / 2) * (W / 2) + x / 2;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) v[e] += 0.25f * cp[e * (plane / 4)];
       }
     }
-    reinterpret_cast<uint4 *>(out0 + t * 32)[gq] = make_uint4(w[0][0], w[0][1], w[0][2], w[0][3]);
-    reinterpret_cast<uint4 *>(out1 + t * 32)[gq] = make_uint4(w[1][0], w[1][1], w[1][2], w[1][3]);
-    reinterpret_cast<uint4 *>(out2 + t * 32)[gq] = make_uint4(w[2][0], w[2][1], w[2][2], w[2][3]);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      v[e] = ap[e * plane] > 0.f ? v[e] : 0.f;
+      sum[e] += v[e];
+    }
+    store_parts<3>(v, out0, out1, out2, t * 32 + 8 * gq);
   }
 #pragma unroll
   for (int e = 0; e < 8; ++e) red[8 * gq + e][px] = sum[e];
@@ -551,23 +576,35 @@ __global__ void __launch_bounds__(256) k_mask_split(const float *__restrict__ g,
   }
 }
 
-// Weights FP32 [Co][Ci][9], output channels co0 .. co0 + cb -> np BF16 parts
-// [9 S][cb][32] in k_pack_tc_weights's block order.
-__global__ void k_pack_split_weights(const float *__restrict__ w, int Co, int Ci, int S, int co0, int cb, int np,
-                                     __nv_bfloat16 *__restrict__ w0, __nv_bfloat16 *__restrict__ w1,
-                                     __nv_bfloat16 *__restrict__ w2) {
-  const long total = (long)9 * S * cb * kTmaSlice;
-  for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < total; t += (long)gridDim.x * blockDim.x) {
-    const int c = (int)(t % kTmaSlice);
-    const long r = t / kTmaSlice;
-    const int co = co0 + (int)(r % cb);
-    const int k = (int)(r / cb);
-    const int tap = k / S, ci = (k - tap * S) * kTmaSlice + c;
+// The split weights of a training step's convolutions in one launch (as one
+// per layer, with the flips of the adjoints: 43 launches, 89 us and as much in
+// the gaps between them).  A job packs 32 output channels co0 .. of one
+// convolution from the FP32 parameters [co][ci][9], as np BF16 parts in
+// k_pack_tc_weights's block order [9 S][32][32], one after the other at out; the
+// adjoint of a layer with zero padding (flip) is the convolution from its
+// outputs to its inputs with the flipped taps.
+struct PackJob {
+  long w_off, out;
+  int Ci, Co, S, co0, np, flip;  // of the convolution packed (the adjoint's own when flip)
+};
+constexpr int kPackJobs = 32;
+struct PackJobs {
+  PackJob job[kPackJobs];
+};
+__global__ void k_pack_split_weights(const __grid_constant__ PackJobs jobs, const float *__restrict__ p,
+                                     __nv_bfloat16 *__restrict__ out) {
+  const PackJob &j = jobs.job[blockIdx.y];
+  const int total = 9 * j.S * 32 * kTmaSlice;
+  const float *w = p + j.w_off;
+  __nv_bfloat16 *o = out + j.out;
+  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < total; t += gridDim.x * blockDim.x) {
+    const int c = t % kTmaSlice, r = t / kTmaSlice, co = j.co0 + r % 32, k = r / 32;
+    const int tap = k / j.S, ci = (k - tap * j.S) * kTmaSlice + c;
+    float v = 0.f;
+    if (ci < j.Ci && co < j.Co) v = j.flip ? w[(ci * j.Co + co) * 9 + 8 - tap] : w[(co * j.Ci + ci) * 9 + tap];
     __nv_bfloat16 part[3];
-    split_parts(ci < Ci && co < Co ? w[((long)co * Ci + ci) * 9 + tap] : 0.f, np, part);
-    w0[t] = part[0];
-    if (np > 1) w1[t] = part[1];
-    if (np > 2) w2[t] = part[2];
+    split_parts(v, j.np, part);
+    for (int q = 0; q < j.np; ++q) o[(long)q * total + t] = part[q];
   }
 }
 
@@ -892,16 +929,32 @@ __global__ void __launch_bounds__(kConvThreads, 1)
 // co] and db[co] += that of part_b[block][32], in a fixed order: block (tap,
 // ci) of each slice, and a last one for db; 8 runs of the partials side by
 // side in FP32 (about 20 terms each), joined in FP64.
-__global__ void __launch_bounds__(256) k_dw_reduce(const float *__restrict__ part, int ctas, int Ci,
-                                                   float *__restrict__ dw, const float *__restrict__ part_b,
-                                                   int blocks, float *__restrict__ db) {
+// (One launch for all layers, blockIdx.y the layer.)
+struct DwJob {
+  long part, part_b;  // the layer's sums in dw_part and db_part
+  long w_off, b_off;
+  int ctas, S, Ci, blocks;
+};
+constexpr int kDwJobs = 32;
+struct DwJobs {
+  DwJob job[kDwJobs];
+};
+__global__ void __launch_bounds__(256) k_dw_reduce(const __grid_constant__ DwJobs jobs,
+                                                   const float *__restrict__ parts,
+                                                   const float *__restrict__ parts_b, float *__restrict__ g) {
   __shared__ double red[8][32];
+  const DwJob &jb = jobs.job[blockIdx.y];
+  const int last = jb.S * 9 * 32;
+  if ((int)blockIdx.x > last) return;
+  const int ctas = jb.ctas, Ci = jb.Ci;
+  const float *part = parts + jb.part;
+  float *dw = g + jb.w_off, *db = g + jb.b_off;
   const int co = threadIdx.x & 31, run = threadIdx.x >> 5;
-  const bool bias = blockIdx.x == gridDim.x - 1;
+  const bool bias = (int)blockIdx.x == last;
   const int slice = blockIdx.x / (9 * 32), r = blockIdx.x % (9 * 32), tap = r / 32, ci = slice * 32 + r % 32;
-  const float *p = bias ? part_b : part + ((size_t)slice * ctas * 9 * 32 + r) * 32;
+  const float *p = bias ? parts_b + jb.part_b : part + ((size_t)slice * ctas * 9 * 32 + r) * 32;
   const size_t step = bias ? 32 : (size_t)9 * 1024;
-  const int n = bias ? blocks : ctas;
+  const int n = bias ? jb.blocks : ctas;
   float f = 0.f;
 #pragma unroll 8
   for (int c = run; c < n; c += 8) f += p[c * step + co];
@@ -957,9 +1010,12 @@ __global__ void k_head_bwd_w(const float *__restrict__ go, const float *__restri
   const int c = blockIdx.x, k = blockIdx.y, K = gridDim.y;
   const long total = (long)B * plane, i0 = total * k / K, i1 = total * (k + 1) / K;
   float s = 0.f;  // a few dozen terms per thread in FP32; the block's sum in FP64
-  for (long i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
-    const long b = i / plane, p = i - b * plane;
-    s += go[i] * (c < C ? d[b * d_bs + c * plane + p] : 1.f);
+  long b = (i0 + threadIdx.x) / plane, p = i0 + threadIdx.x - b * plane;
+  const float *dc = d + c * plane;
+#pragma unroll 4
+  for (long i = i0 + threadIdx.x; i < i1; i += blockDim.x, p += blockDim.x) {
+    for (; p >= plane; p -= plane) ++b;  // (no division per term)
+    s += go[i] * (c < C ? dc[b * d_bs + p] : 1.f);
   }
   red[threadIdx.x] = s;
   __syncthreads();
@@ -1006,6 +1062,35 @@ __global__ void k_avgpool(const float *__restrict__ in, long in_bs, float *__res
   out[b * out_bs + (long)c * (H / 2) * (W / 2) + q] = 0.25f * (r0.x + r0.y + r1.x + r1.y);
 }
 
+// The pooled planes in FP32 and as the next convolution's NHWC input in NP BF16
+// parts (Cp channels, those past C zero): a thread takes 8 channels (blockIdx.y)
+// of one coarse pixel of one image.  H, W: the fine size.
+template <int NP>
+__global__ void k_avgpool_nhwc(const float *__restrict__ in, long in_bs, float *__restrict__ out, long out_bs, int C,
+                               int H, int W, int B, __nv_bfloat16 *__restrict__ out0,
+                               __nv_bfloat16 *__restrict__ out1, __nv_bfloat16 *__restrict__ out2, int Cp) {
+  const int Wo = W / 2, per = (H / 2) * Wo, c0 = 8 * blockIdx.y;
+  const long t = blockIdx.x * (long)blockDim.x + threadIdx.x;
+  if (t >= (long)B * per) return;
+  const int b = (int)(t / per), q = (int)(t - (long)b * per), y = q / Wo, x = q - y * Wo;
+  float v[8];
+#pragma unroll
+  for (int e = 0; e < 8; ++e) v[e] = 0.f;
+  if (c0 < C) {
+    const float *p = in + b * in_bs + ((long)c0 * H + 2 * y) * W + 2 * x;
+    float2 r0[8], r1[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      r0[e] = *reinterpret_cast<const float2 *>(p + (long)e * H * W);
+      r1[e] = *reinterpret_cast<const float2 *>(p + (long)e * H * W + W);
+    }
+    float *o = out + b * out_bs + (long)c0 * per + q;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) o[(long)e * per] = v[e] = 0.25f * (r0[e].x + r0[e].y + r1[e].x + r1[e].y);
+  }
+  store_parts<NP>(v, out0, out1, out2, t * Cp + c0);
+}
+
 // grad of avgpool: g_in (+)= g_out / 4 on each 2x2 block
 __global__ void k_avgpool_bwd(const float *__restrict__ go, long go_bs, float *__restrict__ gi, long gi_bs,
                               int C, int H, int W, int B, int accumulate) {
@@ -1043,14 +1128,16 @@ __global__ void k_upsample_bwd(const float *__restrict__ go, long go_bs, float *
   gi[b * gi_bs + (long)c * (H / 2) * (W / 2) + q] = r0.x + r0.y + r1.x + r1.y;
 }
 
-// The decoder's upsampled half straight into its BF16 NHWC concatenation:
+// The decoder's upsampled half straight into its NHWC concatenation in NP BF16 parts:
 // coarse FP32 planes (image stride in_bs) -> channels 0 .. C (C a multiple of
 // 8) of the 4 fine pixels of each coarse pixel, pixels o_cp channels apart.
 // One thread per (image, coarse pixel, group of 8 channels), the groups
 // fastest, so a warp's stores cover whole 16-byte runs of each fine pixel.
 // H, W: the fine size.
+template <int NP>
 __global__ void k_upsample_nhwc(const float *__restrict__ in, long in_bs, int C, int H, int W, int B,
-                                __nv_bfloat16 *__restrict__ out, long o_bs, int o_cp) {
+                                __nv_bfloat16 *__restrict__ out0, __nv_bfloat16 *__restrict__ out1,
+                                __nv_bfloat16 *__restrict__ out2, long o_bs, int o_cp) {
   const int Wc = W / 2, G8 = C / 8;
   const long per = (long)(H / 2) * Wc;
   for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < (long)B * per * G8;
@@ -1060,18 +1147,14 @@ __global__ void k_upsample_nhwc(const float *__restrict__ in, long in_bs, int C,
     const long b = pq / per;
     const int q = (int)(pq - b * per), y = q / Wc, x = q - y * Wc;
     const float *src = in + b * in_bs + (long)(8 * g8) * per + q;
-    unsigned w4[4];
+    float v[8];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const __nv_bfloat162 q2 = __floats2bfloat162_rn(src[(long)(2 * e) * per], src[(long)(2 * e + 1) * per]);
-      w4[e] = *reinterpret_cast<const unsigned *>(&q2);
-    }
-    const uint4 v = make_uint4(w4[0], w4[1], w4[2], w4[3]);
-    __nv_bfloat16 *o = out + b * o_bs + ((long)(2 * y) * W + 2 * x) * o_cp + 8 * g8;
-    *reinterpret_cast<uint4 *>(o) = v;
-    *reinterpret_cast<uint4 *>(o + o_cp) = v;
-    *reinterpret_cast<uint4 *>(o + (long)W * o_cp) = v;
-    *reinterpret_cast<uint4 *>(o + (long)(W + 1) * o_cp) = v;
+    for (int e = 0; e < 8; ++e) v[e] = src[(long)e * per];
+    const long o = b * o_bs + ((long)(2 * y) * W + 2 * x) * o_cp + 8 * g8;
+    store_parts<NP>(v, out0, out1, out2, o);
+    store_parts<NP>(v, out0, out1, out2, o + o_cp);
+    store_parts<NP>(v, out0, out1, out2, o + (long)W * o_cp);
+    store_parts<NP>(v, out0, out1, out2, o + (long)(W + 1) * o_cp);
   }
 }
 
@@ -1219,9 +1302,6 @@ struct UnetImpl {
   // decoder's concatenation at level l (the upsampled half, then the skip)
   __nv_bfloat16 *hx = nullptr;
   std::vector<__nv_bfloat16 *> hcat;
-  // the input-gradient convolutions of training on the tensor cores (split
-  // precision): the lo half of the converted input, the split weights of
-  // one 32-channel output block
   int train_tc = 0;  // operand parts of the training convolutions on the tensor cores (0: CUDA cores)
   // the split inputs of every convolution, kept by the training forward for
   // the weight gradients, the split gradient of the current output, and the
@@ -1230,7 +1310,16 @@ struct UnetImpl {
   std::vector<__nv_bfloat16 *> xsplit;  // 3 per layer
   __nv_bfloat16 *gsplit[3] = {nullptr, nullptr, nullptr};
   float *dw_part = nullptr, *db_part = nullptr;
-  __nv_bfloat16 *nhwc_lo = nullptr, *nhwc_p2 = nullptr, *wsp_hi = nullptr, *wsp_lo = nullptr, *wsp_p2 = nullptr;
+  std::vector<DwJob> dw_jobs;  // per layer
+  // later parts of a converted input (widths without kept ones)
+  __nv_bfloat16 *nhwc_lo = nullptr, *nhwc_p2 = nullptr;
+  // the split weights of every convolution of a training step and of its
+  // adjoint: packed by the jobs, layer i's at wsp + wsp_f[i] and wsp + wsp_b[i]
+  // (-1: on the CUDA cores)
+  __nv_bfloat16 *wsp = nullptr;
+  std::vector<PackJob> pack_jobs;
+  long wsp_elems = 0;
+  std::vector<long> wsp_f, wsp_b;
   std::vector<MapEntry> maps;
 };
 
@@ -1252,7 +1341,7 @@ void free_acts(UnetImpl *u) {
   u->nhwc = nullptr;
   if (u->hx) vie_free(u->hx);
   u->hx = nullptr;
-  for (__nv_bfloat16 **q : {&u->nhwc_lo, &u->nhwc_p2, &u->wsp_hi, &u->wsp_lo, &u->wsp_p2}) {
+  for (__nv_bfloat16 **q : {&u->nhwc_lo, &u->nhwc_p2, &u->wsp}) {
     if (*q) vie_free(*q);
     *q = nullptr;
   }
@@ -1276,6 +1365,9 @@ void free_acts(UnetImpl *u) {
   u->h_part = nullptr;
   u->B = u->n = 0;
 }
+
+// FP32 convolutions that training takes to the tensor cores in split precision
+bool conv_split_ok(int Ci, int Co) { return Ci <= 2 * kTmaSlice && Co % 32 == 0 && Co <= 64; }
 
 vie_status ensure_acts(UnetImpl *u, int B, int n) {
   if (u->B >= B && u->n == n) return VIE_OK;
@@ -1321,10 +1413,27 @@ vie_status ensure_acts(UnetImpl *u, int B, int n) {
   VIE_CUDA(vie_malloc((void **)&u->nhwc_p2,
                       sizeof(__nv_bfloat16) * (size_t)B * n * n * (size_t)(((2 * C + 31) / 32) * 32)));
   {
-    const size_t wsp = (size_t)9 * ((2 * C + 31) / 32) * 32 * 32;  // 9 S blocks of [32][32]
-    VIE_CUDA(vie_malloc((void **)&u->wsp_hi, sizeof(__nv_bfloat16) * wsp));
-    VIE_CUDA(vie_malloc((void **)&u->wsp_lo, sizeof(__nv_bfloat16) * wsp));
-    VIE_CUDA(vie_malloc((void **)&u->wsp_p2, sizeof(__nv_bfloat16) * wsp));
+    // split weights: three parts for the forward convolutions, two for the adjoints
+    const auto jobs = [u](const ConvLayer &c, bool flip) -> long {
+      const int Ci = flip ? c.co : c.ci, Co = flip ? c.ci : c.co, np = flip ? 2 : 3;
+      if (c.k != 3 || !conv_split_ok(Ci, Co)) return -1;
+      const long at = u->wsp_elems;
+      const int S = (Ci + kTmaSlice - 1) / kTmaSlice;
+      for (int co0 = 0; co0 < Co; co0 += 32) {
+        u->pack_jobs.push_back({c.w_off, u->wsp_elems, Ci, Co, S, co0, np, flip});
+        u->wsp_elems += (long)np * 9 * S * 32 * kTmaSlice;
+      }
+      return at;
+    };
+    u->pack_jobs.clear();
+    u->wsp_f.clear();
+    u->wsp_b.clear();
+    u->wsp_elems = 0;
+    for (const ConvLayer &c : u->layers) {
+      u->wsp_f.push_back(jobs(c, false));
+      u->wsp_b.push_back(jobs(c, true));
+    }
+    VIE_CUDA(vie_malloc((void **)&u->wsp, sizeof(__nv_bfloat16) * (size_t)std::max(1L, u->wsp_elems)));
   }
   // the hand-off buffers, zeroed once: their padding channels are never written
   const size_t cp1 = (size_t)((C + 31) / 32) * 32, cp2 = (size_t)((2 * C + 31) / 32) * 32;
@@ -1403,11 +1512,12 @@ bool conv_on_tensor_cores(const void *wtc, int Ci, int Co, const float *bias) {
 // channels apart (image stride oh_bs elements).
 struct NhwcIo {
   const __nv_bfloat16 *in_h = nullptr;
-  __nv_bfloat16 *out_h = nullptr;
+  __nv_bfloat16 *out_h[3] = {nullptr, nullptr, nullptr};  // (parts past the first: split precision)
   long oh_bs = 0;
   int oh_cp = 0, oh_c0 = 0;
   bool wrote = false;  // set when out_h was written
-  __nv_bfloat16 *const *split = nullptr;  // split-precision convolutions: where the input's parts go (kept)
+  __nv_bfloat16 *const *split = nullptr;  // split-precision convolutions: where the input's parts are kept
+  bool split_ready = false;               // they are there already (else they are written from the FP32 input)
 };
 
 // the input's tensor map: NHWC BF16 at src, S slices; tiles of one row load
@@ -1472,7 +1582,8 @@ vie_status launch_conv_tma(UnetImpl *u, const CUtensorMap *mx, const CUtensorMap
   // per_sm CTAs per SM, each taking every G-th tile
   int tiles = tiles_x * tiles_y * B;
   const int grid = std::min(tiles, per_sm * prop.multiProcessorCount);
-  __nv_bfloat16 *oh = io ? io->out_h : nullptr;
+  __nv_bfloat16 *oh = io ? io->out_h[0] : nullptr, *oh1 = io ? io->out_h[1] : nullptr,
+                *oh2 = io ? io->out_h[2] : nullptr;
   long oh_bs = io ? io->oh_bs : 0;
   int oh_cp = io ? io->oh_cp : 0, oh_c0 = io ? io->oh_c0 : 0;
   int nst_i = nst, S_i = S, Co_i = Co, H_i = H, W_i = W, Wb_i = Wb, R_i = R, tx_i = tiles_x;
@@ -1483,7 +1594,7 @@ vie_status launch_conv_tma(UnetImpl *u, const CUtensorMap *mx, const CUtensorMap
   void *args[] = {(void *)mx, (void *)mw, (void *)x1, (void *)w1, (void *)x2, (void *)w2, (void *)&bias, (void *)&out,
                   (void *)&out_bs, (void *)&Co_i, (void *)&H_i, (void *)&W_i, (void *)&S_i, (void *)&Wb_i,
                   (void *)&R_i, (void *)&tx_i, (void *)&tiles, (void *)&nst_i, (void *)&wl, (void *)&err,
-                  (void *)&oh, (void *)&oh_bs, (void *)&oh_cp, (void *)&oh_c0};
+                  (void *)&oh, (void *)&oh1, (void *)&oh2, (void *)&oh_bs, (void *)&oh_cp, (void *)&oh_c0};
   VIE_CUDA(cudaLaunchKernel(k, dim3((unsigned)grid), dim3(kConvThreads), args, smem, st));
   if (io) io->wrote = oh != nullptr;
   VIE_CHECK_LAUNCH("k_conv3_tma");
@@ -1495,7 +1606,7 @@ vie_status conv3_tma(UnetImpl *u, const float *in, long in_bs, int Ci, const __n
   const int S = (Ci + kTmaSlice - 1) / kTmaSlice, Cp = S * kTmaSlice;
   const long plane = (long)H * W;
   const __nv_bfloat16 *src = io && io->in_h ? io->in_h : u->nhwc;
-  if (src == u->nhwc) {
+  if (!io || !io->in_h) {
     k_to_nhwc_bf16<<<gridn((long)B * plane), 256, 0, st>>>(in, in_bs, Ci, plane, Cp, B, u->nhwc);
     VIE_CHECK_LAUNCH("k_to_nhwc_bf16");
   }
@@ -1505,48 +1616,54 @@ vie_status conv3_tma(UnetImpl *u, const float *in, long in_bs, int Ci, const __n
   return launch_conv_tma(u, &mx, &mw, 1, bias, out, out_bs, Co, H, W, S, B, relu, st, io);
 }
 
-// The FP32 convolution of training on the tensor cores in split precision:
-// the input split into np BF16 NHWC parts, the FP32 weights [Co][Ci][9] split
-// and packed per block of 32 output channels, one launch per block.
-bool conv_split_ok(int Ci, int Co) { return Ci <= 2 * kTmaSlice && Co % 32 == 0 && Co <= 64; }
-
-// the same from an input that is already split (xin: np parts)
-vie_status conv3_split_run(UnetImpl *u, __nv_bfloat16 *const *xin, int Ci, const float *w, const float *bias,
-                           float *out, long out_bs, int Co, int H, int W, int B, bool relu, int np,
-                           cudaStream_t st) {
+// The FP32 convolution of training on the tensor cores in split precision: the
+// input in np BF16 NHWC parts (xin), the weights packed per block of 32 output
+// channels (wsp: np parts of every block), one launch per block.
+vie_status conv3_split_run(UnetImpl *u, __nv_bfloat16 *const *xin, int Ci, const __nv_bfloat16 *wsp,
+                           const float *bias, float *out, long out_bs, int Co, int H, int W, int B, bool relu, int np,
+                           cudaStream_t st, NhwcIo *io = nullptr) {
   const int S = (Ci + kTmaSlice - 1) / kTmaSlice;
-  const long plane = (long)H * W;
-  __nv_bfloat16 *wsp[3] = {u->wsp_hi, u->wsp_lo, u->wsp_p2};
+  const long plane = (long)H * W, part = 9L * S * 32 * kTmaSlice;
   CUtensorMap mx[3], mw[3];
-  for (int q = 0; q < np; ++q) {
-    VIE_TRY(conv_input_map(u, xin[q], S, H, W, B, &mx[q]));
-    VIE_TRY(conv_weight_map(u, wsp[q], S, 32, &mw[q]));
-  }
-  for (int co0 = 0; co0 < Co; co0 += 32) {
-    k_pack_split_weights<<<gridn(9L * S * 32 * kTmaSlice), 256, 0, st>>>(w, Co, Ci, S, co0, 32, np, wsp[0], wsp[1],
-                                                                         wsp[2]);
-    VIE_CHECK_LAUNCH("k_pack_split_weights");
+  for (int q = 0; q < np; ++q) VIE_TRY(conv_input_map(u, xin[q], S, H, W, B, &mx[q]));
+  for (int co0 = 0; co0 < Co; co0 += 32, wsp += np * part) {
+    for (int q = 0; q < np; ++q) VIE_TRY(conv_weight_map(u, wsp + q * part, S, 32, &mw[q]));
     VIE_TRY(launch_conv_tma(u, mx, mw, np, bias ? bias + co0 : nullptr, out + co0 * plane, out_bs, 32, H, W, S, B,
-                            relu, st, nullptr));
+                            relu, st, io));
   }
   return VIE_OK;
 }
 
-vie_status conv3_split(UnetImpl *u, const float *in, long in_bs, int Ci, const float *w, const float *bias,
+vie_status conv3_split(UnetImpl *u, const float *in, long in_bs, int Ci, const __nv_bfloat16 *wsp, const float *bias,
                        float *out, long out_bs, int Co, int H, int W, int B, bool relu, int np, cudaStream_t st,
-                       const NhwcIo *io) {
+                       NhwcIo *io) {
   const int S = (Ci + kTmaSlice - 1) / kTmaSlice, Cp = S * kTmaSlice;
   const long plane = (long)H * W;
   __nv_bfloat16 *own[3] = {u->nhwc, u->nhwc_lo, u->nhwc_p2};
   __nv_bfloat16 *const *xin = io && io->split ? io->split : own;
-  if (np == 3)
-    k_to_nhwc_split<3><<<gridn((long)B * plane), 256, 0, st>>>(in, in_bs, Ci, plane, Cp, B, xin[0], xin[1], xin[2]);
-  else
-    k_to_nhwc_split<2><<<gridn((long)B * plane), 256, 0, st>>>(in, in_bs, Ci, plane, Cp, B, xin[0], xin[1], xin[2]);
-  VIE_CHECK_LAUNCH("k_to_nhwc_split");
-  return conv3_split_run(u, xin, Ci, w, bias, out, out_bs, Co, H, W, B, relu, np, st);
+  if (!(io && io->split && io->split_ready)) {
+    if (np == 3)
+      k_to_nhwc_split<3><<<gridn((long)B * plane), 256, 0, st>>>(in, in_bs, Ci, plane, Cp, B, xin[0], xin[1], xin[2]);
+    else
+      k_to_nhwc_split<2><<<gridn((long)B * plane), 256, 0, st>>>(in, in_bs, Ci, plane, Cp, B, xin[0], xin[1], xin[2]);
+    VIE_CHECK_LAUNCH("k_to_nhwc_split");
+  }
+  return conv3_split_run(u, xin, Ci, wsp, bias, out, out_bs, Co, H, W, B, relu, np, st, io);
 }
 
+// every split weight of a training step
+vie_status pack_split_weights(UnetImpl *u, cudaStream_t st) {
+  for (size_t i = 0; i < u->pack_jobs.size(); i += kPackJobs) {
+    const size_t cnt = std::min<size_t>(kPackJobs, u->pack_jobs.size() - i);
+    PackJobs jobs{};
+    std::copy_n(u->pack_jobs.begin() + i, cnt, jobs.job);
+    k_pack_split_weights<<<dim3(18, (unsigned)cnt), 256, 0, st>>>(jobs, u->p, u->wsp);
+    VIE_CHECK_LAUNCH("k_pack_split_weights");
+  }
+  return VIE_OK;
+}
+
+// wtc: the packed weights (BF16), or the split ones (FP32 in training; nullptr: CUDA cores)
 // io (tensor-core path only; ignored, with io->wrote false, on the CUDA cores)
 template <typename WT>
 vie_status conv3(UnetImpl *u, const float *in, long in_bs, int Ci, const WT *w, const __nv_bfloat16 *wtc,
@@ -1557,8 +1674,8 @@ vie_status conv3(UnetImpl *u, const float *in, long in_bs, int Ci, const WT *w, 
     if (conv_on_tensor_cores(wtc, Ci, Co, bias))
       return conv3_tma(u, in, in_bs, Ci, wtc, bias, out, out_bs, Co, H, W, B, relu, st, io);
   } else {
-    if (u->train_tc > 1 && conv_split_ok(Ci, Co))
-      return conv3_split(u, in, in_bs, Ci, w, bias, out, out_bs, Co, H, W, B, relu, u->train_tc, st, io);
+    if (u->train_tc > 1 && wtc)
+      return conv3_split(u, in, in_bs, Ci, wtc, bias, out, out_bs, Co, H, W, B, relu, u->train_tc, st, io);
   }
   if (relu)
     conv3_shape<true, WT>(in, in_bs, Ci, w, bias, out, out_bs, Co, H, W, B, st);
@@ -1590,54 +1707,70 @@ vie_status forward(UnetImpl *u, const WT *pw, const float *x, int B, int n, cuda
   int li = 0;
   const bool tc = std::is_same<WT, __nv_bfloat16>::value;
   if (tc && (s = pack_tc_weights(u, st)) != VIE_OK) return s;
-  auto wtc = [&](const ConvLayer &c) { return tc ? u->ptc + c.tc_off : nullptr; };
+  // training with kept split inputs: they are written by the layers before
+  const bool split = !tc && u->train_tc == 3 && u->dw_ready;
+  auto wtc = [&](const ConvLayer &c) -> const __nv_bfloat16 * {
+    if (tc) return u->ptc + c.tc_off;
+    const long at = u->train_tc == 3 ? u->wsp_f[&c - u->layers.data()] : -1;
+    return at >= 0 ? u->wsp + at : nullptr;
+  };
   const float *xl = x;
   long xl_bs = 3L * n * n;
-  // BF16 NHWC hand-off (tensor-core path): each convolution also writes the
-  // next one's input, and the encoder's second convolution its skip into the
-  // decoder's concatenation
+  // NHWC hand-off (tensor cores): each convolution also writes the next one's
+  // input, the encoder's second convolution its skip into the decoder's
+  // concatenation, and pooling and upsampling theirs
   const int cp1 = ((C + 31) / 32) * 32, cp2 = ((2 * C + 31) / 32) * 32;
-  const bool handoff = tc && C % 8 == 0;
-  // training: a layer's split input stays for its weight gradient
-  auto kept = [&](const ConvLayer &c) -> __nv_bfloat16 *const * {
-    return u->train_tc == 3 && u->dw_ready ? &u->xsplit[3 * (&c - u->layers.data())] : nullptr;
+  const bool handoff = split || (tc && C % 8 == 0);
+  // a layer's kept split input (3 parts)
+  auto kept = [&](const ConvLayer &c) { return split ? &u->xsplit[3 * (&c - u->layers.data())] : nullptr; };
+  // where a layer's input is handed over: its kept parts, else h
+  auto hand = [&](NhwcIo &io, const ConvLayer &next, __nv_bfloat16 *h, long bs, int cp, int c0) {
+    if (!handoff) return;
+    for (int q = 0; q < (split ? 3 : 1); ++q) io.out_h[q] = split ? kept(next)[q] : h;
+    io.oh_bs = bs;
+    io.oh_cp = cp;
+    io.oh_c0 = c0;
+  };
+  auto take = [&](NhwcIo &io, const ConvLayer &c, bool there, const __nv_bfloat16 *h) {
+    io.split = kept(c);
+    io.split_ready = split && there;
+    io.in_h = tc && there ? h : nullptr;
   };
   std::vector<char> skip_h(L, 0);
+  bool pooled = false;  // the level's input was handed over by the pooling
   for (int l = 0; l < L; ++l) {
     const int H = n >> l;
     const long hw = (long)H * H;
     const ConvLayer &c1 = u->layers[li++], &c2 = u->layers[li++];
-    NhwcIo io1;
-    if (handoff) {
-      io1.out_h = u->hx;
-      io1.oh_bs = hw * cp1;
-      io1.oh_cp = cp1;
-    }
-    io1.split = kept(c1);
+    NhwcIo io1, io2;
+    take(io1, c1, pooled, u->nhwc);
+    hand(io1, c2, u->hx, hw * cp1, cp1, 0);
     if ((s = conv3(u, xl, xl_bs, c1.ci, pw + c1.w_off, wtc(c1), u->p + c1.b_off, u->a[l], (long)C * hw, C, H,
                    H, B, true, st, &io1)) != VIE_OK)
       return s;
     float *e = l < L - 1 ? u->cat[l] + (long)C * hw : u->ebot[0];
     const long e_bs = l < L - 1 ? 2L * C * hw : (long)C * hw;
-    NhwcIo io2;
-    io2.in_h = io1.wrote ? u->hx : nullptr;
-    io2.split = kept(c2);
-    if (handoff && l < L - 1) {
-      io2.out_h = u->hcat[l];
-      io2.oh_bs = hw * cp2;
-      io2.oh_cp = cp2;
-      io2.oh_c0 = C;
-    }
+    take(io2, c2, io1.wrote, u->hx);
+    if (l < L - 1) hand(io2, u->layers[2 * L + 2 * (L - 2 - l)], u->hcat[l], hw * cp2, cp2, C);
     if ((s = conv3(u, u->a[l], (long)C * hw, C, pw + c2.w_off, wtc(c2), u->p + c2.b_off, e, e_bs, C, H, H, B,
                    true, st, &io2)) != VIE_OK)
       return s;
     skip_h[l] = io2.wrote;
     if (l < L - 1) {
-      k_avgpool<<<coarse_grid(H, H, C, B), 256, 0, st>>>(e, e_bs, u->xin[l + 1], (long)C * hw / 4, C, H,
-                                                             H, B);
-      VIE_CHECK_LAUNCH("k_avgpool");
+      const ConvLayer &next = u->layers[li];
       xl = u->xin[l + 1];
       xl_bs = (long)C * hw / 4;
+      const dim3 grid((unsigned)((B * hw / 4 + 255) / 256), (unsigned)(cp1 / 8));
+      pooled = handoff && (split || conv_on_tensor_cores(wtc(next), next.ci, next.co, u->p + next.b_off));
+      if (!pooled)
+        k_avgpool<<<coarse_grid(H, H, C, B), 256, 0, st>>>(e, e_bs, u->xin[l + 1], xl_bs, C, H, H, B);
+      else if (split)
+        k_avgpool_nhwc<3><<<grid, 256, 0, st>>>(e, e_bs, u->xin[l + 1], xl_bs, C, H, H, B, kept(next)[0],
+                                                kept(next)[1], kept(next)[2], cp1);
+      else
+        k_avgpool_nhwc<1><<<grid, 256, 0, st>>>(e, e_bs, u->xin[l + 1], xl_bs, C, H, H, B, u->nhwc, nullptr, nullptr,
+                                                cp1);
+      VIE_CHECK_LAUNCH("k_avgpool");
     }
   }
   const float *d = u->ebot[0];
@@ -1647,29 +1780,28 @@ vie_status forward(UnetImpl *u, const WT *pw, const float *x, int B, int n, cuda
     const long hw = (long)H * H;
     const ConvLayer &c1 = u->layers[li++], &c2 = u->layers[li++];
     NhwcIo io1, io2;
-    io1.split = kept(c1);
-    io2.split = kept(c2);
-    if (skip_h[l] && conv_on_tensor_cores(wtc(c1), c1.ci, c1.co, u->p + c1.b_off)) {
-      // the upsampled half in BF16 beside the skip the encoder wrote; the FP32
+    const bool up_h = skip_h[l] && (split || conv_on_tensor_cores(wtc(c1), c1.ci, c1.co, u->p + c1.b_off));
+    if (up_h) {
+      // the upsampled half beside the skip the encoder wrote; the FP32
       // concatenation's first half is not written (vie_unet_layer_io rebuilds it)
       const long per = hw / 4;
-      k_upsample_nhwc<<<gridn((long)B * per * (C / 8)), 256, 0, st>>>(d, d_bs, C, H, H, B, u->hcat[l], hw * cp2,
-                                                                      cp2);
+      const int grid = gridn((long)B * per * (C / 8));
+      if (split)
+        k_upsample_nhwc<3><<<grid, 256, 0, st>>>(d, d_bs, C, H, H, B, kept(c1)[0], kept(c1)[1], kept(c1)[2],
+                                                 hw * cp2, cp2);
+      else
+        k_upsample_nhwc<1><<<grid, 256, 0, st>>>(d, d_bs, C, H, H, B, u->hcat[l], nullptr, nullptr, hw * cp2, cp2);
       VIE_CHECK_LAUNCH("k_upsample_nhwc");
-      io1.in_h = u->hcat[l];
     } else {
       k_upsample<<<coarse_grid(H, H, C, B), 256, 0, st>>>(d, d_bs, u->cat[l], 2L * C * hw, C, H, H, B);
       VIE_CHECK_LAUNCH("k_upsample");
     }
-    if (handoff) {
-      io1.out_h = u->hx;
-      io1.oh_bs = hw * cp1;
-      io1.oh_cp = cp1;
-    }
+    take(io1, c1, up_h, u->hcat[l]);
+    hand(io1, c2, u->hx, hw * cp1, cp1, 0);
     if ((s = conv3(u, u->cat[l], 2L * C * hw, 2 * C, pw + c1.w_off, wtc(c1), u->p + c1.b_off, u->bl[l],
                    (long)C * hw, C, H, H, B, true, st, &io1)) != VIE_OK)
       return s;
-    io2.in_h = io1.wrote ? u->hx : nullptr;
+    take(io2, c2, io1.wrote, u->hx);
     if ((s = conv3(u, u->bl[l], (long)C * hw, C, pw + c2.w_off, wtc(c2), u->p + c2.b_off, u->dl[l],
                    (long)C * hw, C, H, H, B, true, st, &io2)) != VIE_OK)
       return s;
@@ -1700,8 +1832,20 @@ vie_status alloc_dw(UnetImpl *u) {
   }
   const size_t px = (size_t)u->B * u->n * u->n;
   for (__nv_bfloat16 *&q : u->gsplit) VIE_CUDA(vie_malloc((void **)&q, sizeof(__nv_bfloat16) * px * 32));
-  VIE_CUDA(vie_malloc((void **)&u->dw_part, sizeof(float) * (size_t)prop.multiProcessorCount * 9 * 1024));
-  VIE_CUDA(vie_malloc((void **)&u->db_part, sizeof(float) * 32 * (px / 64 < 1024 ? px / 64 + 1 : std::max<size_t>(1024, px / 512 + 1))));
+  // every layer's partial sums (added up by one launch at the end)
+  long part = 0, part_b = 0;
+  u->dw_jobs.assign(u->layers.size(), DwJob{});
+  for (size_t i = 0; i < u->layers.size(); ++i) {
+    const ConvLayer &c = u->layers[i];
+    if (c.k != 3) continue;
+    const int l = (int)i < 2 * u->L ? (int)i / 2 : u->L - 2 - ((int)i - 2 * u->L) / 2;
+    const long lpx = (long)u->B * (u->n >> l) * (u->n >> l);
+    u->dw_jobs[i] = {part, part_b, c.w_off, c.b_off, 0, (c.ci + 31) / 32, c.ci, 0};
+    part += (long)prop.multiProcessorCount * 9 * 1024;
+    part_b += 32 * (lpx / 64 < 1024 ? lpx / 64 + 1 : std::max(1024L, lpx / 512 + 1));
+  }
+  VIE_CUDA(vie_malloc((void **)&u->dw_part, sizeof(float) * (size_t)part));
+  VIE_CUDA(vie_malloc((void **)&u->db_part, sizeof(float) * (size_t)part_b));
   u->dw_ready = true;
   return VIE_OK;
 }
@@ -1728,12 +1872,28 @@ vie_status conv_row_map(UnetImpl *u, const __nv_bfloat16 *src, int Cp, int H, in
 // tensor cores: gout is masked by act > 0 and split once, for the weight
 // gradient (three parts), the bias gradient's sums and the input gradient (the
 // first two parts).
-vie_status conv3_backward_tc(UnetImpl *u, const ConvLayer &c, const float *gout, long g_bs, const float *act,
-                             long a_bs, float *gin, long gin_bs, int H, int B, cudaStream_t st) {
+struct GradIn {
+  int from = kFromG;  // GradFrom
+  const float *g = nullptr, *g2 = nullptr;
+  long bs = 0, bs2 = 0;
+};
+vie_status conv3_backward_tc(UnetImpl *u, const ConvLayer &c, const GradIn &go, const float *act, long a_bs,
+                             float *gin, long gin_bs, int H, int B, cudaStream_t st) {
   const long hw = (long)H * H;
-  const int blocks = split_blocks(B * hw);
-  k_mask_split<<<blocks, 256, 0, st>>>(gout, g_bs, act, a_bs, hw, B, u->gsplit[0], u->gsplit[1], u->gsplit[2],
-                                       u->db_part, split_steps(B * hw));
+  const int blocks = split_blocks(B * hw), steps = split_steps(B * hw);
+  DwJob &job = u->dw_jobs[&c - u->layers.data()];
+  const auto mask = [&](auto k) {
+    k<<<blocks, 256, 0, st>>>(go.g, go.bs, go.g2, go.bs2, act, a_bs, H, hw, B, u->gsplit[0], u->gsplit[1],
+                              u->gsplit[2], u->db_part + job.part_b, steps);
+  };
+  if (go.from == kFromHead)
+    mask(k_mask_split<kFromHead>);
+  else if (go.from == kFromUp)
+    mask(k_mask_split<kFromUp>);
+  else if (go.from == kFromPool)
+    mask(k_mask_split<kFromPool>);
+  else
+    mask(k_mask_split<kFromG>);
   VIE_CHECK_LAUNCH("k_mask_split");
   DevProps prop;
   VIE_TRY(get_dev_props(u->device, &prop));
@@ -1749,15 +1909,30 @@ vie_status conv3_backward_tc(UnetImpl *u, const ConvLayer &c, const float *gout,
   const size_t smem = dw_smem(Wp);
   VIE_TRY(raise_smem_limit((const void *)k_conv3_dw_tc, smem));
   k_conv3_dw_tc<<<dim3((unsigned)ctas, (unsigned)S), kConvThreads, smem, st>>>(
-      maps, H, H, B, Wp, segs, u->dw_part, wait_limits(u->device), u->dev_err);
+      maps, H, H, B, Wp, segs, u->dw_part + job.part, wait_limits(u->device), u->dev_err);
   VIE_CHECK_LAUNCH("k_conv3_dw_tc");
-  k_dw_reduce<<<S * 9 * 32 + 1, 256, 0, st>>>(u->dw_part, ctas, c.ci, u->g + c.w_off, u->db_part,
-                                                               blocks, u->g + c.b_off);
-  VIE_CHECK_LAUNCH("k_dw_reduce");
-  if (gin) {
-    k_flip<<<gridn((long)c.co * c.ci * 9), 256, 0, st>>>(u->p + c.w_off, c.co, c.ci, u->wt);
-    VIE_CHECK_LAUNCH("k_flip");
-    VIE_TRY(conv3_split_run(u, u->gsplit, c.co, u->wt, nullptr, gin, gin_bs, c.ci, H, H, B, false, 2, st));
+  job.ctas = ctas;
+  job.blocks = blocks;
+  if (gin)
+    VIE_TRY(conv3_split_run(u, u->gsplit, c.co, u->wsp + u->wsp_b[layer], nullptr, gin, gin_bs, c.ci, H, H, B, false, 2,
+                            st));
+  return VIE_OK;
+}
+
+// u->g += the partial sums that conv3_backward_tc left for every layer
+vie_status dw_reduce(UnetImpl *u, cudaStream_t st) {
+  DwJobs jobs{};
+  int cnt = 0, blocks = 0;
+  for (size_t i = 0; i < u->layers.size(); ++i) {
+    if (u->layers[i].k == 3) {
+      blocks = std::max(blocks, u->dw_jobs[i].S * 9 * 32 + 1);
+      jobs.job[cnt++] = u->dw_jobs[i];
+    }
+    if (cnt > 0 && (cnt == kDwJobs || i + 1 == u->layers.size())) {
+      k_dw_reduce<<<dim3((unsigned)blocks, (unsigned)cnt), 256, 0, st>>>(jobs, u->dw_part, u->db_part, u->g);
+      VIE_CHECK_LAUNCH("k_dw_reduce");
+      cnt = 0;
+    }
   }
   return VIE_OK;
 }
@@ -1779,10 +1954,13 @@ vie_status conv3_backward(UnetImpl *u, const ConvLayer &c, const float *in, long
                                   cib, cob, B, splits);
   VIE_CHECK_LAUNCH("k_conv3_dw");
   if (gin) {
-    k_flip<<<gridn((long)c.co * c.ci * 9), 256, 0, st>>>(u->p + c.w_off, c.co, c.ci, u->wt);
-    VIE_CHECK_LAUNCH("k_flip");
-    vie_status s = conv3<float>(u, gout, g_bs, c.co, u->wt, nullptr, nullptr, gin, gin_bs, c.ci, H, H, B, false,
-                                st);
+    const long at = u->wsp_b[&c - u->layers.data()];
+    if (at < 0) {
+      k_flip<<<gridn((long)c.co * c.ci * 9), 256, 0, st>>>(u->p + c.w_off, c.co, c.ci, u->wt);
+      VIE_CHECK_LAUNCH("k_flip");
+    }
+    vie_status s = conv3<float>(u, gout, g_bs, c.co, u->wt, at < 0 ? nullptr : u->wsp + at, nullptr, gin, gin_bs,
+                                c.ci, H, H, B, false, st);
     if (s != VIE_OK) return s;
   }
   return VIE_OK;
@@ -1798,10 +1976,17 @@ vie_status relu_mask(float *g, long g_bs, const float *a, long a_bs, long per, i
 vie_status backward(UnetImpl *u, const float *x, int B, int n, cudaStream_t st) {
   const int L = u->L, C = u->C;
   vie_status s;
-  // one convolution's backward pass; gout is masked by its ReLU's output act first
+  // one convolution's backward pass; gout is masked by its ReLU's output act
+  // first (on the tensor cores that pass also takes the step that gout would
+  // come from, where `from` is given)
   auto back = [&](const ConvLayer &c, const float *in, long in_bs, float *gout, long g_bs, const float *act,
-                  long a_bs, float *gin, long gin_bs, int H) -> vie_status {
-    if (u->dw_ready) return conv3_backward_tc(u, c, gout, g_bs, act, a_bs, gin, gin_bs, H, B, st);
+                  long a_bs, float *gin, long gin_bs, int H, const GradIn *from = nullptr) -> vie_status {
+    if (u->dw_ready) {
+      GradIn go;
+      go.g = gout;
+      go.bs = g_bs;
+      return conv3_backward_tc(u, c, from ? *from : go, act, a_bs, gin, gin_bs, H, B, st);
+    }
     VIE_TRY(relu_mask(gout, g_bs, act, a_bs, (long)C * H * H, B, st));
     return conv3_backward(u, c, in, in_bs, gout, g_bs, gin, gin_bs, H, B, st);
   };
@@ -1819,9 +2004,17 @@ vie_status backward(UnetImpl *u, const float *x, int B, int n, cudaStream_t st) 
     k_head_bwd_w_finish<<<1, ((C + 1 + 31) / 32) * 32, 0, st>>>(u->part, C, K, u->g + hd.w_off, u->g + hd.b_off);
     VIE_CHECK_LAUNCH("k_head_bwd_w_finish");
   }
-  k_head_bwd_data<<<gridn((long)B * C * plane0), 256, 0, st>>>(u->go, C, u->p + hd.w_off, gd, (long)C * plane0,
-                                                                plane0, B);
-  VIE_CHECK_LAUNCH("k_head_bwd_data");
+  // where the next convolution's output gradient comes from (tensor cores)
+  GradIn from;
+  from.from = kFromHead;
+  from.g = u->go;
+  from.bs = plane0;
+  from.g2 = u->p + hd.w_off;
+  if (!u->dw_ready) {
+    k_head_bwd_data<<<gridn((long)B * C * plane0), 256, 0, st>>>(u->go, C, u->p + hd.w_off, gd, (long)C * plane0,
+                                                                  plane0, B);
+    VIE_CHECK_LAUNCH("k_head_bwd_data");
+  }
   --li;
   // decoder, l = 0 .. L-2 (reverse of the forward order)
   for (int l = 0; l <= L - 2; ++l) {
@@ -1830,16 +2023,19 @@ vie_status backward(UnetImpl *u, const float *x, int B, int n, cudaStream_t st) 
     const ConvLayer &c2 = u->layers[li--];
     const ConvLayer &c1 = u->layers[li--];
     if ((s = back(c2, u->bl[l], (long)C * hw, u->gdl[l], (long)C * hw, u->dl[l], (long)C * hw, u->gbl[l],
-                  (long)C * hw, H)) != VIE_OK)
+                  (long)C * hw, H, &from)) != VIE_OK)
       return s;
     if ((s = back(c1, u->cat[l], 2L * C * hw, u->gbl[l], (long)C * hw, u->bl[l], (long)C * hw, u->gcat[l],
                   2L * C * hw, H)) != VIE_OK)
       return s;
     // upsample part of the concat -> gradient of d_{l+1}
     float *gnext = (l + 1 <= L - 2) ? u->gdl[l + 1] : u->gebot[0];
-    k_upsample_bwd<<<coarse_grid(H, H, C, B), 256, 0, st>>>(u->gcat[l], 2L * C * hw, gnext, (long)C * hw / 4,
-                                                                 C, H, H, B);
-    VIE_CHECK_LAUNCH("k_upsample_bwd");
+    from = GradIn{kFromUp, u->gcat[l], nullptr, 2L * C * hw, 0};
+    if (!u->dw_ready) {
+      k_upsample_bwd<<<coarse_grid(H, H, C, B), 256, 0, st>>>(u->gcat[l], 2L * C * hw, gnext, (long)C * hw / 4,
+                                                                   C, H, H, B);
+      VIE_CHECK_LAUNCH("k_upsample_bwd");
+    }
   }
   // encoder, l = L-1 .. 0; grad of e_l: concat slice (l < L-1) + pool path
   for (int l = L - 1; l >= 0; --l) {
@@ -1856,29 +2052,34 @@ vie_status backward(UnetImpl *u, const float *x, int B, int n, cudaStream_t st) 
       e = u->cat[l] + (long)C * hw;
       e_bs = 2L * C * hw;
       // + pool path from level l+1's input gradient
-      k_avgpool_bwd<<<coarse_grid(H, H, C, B), 256, 0, st>>>(u->gx[l + 1], (long)C * hw / 4, ge, ge_bs, C, H, H,
-                                                              B, 1);
-      VIE_CHECK_LAUNCH("k_avgpool_bwd");
+      from = GradIn{kFromPool, ge, u->gx[l + 1], ge_bs, (long)C * hw / 4};
+      if (!u->dw_ready) {
+        k_avgpool_bwd<<<coarse_grid(H, H, C, B), 256, 0, st>>>(u->gx[l + 1], (long)C * hw / 4, ge, ge_bs, C, H, H,
+                                                                B, 1);
+        VIE_CHECK_LAUNCH("k_avgpool_bwd");
+      }
     } else {
       ge = u->gebot[0];
       ge_bs = (long)C * hw;
       e = u->ebot[0];
       e_bs = (long)C * hw;
     }
-    if ((s = back(c2, u->a[l], (long)C * hw, ge, ge_bs, e, e_bs, u->ga[l], (long)C * hw, H)) != VIE_OK) return s;
+    if ((s = back(c2, u->a[l], (long)C * hw, ge, ge_bs, e, e_bs, u->ga[l], (long)C * hw, H, &from)) != VIE_OK)
+      return s;
     const float *xl = l == 0 ? x : u->xin[l];
     const long xl_bs = l == 0 ? 3L * hw : (long)C * hw;
     if ((s = back(c1, xl, xl_bs, u->ga[l], (long)C * hw, u->a[l], (long)C * hw, l > 0 ? u->gx[l] : nullptr,
                   (long)C * hw, H)) != VIE_OK)
       return s;
   }
-  return VIE_OK;
+  return u->dw_ready ? dw_reduce(u, st) : VIE_OK;
 }
 
 vie_status loss_grad(UnetImpl *u, const float *x, const float *t, const float *wts, int B, int n, double *loss,
                      cudaStream_t st) {
   vie_status s;
   if ((s = ensure_acts(u, B, n)) != VIE_OK || (s = ensure_dw(u)) != VIE_OK) return s;
+  if ((s = pack_split_weights(u, st)) != VIE_OK) return s;
   // the training convolutions on the tensor cores in split precision: the
   // forward in three parts (24 significant bits, FP32's own: in two parts its
   // ~1e-5 relative error flipped the ReLU masks of pre-activations near zero,
