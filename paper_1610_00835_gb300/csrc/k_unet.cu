@@ -232,7 +232,8 @@ __global__ void __launch_bounds__(kConvThreads, 2)
                 const float *__restrict__ bias, float *__restrict__ out, long out_bs, int Co, int H, int W, int S,
                 int Wb, int R, int tiles_x, int tiles, int nst, WaitLimits wl, int *err,
                 __nv_bfloat16 *__restrict__ out_h, __nv_bfloat16 *__restrict__ out_h1,
-                __nv_bfloat16 *__restrict__ out_h2, long oh_bs, int oh_cp, int oh_c0) {
+                __nv_bfloat16 *__restrict__ out_h2, long oh_bs, int oh_cp, int oh_c0,
+                const void *__restrict__ head_w, const float *__restrict__ head_b, float *__restrict__ head_o) {
   using namespace tc;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char *smem = (unsigned char *)(((size_t)smem_raw + 1023) & ~(size_t)1023);
@@ -412,6 +413,18 @@ __global__ void __launch_bounds__(kConvThreads, 2)
           if (8 * g8 >= Co) break;
           store_parts<NP == 3 ? 3 : 1>(v + 8 * g8, out_h, out_h1, out_h2, ho + 8 * g8);
         }
+      }
+      if (head_o && pvalid) {
+        // the 1x1 head on this pixel's channels, k_head's sum in its order
+        float s = __ldg(head_b);
+#pragma unroll
+        for (int c = 0; c < 32; ++c) {
+          if (c >= Co) break;
+          const float w = NP == 1 ? (float)static_cast<const __nv_bfloat16 *>(head_w)[c]
+                                  : static_cast<const float *>(head_w)[c];
+          s = fmaf(w, v[c], s);
+        }
+        head_o[img * plane + (long)py * W + px] = s;
       }
     }
   }
@@ -1311,8 +1324,7 @@ struct UnetImpl {
   __nv_bfloat16 *gsplit[3] = {nullptr, nullptr, nullptr};
   float *dw_part = nullptr, *db_part = nullptr;
   std::vector<DwJob> dw_jobs;  // per layer
-  // later parts of a converted input (widths without kept ones)
-  __nv_bfloat16 *nhwc_lo = nullptr, *nhwc_p2 = nullptr;
+  __nv_bfloat16 *nhwc_lo = nullptr;  // second part of a converted input (widths without kept ones)
   // the split weights of every convolution of a training step and of its
   // adjoint: packed by the jobs, layer i's at wsp + wsp_f[i] and wsp + wsp_b[i]
   // (-1: on the CUDA cores)
@@ -1341,7 +1353,7 @@ void free_acts(UnetImpl *u) {
   u->nhwc = nullptr;
   if (u->hx) vie_free(u->hx);
   u->hx = nullptr;
-  for (__nv_bfloat16 **q : {&u->nhwc_lo, &u->nhwc_p2, &u->wsp}) {
+  for (__nv_bfloat16 **q : {&u->nhwc_lo, &u->wsp}) {
     if (*q) vie_free(*q);
     *q = nullptr;
   }
@@ -1409,8 +1421,6 @@ vie_status ensure_acts(UnetImpl *u, int B, int n) {
   VIE_CUDA(vie_malloc((void **)&u->nhwc,
                       sizeof(__nv_bfloat16) * (size_t)B * n * n * (size_t)(((2 * C + 31) / 32) * 32)));
   VIE_CUDA(vie_malloc((void **)&u->nhwc_lo,
-                      sizeof(__nv_bfloat16) * (size_t)B * n * n * (size_t)(((2 * C + 31) / 32) * 32)));
-  VIE_CUDA(vie_malloc((void **)&u->nhwc_p2,
                       sizeof(__nv_bfloat16) * (size_t)B * n * n * (size_t)(((2 * C + 31) / 32) * 32)));
   {
     // split weights: three parts for the forward convolutions, two for the adjoints
@@ -1518,6 +1528,12 @@ struct NhwcIo {
   bool wrote = false;  // set when out_h was written
   __nv_bfloat16 *const *split = nullptr;  // split-precision convolutions: where the input's parts are kept
   bool split_ready = false;               // they are there already (else they are written from the FP32 input)
+  // the 1x1 head on the (at most 32) output channels: weights (BF16, or FP32 in
+  // split precision), bias, result; head_done set when it was computed
+  const void *head_w = nullptr;
+  const float *head_b = nullptr;
+  float *head_o = nullptr;
+  bool head_done = false;
 };
 
 // the input's tensor map: NHWC BF16 at src, S slices; tiles of one row load
@@ -1586,6 +1602,9 @@ vie_status launch_conv_tma(UnetImpl *u, const CUtensorMap *mx, const CUtensorMap
                 *oh2 = io ? io->out_h[2] : nullptr;
   long oh_bs = io ? io->oh_bs : 0;
   int oh_cp = io ? io->oh_cp : 0, oh_c0 = io ? io->oh_c0 : 0;
+  const void *hw = io ? io->head_w : nullptr;
+  const float *hb = io ? io->head_b : nullptr;
+  float *ho = io ? io->head_o : nullptr;
   int nst_i = nst, S_i = S, Co_i = Co, H_i = H, W_i = W, Wb_i = Wb, R_i = R, tx_i = tiles_x;
   int *err = u->dev_err;
   // maps of the parts past np: copies of part 0 (not read)
@@ -1594,9 +1613,13 @@ vie_status launch_conv_tma(UnetImpl *u, const CUtensorMap *mx, const CUtensorMap
   void *args[] = {(void *)mx, (void *)mw, (void *)x1, (void *)w1, (void *)x2, (void *)w2, (void *)&bias, (void *)&out,
                   (void *)&out_bs, (void *)&Co_i, (void *)&H_i, (void *)&W_i, (void *)&S_i, (void *)&Wb_i,
                   (void *)&R_i, (void *)&tx_i, (void *)&tiles, (void *)&nst_i, (void *)&wl, (void *)&err,
-                  (void *)&oh, (void *)&oh1, (void *)&oh2, (void *)&oh_bs, (void *)&oh_cp, (void *)&oh_c0};
+                  (void *)&oh, (void *)&oh1, (void *)&oh2, (void *)&oh_bs, (void *)&oh_cp, (void *)&oh_c0,
+                  (void *)&hw, (void *)&hb, (void *)&ho};
   VIE_CUDA(cudaLaunchKernel(k, dim3((unsigned)grid), dim3(kConvThreads), args, smem, st));
-  if (io) io->wrote = oh != nullptr;
+  if (io) {
+    io->wrote = oh != nullptr;
+    io->head_done = ho != nullptr;
+  }
   VIE_CHECK_LAUNCH("k_conv3_tma");
   return VIE_OK;
 }
@@ -1639,7 +1662,7 @@ vie_status conv3_split(UnetImpl *u, const float *in, long in_bs, int Ci, const _
                        NhwcIo *io) {
   const int S = (Ci + kTmaSlice - 1) / kTmaSlice, Cp = S * kTmaSlice;
   const long plane = (long)H * W;
-  __nv_bfloat16 *own[3] = {u->nhwc, u->nhwc_lo, u->nhwc_p2};
+  __nv_bfloat16 *own[3] = {u->nhwc, u->nhwc_lo, nullptr};  // (three parts: always kept ones)
   __nv_bfloat16 *const *xin = io && io->split ? io->split : own;
   if (!(io && io->split && io->split_ready)) {
     if (np == 3)
@@ -1669,7 +1692,8 @@ template <typename WT>
 vie_status conv3(UnetImpl *u, const float *in, long in_bs, int Ci, const WT *w, const __nv_bfloat16 *wtc,
                  const float *bias, float *out, long out_bs, int Co, int H, int W, int B, bool relu,
                  cudaStream_t st, NhwcIo *io = nullptr) {
-  if (io) io->wrote = false;
+  if (io) io->wrote = io->head_done = false;
+  if (io && Co > 32) io->head_o = nullptr;  // (more than one launch's channels)
   if constexpr (std::is_same<WT, __nv_bfloat16>::value) {
     if (conv_on_tensor_cores(wtc, Ci, Co, bias))
       return conv3_tma(u, in, in_bs, Ci, wtc, bias, out, out_bs, Co, H, W, B, relu, st, io);
@@ -1736,6 +1760,15 @@ vie_status forward(UnetImpl *u, const WT *pw, const float *x, int B, int n, cuda
     io.split_ready = split && there;
     io.in_h = tc && there ? h : nullptr;
   };
+  // the last convolution takes the 1x1 head along (as a pass of its own 40 us
+  // of a forward of 64 images at 128^2)
+  const ConvLayer &hd = u->layers.back();
+  bool head_done = false;
+  auto head = [&](NhwcIo &io) {
+    io.head_w = pw + hd.w_off;
+    io.head_b = u->p + hd.b_off;
+    io.head_o = u->o;
+  };
   std::vector<char> skip_h(L, 0);
   bool pooled = false;  // the level's input was handed over by the pooling
   for (int l = 0; l < L; ++l) {
@@ -1752,9 +1785,11 @@ vie_status forward(UnetImpl *u, const WT *pw, const float *x, int B, int n, cuda
     const long e_bs = l < L - 1 ? 2L * C * hw : (long)C * hw;
     take(io2, c2, io1.wrote, u->hx);
     if (l < L - 1) hand(io2, u->layers[2 * L + 2 * (L - 2 - l)], u->hcat[l], hw * cp2, cp2, C);
+    if (L == 1) head(io2);
     if ((s = conv3(u, u->a[l], (long)C * hw, C, pw + c2.w_off, wtc(c2), u->p + c2.b_off, e, e_bs, C, H, H, B,
                    true, st, &io2)) != VIE_OK)
       return s;
+    head_done = io2.head_done;
     skip_h[l] = io2.wrote;
     if (l < L - 1) {
       const ConvLayer &next = u->layers[li];
@@ -1802,13 +1837,15 @@ vie_status forward(UnetImpl *u, const WT *pw, const float *x, int B, int n, cuda
                    (long)C * hw, C, H, H, B, true, st, &io1)) != VIE_OK)
       return s;
     take(io2, c2, io1.wrote, u->hx);
+    if (l == 0) head(io2);
     if ((s = conv3(u, u->bl[l], (long)C * hw, C, pw + c2.w_off, wtc(c2), u->p + c2.b_off, u->dl[l],
                    (long)C * hw, C, H, H, B, true, st, &io2)) != VIE_OK)
       return s;
+    head_done = io2.head_done;
     d = u->dl[l];
     d_bs = (long)C * hw;
   }
-  const ConvLayer &hd = u->layers[li];
+  if (head_done) return VIE_OK;
   k_head<WT><<<gridn((long)B * n * n), 256, 0, st>>>(d, d_bs, C, pw + hd.w_off, u->p + hd.b_off, u->o,
                                                      (long)n * n, B);
   VIE_CHECK_LAUNCH("k_head");
