@@ -150,6 +150,17 @@ constexpr int kTcM = 128;
 // descriptor reads.  The B operand of the same step is the weights' [Co][32]
 // block of that tap and slice (packed by k_pack_tc_weights).
 //
+// Images of at most 64 pixels a row, BF16 (NP = 1): the flat form.  One box of
+// W + 2 pixels times the tile's rows and two more lies in shared memory as the
+// zero-padded image at pitch P = W + 2; a tile is 128 consecutive positions
+// y P + x of it (those with x >= W are dropped), and the input of tap (dy, dx)
+// is the same rows dy P + dx further on, so one box serves all 9 taps of a
+// slice.  A box per tap (9 times the loads, 63 bytes a clock and SM: the L2
+// path's limit) took 31 us per 32-channel layer of 64 images at 64^2 and 54 for 64
+// channels, this 24 and 34; in
+// split precision the products bound it, and the boxes of all parts would not
+// fit.  The order of the products is the same.
+//
 // Two CTAs per SM (half of its shared memory each) take tiles blockIdx.x,
 // blockIdx.x + G, ... in a warp-specialised pipeline: the weights are loaded once; warp 4 streams the A
 // boxes of its tiles into a ring of nst stages (a tile of one image row
@@ -170,16 +181,29 @@ constexpr int kConvThreads = 192;
 
 // one ring stage: a tap box of 128 pixels, or a halo box of Wb + 2 (Wb = 128)
 // rounded up to 1024 bytes
-__host__ __device__ inline int conv_stage_bytes(int Wb) { return Wb == kTcM ? 9216 : kTcM * 64; }
+// (flat form, fr box rows: every position a tap of the tile reaches)
+__host__ __device__ inline int conv_stage_bytes(int Wb, int fr = 0) {
+  if (fr > 0) {
+    const int rows = fr * (Wb + 2), reach = kTcM + 3 * (Wb + 2) + 2;
+    return ((rows > reach ? rows : reach) * 64 + 1023) & ~1023;
+  }
+  return Wb == kTcM ? 9216 : kTcM * 64;
+}
+// box rows of the flat form: the most image rows 128 positions touch, and two; 0: another form
+inline int conv_flat_rows(int H, int W, int np) {
+  if (np != 1 || W > kTcM / 2 || H < 2) return 0;
+  const int P = W + 2;
+  return std::min((kTcM - 1 + P - 1) / P + 1, H) + 2;
+}
 // ring stages of a CTA with `budget` bytes of shared memory
 // (np = 2: split precision, operands in two parts)
-int conv_stages(int S, int Co, int Wb, size_t budget, int np = 1) {
+int conv_stages(int S, int Co, int Wb, size_t budget, int np, int fr) {
   const size_t b = (size_t)np * 9 * S * Co * 64, fixed = 1024 + b + 1024;
   if (budget <= fixed) return 0;
-  return (int)std::min<size_t>(32, (budget - fixed) / ((size_t)np * conv_stage_bytes(Wb)));
+  return (int)std::min<size_t>(32, (budget - fixed) / ((size_t)np * conv_stage_bytes(Wb, fr)));
 }
-size_t conv_tma_smem(int S, int Co, int Wb, int nst, int np = 1) {
-  return 1024 + (size_t)np * 9 * S * Co * 64 + (size_t)nst * np * conv_stage_bytes(Wb) + 8 * (2 * nst + 2 * kAcc + 2) +
+size_t conv_tma_smem(int S, int Co, int Wb, int nst, int np, int fr) {
+  return 1024 + (size_t)np * 9 * S * Co * 64 + (size_t)nst * np * conv_stage_bytes(Wb, fr) + 8 * (2 * nst + 2 * kAcc + 2) +
          16;
 }
 
@@ -230,7 +254,7 @@ __global__ void __launch_bounds__(kConvThreads, 2)
                 const __grid_constant__ CUtensorMap map_x1, const __grid_constant__ CUtensorMap map_w1,
                 const __grid_constant__ CUtensorMap map_x2, const __grid_constant__ CUtensorMap map_w2,
                 const float *__restrict__ bias, float *__restrict__ out, long out_bs, int Co, int H, int W, int S,
-                int Wb, int R, int tiles_x, int tiles, int nst, WaitLimits wl, int *err,
+                int Wb, int R, int fr, int tiles_x, int tiles, int nst, WaitLimits wl, int *err,
                 __nv_bfloat16 *__restrict__ out_h, __nv_bfloat16 *__restrict__ out_h1,
                 __nv_bfloat16 *__restrict__ out_h2, long oh_bs, int oh_cp, int oh_c0,
                 const void *__restrict__ head_w, const float *__restrict__ head_b, float *__restrict__ head_o) {
@@ -240,10 +264,11 @@ __global__ void __launch_bounds__(kConvThreads, 2)
   // halo: tiles of one image row take, per slice, the 3 input rows once
   // (Wb + 2 pixels each) and the 3 taps of a row as 64-byte offsets into
   // that box; other tiles take one box per tap and slice
-  const bool halo = R == 1;
-  const int steps = (halo ? 3 : 9) * S, taps_step = halo ? 3 : 1;
-  const int tiles_img = tiles_x * ((H + R - 1) / R);
-  const int a_part = conv_stage_bytes(Wb), a_bytes = NP * a_part, b_bytes = Co * 64;
+  const bool halo = R == 1, flat = NP == 1 && fr > 0;
+  const int P = W + 2;  // (flat)
+  const int steps = flat ? S : (halo ? 3 : 9) * S, taps_step = halo ? 3 : 1;
+  const int tiles_img = flat ? (H * P + kTcM - 1) / kTcM : tiles_x * ((H + R - 1) / R);
+  const int a_part = conv_stage_bytes(Wb, fr), a_bytes = NP * a_part, b_bytes = Co * 64;
   const size_t b_part = (size_t)9 * S * b_bytes;  // one part of the weights
   unsigned char *Bs = smem;
   unsigned char *As = smem + (size_t)NP * b_part;
@@ -278,7 +303,7 @@ __global__ void __launch_bounds__(kConvThreads, 2)
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const unsigned tmem = *tmem_slot;
-  const unsigned box_bytes = (unsigned)(kTmaSlice * 2 * (halo ? Wb + 2 : Wb * R));
+  const unsigned box_bytes = (unsigned)(kTmaSlice * 2 * (flat ? P * fr : halo ? Wb + 2 : Wb * R));
   int issued_loads = 0;
   if (warp == 4 && lane == 0) {
     // TMA producer: the weights once, then every step's shifted input box
@@ -292,7 +317,7 @@ __global__ void __launch_bounds__(kConvThreads, 2)
     bool go = true;
     for (int t = blockIdx.x; t < tiles && go; t += G) {
       const int img = t / tiles_img, r = t - img * tiles_img;
-      const int x0 = (r % tiles_x) * Wb, y0 = (r / tiles_x) * R;
+      int x0 = (r % tiles_x) * Wb, y0 = (r / tiles_x) * R;
       for (int k = 0; k < steps; ++k, ++g) {
         const int st = g % nst, use = g / nst;
         if (use > 0 && !mbar_wait(su32(empty + st), (use - 1) & 1, abort_flag, wl.limit)) {
@@ -302,8 +327,13 @@ __global__ void __launch_bounds__(kConvThreads, 2)
           break;
         }
         // step k: slice sl of input row dy (halo) or of tap (dy, dx)
-        const int q = k / S, sl = k - q * S;
+        // (flat: slice k of the tile's rows and their neighbours)
+        const int q = flat ? 0 : k / S, sl = k - q * S;
         const int dy = halo ? q : q / 3, dx = halo ? 0 : q % 3;
+        if (flat) {
+          x0 = 0;
+          y0 = r * kTcM / P;
+        }
         mbar_arrive_expect_tx(su32(full + st), NP * box_bytes);
         tma_load_4d(su32(As + (size_t)st * a_bytes), &map_x, su32(full + st), sl * kTmaSlice, x0 + dx - 1,
                     y0 + dy - 1, img);
@@ -331,6 +361,29 @@ __global__ void __launch_bounds__(kConvThreads, 2)
       }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const unsigned d = tmem + (unsigned)(b * 32);
+      if (flat) {
+        // every slice of the tile (at most nst), then tap by tap in the other forms' order
+        for (int sl = 0; sl < S && go; ++sl)
+          go = mbar_wait(su32(full + (g + sl) % nst), ((g + sl) / nst) & 1, abort_flag,
+                         g + sl == 0 ? wl.first : wl.limit);
+        if (!go) break;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const int v0 = (t % tiles_img) * kTcM, s0 = v0 - v0 / P * P;  // the tile's first position in the box
+        for (int tap = 0; tap < 9; ++tap) {
+          const unsigned row = 64u * (unsigned)(s0 + tap / 3 * P + tap % 3);
+          for (int sl = 0; sl < S; ++sl) {
+            const unsigned long long ad = smem_desc_sw64(su32(As + (size_t)((g + sl) % nst) * a_bytes) + row);
+            const unsigned long long bd = smem_desc_sw64(su32(Bs + (size_t)(tap * S + sl) * b_bytes));
+#pragma unroll
+            for (int kk = 0; kk < 2; ++kk)
+              mma_bf16(d, ad + (unsigned)(kk * 2), bd + (unsigned)(kk * 2), idesc,
+                       (tap > 0 || sl > 0 || kk > 0) ? 1u : 0u);
+          }
+        }
+        for (int sl = 0; sl < S; ++sl, ++g) mma_commit(su32(empty + g % nst));
+        mma_commit(su32(tfull + b));
+        continue;
+      }
       for (int k = 0; k < steps; ++k, ++g) {
         const int st = g % nst;
         if (!mbar_wait(su32(full + st), (g / nst) & 1, abort_flag, g == 0 ? wl.first : wl.limit)) {
@@ -378,8 +431,12 @@ __global__ void __launch_bounds__(kConvThreads, 2)
     for (int t = blockIdx.x; t < tiles; t += G, ++j) {
       const int b = j % kAcc;
       const int img = t / tiles_img, r = t - img * tiles_img;
-      const int px = (r % tiles_x) * Wb + i % Wb, py = (r / tiles_x) * R + i / Wb;
-      const bool pvalid = i < Wb * R && px < W && py < H;
+      int px = (r % tiles_x) * Wb + i % Wb, py = (r / tiles_x) * R + i / Wb;
+      if (flat) {
+        py = (r * kTcM + i) / P;
+        px = r * kTcM + i - py * P;
+      }
+      const bool pvalid = (flat || i < Wb * R) && px < W && py < H;
       bool ok = *abort_flag == 0 && mbar_wait(su32(tfull + b), (j / kAcc) & 1, abort_flag, wl.limit);
       ok = __all_sync(0xffffffffu, ok);  // tcgen05.ld is warp-collective
       float v[32];
@@ -1538,11 +1595,14 @@ struct NhwcIo {
 
 // the input's tensor map: NHWC BF16 at src, S slices; tiles of one row load
 // halo boxes of Wb + 2 pixels (the kernel's halo mode)
-vie_status conv_input_map(UnetImpl *u, const __nv_bfloat16 *src, int S, int H, int W, int B, CUtensorMap *mx) {
-  const int Cp = S * kTmaSlice, Wb = std::min(W, kTcM), R = std::min(kTcM / Wb, H);
-  const unsigned bw = R == 1 ? (unsigned)Wb + 2 : (unsigned)Wb;
-  const unsigned long long key[4] = {(unsigned long long)Cp | ((unsigned long long)bw << 32), (unsigned long long)W,
-                                     (unsigned long long)H, (unsigned long long)B};
+// (fr > 0: the flat form's boxes of W + 2 pixels and fr rows)
+vie_status conv_input_map(UnetImpl *u, const __nv_bfloat16 *src, int S, int H, int W, int B, int fr,
+                          CUtensorMap *mx) {
+  const int Cp = S * kTmaSlice, Wb = std::min(W, kTcM), R = fr > 0 ? fr : std::min(kTcM / Wb, H);
+  const unsigned bw = R == 1 || fr > 0 ? (unsigned)Wb + 2 : (unsigned)Wb;
+  const unsigned long long key[4] = {(unsigned long long)Cp | ((unsigned long long)bw << 32),
+                                     (unsigned long long)W | ((unsigned long long)R << 32), (unsigned long long)H,
+                                     (unsigned long long)B};
   const unsigned long long dims[4] = {(unsigned long long)Cp, (unsigned long long)W, (unsigned long long)H,
                                       (unsigned long long)B};
   const unsigned long long strides[3] = {2ull * Cp, 2ull * Cp * W, 2ull * Cp * W * H};
@@ -1565,6 +1625,7 @@ vie_status launch_conv_tma(UnetImpl *u, const CUtensorMap *mx, const CUtensorMap
                            float *out, long out_bs, int Co, int H, int W, int S, int B, bool relu, cudaStream_t st,
                            NhwcIo *io) {
   const int Wb = std::min(W, kTcM), R = std::min(kTcM / Wb, H);
+  const int fr = conv_flat_rows(H, W, np);
   const int tiles_x = (W + Wb - 1) / Wb, tiles_y = (H + R - 1) / R;
   int dev = 0;
   VIE_CUDA(cudaGetDevice(&dev));
@@ -1578,16 +1639,16 @@ vie_status launch_conv_tma(UnetImpl *u, const CUtensorMap *mx, const CUtensorMap
   // two run side by side all the same, and a grid they could not share would
   // only run in two waves, each CTA taking every G-th tile.)
   const size_t optin = (size_t)prop.sharedMemPerBlockOptin;
-  int per_sm = 2, nst = conv_stages(S, Co, Wb, (optin + 1024) / 2 - 1024, np);
+  int per_sm = 2, nst = conv_stages(S, Co, Wb, (optin + 1024) / 2 - 1024, np, fr);
   if (nst < 3) {
     per_sm = 1;
-    nst = conv_stages(S, Co, Wb, optin, np);
+    nst = conv_stages(S, Co, Wb, optin, np, fr);
   }
-  if (nst < 2) {
+  if (nst < 2 || (fr > 0 && nst < S)) {
     set_error("BF16 convolution: not enough shared memory for two stages");
     return VIE_ERR_UNSUPPORTED;
   }
-  const size_t smem = conv_tma_smem(S, Co, Wb, nst, np);
+  const size_t smem = conv_tma_smem(S, Co, Wb, nst, np, fr);
   const void *k = np == 3   ? (relu ? (const void *)k_conv3_tma<true, 3> : (const void *)k_conv3_tma<false, 3>)
                   : np == 2 ? (relu ? (const void *)k_conv3_tma<true, 2> : (const void *)k_conv3_tma<false, 2>)
                             : (relu ? (const void *)k_conv3_tma<true, 1> : (const void *)k_conv3_tma<false, 1>);
@@ -1596,7 +1657,7 @@ vie_status launch_conv_tma(UnetImpl *u, const CUtensorMap *mx, const CUtensorMap
   VIE_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
   WaitLimits wl = wait_limits(dev);
   // per_sm CTAs per SM, each taking every G-th tile
-  int tiles = tiles_x * tiles_y * B;
+  int tiles = (fr > 0 ? (H * (W + 2) + kTcM - 1) / kTcM : tiles_x * tiles_y) * B;
   const int grid = std::min(tiles, per_sm * prop.multiProcessorCount);
   __nv_bfloat16 *oh = io ? io->out_h[0] : nullptr, *oh1 = io ? io->out_h[1] : nullptr,
                 *oh2 = io ? io->out_h[2] : nullptr;
@@ -1605,14 +1666,14 @@ vie_status launch_conv_tma(UnetImpl *u, const CUtensorMap *mx, const CUtensorMap
   const void *hw = io ? io->head_w : nullptr;
   const float *hb = io ? io->head_b : nullptr;
   float *ho = io ? io->head_o : nullptr;
-  int nst_i = nst, S_i = S, Co_i = Co, H_i = H, W_i = W, Wb_i = Wb, R_i = R, tx_i = tiles_x;
+  int nst_i = nst, S_i = S, Co_i = Co, H_i = H, W_i = W, Wb_i = Wb, R_i = R, fr_i = fr, tx_i = tiles_x;
   int *err = u->dev_err;
   // maps of the parts past np: copies of part 0 (not read)
   const CUtensorMap *x1 = np > 1 ? mx + 1 : mx, *w1 = np > 1 ? mw + 1 : mw;
   const CUtensorMap *x2 = np > 2 ? mx + 2 : mx, *w2 = np > 2 ? mw + 2 : mw;
   void *args[] = {(void *)mx, (void *)mw, (void *)x1, (void *)w1, (void *)x2, (void *)w2, (void *)&bias, (void *)&out,
                   (void *)&out_bs, (void *)&Co_i, (void *)&H_i, (void *)&W_i, (void *)&S_i, (void *)&Wb_i,
-                  (void *)&R_i, (void *)&tx_i, (void *)&tiles, (void *)&nst_i, (void *)&wl, (void *)&err,
+                  (void *)&R_i, (void *)&fr_i, (void *)&tx_i, (void *)&tiles, (void *)&nst_i, (void *)&wl, (void *)&err,
                   (void *)&oh, (void *)&oh1, (void *)&oh2, (void *)&oh_bs, (void *)&oh_cp, (void *)&oh_c0,
                   (void *)&hw, (void *)&hb, (void *)&ho};
   VIE_CUDA(cudaLaunchKernel(k, dim3((unsigned)grid), dim3(kConvThreads), args, smem, st));
@@ -1634,7 +1695,7 @@ vie_status conv3_tma(UnetImpl *u, const float *in, long in_bs, int Ci, const __n
     VIE_CHECK_LAUNCH("k_to_nhwc_bf16");
   }
   CUtensorMap mx, mw;
-  VIE_TRY(conv_input_map(u, src, S, H, W, B, &mx));
+  VIE_TRY(conv_input_map(u, src, S, H, W, B, conv_flat_rows(H, W, 1), &mx));
   VIE_TRY(conv_weight_map(u, wtc, S, Co, &mw));
   return launch_conv_tma(u, &mx, &mw, 1, bias, out, out_bs, Co, H, W, S, B, relu, st, io);
 }
@@ -1648,7 +1709,7 @@ vie_status conv3_split_run(UnetImpl *u, __nv_bfloat16 *const *xin, int Ci, const
   const int S = (Ci + kTmaSlice - 1) / kTmaSlice;
   const long plane = (long)H * W, part = 9L * S * 32 * kTmaSlice;
   CUtensorMap mx[3], mw[3];
-  for (int q = 0; q < np; ++q) VIE_TRY(conv_input_map(u, xin[q], S, H, W, B, &mx[q]));
+  for (int q = 0; q < np; ++q) VIE_TRY(conv_input_map(u, xin[q], S, H, W, B, 0, &mx[q]));
   for (int co0 = 0; co0 < Co; co0 += 32, wsp += np * part) {
     for (int q = 0; q < np; ++q) VIE_TRY(conv_weight_map(u, wsp + q * part, S, 32, &mw[q]));
     VIE_TRY(launch_conv_tma(u, mx, mw, np, bias ? bias + co0 : nullptr, out + co0 * plane, out_bs, 32, H, W, S, B,
