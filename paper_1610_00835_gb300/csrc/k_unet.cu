@@ -247,14 +247,20 @@ __device__ __forceinline__ void store_parts(const float *v, __nv_bfloat16 *__res
 // the later parts), every tap the products of parts i, j with i + j < NP
 // into the FP32 accumulator (the terms left out are below 2^-8 NP of the
 // kept ones: 2^-16 for two parts, 2^-24 for three); a stage holds the parts'
-// boxes one after the other.
+// boxes one after the other.  A product of 128 pixels takes about 65 cycles to
+// read its operand however few columns it has, so two parts (the input
+// gradients) take p0 against both weight parts at once, in 64 columns whose
+// halves the epilogue adds (16 images at 128^2, 13 layers: 222 us with a product
+// per pair of parts, 206 so).  Three parts keep one accumulator: the
+// training loss keeps its bits.  Inputs of at most 16 channels skip the second
+// half of their slice, all zeros.
 template <bool RELU, int NP>
 __global__ void __launch_bounds__(kConvThreads, 2)
     k_conv3_tma(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w,
                 const __grid_constant__ CUtensorMap map_x1, const __grid_constant__ CUtensorMap map_w1,
                 const __grid_constant__ CUtensorMap map_x2, const __grid_constant__ CUtensorMap map_w2,
                 const float *__restrict__ bias, float *__restrict__ out, long out_bs, int Co, int H, int W, int S,
-                int Wb, int R, int fr, int tiles_x, int tiles, int nst, WaitLimits wl, int *err,
+                int Wb, int R, int fr, int kks, int tiles_x, int tiles, int nst, WaitLimits wl, int *err,
                 __nv_bfloat16 *__restrict__ out_h, __nv_bfloat16 *__restrict__ out_h1,
                 __nv_bfloat16 *__restrict__ out_h2, long oh_bs, int oh_cp, int oh_c0,
                 const void *__restrict__ head_w, const float *__restrict__ head_b, float *__restrict__ head_o) {
@@ -269,9 +275,12 @@ __global__ void __launch_bounds__(kConvThreads, 2)
   const int steps = flat ? S : (halo ? 3 : 9) * S, taps_step = halo ? 3 : 1;
   const int tiles_img = flat ? (H * P + kTcM - 1) / kTcM : tiles_x * ((H + R - 1) / R);
   const int a_part = conv_stage_bytes(Wb, fr), a_bytes = NP * a_part, b_bytes = Co * 64;
-  const size_t b_part = (size_t)9 * S * b_bytes;  // one part of the weights
+  // weights: block k's parts one part apart, two parts side by side
+  constexpr int kCols = NP == 2 ? 64 : 32;  // columns of an accumulator
+  const size_t b_part = NP == 2 ? (size_t)b_bytes : (size_t)9 * S * b_bytes;
+  const int b_step = NP == 2 ? 2 * b_bytes : b_bytes;
   unsigned char *Bs = smem;
-  unsigned char *As = smem + (size_t)NP * b_part;
+  unsigned char *As = smem + (size_t)NP * 9 * S * b_bytes;
   unsigned long long *full = (unsigned long long *)(As + (size_t)nst * a_bytes);
   unsigned long long *empty = full + nst, *tfull = empty + nst, *tempty = tfull + kAcc;
   unsigned long long *wbar = tempty + kAcc, *done = wbar + 1;
@@ -295,7 +304,7 @@ __global__ void __launch_bounds__(kConvThreads, 2)
   }
   if (warp == 5) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tmem_slot)),
-                 "r"(kAcc * 32)
+                 "r"(kAcc * kCols)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -309,9 +318,9 @@ __global__ void __launch_bounds__(kConvThreads, 2)
     // TMA producer: the weights once, then every step's shifted input box
     mbar_arrive_expect_tx(su32(wbar), (unsigned)(NP * 9 * S * b_bytes));
     for (int k = 0; k < 9 * S; ++k) {
-      tma_load_2d(su32(Bs + (size_t)k * b_bytes), &map_w, su32(wbar), 0, k * Co);
-      if (NP > 1) tma_load_2d(su32(Bs + b_part + (size_t)k * b_bytes), &map_w1, su32(wbar), 0, k * Co);
-      if (NP > 2) tma_load_2d(su32(Bs + 2 * b_part + (size_t)k * b_bytes), &map_w2, su32(wbar), 0, k * Co);
+      tma_load_2d(su32(Bs + (size_t)k * b_step), &map_w, su32(wbar), 0, k * Co);
+      if (NP > 1) tma_load_2d(su32(Bs + b_part + (size_t)k * b_step), &map_w1, su32(wbar), 0, k * Co);
+      if (NP > 2) tma_load_2d(su32(Bs + 2 * b_part + (size_t)k * b_step), &map_w2, su32(wbar), 0, k * Co);
     }
     int g = 0;
     bool go = true;
@@ -360,7 +369,7 @@ __global__ void __launch_bounds__(kConvThreads, 2)
         break;
       }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const unsigned d = tmem + (unsigned)(b * 32);
+      const unsigned d = tmem + (unsigned)(b * kCols);
       if (flat) {
         // every slice of the tile (at most nst), then tap by tap in the other forms' order
         for (int sl = 0; sl < S && go; ++sl)
@@ -373,11 +382,12 @@ __global__ void __launch_bounds__(kConvThreads, 2)
           const unsigned row = 64u * (unsigned)(s0 + tap / 3 * P + tap % 3);
           for (int sl = 0; sl < S; ++sl) {
             const unsigned long long ad = smem_desc_sw64(su32(As + (size_t)((g + sl) % nst) * a_bytes) + row);
-            const unsigned long long bd = smem_desc_sw64(su32(Bs + (size_t)(tap * S + sl) * b_bytes));
+            const unsigned long long bd = smem_desc_sw64(su32(Bs + (size_t)(tap * S + sl) * b_step));
 #pragma unroll
             for (int kk = 0; kk < 2; ++kk)
-              mma_bf16(d, ad + (unsigned)(kk * 2), bd + (unsigned)(kk * 2), idesc,
-                       (tap > 0 || sl > 0 || kk > 0) ? 1u : 0u);
+              if (kk < kks)
+                mma_bf16(d, ad + (unsigned)(kk * 2), bd + (unsigned)(kk * 2), idesc,
+                         (tap > 0 || sl > 0 || kk > 0) ? 1u : 0u);
           }
         }
         for (int sl = 0; sl < S; ++sl, ++g) mma_commit(su32(empty + g % nst));
@@ -397,9 +407,16 @@ __global__ void __launch_bounds__(kConvThreads, 2)
           const int tap = halo ? 3 * q + e : q;
           // (descriptors by addition to the start address field, in 16-byte units)
           const unsigned long long ad = smem_desc_sw64(su32(As + (size_t)st * a_bytes) + 64u * (unsigned)e);
-          const unsigned long long bd = smem_desc_sw64(su32(Bs + (size_t)(tap * S + sl) * b_bytes));
+          const unsigned long long bd = smem_desc_sw64(su32(Bs + (size_t)(tap * S + sl) * b_step));
 #pragma unroll
           for (int kk = 0; kk < 2; ++kk) {
+            if (kk >= kks) break;
+            if constexpr (NP == 2) {
+              mma_bf16(d, ad + (unsigned)(kk * 2), bd + (unsigned)(kk * 2), idesc_bf16(kTcM, kCols),
+                       (k > 0 || e > 0 || kk > 0) ? 1u : 0u);
+              mma_bf16(d, ad + (unsigned)((a_part >> 4) + kk * 2), bd + (unsigned)(kk * 2), idesc, 1u);
+              continue;
+            }
             // parts i of the input and j of the weights, i + j < NP
 #pragma unroll
             for (int i = 0; i < NP; ++i)
@@ -427,6 +444,13 @@ __global__ void __launch_bounds__(kConvThreads, 2)
     float bv[32];
 #pragma unroll
     for (int c = 0; c < 32; ++c) bv[c] = bias && c < Co ? bias[c] : 0.f;
+    float hv[32];  // the head's weights
+#pragma unroll
+    for (int c = 0; c < 32; ++c) {
+      hv[c] = 0.f;
+      if (head_o && c < Co)
+        hv[c] = NP == 1 ? (float)static_cast<const __nv_bfloat16 *>(head_w)[c] : static_cast<const float *>(head_w)[c];
+    }
     int j = 0;
     for (int t = blockIdx.x; t < tiles; t += G, ++j) {
       const int b = j % kAcc;
@@ -442,9 +466,16 @@ __global__ void __launch_bounds__(kConvThreads, 2)
       float v[32];
       if (ok) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const unsigned ta = tmem + ((unsigned)(warp * 32) << 16) + (unsigned)(b * 32);
+        const unsigned ta = tmem + ((unsigned)(warp * 32) << 16) + (unsigned)(b * kCols);
         tmem_ld16(ta, v);
         if (Co > 16) tmem_ld16(ta + 16, v + 16);
+        if constexpr (NP == 2) {
+          float v1[32];
+          tmem_ld16(ta + 32, v1);
+          tmem_ld16(ta + 48, v1 + 16);
+#pragma unroll
+          for (int c = 0; c < 32; ++c) v[c] += v1[c];
+        }
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncwarp();
         if (lane == 0) mbar_arrive(su32(tempty + b));  // the accumulator may be overwritten
@@ -477,9 +508,7 @@ __global__ void __launch_bounds__(kConvThreads, 2)
 #pragma unroll
         for (int c = 0; c < 32; ++c) {
           if (c >= Co) break;
-          const float w = NP == 1 ? (float)static_cast<const __nv_bfloat16 *>(head_w)[c]
-                                  : static_cast<const float *>(head_w)[c];
-          s = fmaf(w, v[c], s);
+          s = fmaf(hv[c], v[c], s);
         }
         head_o[img * plane + (long)py * W + px] = s;
       }
@@ -507,7 +536,7 @@ __global__ void __launch_bounds__(kConvThreads, 2)
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   if (warp == 5) {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kAcc * 32) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kAcc * kCols) : "memory");
   }
 }
 
@@ -1622,8 +1651,9 @@ vie_status conv_weight_map(UnetImpl *u, const __nv_bfloat16 *wtc, int S, int Co,
 // Launch k_conv3_tma with np operand parts (maps mx[p], mw[p]; np > 1: the
 // split-precision form).
 vie_status launch_conv_tma(UnetImpl *u, const CUtensorMap *mx, const CUtensorMap *mw, int np, const float *bias,
-                           float *out, long out_bs, int Co, int H, int W, int S, int B, bool relu, cudaStream_t st,
+                           float *out, long out_bs, int Co, int H, int W, int Ci, int B, bool relu, cudaStream_t st,
                            NhwcIo *io) {
+  const int S = (Ci + kTmaSlice - 1) / kTmaSlice;
   const int Wb = std::min(W, kTcM), R = std::min(kTcM / Wb, H);
   const int fr = conv_flat_rows(H, W, np);
   const int tiles_x = (W + Wb - 1) / Wb, tiles_y = (H + R - 1) / R;
@@ -1667,13 +1697,14 @@ vie_status launch_conv_tma(UnetImpl *u, const CUtensorMap *mx, const CUtensorMap
   const float *hb = io ? io->head_b : nullptr;
   float *ho = io ? io->head_o : nullptr;
   int nst_i = nst, S_i = S, Co_i = Co, H_i = H, W_i = W, Wb_i = Wb, R_i = R, fr_i = fr, tx_i = tiles_x;
+  int kks = Ci <= 16 ? 1 : 2;  // 16-channel halves of a slice that are not all padding
   int *err = u->dev_err;
   // maps of the parts past np: copies of part 0 (not read)
   const CUtensorMap *x1 = np > 1 ? mx + 1 : mx, *w1 = np > 1 ? mw + 1 : mw;
   const CUtensorMap *x2 = np > 2 ? mx + 2 : mx, *w2 = np > 2 ? mw + 2 : mw;
   void *args[] = {(void *)mx, (void *)mw, (void *)x1, (void *)w1, (void *)x2, (void *)w2, (void *)&bias, (void *)&out,
                   (void *)&out_bs, (void *)&Co_i, (void *)&H_i, (void *)&W_i, (void *)&S_i, (void *)&Wb_i,
-                  (void *)&R_i, (void *)&fr_i, (void *)&tx_i, (void *)&tiles, (void *)&nst_i, (void *)&wl, (void *)&err,
+                  (void *)&R_i, (void *)&fr_i, (void *)&kks, (void *)&tx_i, (void *)&tiles, (void *)&nst_i, (void *)&wl, (void *)&err,
                   (void *)&oh, (void *)&oh1, (void *)&oh2, (void *)&oh_bs, (void *)&oh_cp, (void *)&oh_c0,
                   (void *)&hw, (void *)&hb, (void *)&ho};
   VIE_CUDA(cudaLaunchKernel(k, dim3((unsigned)grid), dim3(kConvThreads), args, smem, st));
@@ -1697,7 +1728,7 @@ vie_status conv3_tma(UnetImpl *u, const float *in, long in_bs, int Ci, const __n
   CUtensorMap mx, mw;
   VIE_TRY(conv_input_map(u, src, S, H, W, B, conv_flat_rows(H, W, 1), &mx));
   VIE_TRY(conv_weight_map(u, wtc, S, Co, &mw));
-  return launch_conv_tma(u, &mx, &mw, 1, bias, out, out_bs, Co, H, W, S, B, relu, st, io);
+  return launch_conv_tma(u, &mx, &mw, 1, bias, out, out_bs, Co, H, W, Ci, B, relu, st, io);
 }
 
 // The FP32 convolution of training on the tensor cores in split precision: the
@@ -1712,7 +1743,7 @@ vie_status conv3_split_run(UnetImpl *u, __nv_bfloat16 *const *xin, int Ci, const
   for (int q = 0; q < np; ++q) VIE_TRY(conv_input_map(u, xin[q], S, H, W, B, 0, &mx[q]));
   for (int co0 = 0; co0 < Co; co0 += 32, wsp += np * part) {
     for (int q = 0; q < np; ++q) VIE_TRY(conv_weight_map(u, wsp + q * part, S, 32, &mw[q]));
-    VIE_TRY(launch_conv_tma(u, mx, mw, np, bias ? bias + co0 : nullptr, out + co0 * plane, out_bs, 32, H, W, S, B,
+    VIE_TRY(launch_conv_tma(u, mx, mw, np, bias ? bias + co0 : nullptr, out + co0 * plane, out_bs, 32, H, W, Ci, B,
                             relu, st, io));
   }
   return VIE_OK;
