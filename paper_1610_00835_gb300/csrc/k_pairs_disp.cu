@@ -113,11 +113,28 @@ inline int shared_pitch(int n, int R) {
 // rows of an odd pitch: s R = 16 (mod 32) for pairs and 8 or 24 for quads,
 // so the groups load from disjoint banks.
 __host__ __device__ constexpr int group_stride(int R, int lg) { return lg == 1 ? (R == 8 ? 2 : 4) : (R == 8 ? 1 : 2); }
-// Grids whose lattice does not fit in shared memory read it from global
-// memory: a square lattice of pitch disp_pitch(kGlobalMaxN, R) (odd, like the
-// shared one, so that the lane groups of a ragged block get the same
-// strides), for n <= kGlobalMaxN.
+// Grids whose lattice does not fit in shared memory (up to kGlobalMaxN): a
+// square lattice of pitch disp_pitch(kGlobalMaxN, R) in global memory.  Most
+// tiles read rows of one of two windows that do fit, the first rows of the
+// lattice or its last ones: each window's units run as a launch of their own
+// with the window in shared memory, the rest (tiles that span more: at 256^2 a
+// tenth of the units, 17 % of the march) reads the lattice through L1, with a
+// transposed copy for the runs along x.  An apply at 256^2 with every unit
+// through L1 took 28.3 ms, with windows 25.1.
 constexpr int kGlobalMaxN = 258;
+constexpr int kGlobalPitch = 271;  // disp_pitch(kGlobalMaxN, 12)
+// rows of a window, and the first row of the second one (a multiple of 4: its
+// copy to shared memory reads 16 bytes at a time), R - 1 rows past the grid
+// included; 4 kGlobalPitch bytes a row
+struct Windows {
+  int rows = 0, row_b = 0;
+};
+inline Windows disp_windows(int n, int R, size_t optin) {
+  Windows w;
+  w.rows = std::min(n + R, (int)((optin - 16) / (4 * kGlobalPitch)));
+  w.row_b = (n + R - w.rows + 3) & ~3;
+  return w;
+}
 
 struct DispArgs {
   const float *lat;            // [n + R][ldp] sigma_t on the cell lattice, edge repeated
@@ -139,6 +156,8 @@ struct DispArgs {
   long n_units;
   int n, ldp;
   int grab;                    // units a warp takes from the counter at a time
+  int row0;                    // first lattice row that lat holds (windows)
+  int last;                    // the last launch of this apply (clears smax)
   long lat_elems;
   float tau_scale2, wcoef;
 };
@@ -300,7 +319,7 @@ __device__ __forceinline__ void disp_body(const DispArgs &a) {
   __syncthreads();
   const float scale = MODE != kStore ? (float)scale_s : 1.f;
   const int ldp = LDP > 0 ? LDP : a.ldp;
-  const unsigned lat_base = (unsigned)__cvta_generic_to_shared(lat);
+  const unsigned lat_base = (unsigned)__cvta_generic_to_shared(lat) - 4u * (unsigned)(ldp * a.row0);
   long u0 = 0, u_end = 0;
   for (;;) {
     if (u0 >= u_end) {
@@ -388,7 +407,7 @@ __device__ __forceinline__ void disp_body(const DispArgs &a) {
     if (atomicAdd(a.counter + 1, 1) == (int)gridDim.x - 1) {
       a.counter[0] = 0;
       a.counter[1] = 0;
-      if (MODE != kStore) *a.smax = 0u;  // every CTA read it before this, the next source kernel sets it
+      if (MODE != kStore && a.last) *a.smax = 0u;  // every CTA read it before this, the next source kernel sets it
       __threadfence();
     }
   }
@@ -836,6 +855,7 @@ namespace {
 // that size (kept after the last handle goes, at most kGeoKeep unused ones).
 struct Geometry {
   int device = -1, n = 0, ldp = 0, global = 0, depth = 0, refs = 0;
+  long window_end[2] = {0, 0};  // global: units of the first window, of the first and second
   int4 *units = nullptr;
   float *stencil = nullptr;
   long long *doff = nullptr;  // first stored weight of each D (displacement-major storage)
@@ -870,13 +890,15 @@ void geometry_trim() {
   }
 }
 
-// global: the lattice-in-global-memory layout (runs along x address lat_t)
-vie_status geometry_build(int n, int ldp, bool global, int R, Geometry *geo) {
+// global: units by window (win), the others' records in the
+// lattice-in-global-memory layout (runs along x address lat_t)
+vie_status geometry_build(int n, int ldp, bool global, const Windows &win, int R, Geometry *geo) {
   // stencils and work units, the run axis of each D chosen by estimated cost
   const int T = disp_tiles(n);
   struct U {
     int4 u;
     long cost;
+    int cls;  // 0: first window (or no windows), 1: second, 2: global memory
   };
   // first stored weight of each D, in the half plane's order
   std::vector<long long> doff;
@@ -901,7 +923,7 @@ vie_status geometry_build(int n, int ldp, bool global, int R, Geometry *geo) {
     std::vector<float> &rec = o.rec;
     double &taps = o.taps;
     std::vector<Cell> cy_cells, cx_cells;
-    std::vector<int> cy_runs, cx_runs, tiles;
+    std::vector<int> cy_runs, cx_runs, tiles, split[3];
     for (int dx = -(n - 1); dx < n; ++dx) {
       if (dy == 0 && dx <= 0) continue;
       const int wx = n - std::abs(dx), wy = n - dy;
@@ -915,25 +937,29 @@ vie_status geometry_build(int n, int ldp, bool global, int R, Geometry *geo) {
       taps += (double)cells.size() * wx * wy;
       const std::vector<int> &runs = along_y ? cy_runs : cx_runs;
       const Plan &pl = along_y ? py : px;
-      const int off = (int)(rec.size() / 4);
-      // header: chunks per length (16 bits per length 1..8), then the chunks
-      // grouped by length, each group in run order
-      unsigned counts[4] = {0u, 0u, 0u, 0u};
-      for_each_chunk(runs, [&](int, int lc) { counts[(lc - 1) >> 1] += 1u << (16 * ((lc - 1) & 1)); });
-      float hbits[4];
-      memcpy(hbits, counts, sizeof hbits);
-      for (float f : hbits) rec.push_back(f);
-      for (int len = 1; len <= kMaxChunk; ++len)
-        for_each_chunk(runs, [&](int c0, int lc) {
-          if (lc != len) return;
-          const int eoff =
-              global && !along_y ? cells[c0].cy + ldp * cells[c0].cx : cells[c0].cx + ldp * cells[c0].cy;
-          float obits;
-          memcpy(&obits, &eoff, sizeof obits);
-          rec.push_back(obits);
-          for (int i = 0; i < lc; ++i) rec.push_back((float)cells[c0 + i].w);
-          for (int i = lc + 1; i < 4 * ((lc + 4) / 4); ++i) rec.push_back(0.f);
-        });
+      // the D's records, offsets in lat's layout or lat_t's
+      const auto records = [&](bool transposed) {
+        const int off = (int)(rec.size() / 4);
+        // header: chunks per length (16 bits per length 1..8), then the chunks
+        // grouped by length, each group in run order
+        unsigned counts[4] = {0u, 0u, 0u, 0u};
+        for_each_chunk(runs, [&](int, int lc) { counts[(lc - 1) >> 1] += 1u << (16 * ((lc - 1) & 1)); });
+        float hbits[4];
+        memcpy(hbits, counts, sizeof hbits);
+        for (float f : hbits) rec.push_back(f);
+        for (int len = 1; len <= kMaxChunk; ++len)
+          for_each_chunk(runs, [&](int c0, int lc) {
+            if (lc != len) return;
+            const int eoff =
+                transposed ? cells[c0].cy + ldp * cells[c0].cx : cells[c0].cx + ldp * cells[c0].cy;
+            float obits;
+            memcpy(&obits, &eoff, sizeof obits);
+            rec.push_back(obits);
+            for (int i = 0; i < lc; ++i) rec.push_back((float)cells[c0 + i].w);
+            for (int i = lc + 1; i < 4 * ((lc + 4) / 4); ++i) rec.push_back(0.f);
+          });
+        return off;
+      };
       int per_len[kMaxChunk + 1] = {};
       for_each_chunk(runs, [&](int, int lc) { ++per_len[lc]; });
       if (*std::max_element(per_len, per_len + kMaxChunk + 1) > 65535 || pl.recs + 1 > 524287) {
@@ -960,11 +986,47 @@ vie_status geometry_build(int n, int ldp, bool global, int R, Geometry *geo) {
           for (int j = 0; j < (lg == 0 ? 1 : sstride) && base + j < nfb; ++j)
             tiles.push_back(tile_code(full, R * (base + j), lg));
       }
-      for (size_t i = 0; i < tiles.size(); i += T) {
-        const bool two = T == 2 && i + 1 < tiles.size();
-        const int z = tiles[i] | (two ? 0x8000 | (tiles[i + 1] << 16) : 0);
-        units.push_back({make_int4(off, dxy, z, w), two ? 2 * pl.cost : pl.cost});
+      for (std::vector<int> &v : split) v.clear();
+      size_t both = 0;  // tiles of split[0] that either window holds, kept at its end
+      for (int code : tiles) {
+        if (!global) {
+          split[0].push_back(code);
+          continue;
+        }
+        // lattice rows the tile reads, from the first stacked target's or lane's
+        // to the last one's partner
+        const int row0 = (code >> 4) & 511, lg = (code >> 13) & 3, lb = code & 15;
+        int y0 = 32 * lb, y1 = std::min(32 * lb + 31, wy - 1) + dy;
+        if (along_y) {
+          y0 = y1 = row0;
+          for (int g = 1; g < (1 << lg); ++g)
+            if (row0 + R * group_stride(R, lg) * g < stack) y1 = row0 + R * group_stride(R, lg) * g;
+          y1 += R - 1 + dy;
+        }
+        const bool in_a = y1 < win.rows, in_b = y0 >= win.row_b && y1 < win.row_b + win.rows;
+        if (in_a && in_b) {
+          split[0].push_back(code);
+          ++both;
+        } else if (in_a) {
+          split[0].insert(split[0].end() - both, code);
+        } else {
+          split[in_b ? 1 : 2].push_back(code);
+        }
       }
+      // a unit of one tile marches it twice: even out the windows
+      if (T == 2 && both > 0 && split[0].size() % 2 == 1 && split[1].size() % 2 == 1) {
+        split[1].push_back(split[0].back());
+        split[0].pop_back();
+      }
+      int off[2] = {-1, -1};
+      for (int c = 0; c < 3; ++c)
+        for (size_t i = 0; i < split[c].size(); i += T) {
+          int &o2 = off[c == 2 && !along_y];
+          if (o2 < 0) o2 = records(c == 2 && !along_y);
+          const bool two = T == 2 && i + 1 < split[c].size();
+          const int z = split[c][i] | (two ? 0x8000 | (split[c][i + 1] << 16) : 0);
+          units.push_back({make_int4(o2, dxy, z, w), two ? 2 * pl.cost : pl.cost, c});
+        }
     }
   };
   {
@@ -997,6 +1059,7 @@ vie_status geometry_build(int n, int ldp, bool global, int R, Geometry *geo) {
   }
   for (int i = 0; i < 32; ++i) rec.push_back(0.f);  // the L1 prefetch may reach 127 bytes past a stencil
   std::stable_sort(units.begin(), units.end(), [T](const U &p, const U &q) {
+    if (p.cls != q.cls) return p.cls < q.cls;
     if (T == 2 && (p.u.w & 1) != (q.u.w & 1)) return (p.u.w & 1) > (q.u.w & 1);
     return p.cost > q.cost;
   });
@@ -1009,6 +1072,8 @@ vie_status geometry_build(int n, int ldp, bool global, int R, Geometry *geo) {
   VIE_CUDA(vie_malloc((void **)&geo->doff, sizeof(long long) * doff.size()));
   VIE_CUDA(cudaMemcpy(geo->doff, doff.data(), sizeof(long long) * doff.size(), cudaMemcpyHostToDevice));
   geo->n_units = (long)uv.size();
+  for (int c = 0; c < 2; ++c)
+    geo->window_end[c] = std::count_if(units.begin(), units.end(), [c](const U &u) { return u.cls <= c; });
   double rb = 0.0;
   for (int dy = -(n - 1); dy < n; ++dy)
     for (int dx = -(n - 1); dx < n; ++dx)
@@ -1019,7 +1084,7 @@ vie_status geometry_build(int n, int ldp, bool global, int R, Geometry *geo) {
   return VIE_OK;
 }
 
-vie_status geometry_acquire(int device, int n, int ldp, bool global, int R, Geometry **out) {
+vie_status geometry_acquire(int device, int n, int ldp, bool global, const Windows &win, int R, Geometry **out) {
   std::lock_guard<std::mutex> lock(g_geo_mu);
   for (Geometry *g : g_geo)
     if (g->device == device && g->n == n && g->ldp == ldp && g->global == (int)global && g->depth == R) {
@@ -1033,7 +1098,7 @@ vie_status geometry_acquire(int device, int n, int ldp, bool global, int R, Geom
   g->ldp = ldp;
   g->global = global;
   g->depth = R;
-  const vie_status s = geometry_build(n, ldp, global, R, g);
+  const vie_status s = geometry_build(n, ldp, global, win, R, g);
   if (s != VIE_OK) {
     geometry_free(g);
     return s;
@@ -1108,7 +1173,9 @@ vie_status disp_prepare(DispPlan *dp, int n, const float *sig_padded, int device
   if (disp_smem_bytes(n, R) > optin && disp_smem_bytes(n, 8) <= optin) R = 8;
   const bool global = disp_smem_bytes(n, R) > optin;
   if (global && n > kGlobalMaxN) return VIE_OK;
-  const int ldp = global ? disp_pitch(kGlobalMaxN, R) : shared_pitch(n, R), rows = global ? ldp : n + R;
+  static_assert(kGlobalPitch == disp_pitch(kGlobalMaxN, 12), "the pitch of global lattices");
+  const int ldp = global ? kGlobalPitch : shared_pitch(n, R), rows = global ? ldp : n + R;
+  const Windows win = global ? disp_windows(n, R, optin) : Windows{};
   const size_t smem = global ? 16 : disp_smem_bytes(n, R);
   const int T = disp_tiles(n);
   DispKernel k = global ? k_pairs_disp_global<12, 2> : pick_disp(ldp, R, T, false);
@@ -1134,7 +1201,7 @@ vie_status disp_prepare(DispPlan *dp, int n, const float *sig_padded, int device
   VIE_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps_stream, kst, kThreads, smem_stream));
   if (bps_store < 1 || bps_stream < 1) return VIE_OK;
   Geometry *geo = nullptr;
-  vie_status s = geometry_acquire(device, n, ldp, global, R, &geo);
+  vie_status s = geometry_acquire(device, n, ldp, global, win, R, &geo);
   if (s != VIE_OK) return s;
   dp->geometry = geo;
   dp->doff = geo->doff;
@@ -1157,6 +1224,17 @@ vie_status disp_prepare(DispPlan *dp, int n, const float *sig_padded, int device
     VIE_CHECK_LAUNCH("k_make_lattice");
   }
   dp->global = global;
+  if (global) {
+    dp->kernel_window = (const void *)k_pairs_disp<kGlobalPitch, 12, 2>;
+    dp->kernel_window_store = (const void *)k_store_disp<kGlobalPitch, 12, 2>;
+    dp->smem_window = sizeof(float) * (size_t)win.rows * kGlobalPitch;
+    dp->window_rows = win.rows;
+    dp->window_row_b = win.row_b;
+    for (int c = 0; c < 2; ++c) dp->window_end[c] = geo->window_end[c];
+    VIE_TRY(raise_smem_limit(dp->kernel_window, dp->smem_window));
+    VIE_TRY(raise_smem_limit(dp->kernel_window_store, dp->smem_window));
+    dp->grid_window = prop.multiProcessorCount;
+  }
   VIE_CUDA(vie_malloc((void **)&dp->smax, sizeof(unsigned)));
   VIE_CUDA(cudaMemset(dp->smax, 0, sizeof(unsigned)));
   VIE_CUDA(vie_malloc((void **)&dp->scale, sizeof(double)));
@@ -1318,6 +1396,8 @@ DispArgs disp_args(const DispPlan &dp, int n, float tau_scale2, float wcoef, flo
   a.n_units = dp.n_units;
   a.n = n;
   a.ldp = dp.ldp;
+  a.row0 = 0;
+  a.last = 1;
   a.lat_elems = dp.lat_elems;
   a.tau_scale2 = tau_scale2;
   a.wcoef = wcoef;
@@ -1326,20 +1406,49 @@ DispArgs disp_args(const DispPlan &dp, int n, float tau_scale2, float wcoef, flo
 
 }  // namespace
 
-vie_status disp_launch(const DispPlan &dp, int n, float tau_scale2, float wcoef, cudaStream_t st) {
-  DispArgs a = disp_args(dp, n, tau_scale2, wcoef, nullptr);
+namespace {
+
+// the marching launches of an apply or a store: one, or with a lattice past
+// shared memory one per window and one for the units that no window holds
+vie_status disp_march_launch(const DispPlan &dp, DispArgs a, const void *kernel, const void *window, int grid,
+                             size_t smem, cudaStream_t st) {
+  const dim3 threads(disp_threads(disp_tiles(a.n)));
+  const long n_units = a.n_units;
+  const int4 *units = a.units;
+  const float *lat = a.lat;
+  const long lat_elems = a.lat_elems;
   void *args[] = {&a};
-  VIE_CUDA(cudaLaunchKernel(dp.kernel, dim3(dp.grid), dim3(disp_threads(disp_tiles(n))), args, dp.smem, st));
-  count_launch();
+  long from = 0;
+  for (int c = 0; c < 3; ++c) {
+    const bool win = dp.global && c < 2;
+    const long to = win ? dp.window_end[c] : n_units;
+    if (to > from) {
+      a.units = units + from;
+      a.n_units = to - from;
+      a.last = to == n_units;
+      a.row0 = win && c == 1 ? dp.window_row_b : 0;
+      a.lat = lat + (long)a.row0 * a.ldp;
+      a.lat_elems = win ? (long)dp.window_rows * a.ldp : lat_elems;
+      VIE_CUDA(cudaLaunchKernel(win ? window : kernel, dim3(win ? dp.grid_window : grid), threads, args,
+                                win ? dp.smem_window : smem, st));
+      count_launch();
+    }
+    from = to;
+    if (!win) break;
+  }
   return VIE_OK;
 }
 
+}  // namespace
+
+vie_status disp_launch(const DispPlan &dp, int n, float tau_scale2, float wcoef, cudaStream_t st) {
+  return disp_march_launch(dp, disp_args(dp, n, tau_scale2, wcoef, nullptr), dp.kernel, dp.kernel_window, dp.grid,
+                           dp.smem, st);
+}
+
 vie_status disp_store(const DispPlan &dp, int n, float tau_scale2, float wcoef, float *wbuf, cudaStream_t st) {
-  DispArgs a = disp_args(dp, n, tau_scale2, wcoef, wbuf);
-  void *args[] = {&a};
-  VIE_CUDA(cudaLaunchKernel(dp.kernel_store, dim3(dp.grid_store), dim3(disp_threads(disp_tiles(n))), args, dp.smem_store, st));
-  count_launch();
-  return VIE_OK;
+  return disp_march_launch(dp, disp_args(dp, n, tau_scale2, wcoef, wbuf), dp.kernel_store, dp.kernel_window_store,
+                           dp.grid_store, dp.smem_store, st);
 }
 
 vie_status disp_stream(const DispPlan &dp, int n, const float *wbuf, cudaStream_t st) {

@@ -181,6 +181,13 @@ struct DispPlan {
   void *lattice = nullptr;
   void *lattice_t = nullptr;  // lattice with y fastest (global-lattice kernels only)
   int global = 0;             // lattice read from global memory (grids past shared memory, n <= 258)
+  // global: the units up to window_end[0] run with the first window_rows rows of
+  // the lattice in shared memory, those up to window_end[1] with window_rows
+  // rows from window_row_b on, the rest from global memory
+  const void *kernel_window = nullptr, *kernel_window_store = nullptr;
+  size_t smem_window = 0;
+  int grid_window = 0, window_rows = 0, window_row_b = 0;
+  long window_end[2] = {0, 0};
   unsigned *smax = nullptr;   // max |s| of the current apply (float bits)
   double *scale = nullptr;    // fixed-point scale of the current apply
   double rbound = 0.0;        // bound on every row sum of A

@@ -36,8 +36,9 @@ def check(dim, n, m, rows):
     np.testing.assert_array_equal(gpu_apply(h, g), got)
 
 
-# two tiles per unit from n = 96 on; compiled pitches per class of n
-@pytest.mark.parametrize("n", [32, 33, 64, 65, 95, 96, 97, 128, 129, 140, 141, 161, 162])
+# two tiles per unit from n = 96 on; compiled pitches per class of n; from n = 234
+# on two windows of the lattice in shared memory, the rest from global memory
+@pytest.mark.parametrize("n", [32, 33, 64, 65, 95, 96, 97, 128, 129, 140, 141, 161, 162, 233, 234, 235, 247, 258])
 def test_2d_tiles(n):
     m = V.heterogeneous_2d(n=n, seed=31)
     rows = np.unique(np.r_[0, n - 1, m.N - 1, np.random.default_rng(n).integers(0, m.N, 13)])
