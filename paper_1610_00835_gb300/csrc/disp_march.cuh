@@ -75,7 +75,7 @@ struct Acc2 {
     for (int p = 0; p < R / 2 - 1; ++p) b[p] = 0ull;
     c0 = cl = 0.f;
   }
-  __device__ __forceinline__ void sum(float (&acc)[R]) const {
+  __device__ __forceinline__ void sum(float *acc) const {
     float al[R / 2], ah[R / 2], bl[R / 2 - 1], bh[R / 2 - 1];
 #pragma unroll
     for (int p = 0; p < R / 2; ++p) unpack2(a[p], al[p], ah[p]);
@@ -153,6 +153,50 @@ __device__ __forceinline__ const float4 *chunks2_smem(const float4 *__restrict__
     float v[LC + R - 1];
     LoadRun<ST, 0, LC + R - 1>::go(base + 4u * (unsigned)off, st, v);
     taps2<LC, R>(w, v, s);
+  }
+  return rec;
+}
+
+// the taps of one chunk for the stacked sums a[P0 .. P1), b[P0 .. P1) (b one
+// shorter at the end): v[2 P0 .. )
+template <int LC, int R, int P0, int P1>
+__device__ __forceinline__ void taps2_part(const float *w, const float *v, Acc2<R> &s) {
+  constexpr int B1 = P1 < R / 2 ? P1 : R / 2 - 1;
+#pragma unroll
+  for (int t = 0; t < LC; ++t) {
+    const u64 W = pack2(w[t], w[t]);
+    if ((t & 1) == 0) {
+#pragma unroll
+      for (int p = P0; p < P1; ++p) ffma2(s.a[p], W, pack2(v[t + 2 * p], v[t + 2 * p + 1]));
+    } else {
+#pragma unroll
+      for (int p = P0; p < B1; ++p) ffma2(s.b[p], W, pack2(v[t + 2 * p + 1], v[t + 2 * p + 2]));
+      if (P0 == 0) s.c0 = fmaf(w[t], v[t], s.c0);
+      if (P1 == R / 2) s.cl = fmaf(w[t], v[t + R - 1], s.cl);
+    }
+  }
+}
+
+// Two stack blocks that follow each other, R targets in all: a chunk takes LC +
+// R - 1 lattice loads instead of the two tiles' LC + R / 2 - 1 each.  In two
+// halves, so that the values of the second are loaded once the first are used
+// (all at once they spill).  Every target's sum is the one a tile of its own
+// forms, tap by tap.
+template <int LC, int ST, int R>
+__device__ __forceinline__ const float4 *chunks2_smem_stacked(const float4 *__restrict__ rec, int cnt, unsigned base,
+                                                              int st, Acc2<R> &s) {
+  constexpr int RS = (LC + 4) / 4, H = R / 4;  // H pairs of targets in the first half
+#pragma unroll 1
+  for (int c = 0; c < cnt; ++c, rec += RS) {
+    int off;
+    float w[LC];
+    load_chunk<LC>(rec, off, w);
+    float v[LC + R - 1];
+    const unsigned at = base + 4u * (unsigned)off;
+    LoadRun<ST, 0, LC + 2 * H>::go(at, st, v);
+    taps2_part<LC, R, 0, H>(w, v, s);
+    LoadRun<ST, LC + 2 * H, LC + R - 1>::go(at, st, v);
+    taps2_part<LC, R, H, R / 2>(w, v, s);
   }
   return rec;
 }
@@ -250,6 +294,23 @@ __device__ __forceinline__ void march_runs(const float4 *__restrict__ rec, unsig
   if ((c = chunk_count<6>(hdr)) > 0) rec = chunks2_smem<6, ST, R>(rec, c, base, st, s);
   if ((c = chunk_count<7>(hdr)) > 0) rec = chunks2_smem<7, ST, R>(rec, c, base, st, s);
   if ((c = chunk_count<8>(hdr)) > 0) rec = chunks2_smem<8, ST, R>(rec, c, base, st, s);
+}
+
+// the same for two stack blocks that follow each other
+template <int ST, int R>
+__device__ __forceinline__ void march_runs_stacked(const float4 *__restrict__ rec, unsigned base, int st,
+                                                   Acc2<R> &s) {
+  const float4 hdr = __ldg(rec);
+  ++rec;
+  int c;
+  if ((c = chunk_count<1>(hdr)) > 0) rec = chunks2_smem_stacked<1, ST, R>(rec, c, base, st, s);
+  if ((c = chunk_count<2>(hdr)) > 0) rec = chunks2_smem_stacked<2, ST, R>(rec, c, base, st, s);
+  if ((c = chunk_count<3>(hdr)) > 0) rec = chunks2_smem_stacked<3, ST, R>(rec, c, base, st, s);
+  if ((c = chunk_count<4>(hdr)) > 0) rec = chunks2_smem_stacked<4, ST, R>(rec, c, base, st, s);
+  if ((c = chunk_count<5>(hdr)) > 0) rec = chunks2_smem_stacked<5, ST, R>(rec, c, base, st, s);
+  if ((c = chunk_count<6>(hdr)) > 0) rec = chunks2_smem_stacked<6, ST, R>(rec, c, base, st, s);
+  if ((c = chunk_count<7>(hdr)) > 0) rec = chunks2_smem_stacked<7, ST, R>(rec, c, base, st, s);
+  if ((c = chunk_count<8>(hdr)) > 0) rec = chunks2_smem_stacked<8, ST, R>(rec, c, base, st, s);
 }
 
 // Integer add whose old value nobody reads: the reduction form, with no

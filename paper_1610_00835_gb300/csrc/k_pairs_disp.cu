@@ -76,6 +76,7 @@ using dmarch::Acc2;
 using dmarch::march_runs;
 using dmarch::march_runs_global_pair;
 using dmarch::march_runs_pair;
+using dmarch::march_runs_stacked;
 // R, the targets stacked along the run axis in one thread: 12 on grids of
 // 96 and more, 8 below (measured per apply: 8 / 12 took 0.100 / 0.107 ms at
 // 64^2, 0.550 / 0.519 at 100^2, 1.41 / 1.38 at 128^2, 42.9 / 38.3 at 256^2;
@@ -97,6 +98,15 @@ constexpr int kThreads = 1024;
 // 160^2, 10075 / 9916 at 200^2.  Small grids have too few units per warp.
 __host__ __device__ constexpr int disp_tiles(int n) { return n >= 96 ? 2 : 1; }
 __host__ __device__ constexpr int disp_threads(int T) { return T == 2 ? 640 : kThreads; }
+// Two tiles whose blocks follow each other along the run axis are one march of 2 R
+// stacked targets: L + 2 R - 1 lattice loads per chunk of L cells instead of
+// 2 (L + R - 1), 7 % of the data path's wavefronts.  It takes the march's code a
+// third time, which pays from 130^2 on, where most units are such pairs: an
+// apply (with, without) 462 and 432 us at 97^2, 1277 and 1294 at 128^2, 1682 and
+// 1723 at 136^2, 3365 and 3531 at 160^2, 9763 and 10195 at 200^2.  Below, the
+// kernels (lattice pitches up to 141) leave the code out.
+__host__ __device__ constexpr bool disp_stacked(int n, int R) { return R == 12 && n >= 130; }
+constexpr int kStackedPitch = 173;  // the least pitch of those grids
 __host__ __device__ constexpr int disp_depth(int n) { return n >= 96 ? 12 : 8; }
 // lattice pitch: room for R - 1 stacked targets past the grid, odd so that
 // 32 consecutive rows of one column fall in 32 different banks
@@ -149,7 +159,8 @@ struct DispArgs {
   unsigned long long *yacc;    // [2 N] int64 sums (x fastest, then y fastest), zero between applies
   const int4 *units;           // {the D's record header (float4 index), dx | dy << 16,
                                //  tile | second tile << 16 (tile_code; bit 15: there is one),
-                               //  runs along y | record float4s << 12}
+                               //  runs along y | second tile's blocks follow the first's << 1 |
+                               //  record float4s << 12}
   int *counter;                // [2]
   float *wbuf;                 // stored weights (store: written, stream: read)
   const long long *doff;       // first stored weight of each D of the half plane
@@ -219,7 +230,7 @@ __device__ __forceinline__ TileAt tile_at(int code, const Rect &b, bool along_y,
 
 // what becomes of a tile's pairs (acc: their tau sums; not read when streaming)
 template <int MODE, int R>
-__device__ __forceinline__ void tile_pairs(const DispArgs &a, const float (&acc)[R], const TileAt &t, const Rect &b,
+__device__ __forceinline__ void tile_pairs(const DispArgs &a, const float *acc, const TileAt &t, const Rect &b,
                                            int dx, int dy, bool along_y, float scale, float tscale, float wk,
                                            long woff) {
   const int wx = b.xhi - b.xlo, x = t.x, y = t.y, n = a.n;
@@ -335,7 +346,7 @@ __device__ __forceinline__ void disp_body(const DispArgs &a) {
     const bool along_y = (un.w & 1) != 0;
     const int nrec = un.w >> 12;
     const Rect rect(dx, dy, n);
-    Acc2<R> sa, sb;
+    float acc[T * R];  // the tau sums of the unit's tiles
     const TileAt ta = tile_at<R>(un.z, rect, along_y, lane);
     if constexpr (MODE != kStream) {
       // a unit of one tile (T = 2) marches it twice
@@ -346,27 +357,49 @@ __device__ __forceinline__ void disp_body(const DispArgs &a) {
         const int lines = (int)(((reinterpret_cast<size_t>(r0) & 127) + 16L * nrec + 127) >> 7);
         for (int l = lane; l < lines; l += 32) asm volatile("prefetch.global.L1 [%0];" ::"l"(r0 + 128L * l));
       }
-      sa.zero();
-      sb.zero();
       const float4 *rec = a.stencil + un.x;
       if constexpr (GLAT) {
+        Acc2<R> sa, sb;
+        sa.zero();
+        sb.zero();
         const float *lt = along_y ? a.lat : a.lat_t;
         const long oa = along_y ? ta.x + (long)LDP * ta.y : ta.y + (long)LDP * ta.x;
         const long ob = along_y ? tb.x + (long)LDP * tb.y : tb.y + (long)LDP * tb.x;
         march_runs_global_pair<LDP, R>(rec, lt + oa, lt + ob, sa, sb);
+        sa.sum(acc);
+        sb.sum(acc + R);
       } else {
         const unsigned ba = lat_base + 4u * (unsigned)(ta.x + ldp * ta.y);
         const unsigned bb = lat_base + 4u * (unsigned)(tb.x + ldp * tb.y);
         if constexpr (T == 2) {
-          if (along_y)
-            march_runs_pair<LDP, R>(rec, ba, bb, ldp, sa, sb);
-          else
-            march_runs_pair<1, R>(rec, ba, bb, 1, sa, sb);
+          if (LDP >= kStackedPitch && (un.w & 2)) {
+            // 2 R stacked targets in one march
+            Acc2<2 * R> s2;
+            s2.zero();
+            if (along_y)
+              march_runs_stacked<LDP, 2 * R>(rec, ba, ldp, s2);
+            else
+              march_runs_stacked<1, 2 * R>(rec, ba, 1, s2);
+            s2.sum(acc);
+          } else {
+            Acc2<R> sa, sb;
+            sa.zero();
+            sb.zero();
+            if (along_y)
+              march_runs_pair<LDP, R>(rec, ba, bb, ldp, sa, sb);
+            else
+              march_runs_pair<1, R>(rec, ba, bb, 1, sa, sb);
+            sa.sum(acc);
+            sb.sum(acc + R);
+          }
         } else {
+          Acc2<R> sa;
+          sa.zero();
           if (along_y)
             march_runs<LDP, R>(rec, ba, ldp, sa);
           else
             march_runs<1, R>(rec, ba, 1, sa);
+          sa.sum(acc);
         }
       }
     }
@@ -381,18 +414,18 @@ __device__ __forceinline__ void disp_body(const DispArgs &a) {
     long woff = 0;
     if constexpr (MODE != kApply) woff = a.doff[disp_index(dx, dy, n)];
     if constexpr (T == 1) {
-      float acc[R];
-      if constexpr (MODE != kStream) sa.sum(acc);
       tile_pairs<MODE, R>(a, acc, ta, rect, dx, dy, along_y, scale, tscale, wk, woff);
     } else {
       // one copy of the epilogue's code for both tiles
 #pragma unroll 1
-      for (int z = un.z;; z >>= 16, sa = sb) {
-        float acc[R];
-        if constexpr (MODE != kStream) sa.sum(acc);
+      for (int z = un.z;; z >>= 16) {
         tile_pairs<MODE, R>(a, acc, tile_at<R>(z, rect, along_y, lane), rect, dx, dy, along_y, scale, tscale, wk,
                             woff);
         if (!(z & 0x8000)) break;
+        if constexpr (MODE != kStream) {
+#pragma unroll
+          for (int q = 0; q < R; ++q) acc[q] = acc[R + q];
+        }
       }
     }
   }
@@ -986,6 +1019,17 @@ vie_status geometry_build(int n, int ldp, bool global, const Windows &win, int R
           for (int j = 0; j < (lg == 0 ? 1 : sstride) && base + j < nfb; ++j)
             tiles.push_back(tile_code(full, R * (base + j), lg));
       }
+      // b's block follows a's in every lane group that has one (its reads stay
+      // where b's own are)
+      const auto stacked = [&](int a, int b) {
+        const int row0 = (a >> 4) & 511, lg = (a >> 13) & 3;
+        if (!disp_stacked(n, R) || b != tile_code(a & 15, row0 + R, lg)) return false;
+        for (int g = 0; g < (1 << lg); ++g) {
+          const int row = row0 + (lg > 0 ? R * group_stride(R, lg) * g : 0);
+          if (row < stack && row + R >= stack) return false;
+        }
+        return true;
+      };
       for (std::vector<int> &v : split) v.clear();
       size_t both = 0;  // tiles of split[0] that either window holds, kept at its end
       for (int code : tiles) {
@@ -1019,14 +1063,39 @@ vie_status geometry_build(int n, int ldp, bool global, const Windows &win, int R
         split[0].pop_back();
       }
       int off[2] = {-1, -1};
-      for (int c = 0; c < 3; ++c)
-        for (size_t i = 0; i < split[c].size(); i += T) {
-          int &o2 = off[c == 2 && !along_y];
-          if (o2 < 0) o2 = records(c == 2 && !along_y);
-          const bool two = T == 2 && i + 1 < split[c].size();
-          const int z = split[c][i] | (two ? 0x8000 | (split[c][i + 1] << 16) : 0);
-          units.push_back({make_int4(o2, dxy, z, w), two ? 2 * pl.cost : pl.cost, c});
+      const auto unit = [&](int c, int a, int b) {  // b < 0: one tile
+        int &o2 = off[c == 2 && !along_y];
+        if (o2 < 0) o2 = records(c == 2 && !along_y);
+        const int z = a | (b >= 0 ? 0x8000 | (b << 16) : 0);
+        units.push_back({make_int4(o2, dxy, z, w | (b >= 0 && stacked(a, b) ? 2 : 0)), b >= 0 ? 2 * pl.cost : pl.cost,
+                         c});
+      };
+      for (int c = 0; c < 3; ++c) {
+        std::vector<int> &v = split[c];
+        if (T == 1) {
+          for (int code : v) unit(c, code, -1);
+          continue;
         }
+        // tiles whose blocks follow each other first, the others as they come
+        // (by lane block, then by first row: the low bits of the code, then the next)
+        if (disp_stacked(n, R))
+          std::sort(v.begin(), v.end(), [](int a, int b) {
+            return (a & 15) != (b & 15) ? (a & 15) < (b & 15) : a < b;
+          });
+        int left = -1;
+        for (size_t i = 0; i < v.size(); ++i) {
+          if (i + 1 < v.size() && stacked(v[i], v[i + 1])) {
+            unit(c, v[i], v[i + 1]);
+            ++i;
+          } else if (left < 0) {
+            left = v[i];
+          } else {
+            unit(c, left, v[i]);
+            left = -1;
+          }
+        }
+        if (left >= 0) unit(c, left, -1);
+      }
     }
   };
   {
@@ -1060,7 +1129,7 @@ vie_status geometry_build(int n, int ldp, bool global, const Windows &win, int R
   for (int i = 0; i < 32; ++i) rec.push_back(0.f);  // the L1 prefetch may reach 127 bytes past a stencil
   std::stable_sort(units.begin(), units.end(), [T](const U &p, const U &q) {
     if (p.cls != q.cls) return p.cls < q.cls;
-    if (T == 2 && (p.u.w & 1) != (q.u.w & 1)) return (p.u.w & 1) > (q.u.w & 1);
+    if (T == 2 && (p.u.w & 3) != (q.u.w & 3)) return (p.u.w & 3) > (q.u.w & 3);
     return p.cost > q.cost;
   });
   std::vector<int4> uv(units.size());
