@@ -254,12 +254,13 @@ __device__ __forceinline__ void tile_pairs(const DispArgs &a, const float *acc, 
   const int wstep = along_y ? wx : 1;
   if constexpr (MODE != kApply) wp = a.wbuf + woff + (long)(y - b.ylo) * wx + (x - b.xlo);
   if constexpr (MODE == kStream) {
-    // four targets at a time: their global loads are issued before their atomics
+    // QB targets at a time: their global loads are issued before their atomics
+    constexpr int QB = R == 12 ? 6 : 8;
 #pragma unroll
-    for (int q0 = 0; q0 < R; q0 += 4) {
-      float wv[4], sjv[4], skv[4];
+    for (int q0 = 0; q0 < R; q0 += QB) {
+      float wv[QB], sjv[QB], skv[QB];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
+      for (int i = 0; i < QB; ++i) {
         const int q = q0 + i;
         wv[i] = sjv[i] = skv[i] = 0.f;
         if (q < cnt) {
@@ -269,7 +270,7 @@ __device__ __forceinline__ void tile_pairs(const DispArgs &a, const float *acc, 
         }
       }
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
+      for (int i = 0; i < QB; ++i) {
         const int q = q0 + i;
         if (q < cnt) {
           const float w = wv[i] * scale;
@@ -890,6 +891,7 @@ struct Geometry {
   int device = -1, n = 0, ldp = 0, global = 0, depth = 0, refs = 0;
   long window_end[2] = {0, 0};  // global: units of the first window, of the first and second
   int4 *units = nullptr;
+  int4 *units_stream = nullptr;  // the units in the order of the stored weights' applies
   float *stencil = nullptr;
   long long *doff = nullptr;  // first stored weight of each D (displacement-major storage)
   long n_units = 0;
@@ -903,6 +905,7 @@ constexpr int kGeoKeep = 4;
 
 void geometry_free(Geometry *g) {
   if (g->units) vie_free(g->units);
+  if (g->units_stream) vie_free(g->units_stream);
   if (g->stencil) vie_free(g->stencil);
   if (g->doff) vie_free(g->doff);
   delete g;
@@ -930,7 +933,7 @@ vie_status geometry_build(int n, int ldp, bool global, const Windows &win, int R
   const int T = disp_tiles(n);
   struct U {
     int4 u;
-    long cost;
+    long cost, tile_cost;
     int cls;  // 0: first window (or no windows), 1: second, 2: global memory
   };
   // first stored weight of each D, in the half plane's order
@@ -1068,7 +1071,7 @@ vie_status geometry_build(int n, int ldp, bool global, const Windows &win, int R
         if (o2 < 0) o2 = records(c == 2 && !along_y);
         const int z = a | (b >= 0 ? 0x8000 | (b << 16) : 0);
         units.push_back({make_int4(o2, dxy, z, w | (b >= 0 && stacked(a, b) ? 2 : 0)), b >= 0 ? 2 * pl.cost : pl.cost,
-                         c});
+                         pl.cost, c});
       };
       for (int c = 0; c < 3; ++c) {
         std::vector<int> &v = split[c];
@@ -1127,12 +1130,21 @@ vie_status geometry_build(int n, int ldp, bool global, const Windows &win, int R
     std::vector<float>().swap(o.rec);
   }
   for (int i = 0; i < 32; ++i) rec.push_back(0.f);  // the L1 prefetch may reach 127 bytes past a stencil
+  std::vector<int4> uv(units.size());
+  // the applies of stored weights run by cost alone: they read no lattice and no
+  // records, and units of both run axes in turn spread the reductions over both
+  // halves of the sums (in the march's order 609 us at 128^2, so 511; small grids
+  // take them from both ends of that order in turn, 72 and 70 us at 64^2)
+  std::stable_sort(units.begin(), units.end(), [](const U &p, const U &q) { return p.tile_cost > q.tile_cost; });
+  for (size_t i = 0; i < units.size(); ++i)
+    uv[i] = units[T == 2 ? i : i % 2 == 0 ? i / 2 : units.size() - 1 - i / 2].u;
+  VIE_CUDA(vie_malloc((void **)&geo->units_stream, sizeof(int4) * uv.size()));
+  VIE_CUDA(cudaMemcpy(geo->units_stream, uv.data(), sizeof(int4) * uv.size(), cudaMemcpyHostToDevice));
   std::stable_sort(units.begin(), units.end(), [T](const U &p, const U &q) {
     if (p.cls != q.cls) return p.cls < q.cls;
     if (T == 2 && (p.u.w & 3) != (q.u.w & 3)) return (p.u.w & 3) > (q.u.w & 3);
     return p.cost > q.cost;
   });
-  std::vector<int4> uv(units.size());
   for (size_t i = 0; i < units.size(); ++i) uv[i] = units[i].u;
   VIE_CUDA(vie_malloc((void **)&geo->units, sizeof(int4) * uv.size()));
   VIE_CUDA(cudaMemcpy(geo->units, uv.data(), sizeof(int4) * uv.size(), cudaMemcpyHostToDevice));
@@ -1275,6 +1287,7 @@ vie_status disp_prepare(DispPlan *dp, int n, const float *sig_padded, int device
   dp->geometry = geo;
   dp->doff = geo->doff;
   dp->units = geo->units;
+  dp->units_stream = geo->units_stream;
   dp->stencil = geo->stencil;
   dp->n_units = geo->n_units;
   dp->taps = geo->taps;
@@ -1350,6 +1363,7 @@ void disp_release(DispPlan *dp) {
   dp->smax = nullptr;
   dp->scale = nullptr;
   dp->units = nullptr;
+  dp->units_stream = nullptr;
   dp->stencil = nullptr;
   dp->doff = nullptr;
   dp->counter = nullptr;
@@ -1522,6 +1536,7 @@ vie_status disp_store(const DispPlan &dp, int n, float tau_scale2, float wcoef, 
 
 vie_status disp_stream(const DispPlan &dp, int n, const float *wbuf, cudaStream_t st) {
   DispArgs a = disp_args(dp, n, 0.f, 0.f, const_cast<float *>(wbuf));
+  a.units = (const int4 *)dp.units_stream;
   void *args[] = {&a};
   VIE_CUDA(cudaLaunchKernel(dp.kernel_stream, dim3(dp.grid_stream), dim3(kThreads), args, dp.smem_stream, st));
   count_launch();

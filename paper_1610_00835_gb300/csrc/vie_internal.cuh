@@ -175,6 +175,7 @@ struct DispPlan {
   void *yacc = nullptr;       // int64 [2 N]: fixed-point sums (x fastest, then y fastest), zero between applies
   void *geometry = nullptr;   // shared stencils and units of this n (owned by a cache)
   void *units = nullptr;
+  void *units_stream = nullptr;  // the same units in the order of k_stream_disp
   void *stencil = nullptr;    // per-displacement chunk records (float4)
   size_t stencil_bytes = 0;
   int *counter = nullptr;
