@@ -160,13 +160,14 @@ __global__ void k_fmm_m2l_fill(FillArgs a, int level, int p, const float *__rest
 // matrix is read transposed, so that a warp's loads are consecutive (with one
 // CTA of 128 threads per box and the rows m apart, 36 threads worked and every
 // load touched 32 lines: 34 us for P2M and 9 us per M2M level at 512^2, order
-// 6; now 6.6 and 8 us).
+// 6; now 6.6 and 7 us).
 constexpr int kBoxThreads = 256;
 
-// boxes per CTA, `floats` of shared memory each (at most 48 KB in all)
-__host__ __device__ __forceinline__ int boxes_per_cta(int P2, int floats) {
-  const int g = kBoxThreads / P2, fit = 12288 / floats;
-  return g < 1 ? 1 : g < fit ? g : fit < 1 ? 1 : fit;
+// boxes per CTA, `floats` of shared memory each (at most 48 KB in all), and
+// fewer where that leaves less than a CTA for each of about 152 SMs (P2M of 256
+// leaves at order 2: 12 us with 64 boxes per CTA, 4.9 so)
+inline int boxes_per_cta(int P2, int floats, long boxes) {
+  return (int)std::max(1L, std::min({(long)(kBoxThreads / P2), 12288L / floats, boxes / 152}));
 }
 
 // P2M: W[leaf][m] = sum_k Pt[k][m] s_leaf[k]
@@ -192,9 +193,10 @@ __global__ void __launch_bounds__(kBoxThreads) k_fmm_p2m(int n, int L, int b, in
 }
 
 // M2M: parent boxes at level l from their children at l + 1; Ct[q][m'][m]
-__global__ void __launch_bounds__(kBoxThreads) k_fmm_m2m(int level, int P2, int G, const float *__restrict__ Ct,
+__global__ void __launch_bounds__(kBoxThreads) k_fmm_m2m(int level, int P2, int G, int staged,
+                                                         const float *__restrict__ Ct,
                                                          const float *__restrict__ Wc, float *__restrict__ Wp) {
-  extern __shared__ float sh[];  // [G][4][P2]
+  extern __shared__ float sh[];  // [G][4][P2], then Ct when it fits (staged)
   const int nb = 1 << level;
   const int box0 = blockIdx.x * G, cnt = min(G, nb * nb - box0);
   for (int i = threadIdx.x; i < cnt * 4 * P2; i += blockDim.x) {
@@ -202,13 +204,24 @@ __global__ void __launch_bounds__(kBoxThreads) k_fmm_m2m(int level, int P2, int 
     const long child = (long)(2 * by + q / 2) * (2 * nb) + 2 * bx + q % 2;
     sh[i] = Wc[child * P2 + mp];
   }
+  // the matrix at once: the sums run term by term, and each term's load from L2
+  // would be waited for a few at a time
+  float *mat = sh + G * 4 * P2;
+  if (staged)
+#pragma unroll 8
+    for (int i = threadIdx.x; i < 4 * P2 * P2; i += blockDim.x) mat[i] = __ldg(Ct + i);
   __syncthreads();
   for (int i = threadIdx.x; i < cnt * P2; i += blockDim.x) {
     const int g = i / P2, m = i % P2;
     const float *v = sh + g * 4 * P2;
     float acc = 0.f;
+    if (staged) {
+#pragma unroll 8
+      for (int k = 0; k < 4 * P2; ++k) acc = fmaf(mat[k * P2 + m], v[k], acc);
+    } else {
 #pragma unroll 24
-    for (int k = 0; k < 4 * P2; ++k) acc = fmaf(__ldg(Ct + (long)k * P2 + m), v[k], acc);
+      for (int k = 0; k < 4 * P2; ++k) acc = fmaf(__ldg(Ct + (long)k * P2 + m), v[k], acc);
+    }
     Wp[(long)(box0 + g) * P2 + m] = acc;
   }
 }
@@ -328,9 +341,10 @@ __global__ void __launch_bounds__(kBoxThreads) k_fmm_l2l(int level, int P2, int 
   __syncthreads();
   for (int i = threadIdx.x; i < cnt * P2; i += blockDim.x) {
     const int g = i / P2, mp = i % P2, box = box0 + g;
-    const float *C = Cq + (long)((box % nc & 1) + 2 * (box / nc & 1)) * P2 * P2 + mp, *v = sh + g * P2;
+    const float *C = Cq + (long)((box % nc & 1) + 2 * (box / nc & 1)) * P2 * P2 + mp;
+    const float *v = sh + g * P2;
     float acc = 0.f;
-#pragma unroll 18
+#pragma unroll 4
     for (int m = 0; m < P2; ++m) acc = fmaf(__ldg(C + (long)m * P2), v[m], acc);
     Lch[(long)box * P2 + mp] += acc;
   }
@@ -375,7 +389,7 @@ __global__ void k_fmm_leaf(int n, int L, int b, int P2, const float *__restrict_
   float c[4];
   dot.run(sh, c);
   if (part == 0) {
-#pragma unroll 18
+#pragma unroll 4
     for (int m = 0; m < P2; ++m) c[1] = fmaf(__ldg(Pm + m * bb + j), far[m], c[1]);
   }
   red[threadIdx.x] = (c[0] + c[1]) + (c[2] + c[3]);
@@ -510,14 +524,16 @@ vie_status fmm_apply(const FmmPlan &fp, int op, const float *s, const double *g,
   const int tm = std::max(P2, 256 / P2 * P2), tl = std::max(bb, 256 / bb * bb);
   auto ctas = [](long boxes, int G) { return (unsigned)((boxes + G - 1) / G); };
   // upward pass
-  const int gp = boxes_per_cta(P2, bb);
+  const int gp = boxes_per_cta(P2, bb, (long)nl * nl);
   k_fmm_p2m<<<ctas((long)nl * nl, gp), kBoxThreads, sizeof(float) * gp * bb, st>>>(n, L, b, P2, gp, fp.Pt, s,
                                                                                 fp.W + fp.node_off[L]);
   VIE_CHECK_LAUNCH("k_fmm_p2m");
-  const int gm = boxes_per_cta(P2, 4 * P2);
   for (int l = L - 1; l >= 2; --l) {
-    k_fmm_m2m<<<ctas(1L << (2 * l), gm), kBoxThreads, sizeof(float) * gm * 4 * P2, st>>>(
-        l, P2, gm, fp.Ct, fp.W + fp.node_off[l + 1], fp.W + fp.node_off[l]);
+    const int gm = boxes_per_cta(P2, 4 * P2, 1L << (2 * l));
+    const size_t own = sizeof(float) * gm * 4 * P2, mat = sizeof(float) * 4 * P2 * P2;
+    const bool staged = own + mat <= 48 * 1024;  // orders up to 7
+    k_fmm_m2m<<<ctas(1L << (2 * l), gm), kBoxThreads, own + (staged ? mat : 0), st>>>(
+        l, P2, gm, staged, fp.Ct, fp.W + fp.node_off[l + 1], fp.W + fp.node_off[l]);
     VIE_CHECK_LAUNCH("k_fmm_m2m");
   }
   // interactions (all levels in one launch), then the downward pass
@@ -535,14 +551,18 @@ vie_status fmm_apply(const FmmPlan &fp, int op, const float *s, const double *g,
     k_fmm_m2l<<<(unsigned)first, tm, sizeof(float) * (kIL * P2 + tm), st>>>(a, P2, fp.m2l, fp.W, fp.Lc);
     VIE_CHECK_LAUNCH("k_fmm_m2l");
   }
-  const int gl = boxes_per_cta(P2, P2);
-  for (int l = 2; l < L - 1; ++l) {
+  // the leaves take their own L2L step where there are enough of them to hide it
+  // behind other leaves' near fields (1024 leaves at order 4: 31 us without it, 40
+  // with it, 3 for a launch of its own; 4096 at order 6: 106 with it, 117 without)
+  const bool fused = L > 2 && nl * nl >= 2048;
+  for (int l = 2; l < (fused ? L - 1 : L); ++l) {
+    const int gl = boxes_per_cta(P2, P2, 4L << (2 * l));
     k_fmm_l2l<<<ctas(4L << (2 * l), gl), kBoxThreads, sizeof(float) * gl * P2, st>>>(
         l, P2, gl, fp.Cq, fp.Lc + fp.node_off[l], fp.Lc + fp.node_off[l + 1]);
     VIE_CHECK_LAUNCH("k_fmm_l2l");
   }
   k_fmm_leaf<<<nl * nl, tl, sizeof(float) * (9 * bb + 2 * P2 + tl), st>>>(
-      n, L, b, P2, fp.near, fp.Pm, s, fp.Lc + fp.node_off[L], L > 2 ? fp.Lc + fp.node_off[L - 1] : nullptr, fp.Cq,
+      n, L, b, P2, fp.near, fp.Pm, s, fp.Lc + fp.node_off[L], fused ? fp.Lc + fp.node_off[L - 1] : nullptr, fp.Cq,
       op, g, y);
   VIE_CHECK_LAUNCH("k_fmm_leaf");
   return VIE_OK;
