@@ -1133,13 +1133,14 @@ vie_status geometry_build(int n, int ldp, bool global, const Windows &win, int R
   std::vector<int4> uv(units.size());
   // the applies of stored weights run by cost alone: they read no lattice and no
   // records, and units of both run axes in turn spread the reductions over both
-  // halves of the sums (in the march's order 609 us at 128^2, so 511; small grids
-  // take them from both ends of that order in turn, 72 and 70 us at 64^2)
+  // halves of the sums (in the march's order 609 us at 128^2, so 511); with one
+  // tile a unit the march's order is that order
   std::stable_sort(units.begin(), units.end(), [](const U &p, const U &q) { return p.tile_cost > q.tile_cost; });
-  for (size_t i = 0; i < units.size(); ++i)
-    uv[i] = units[T == 2 ? i : i % 2 == 0 ? i / 2 : units.size() - 1 - i / 2].u;
-  VIE_CUDA(vie_malloc((void **)&geo->units_stream, sizeof(int4) * uv.size()));
-  VIE_CUDA(cudaMemcpy(geo->units_stream, uv.data(), sizeof(int4) * uv.size(), cudaMemcpyHostToDevice));
+  if (T == 2) {
+    for (size_t i = 0; i < units.size(); ++i) uv[i] = units[i].u;
+    VIE_CUDA(vie_malloc((void **)&geo->units_stream, sizeof(int4) * uv.size()));
+    VIE_CUDA(cudaMemcpy(geo->units_stream, uv.data(), sizeof(int4) * uv.size(), cudaMemcpyHostToDevice));
+  }
   std::stable_sort(units.begin(), units.end(), [T](const U &p, const U &q) {
     if (p.cls != q.cls) return p.cls < q.cls;
     if (T == 2 && (p.u.w & 3) != (q.u.w & 3)) return (p.u.w & 3) > (q.u.w & 3);
@@ -1287,7 +1288,7 @@ vie_status disp_prepare(DispPlan *dp, int n, const float *sig_padded, int device
   dp->geometry = geo;
   dp->doff = geo->doff;
   dp->units = geo->units;
-  dp->units_stream = geo->units_stream;
+  dp->units_stream = geo->units_stream ? geo->units_stream : geo->units;
   dp->stencil = geo->stencil;
   dp->n_units = geo->n_units;
   dp->taps = geo->taps;
