@@ -2210,7 +2210,8 @@ vie_status loss_grad(UnetImpl *u, const float *x, const float *t, const float *w
   if ((s = ensure_acts(u, B, n)) != VIE_OK || (s = ensure_dw(u)) != VIE_OK) return s;
   if ((s = pack_split_weights(u, st)) != VIE_OK) return s;
   // the training convolutions on the tensor cores in split precision: the
-  // forward in three parts (24 significant bits, FP32's own: in two parts its
+  // forward in three parts (24 bits an operand, FP32's own; the tensor cores'
+  // accumulation truncates, about 1e-5 of the loss: in two parts its
   // ~1e-5 relative error flipped the ReLU masks of pre-activations near zero,
   // each flip moving a gradient entry by a whole term, 3.6e-3 relative
   // against the FP64 reference, 1e-4 allowed), the input gradients in two
