@@ -334,6 +334,8 @@ vie_status diffusion_prepare(DiffPre *dp, int n, const double *sigma_t, const do
     VIE_CUDA(vie_malloc((void **)&dp->map, sizeof(double) * (size_t)Nc * Nc));
     k_dp_coarse_map<<<Nc, (Nc + 31) / 32 * 32, 0, st>>>(C.n, C.c, dp->map);
     VIE_CHECK_LAUNCH("k_dp_coarse_map");
+    // applies may come on another stream
+    VIE_CUDA(cudaStreamSynchronize(st));
   }
   dp->on = 1;
   return VIE_OK;
