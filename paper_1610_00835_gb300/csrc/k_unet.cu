@@ -1467,7 +1467,7 @@ void free_acts(UnetImpl *u) {
 // FP32 convolutions that training takes to the tensor cores in split precision
 bool conv_split_ok(int Ci, int Co) { return Ci <= 2 * kTmaSlice && Co % 32 == 0 && Co <= 64; }
 
-vie_status ensure_acts(UnetImpl *u, int B, int n) {
+vie_status ensure_acts(UnetImpl *u, int B, int n, cudaStream_t st) {
   if (u->B >= B && u->n == n) return VIE_OK;
   free_acts(u);
   const int L = u->L, C = u->C;
@@ -1534,12 +1534,12 @@ vie_status ensure_acts(UnetImpl *u, int B, int n) {
   // the hand-off buffers, zeroed once: their padding channels are never written
   const size_t cp1 = (size_t)((C + 31) / 32) * 32, cp2 = (size_t)((2 * C + 31) / 32) * 32;
   VIE_CUDA(vie_malloc((void **)&u->hx, sizeof(__nv_bfloat16) * (size_t)B * n * n * cp1));
-  VIE_CUDA(cudaMemset(u->hx, 0, sizeof(__nv_bfloat16) * (size_t)B * n * n * cp1));
+  VIE_CUDA(cudaMemsetAsync(u->hx, 0, sizeof(__nv_bfloat16) * (size_t)B * n * n * cp1, st));
   u->hcat.assign(L, nullptr);
   for (int l = 0; l < L - 1; ++l) {
     const size_t bytes = sizeof(__nv_bfloat16) * (size_t)B * (n >> l) * (n >> l) * cp2;
     VIE_CUDA(vie_malloc((void **)&u->hcat[l], bytes));
-    VIE_CUDA(cudaMemset(u->hcat[l], 0, bytes));
+    VIE_CUDA(cudaMemsetAsync(u->hcat[l], 0, bytes, st));
   }
   u->B = B;
   u->n = n;
@@ -2207,7 +2207,7 @@ vie_status backward(UnetImpl *u, const float *x, int B, int n, cudaStream_t st) 
 vie_status loss_grad(UnetImpl *u, const float *x, const float *t, const float *wts, int B, int n, double *loss,
                      cudaStream_t st) {
   vie_status s;
-  if ((s = ensure_acts(u, B, n)) != VIE_OK || (s = ensure_dw(u)) != VIE_OK) return s;
+  if ((s = ensure_acts(u, B, n, st)) != VIE_OK || (s = ensure_dw(u)) != VIE_OK) return s;
   if ((s = pack_split_weights(u, st)) != VIE_OK) return s;
   // the training convolutions on the tensor cores in split precision: the
   // forward in three parts (24 bits an operand, FP32's own; the tensor cores'
@@ -2249,7 +2249,7 @@ vie_status unet_precondition(UnetImpl *u, const double *sigma_t, const double *s
                              const double *v, const double *vnorm2, int n, float *xbuf, const double *base,
                              double *z, cudaStream_t st) {
   vie_status s;
-  if ((s = ensure_acts(u, 1, n)) != VIE_OK) return s;
+  if ((s = ensure_acts(u, 1, n, st)) != VIE_OK) return s;
   const long N = (long)n * n;
   k_net_input<<<gridn(N), 256, 0, st>>>(sigma_t, sigma_s, v, vnorm2, N, (float)inv_ref, xbuf);
   VIE_CHECK_LAUNCH("k_net_input");
@@ -2267,7 +2267,7 @@ vie_status unet_precondition_batch(UnetImpl *u, const double *sigma_t, const dou
                                    const double *v, long ldv, const double *scal, int slot, int R, int n,
                                    float *xbuf, const double *base, long ldb, double *z, long ldz, cudaStream_t st) {
   vie_status s;
-  if ((s = ensure_acts(u, R, n)) != VIE_OK) return s;
+  if ((s = ensure_acts(u, R, n, st)) != VIE_OK) return s;
   const long N = (long)n * n;
   const dim3 grid((unsigned)std::max(1L, std::min((N + 255) / 256, 1024L)), (unsigned)R);
   k_net_input_b<<<grid, 256, 0, st>>>(sigma_t, sigma_s, v, ldv, scal, slot, N, (float)inv_ref, xbuf);
@@ -2433,7 +2433,7 @@ vie_status vie_unet_forward(vie_unet *u, const float *x, float *o, int B, int n,
   }
   VIE_CUDA(cudaSetDevice(u->impl.device));
   cudaStream_t st = (cudaStream_t)stream;
-  vie_status s = ensure_acts(&u->impl, B, n);
+  vie_status s = ensure_acts(&u->impl, B, n, st);
   if (s != VIE_OK) return s;
   s = use_bf16 ? forward<__nv_bfloat16>(&u->impl, u->impl.pb, x, B, n, st)
                : forward<float>(&u->impl, u->impl.p, x, B, n, st);

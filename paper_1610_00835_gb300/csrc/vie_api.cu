@@ -294,7 +294,7 @@ void free_all(vie_handle *h) {
   h->events.clear();
 }
 
-vie_status ensure_gmres(vie_handle *h, int m) {
+vie_status ensure_gmres(vie_handle *h, int m, cudaStream_t st) {
   if (h->gm_m >= m) return VIE_OK;
   free_gmres(h);
   const long N = h->N;
@@ -312,11 +312,11 @@ vie_status ensure_gmres(vie_handle *h, int m) {
   if ((s = dalloc(&h->scal, 8)) != VIE_OK) return s;
   if (!h->ticket) {
     if ((s = dalloc(&h->ticket, 1)) != VIE_OK) return s;
-    VIE_CUDA(cudaMemset(h->ticket, 0, sizeof(int)));
+    VIE_CUDA(cudaMemsetAsync(h->ticket, 0, sizeof(int), st));
   }
   if (!h->bar) {
     if ((s = dalloc(&h->bar, 2)) != VIE_OK) return s;
-    VIE_CUDA(cudaMemset(h->bar, 0, 2 * sizeof(unsigned)));
+    VIE_CUDA(cudaMemsetAsync(h->bar, 0, 2 * sizeof(unsigned), st));
   }
   VIE_CUDA(vie_malloc_host((void **)&h->h_pinned, sizeof(double) * (m + 1 + 8)));
   VIE_CUDA(vie_malloc_host((void **)&h->slots, sizeof(double) * 4));
@@ -547,15 +547,15 @@ vie_status wait_slots(vie_handle *h, const double *slots, int R, const int *act,
     return take_errors(h, st);
   }
   if (gave_up) {
+    VIE_CUDA(cudaMemsetAsync(h->bar, 0, 2 * sizeof(unsigned), st));
     VIE_CUDA(cudaStreamSynchronize(st));
-    VIE_CUDA(cudaMemset(h->bar, 0, 2 * sizeof(unsigned)));
     set_error("vie_solve_gmres: a bounded device wait of the Arnoldi step ran out");
     return VIE_ERR_TIMEOUT;
   }
   return VIE_OK;
 }
 
-vie_status ensure_multi(vie_handle *h, int R, int m, bool need_z, bool need_net) {
+vie_status ensure_multi(vie_handle *h, int R, int m, bool need_z, bool need_net, cudaStream_t st) {
   MultiGmres &g = h->mg;
   if (g.R >= R && g.m >= m && (g.has_z || !need_z) && (g.has_net || !need_net)) return VIE_OK;
   free_multi(g);
@@ -581,7 +581,7 @@ vie_status ensure_multi(vie_handle *h, int R, int m, bool need_z, bool need_net)
   if ((s = dalloc(&b.act, (size_t)R)) != VIE_OK) return s;
   if ((s = dalloc(&g.kk, (size_t)R)) != VIE_OK) return s;
   if (need_net && (s = dalloc(&g.net_x, (size_t)R * 3 * N)) != VIE_OK) return s;
-  VIE_CUDA(cudaMemset(b.ticket, 0, sizeof(int) * R));
+  VIE_CUDA(cudaMemsetAsync(b.ticket, 0, sizeof(int) * R, st));
   VIE_CUDA(vie_malloc_host((void **)&g.h_scal, sizeof(double) * 8 * R));
   VIE_CUDA(vie_malloc_host((void **)&g.h_gv, sizeof(double) * (size_t)R * (m + 1)));
   VIE_CUDA(vie_malloc_host((void **)&g.h_act, sizeof(int) * 2 * R));
@@ -675,7 +675,7 @@ vie_status solve_multi(vie_handle *h, const double *fdev, double *x, int R, cons
   const int m = opt.restart;
   const bool has_precond = h->precond || h->fft.on || h->diff.on;
   vie_status s;
-  if ((s = ensure_multi(h, R, m, has_precond, h->precond != nullptr)) != VIE_OK) return s;
+  if ((s = ensure_multi(h, R, m, has_precond, h->precond != nullptr, st)) != VIE_OK) return s;
   MultiGmres &g = h->mg;
   KBatch b = g.kb;
   b.R = R;
@@ -1520,7 +1520,7 @@ vie_status vie_solve_gmres(vie_handle *h, const double *f, double *U, const vie_
     }
     return s;
   }
-  if ((s = ensure_gmres(h, m)) != VIE_OK) return s;
+  if ((s = ensure_gmres(h, m, st)) != VIE_OK) return s;
   const bool has_precond = h->precond || h->fft.on || h->diff.on;
   if (has_precond && h->z_m < m) {
     dfree(h->Z);
