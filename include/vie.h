@@ -477,12 +477,16 @@ vie_status vie_diffusion_precondition(vie_handle *h, const double *v, double *z,
  * Arnoldi step), vie_apply with host pointers, vie_unet_forward with
  * use_bf16 (which synchronises its stream) and vie_check_device; the word is
  * cleared when reported, so the next call runs normally.
+ * The grid-wide barriers of vie_solve_gmres's Arnoldi step (one source, more
+ * than 16384 cells) are bounded by the same limits: no block passes a barrier that
+ * ran out, and the solve returns VIE_ERR_TIMEOUT.
  *
  * vie_set_wait_limits sets the bounds for later launches, process-wide, in
  * milliseconds (converted with the device's clock rate): limit_ms for every
  * wait (default 1000), first_wait_ms for the first producer/consumer wait of
- * each CTA (negative: the same as limit_ms; 0: that wait gives up at once,
- * which lets a test exercise the failure path without a fault).
+ * each CTA and the first barrier of an Arnoldi step (negative: the same as
+ * limit_ms; 0: that wait gives up at once, which lets a test exercise the failure
+ * path without a fault).
  * Errors: INVALID_ARG (0 < limit_ms <= 60000 and first_wait_ms <= limit_ms
  * required). */
 vie_status vie_set_wait_limits(double limit_ms, double first_wait_ms);

@@ -172,30 +172,35 @@ __device__ __forceinline__ void by_count(int n, F &&f) {
 // how the blocks of one right-hand side wait for one another
 enum StepSync { kOneBlock = 0, kCluster = 1, kGridWide = 2 };
 
-// Grid-wide barrier of a cooperative launch: bar[0] counts arrivals, `target`
-// of them must have come.  The wait is bounded; false: it ran out.
-__device__ __forceinline__ bool grid_wait(unsigned *bar, unsigned target) {
+// Grid-wide barrier of a cooperative launch: bar counts arrivals, `target` of
+// them must have come.  The wait is bounded (a limit of zero gives up at once);
+// false: it ran out.  All blocks get the same answer: a block whose time is up
+// sets the top bit of the counter, in one atomic step only while arrivals are
+// missing, and with the bit set nobody passes.  (Each block deciding for itself,
+// one could give up just before the last arrival while the others went on.)
+constexpr unsigned kGaveUp = 0x80000000u;
+__device__ __forceinline__ bool grid_wait(unsigned *bar, unsigned target, long long limit) {
   __shared__ int ok;
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
     atomicAdd(bar, 1u);
     const long long t0 = clock64();
-    int good = 1;
-    while (atomicAdd(bar, 0u) < target)
-      if (clock64() - t0 > 4000000000ll) {
-        good = 0;
-        break;
-      }
+    unsigned seen = 0;
+    if (limit <= 0) seen = atomicOr(bar, kGaveUp) | kGaveUp;
+    while (seen < target) {
+      seen = atomicAdd(bar, 0u);
+      if (seen < target && clock64() - t0 > limit && atomicCAS(bar, seen, seen | kGaveUp) == seen) seen |= kGaveUp;
+    }
     __threadfence();
-    ok = good;
+    ok = !(seen & kGaveUp);
   }
   __syncthreads();
   return ok != 0;
 }
 
 template <int SYNC>
-__device__ __forceinline__ bool step_wait(unsigned *bar, unsigned &target) {
+__device__ __forceinline__ bool step_wait(unsigned *bar, unsigned &target, long long limit) {
   if constexpr (SYNC == kOneBlock) {
     __syncthreads();
     return true;
@@ -205,7 +210,7 @@ __device__ __forceinline__ bool step_wait(unsigned *bar, unsigned &target) {
     return true;
   } else {
     target += gridDim.x;
-    return grid_wait(bar, target);
+    return grid_wait(bar, target, limit);
   }
 }
 
@@ -220,7 +225,7 @@ __device__ __forceinline__ bool step_wait(unsigned *bar, unsigned &target) {
 template <int SYNC, bool REG, int VB>
 __global__ void __launch_bounds__(kDotThreads, 4) k_arnoldi(KBatch b, double *__restrict__ V, long ldv_r, int k,
                                                             double inv_bnorm1, const int *err0, const int *err1,
-                                                            unsigned long long seq, unsigned *bar) {
+                                                            unsigned long long seq, unsigned *bar, WaitLimits wl) {
   static_assert(REG || VB == 1, "one block per CTA without the registers");
   __shared__ double red[8][kDotThreads];
   __shared__ double hs[256], hc[256];
@@ -323,7 +328,7 @@ __global__ void __launch_bounds__(kDotThreads, 4) k_arnoldi(KBatch b, double *__
   };
   double n2 = 0.0;
   dots(partA);
-  bool ok = step_wait<SYNC>(bar, target);
+  bool ok = step_wait<SYNC>(bar, target, wl.first);
   if (ok) {
     sums(partA, false);
     if (REG && nv <= 8) {
@@ -357,7 +362,7 @@ __global__ void __launch_bounds__(kDotThreads, 4) k_arnoldi(KBatch b, double *__
       update();
       dots(partB);
     }
-    ok = step_wait<SYNC>(bar, target);
+    ok = step_wait<SYNC>(bar, target, wl.limit);
   }
   if (ok) {
     sums(partB, true);
@@ -376,7 +381,7 @@ __global__ void __launch_bounds__(kDotThreads, 4) k_arnoldi(KBatch b, double *__
       s = block_sum(s, red[0]);
       if (tid == 0) partA[(long)blockIdx.x + (long)vb * gridDim.x] = s;
     }
-    ok = step_wait<SYNC>(bar, target);
+    ok = step_wait<SYNC>(bar, target, wl.limit);
   }
   if (ok) {
     if (warp == 0) {
@@ -633,6 +638,9 @@ bool arnoldi_fused(const KBatch &b) { return b.R == 1 || b.blocks <= kMaxCluster
 vie_status launch_arnoldi(const KBatch &b, double *V, long ldv_r, int k, double inv_bnorm1, const int *err0,
                           const int *err1, unsigned long long seq, unsigned *bar, cudaStream_t st) {
   const bool reg = b.N <= (long)kRegElems * b.blocks * kDotThreads;
+  int dev = 0;
+  VIE_CUDA(cudaGetDevice(&dev));
+  const WaitLimits wl = wait_limits(dev);
   // large batches: two blocks per CTA (and clusters of 8)
   const int vb = b.R > 1 && b.blocks == kMaxCluster ? 2 : 1;
   cudaLaunchConfig_t cfg{};
@@ -642,7 +650,7 @@ vie_status launch_arnoldi(const KBatch &b, double *V, long ldv_r, int k, double 
   cudaLaunchAttribute at[1];
   cfg.attrs = at;
   auto go = [&](auto kernel) {
-    return cudaLaunchKernelEx(&cfg, kernel, b, V, ldv_r, k, inv_bnorm1, err0, err1, seq, bar);
+    return cudaLaunchKernelEx(&cfg, kernel, b, V, ldv_r, k, inv_bnorm1, err0, err1, seq, bar, wl);
   };
   if (b.blocks == 1) {
     VIE_CUDA(go(k_arnoldi<kOneBlock, true, 1>));

@@ -547,8 +547,7 @@ vie_status wait_slots(vie_handle *h, const double *slots, int R, const int *act,
     return take_errors(h, st);
   }
   if (gave_up) {
-    VIE_CUDA(cudaMemsetAsync(h->bar, 0, 2 * sizeof(unsigned), st));
-    VIE_CUDA(cudaStreamSynchronize(st));
+    VIE_CUDA(cudaStreamSynchronize(st));  // (the kernel's last block leaves the barrier at zero)
     set_error("vie_solve_gmres: a bounded device wait of the Arnoldi step ran out");
     return VIE_ERR_TIMEOUT;
   }
