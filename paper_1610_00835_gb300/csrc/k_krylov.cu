@@ -22,6 +22,7 @@
 
 #include <atomic>
 
+#include "arnoldi_form.cuh"
 #include "vie_internal.cuh"
 
 namespace vie {
@@ -146,7 +147,6 @@ __device__ void backsolve_warp(const double *__restrict__ H, int m, int k, const
 }
 
 constexpr int kRegElems = 4;       // elements of w a thread keeps in registers
-constexpr int kMaxCluster = 16;    // blocks of the cluster form
 
 // f(Count<1>) .. f(Count<8>) for min(n, 8): the sweeps over up to eight basis
 // vectors are compiled for their number (predicated off, the operations of the
@@ -607,15 +607,46 @@ __global__ void k_baxpby(KBatch b, double a, const double *__restrict__ x, long 
 
 }  // namespace
 
-// Clusters of more than 8 blocks need a per-kernel opt-in, once per device.
-static vie_status allow_large_clusters(const void *kernel) {
-  static std::atomic<unsigned long long> done{0};
+// What the current device has room for, asked once per device (two words, no
+// state of a solve).  Clusters of more than 8 blocks need a per-kernel opt-in.
+static vie_status arnoldi_room(ArnoldiRoom *room) {
+  static std::atomic<int> known[64];  // 1 + cluster + 32 resident
   int dev = 0;
   VIE_CUDA(cudaGetDevice(&dev));
-  const unsigned long long bit = 1ull << (dev & 63);
-  if (done.load() & bit) return VIE_OK;
-  VIE_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-  done.fetch_or(bit);
+  int v = known[dev & 63].load();
+  if (v == 0) {
+    const void *wide = (const void *)k_arnoldi<kCluster, true, 1>;
+    VIE_CUDA(cudaFuncSetAttribute(wide, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    auto clusters = [&](const void *kernel, unsigned size) {
+      cudaLaunchAttribute at[1];
+      at[0].id = cudaLaunchAttributeClusterDimension;
+      at[0].val.clusterDim.x = size;
+      at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+      cudaLaunchConfig_t cfg{};
+      cfg.gridDim = dim3(size);
+      cfg.blockDim = dim3(kDotThreads);
+      cfg.attrs = at;
+      cfg.numAttrs = 1;
+      int n = 0;
+      if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
+        cudaGetLastError();  // a size the device does not run
+        n = 0;
+      }
+      return n;
+    };
+    const int cluster = clusters(wide, 16) > 0                                                         ? 16
+                        : clusters(wide, 8) > 0 && clusters((const void *)k_arnoldi<kCluster, true, 2>, 8) > 0 ? 8
+                                                                                                       : 0;
+    int per_sm = 0, per_sm_reg = 0;
+    DevProps prop;
+    VIE_TRY(get_dev_props(dev, &prop));
+    VIE_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_arnoldi<kGridWide, false, 1>, kDotThreads, 0));
+    VIE_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_reg, k_arnoldi<kGridWide, true, 1>, kDotThreads, 0));
+    v = 1 + cluster + 32 * ((per_sm < per_sm_reg ? per_sm : per_sm_reg) * prop.multiProcessorCount);
+    known[dev & 63].store(v);
+  }
+  room->cluster = (v - 1) % 32;
+  room->resident = (v - 1) / 32;
   return VIE_OK;
 }
 
@@ -623,7 +654,8 @@ static vie_status allow_large_clusters(const void *kernel) {
 // as long as a thread then holds at most four elements: with one block the
 // narrow FP64 pipe of its SM bounds the step (17.7 us at N = 1024; four blocks
 // 13.3).  Above, four elements per thread: the block sums add one
-// operation per thread to them (25 %); past one block per SM, two on every SM.
+// operation per thread to them (25 %); past one block per SM, two on every SM
+// (152; the same on a part of the device, so that the sums keep their order).
 int dot_blocks(long N) {
   const long one = (N + kDotThreads - 1) / kDotThreads;
   if (one <= kMaxCluster) return (int)(one < 1 ? 1 : one);
@@ -631,9 +663,12 @@ int dot_blocks(long N) {
   return (int)(four <= kMaxCluster ? kMaxCluster : four <= 152 ? four : 304);
 }
 
-// the Arnoldi step of column k for every active r in one launch (R = 1: any
-// N; R > 1: up to kMaxCluster blocks, else false and nothing is launched)
-bool arnoldi_fused(const KBatch &b) { return b.R == 1 || b.blocks <= kMaxCluster; }
+vie_status arnoldi_fused(long N, int R, bool *fused) {
+  ArnoldiRoom room;
+  VIE_TRY(arnoldi_room(&room));
+  *fused = arnoldi_one_launch(dot_blocks(N), R, room);
+  return VIE_OK;
+}
 
 vie_status launch_arnoldi(const KBatch &b, double *V, long ldv_r, int k, double inv_bnorm1, const int *err0,
                           const int *err1, unsigned long long seq, unsigned *bar, cudaStream_t st) {
@@ -642,7 +677,7 @@ vie_status launch_arnoldi(const KBatch &b, double *V, long ldv_r, int k, double 
   VIE_CUDA(cudaGetDevice(&dev));
   const WaitLimits wl = wait_limits(dev);
   // large batches: two blocks per CTA (and clusters of 8)
-  const int vb = b.R > 1 && b.blocks == kMaxCluster ? 2 : 1;
+  const int vb = b.blocks <= kMaxCluster ? b.blocks / arnoldi_cluster(b.blocks, b.R) : 1;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)(b.blocks / vb), (unsigned)b.R);
   cfg.blockDim = dim3(kDotThreads);
@@ -655,7 +690,6 @@ vie_status launch_arnoldi(const KBatch &b, double *V, long ldv_r, int k, double 
   if (b.blocks == 1) {
     VIE_CUDA(go(k_arnoldi<kOneBlock, true, 1>));
   } else if (b.blocks <= kMaxCluster) {
-    VIE_TRY(allow_large_clusters((const void *)k_arnoldi<kCluster, true, 1>));
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = cfg.gridDim.x;
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;

@@ -599,12 +599,12 @@ vie_status ensure_multi(vie_handle *h, int R, int m, bool need_z, bool need_net,
 
 // Operator applies to R vectors, column r of g at g + r ldg and of y at
 // y + r ldy.  With the assembled BF16 hi/lo operator every product of K goes
-// through the tensor cores, all columns in one product (up to 128); otherwise
-// one apply per column with act[r] != 0 (act NULL: every column).
+// through the tensor cores, all columns in one product (up to 128); otherwise (and
+// for a single column) one apply per column with act[r] != 0 (act NULL: every column).
 vie_status apply_multi(vie_handle *h, int op, const double *g, long ldg, double *y, long ldy, int R,
                        const int *act, cudaStream_t st, bool timed) {
   vie_status s;
-  if (h->asm_mode == VIE_OPERATOR_BF16X3 && op != VIE_OP_A_RAW) {
+  if (h->asm_mode == VIE_OPERATOR_BF16X3 && op != VIE_OP_A_RAW && R > 1) {
     ApplyEvents *ev = nullptr;
     if (timed) {
       if (h->events.empty()) {
@@ -675,6 +675,8 @@ vie_status solve_multi(vie_handle *h, const double *fdev, double *x, int R, cons
   const bool has_precond = h->precond || h->fft.on || h->diff.on;
   vie_status s;
   if ((s = ensure_multi(h, R, m, has_precond, h->precond != nullptr, st)) != VIE_OK) return s;
+  bool fused = false;
+  if ((s = arnoldi_fused(N, R, &fused)) != VIE_OK) return s;
   MultiGmres &g = h->mg;
   KBatch b = g.kb;
   b.R = R;
@@ -805,7 +807,7 @@ vie_status solve_multi(vie_handle *h, const double *fdev, double *x, int R, cons
         return s;
       for (int r = 0; r < R; ++r) napply[r] += act[r];
       // CGS2 (two passes of h = V^T w, w -= V h), the norm and the Givens step
-      if (arnoldi_fused(b)) {
+      if (fused) {
         const int *err1 = h->precond ? unet_error_word(h->precond) : nullptr;
         if ((s = launch_arnoldi(b, g.V, ldv, k, 0.0, h->dev_err, err1, ++h->step_seq, nullptr, st)) != VIE_OK)
           return s;
@@ -1491,8 +1493,11 @@ vie_status vie_solve_gmres(vie_handle *h, const double *f, double *U, const vie_
   const long N = h->N;
   const int m = opt.restart;
   vie_status s;
-  if (opt.nrhs > 1) {
-    // several sources on this medium: lockstep solves
+  bool one_launch = true;
+  if (opt.nrhs == 1 && (s = arnoldi_fused(N, 1, &one_launch)) != VIE_OK) return s;
+  if (opt.nrhs > 1 || !one_launch) {
+    // several sources on this medium: lockstep solves (which also take the
+    // Arnoldi step in separate launches, where one launch has no room)
     const int R = opt.nrhs;
     const size_t total = (size_t)R * N;
     h->t_apply_ms = h->t_kernel_ms = 0.0;

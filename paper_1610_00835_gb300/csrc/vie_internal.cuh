@@ -347,10 +347,10 @@ vie_status launch_bscale(const KBatch &b, const double *x, long ldx_r, int slot,
                          cudaStream_t st);
 vie_status launch_baxpby(const KBatch &b, double a, const double *x, long ldx_r, double c, const double *y,
                          long ldy_r, double *z, long ldz_r, cudaStream_t st);
-// one launch for the whole Arnoldi step (arnoldi_fused), or the separate ones
-// above; bar: two zeroed device words; err0, err1: device error words to
-// report or null
-bool arnoldi_fused(const KBatch &b);
+// one launch for the whole Arnoldi step where the current device has room for
+// it (arnoldi_form.cuh), or the separate ones above; bar: two zeroed device
+// words; err0, err1: device error words to report or null
+vie_status arnoldi_fused(long N, int R, bool *fused);
 vie_status launch_arnoldi(const KBatch &b, double *V, long ldv_r, int k, double inv_bnorm1, const int *err0,
                           const int *err1, unsigned long long seq, unsigned *bar, cudaStream_t st);
 // the triangular solve and x_r += sum_{v < k} y_v B_r[v] (k_all >= 0, else kk[r])
