@@ -92,7 +92,8 @@ __device__ double givens_step(double *H, int m, int k, const double *hcol, doubl
     c[i] = ci * a + si * b;
     a = -si * a + ci * b;
   }
-  const double b = hk1sq > 0.0 ? hk1sq * rsqrt(hk1sq) : hk1sq;
+  // (an overflowed norm stays infinite: the rotation below and the estimate are NaN)
+  const double b = hk1sq > 0.0 && hk1sq <= 1.7976931348623157e308 ? hk1sq * rsqrt(hk1sq) : hk1sq;
   const double big = fmax(fabs(a), fabs(b));
   // 2^-e with 2^e <= big < 2^(e+1), clamped so that it and its inverse are normal
   const int e = max(2, min(2044, (int)((__double_as_longlong(big) >> 52) & 0x7ff)));
