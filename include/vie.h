@@ -388,12 +388,13 @@ vie_status vie_unet_layer_io(vie_unet *u, int layer, float *in, float *out, void
 
 /* Mean squared error of Net(x) against t (device FP32 [B][n][n]) and, if
  * grads_host is not NULL, its gradient with respect to every parameter
- * (host FP32 [num_params]). Synchronous. */
+ * (host FP32 [num_params]). Synchronous; VIE_ERR_TIMEOUT if a tensor-core kernel
+ * gave up on a bounded wait. */
 vie_status vie_unet_loss_grad(vie_unet *u, const float *x, const float *t, int B, int n, float *grads_host,
                               double *loss, void *stream);
 /* One Adam step (beta 0.9 / 0.999, eps 1e-8) on the batch; returns the loss
  * mean_b w_b mean_p (o - t)^2, w_b = weights[b] (device FP32 [B]) or 1 if
- * weights is NULL. */
+ * weights is NULL.  After an error the parameters and moments are as before. */
 vie_status vie_unet_train_step(vie_unet *u, const float *x, const float *t, const float *weights, int B,
                                int n, float lr, double *loss, void *stream);
 /* Checkpoint: the parameters and the Adam state (step count, first and
@@ -468,14 +469,15 @@ vie_status vie_diffusion_precondition(vie_handle *h, const double *v, double *z,
 
 /* ---- Failure detection of the tensor-core kernels (no paper counterpart).
  * Every wait of the kernels that issue tcgen05.mma (the multi-RHS product of
- * VIE_OPERATOR_BF16X3 and the BF16 convolutions of the learned
- * preconditioner) on an mbarrier is bounded.  A CTA whose wait runs out stops
- * issuing work, waits (bounded by the full limit) for the copies and
+ * VIE_OPERATOR_BF16X3, the BF16 convolutions of the learned
+ * preconditioner and its training) on an mbarrier is bounded.  A CTA whose wait
+ * runs out stops issuing work, waits (bounded by the full limit) for the copies and
  * products it already issued, frees its tensor memory, writes NaN into its
  * outputs and sets the error word of its handle or network.  Synchronous
  * calls report that as VIE_ERR_TIMEOUT: vie_solve_gmres (checked at every
  * Arnoldi step), vie_apply with host pointers, vie_unet_forward with
- * use_bf16 (which synchronises its stream) and vie_check_device; the word is
+ * use_bf16 (which synchronises its stream), vie_unet_loss_grad,
+ * vie_unet_train_step and vie_check_device; the word is
  * cleared when reported, so the next call runs normally.
  * The grid-wide barriers of vie_solve_gmres's Arnoldi step (one source, more
  * than 16384 cells) are bounded by the same limits: no block passes a barrier that

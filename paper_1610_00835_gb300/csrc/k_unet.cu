@@ -2235,7 +2235,11 @@ vie_status loss_grad(UnetImpl *u, const float *x, const float *t, const float *w
     TrainTc tc2(u, 2);
     if ((s = backward(u, x, B, n, st)) != VIE_OK) return s;
   }
+  // a tensor-core kernel that gave up on a wait left NaN in the gradients
+  int *e = reinterpret_cast<int *>(u->h_part + blocks);
+  VIE_CUDA(cudaMemcpyAsync(e, u->dev_err, sizeof(int), cudaMemcpyDeviceToHost, st));
   VIE_CUDA(cudaStreamSynchronize(st));
+  if (*e != 0) return unet_take_error(u, st);
   double sum = 0.0;
   for (int i = 0; i < blocks; ++i) sum += u->h_part[i];
   *loss = sum / (double)cnt;
