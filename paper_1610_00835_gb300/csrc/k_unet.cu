@@ -807,9 +807,12 @@ __global__ void __launch_bounds__(256, 3) k_conv3_dw(const float *__restrict__ x
 // input row of Wp + 2 pixels serves three output rows; zero fill outside the
 // image is the convolution's padding and pads Wp to a multiple of 16), warp 5
 // issues the products of one row and one ky into one of kDwAcc accumulators of
-// 96 columns, warps 0-2 add the finished ones to FP32 sums in registers (after
-// at most 24 products per column: the accumulation of tcgen05 truncates, long
-// chains would drift).  The CTAs' sums are added by k_dw_reduce, in order.
+// 96 columns, warps 0-2 add the finished ones to FP32 sums in registers.  The
+// accumulation of tcgen05 truncates, so chains are short (a row) and each column
+// block has products of one size, parts i + j = 0, 1 and 2: the large ones are
+// not truncated again for every small one (against FP64 6e-8 to 9e-8 relative at
+// 128^2 and 136^2; with all parts of the input against the same columns 3.5e-7,
+// the CUDA-core form 1.8e-7).  The CTAs' sums are added by k_dw_reduce, in order.
 // What bounds it is the operand traffic of the products.  The CUDA-core form
 // (k_conv3_dw, other widths) took 95 us per layer of 16 images at 128^2 on
 // average; this takes 30 us (50 us for a 32 -> 32 layer at 128^2).
@@ -937,8 +940,8 @@ __global__ void __launch_bounds__(kConvThreads, 1)
         for (int s = 0; s < Wp / 16; ++s, xd += 1024 >> 4, gd += 1024 >> 4)
 #pragma unroll
           for (int a = 0; a < kDwParts; ++a)
-            mma_bf16(d, xd + (unsigned)(a * (xp >> 4)), gd, idesc_bf16(kTcM, 32 * (kDwParts - a), true),
-                     a > 0 || s > 0 ? 1u : 0u);
+            mma_bf16(d + 32u * (unsigned)a, xd + (unsigned)(a * (xp >> 4)), gd,
+                     idesc_bf16(kTcM, 32 * (kDwParts - a), true), a > 0 || s > 0 ? 1u : 0u);
         mma_commit(su32(tfull + st));
       }
       if (!go) break;
