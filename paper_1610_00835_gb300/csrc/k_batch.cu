@@ -387,7 +387,7 @@ vie_status enqueue_one(vie_batch *b, int op, const double *g, double *y, cudaStr
       if ((s = disp_launch(dp, G.n, (float)(h / kS * 1.4426950408889634), (float)(h / (2.0 * kPi)), st)) != VIE_OK)
         return s;
       if ((s = disp_reduce(dp, G.N, op, b->diag + off, b->sig_s + off, g + off, y + off, st)) != VIE_OK) return s;
-      k += 3;
+      k += 2 + disp_march_launches(dp);
     } else {
       if ((s = launch_reduce(G.N, G.T, op, b->partial + b->part_off[i], b->diag + off, b->sig_s + off, g + off,
                              y + off, st)) != VIE_OK)

@@ -1525,6 +1525,11 @@ vie_status disp_march_launch(const DispPlan &dp, DispArgs a, const void *kernel,
 
 }  // namespace
 
+int disp_march_launches(const DispPlan &dp) {
+  if (!dp.global) return 1;
+  return (dp.window_end[0] > 0) + (dp.window_end[1] > dp.window_end[0]) + (dp.n_units > dp.window_end[1]);
+}
+
 vie_status disp_launch(const DispPlan &dp, int n, float tau_scale2, float wcoef, cudaStream_t st) {
   return disp_march_launch(dp, disp_args(dp, n, tau_scale2, wcoef, nullptr), dp.kernel, dp.kernel_window, dp.grid,
                            dp.smem, st);

@@ -252,6 +252,7 @@ vie_status disp_prepare(DispPlan *dp, int n, const float *sig_padded, int device
 vie_status disp_mii_prepare(DispPlan *dp, int n, double *diag_value, cudaStream_t st);
 void disp_release(DispPlan *dp);
 vie_status disp_launch(const DispPlan &dp, int n, float tau_scale2, float wcoef, cudaStream_t st);
+int disp_march_launches(const DispPlan &dp);  // the kernels that disp_launch queues
 vie_status disp_store(const DispPlan &dp, int n, float tau_scale2, float wcoef, float *wbuf, cudaStream_t st);
 int symv_max_n();  // largest grid the symmetric-block product takes (160)
 size_t symv_block_floats(int n);
