@@ -1030,7 +1030,7 @@ __global__ void __launch_bounds__(kConvThreads, 1)
 // dw[co][ci][tap] += the sum of the CTAs' partials [slice][cta][tap][32 ci][32
 // co] and db[co] += that of part_b[block][32], in a fixed order: block (tap,
 // ci) of each slice, and a last one for db; 8 runs of the partials side by
-// side in FP32 (about 20 terms each), joined in FP64.
+// side, at most 64 terms at a time in FP32, joined in FP64.
 // (One launch for all layers, blockIdx.y the layer.)
 struct DwJob {
   long part, part_b;  // the layer's sums in dw_part and db_part
@@ -1057,10 +1057,14 @@ __global__ void __launch_bounds__(256) k_dw_reduce(const __grid_constant__ DwJob
   const float *p = bias ? parts_b + jb.part_b : part + ((size_t)slice * ctas * 9 * 32 + r) * 32;
   const size_t step = bias ? 32 : (size_t)9 * 1024;
   const int n = bias ? jb.blocks : ctas;
-  float f = 0.f;
+  double s = 0.0;
+  for (int c = run; c < n;) {
+    const int end = min(n, c + 512);
+    float f = 0.f;
 #pragma unroll 8
-  for (int c = run; c < n; c += 8) f += p[c * step + co];
-  double s = f;
+    for (; c < end; c += 8) f += p[c * step + co];
+    s += f;
+  }
   red[run][co] = s;
   __syncthreads();
   if (run > 0 || (!bias && ci >= Ci)) return;
@@ -1111,13 +1115,19 @@ __global__ void k_head_bwd_w(const float *__restrict__ go, const float *__restri
   __shared__ double red[256];
   const int c = blockIdx.x, k = blockIdx.y, K = gridDim.y;
   const long total = (long)B * plane, i0 = total * k / K, i1 = total * (k + 1) / K;
-  float s = 0.f;  // a few dozen terms per thread in FP32; the block's sum in FP64
+  double s = 0.0;
   long b = (i0 + threadIdx.x) / plane, p = i0 + threadIdx.x - b * plane;
   const float *dc = d + c * plane;
+  // 64 terms at a time in FP32, the rest in FP64: the rounding does not grow with the image
+  for (long i = i0 + threadIdx.x; i < i1;) {
+    const long end = min(i1, i + 64L * blockDim.x);
+    float f = 0.f;
 #pragma unroll 4
-  for (long i = i0 + threadIdx.x; i < i1; i += blockDim.x, p += blockDim.x) {
-    for (; p >= plane; p -= plane) ++b;  // (no division per term)
-    s += go[i] * (c < C ? dc[b * d_bs + p] : 1.f);
+    for (; i < end; i += blockDim.x, p += blockDim.x) {
+      for (; p >= plane; p -= plane) ++b;  // (no division per term)
+      f += go[i] * (c < C ? dc[b * d_bs + p] : 1.f);
+    }
+    s += f;
   }
   red[threadIdx.x] = s;
   __syncthreads();
