@@ -1415,15 +1415,17 @@ struct UnetImpl {
   __nv_bfloat16 *hx = nullptr;
   std::vector<__nv_bfloat16 *> hcat;
   int train_tc = 0;  // operand parts of the training convolutions on the tensor cores (0: CUDA cores)
-  // the split inputs of every convolution, kept by the training forward for
-  // the weight gradients, the split gradient of the current output, and the
-  // partial sums (dw_ready: allocated for the current (B, n))
-  bool dw_ready = false;
+  // training buffers for the current (B, n), by form.  Tensor cores (dw_ready):
+  // the split inputs of every convolution, kept by the forward for the weight
+  // gradients, the split gradient of the current output, the partial sums.  CUDA
+  // cores (core_ready): the FP32 gradient planes gdl and gebot, and the later
+  // parts of a converted input.
+  bool dw_ready = false, core_ready = false;
   std::vector<__nv_bfloat16 *> xsplit;  // 3 per layer
   __nv_bfloat16 *gsplit[3] = {nullptr, nullptr, nullptr};
   float *dw_part = nullptr, *db_part = nullptr;
   std::vector<DwJob> dw_jobs;  // per layer
-  __nv_bfloat16 *nhwc_lo = nullptr;  // second part of a converted input (widths without kept ones)
+  __nv_bfloat16 *nhwc_lo = nullptr, *nhwc_p2 = nullptr;
   // the split weights of every convolution of a training step and of its
   // adjoint: packed by the jobs, layer i's at wsp + wsp_f[i] and wsp + wsp_b[i]
   // (-1: on the CUDA cores)
@@ -1435,6 +1437,20 @@ struct UnetImpl {
 };
 
 namespace {
+
+void free_dw(UnetImpl *u) {
+  for (__nv_bfloat16 *q : u->xsplit)
+    if (q) vie_free(q);
+  u->xsplit.clear();
+  for (__nv_bfloat16 *&q : u->gsplit) {
+    if (q) vie_free(q);
+    q = nullptr;
+  }
+  if (u->dw_part) vie_free(u->dw_part);
+  if (u->db_part) vie_free(u->db_part);
+  u->dw_part = u->db_part = nullptr;
+  u->dw_ready = false;
+}
 
 void free_acts(UnetImpl *u) {
   auto fr = [](std::vector<float *> &vv) {
@@ -1452,24 +1468,15 @@ void free_acts(UnetImpl *u) {
   u->nhwc = nullptr;
   if (u->hx) vie_free(u->hx);
   u->hx = nullptr;
-  for (__nv_bfloat16 **q : {&u->nhwc_lo, &u->wsp}) {
+  for (__nv_bfloat16 **q : {&u->nhwc_lo, &u->nhwc_p2, &u->wsp}) {
     if (*q) vie_free(*q);
     *q = nullptr;
   }
   for (__nv_bfloat16 *q : u->hcat)
     if (q) vie_free(q);
   u->hcat.clear();
-  for (__nv_bfloat16 *q : u->xsplit)
-    if (q) vie_free(q);
-  u->xsplit.clear();
-  for (__nv_bfloat16 *&q : u->gsplit) {
-    if (q) vie_free(q);
-    q = nullptr;
-  }
-  if (u->dw_part) vie_free(u->dw_part);
-  if (u->db_part) vie_free(u->db_part);
-  u->dw_part = u->db_part = nullptr;
-  u->dw_ready = false;
+  free_dw(u);
+  u->core_ready = false;
   u->maps.clear();
   u->o = u->go = nullptr;
   u->part = nullptr;
@@ -1506,20 +1513,16 @@ vie_status ensure_acts(UnetImpl *u, int B, int n, cudaStream_t st) {
       if ((s = al(&u->dl[l], (long)B * C * hw)) != VIE_OK) return s;
       if ((s = al(&u->gcat[l], (long)B * 2 * C * hw)) != VIE_OK) return s;
       if ((s = al(&u->gbl[l], (long)B * C * hw)) != VIE_OK) return s;
-      if ((s = al(&u->gdl[l], (long)B * C * hw)) != VIE_OK) return s;
     }
   }
   const long hwb = (long)(n >> (L - 1)) * (n >> (L - 1));
   if ((s = al(&u->ebot[0], (long)B * C * hwb)) != VIE_OK) return s;
-  if ((s = al(&u->gebot[0], (long)B * C * hwb)) != VIE_OK) return s;
   if ((s = al(&u->o, (long)B * n * n)) != VIE_OK) return s;
   if ((s = al(&u->go, (long)B * n * n)) != VIE_OK) return s;
   VIE_CUDA(vie_malloc((void **)&u->part, sizeof(double) * 1024));
   VIE_CUDA(vie_malloc_host((void **)&u->h_part, sizeof(double) * 1024));
   // the widest convolution input: 2 C channels (a decoder's concatenation), padded to slices
   VIE_CUDA(vie_malloc((void **)&u->nhwc,
-                      sizeof(__nv_bfloat16) * (size_t)B * n * n * (size_t)(((2 * C + 31) / 32) * 32)));
-  VIE_CUDA(vie_malloc((void **)&u->nhwc_lo,
                       sizeof(__nv_bfloat16) * (size_t)B * n * n * (size_t)(((2 * C + 31) / 32) * 32)));
   {
     // split weights: three parts for the forward convolutions, two for the adjoints
@@ -1767,7 +1770,7 @@ vie_status conv3_split(UnetImpl *u, const float *in, long in_bs, int Ci, const _
                        NhwcIo *io) {
   const int S = (Ci + kTmaSlice - 1) / kTmaSlice, Cp = S * kTmaSlice;
   const long plane = (long)H * W;
-  __nv_bfloat16 *own[3] = {u->nhwc, u->nhwc_lo, nullptr};  // (three parts: always kept ones)
+  __nv_bfloat16 *own[3] = {u->nhwc, u->nhwc_lo, u->nhwc_p2};
   __nv_bfloat16 *const *xin = io && io->split ? io->split : own;
   if (!(io && io->split && io->split_ready)) {
     if (np == 3)
@@ -1992,9 +1995,31 @@ vie_status alloc_dw(UnetImpl *u) {
   return VIE_OK;
 }
 
-vie_status ensure_dw(UnetImpl *u) {
-  if (u->dw_ready || !dw_on_tensor_cores(u)) return VIE_OK;
-  const vie_status s = alloc_dw(u);
+// buffers of the training step on the CUDA cores
+vie_status alloc_core(UnetImpl *u) {
+  const size_t B = (size_t)u->B, C = (size_t)u->C, n = (size_t)u->n;
+  for (int l = 0; l < u->L; ++l) {
+    const size_t hw = (n >> l) * (n >> l);
+    VIE_CUDA(vie_malloc((void **)(l < u->L - 1 ? &u->gdl[l] : &u->gebot[0]), sizeof(float) * B * C * hw));
+  }
+  const size_t bytes = sizeof(__nv_bfloat16) * B * n * n * ((2 * C + 31) / 32 * 32);
+  VIE_CUDA(vie_malloc((void **)&u->nhwc_lo, bytes));
+  if (u->C == 32) VIE_CUDA(vie_malloc((void **)&u->nhwc_p2, bytes));  // (its forward has three parts)
+  u->core_ready = true;
+  return VIE_OK;
+}
+
+// The tensor-core form keeps every layer's split input (with four levels 1 KB a pixel of
+// the batch more than the other form needs); where that does not fit, 32 channels
+// train on the CUDA cores as the other widths do.
+vie_status ensure_train(UnetImpl *u) {
+  if (u->dw_ready || u->core_ready) return VIE_OK;
+  vie_status s = VIE_ERR_OOM;
+  if (dw_on_tensor_cores(u)) {
+    if ((s = alloc_dw(u)) == VIE_OK) return VIE_OK;
+    free_dw(u);
+  }
+  if (s == VIE_ERR_OOM) s = alloc_core(u);
   if (s != VIE_OK) free_acts(u);  // what was allocated goes with the activations
   return s;
 }
@@ -2220,7 +2245,7 @@ vie_status backward(UnetImpl *u, const float *x, int B, int n, cudaStream_t st) 
 vie_status loss_grad(UnetImpl *u, const float *x, const float *t, const float *wts, int B, int n, double *loss,
                      cudaStream_t st) {
   vie_status s;
-  if ((s = ensure_acts(u, B, n, st)) != VIE_OK || (s = ensure_dw(u)) != VIE_OK) return s;
+  if ((s = ensure_acts(u, B, n, st)) != VIE_OK || (s = ensure_train(u)) != VIE_OK) return s;
   if ((s = pack_split_weights(u, st)) != VIE_OK) return s;
   // the training convolutions on the tensor cores in split precision: the
   // forward in three parts (24 bits an operand, FP32's own; the tensor cores'

@@ -94,7 +94,10 @@ cudaError_t cached_alloc(void **p, size_t bytes, bool host) {
     cudaGetLastError();  // the failed allocation's error is not sticky
     release_cached();
     e = host ? cudaMallocHost(p, cls) : cudaMalloc(p, cls);
-    if (e != cudaSuccess) return e;
+    if (e != cudaSuccess) {
+      cudaGetLastError();  // nor is this one's: a caller with another plan may go on
+      return e;
+    }
   }
   g_live[*p] = {dev, cls};
   return cudaSuccess;
