@@ -33,7 +33,8 @@
 //
 // The coarsest grid's sweeps from zero are a fixed linear map f -> u.  Up to
 // kMapCells cells it is set up as a matrix (the sweeps applied to the unit
-// vectors, once per medium) and applied as one product: 200 sweeps in one CTA
+// vectors, once per medium: 60 us for 8 x 8 cells, 0.6 ms for 25 x 25) and
+// applied as one product: 200 sweeps in one CTA
 // took 160 us of each V-cycle at 128^2 (an 8 x 8 grid).  Larger coarsest grids
 // (odd sizes of 27 and more) run the sweeps on tiles, kCoarseSweeps / 4
 // launches of four.
@@ -53,7 +54,7 @@ namespace {
 constexpr int kCoarseSweeps = 200;
 constexpr int kT = 256;
 constexpr int kTile = 16;        // tile side of the smoothing kernels (even: colours and children align)
-constexpr int kMapCells = 625;   // largest coarsest grid (25 x 25) kept as a matrix: 3.1 MB, set up in < 1 ms
+constexpr int kMapCells = 625;   // largest coarsest grid (25 x 25) kept as a matrix: 3.1 MB, set up in half a ms
 
 __device__ __forceinline__ double neighbour_sum(const double *__restrict__ c, const double *__restrict__ u, int n,
                                                long N, int ix, int iy, long j) {
@@ -207,21 +208,50 @@ __global__ void __launch_bounds__(kT) k_dp_sweeps(int n, const double *__restric
 }
 
 // The coarsest grid's map, column by column: CTA k runs kCoarseSweeps
-// red-black sweeps from zero on the unit vector of cell k into G[k][.].
-__global__ void k_dp_coarse_map(int n, const double *__restrict__ c, double *__restrict__ G) {
-  const long N = (long)n * n, k = blockIdx.x;
-  double *u = G + k * N;
-  for (long j = threadIdx.x; j < N; j += blockDim.x) u[j] = 0.0;
+// red-black sweeps from zero on the unit vector of cell k into G[k][.].  Thread t
+// owns cells 2 t and 2 t + 1, one of each colour, with their couplings times
+// 1 / diagonal in registers; u lies in shared memory with a border of zeros, so
+// that a half-sweep is four multiply-adds and a barrier.  The FP64 pipe bounds
+// it on large grids (25 x 25: 0.5 ms for 3.1e8 multiply-adds), the chain of
+// half-sweeps on small ones.
+constexpr int kMapSide = 25;
+static_assert(kMapSide * kMapSide == kMapCells, "the border fits");
+constexpr int map_threads(int cells) { return ((cells + 1) / 2 + 31) / 32 * 32; }
+__global__ void __launch_bounds__(map_threads(kMapCells)) k_dp_coarse_map(int n, const double *__restrict__ c,
+                                                                         double *__restrict__ G) {
+  __shared__ double U[(kMapSide + 2) * (kMapSide + 2)];
+  const int N = n * n, P = n + 2, k = blockIdx.x;  // (N <= kMapCells)
+  for (int l = threadIdx.x; l < P * P; l += blockDim.x) U[l] = 0.0;
+  int at[2], cell[2];  // by colour: place in U, index
+  double w[2][4], b[2];
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const int j0 = 2 * threadIdx.x, j = j0 + ((j0 % n + j0 / n + q) & 1), x = j % n, y = j / n;
+    cell[q] = j < N ? j : -1;
+    at[q] = (y + 1) * P + x + 1;
+    b[q] = 0.0;
+    if (j < N) {
+      const double inv = c[5L * N + j];
+      w[q][0] = x > 0 ? c[N + j] * inv : 0.0;
+      w[q][1] = x < n - 1 ? c[2 * N + j] * inv : 0.0;
+      w[q][2] = y > 0 ? c[3 * N + j] * inv : 0.0;
+      w[q][3] = y < n - 1 ? c[4 * N + j] * inv : 0.0;
+      if (j == k) b[q] = inv;
+    }
+  }
   __syncthreads();
   for (int s = 0; s < kCoarseSweeps; ++s)
-    for (int colour = 0; colour < 2; ++colour) {
-      for (long j = threadIdx.x; j < N; j += blockDim.x) {
-        const int ix = (int)(j % n), iy = (int)(j / n);
-        if (((ix + iy) & 1) == colour)
-          u[j] = ((j == k ? 1.0 : 0.0) + neighbour_sum(c, u, n, N, ix, iy, j)) * c[5 * N + j];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      if (cell[q] >= 0) {
+        const double *u = U + at[q];
+        U[at[q]] = fma(w[q][0], u[-1], fma(w[q][1], u[1], fma(w[q][2], u[-P], fma(w[q][3], u[P], b[q]))));
       }
       __syncthreads();
     }
+#pragma unroll
+  for (int q = 0; q < 2; ++q)
+    if (cell[q] >= 0) G[(long)k * N + cell[q]] = U[at[q]];
 }
 
 // u = sum_k f_k G[k][.]: a CTA takes 32 cells, its 8 warps every 8th k, and
@@ -332,7 +362,7 @@ vie_status diffusion_prepare(DiffPre *dp, int n, const double *sigma_t, const do
   const int Nc = C.n * C.n;
   if (Nc <= kMapCells) {
     VIE_CUDA(vie_malloc((void **)&dp->map, sizeof(double) * (size_t)Nc * Nc));
-    k_dp_coarse_map<<<Nc, (Nc + 31) / 32 * 32, 0, st>>>(C.n, C.c, dp->map);
+    k_dp_coarse_map<<<Nc, map_threads(Nc), 0, st>>>(C.n, C.c, dp->map);
     VIE_CHECK_LAUNCH("k_dp_coarse_map");
     // applies may come on another stream
     VIE_CUDA(cudaStreamSynchronize(st));
