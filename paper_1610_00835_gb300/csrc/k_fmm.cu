@@ -22,8 +22,8 @@
 // S-step midpoint march of the bilinear sigma_t with the sample points
 // clamped to the hull of the cell centres (nodes near the boundary lie
 // outside it).  Setup fills the near blocks and the M2L blocks on the device
-// (FP32); an apply is 2 L - 2 launches of small dense products that read the
-// cached blocks once (M2L of all levels in one of them).
+// (FP32); an apply is the source kernel and 2 L - 2 launches (L = 2: 3) of small
+// dense products that read the cached blocks once (M2L of all levels in one of them).
 #include <math.h>
 
 #include <algorithm>
@@ -551,10 +551,11 @@ vie_status fmm_apply(const FmmPlan &fp, int op, const float *s, const double *g,
     k_fmm_m2l<<<(unsigned)first, tm, sizeof(float) * (kIL * P2 + tm), st>>>(a, P2, fp.m2l, fp.W, fp.Lc);
     VIE_CHECK_LAUNCH("k_fmm_m2l");
   }
-  // the leaves take their own L2L step where there are enough of them to hide it
-  // behind other leaves' near fields (1024 leaves at order 4: 31 us without it, 40
-  // with it, 3 for a launch of its own; 4096 at order 6: 106 with it, 117 without)
-  const bool fused = L > 2 && nl * nl >= 2048;
+  // the leaves take their own L2L step: a launch fewer, hidden behind other leaves'
+  // near fields.  Per apply with it and as a launch of its own: 42.0 and 46.2 us at
+  // 128^2 (256 leaves) and 86.8 and 87.5 at 256^2 (1024) at order 4, 62.1 and 66.2,
+  // 121.4 and 126.5, and 287 and 293 at 512^2 (4096) at order 6
+  const bool fused = L > 2;
   for (int l = 2; l < (fused ? L - 1 : L); ++l) {
     const int gl = boxes_per_cta(P2, P2, 4L << (2 * l));
     k_fmm_l2l<<<ctas(4L << (2 * l), gl), kBoxThreads, sizeof(float) * gl * P2, st>>>(
