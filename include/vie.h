@@ -317,7 +317,7 @@ typedef struct vie_batch vie_batch;
  * be FP32 tiles with the S = 64 march and M-iii.  o->kernel selects how the
  * grids run: VIE_KERNEL_SYMMETRIC puts every grid's tile pairs into one
  * persistent launch; VIE_KERNEL_AUTO (and DISPLACEMENT) give each grid that
- * the displacement kernel takes (2 <= n <= 258) a launch of that kernel and
+ * the displacement kernel takes (2 <= n <= 258) launches of that kernel and
  * put only the others into the persistent launch; all of them are replayed
  * from one CUDA graph.  Vectors of the batch are packed: medium i occupies
  * cells [offsets[i], offsets[i+1]) (vie_batch_layout).

@@ -312,8 +312,8 @@ __global__ void __launch_bounds__(128, 1)
       ++issued_loads;
     }
   } else if (warp == 1 && elect_one()) {
-    // MMA issuer (one elected lane: the compiler then keeps the descriptors in
-    // uniform registers)
+    // MMA issuer: one elected lane, descriptors by addition (207 to 201 us for 64
+    // sources at 128^2 against a lane chosen by its number)
     for (int i = 0; i < nkb; ++i) {
       const int s = i % STAGES, use = i / STAGES;
       if (!mbar_wait(su32(bars + s), use & 1, abort_flag, i == 0 ? a.wl.first : a.wl.limit)) {

@@ -93,18 +93,21 @@ constexpr int kThreads = 1024;
 // take 96 registers, so 640 threads; the code of the march doubles, which the
 // instruction cache only bears because units are sorted by run axis (warps run
 // one axis' loops at a time; unsorted 1977 us at 128^2) and the epilogue is one
-// loop over the tiles.  Measured per apply with one and two tiles: 424 / 419 us
-// at 97^2, 1282 / 1254 at 128^2 (512 threads 1374, 768 1263), 3470 / 3378 at
-// 160^2, 10075 / 9916 at 200^2.  Small grids have too few units per warp.
+// loop over the tiles.  Measured per apply with one and two tiles, both on one
+// box: 424 / 419 us at 97^2, 1282 / 1254 at 128^2 (512 threads 1374, 768 1263),
+// 3470 / 3378 at 160^2, 10075 / 9916 at 200^2 (boxes differ by 2 %: 1282 with two
+// tiles at 128^2 on another).  Small grids have too few units per warp.
 __host__ __device__ constexpr int disp_tiles(int n) { return n >= 96 ? 2 : 1; }
 __host__ __device__ constexpr int disp_threads(int T) { return T == 2 ? 640 : kThreads; }
 // Two tiles whose blocks follow each other along the run axis are one march of 2 R
 // stacked targets: L + 2 R - 1 lattice loads per chunk of L cells instead of
 // 2 (L + R - 1), 7 % of the data path's wavefronts.  It takes the march's code a
-// third time, which pays from 130^2 on, where most units are such pairs: an
-// apply (with, without) 462 and 432 us at 97^2, 1277 and 1294 at 128^2, 1682 and
-// 1723 at 136^2, 3365 and 3531 at 160^2, 9763 and 10195 at 200^2.  Below, the
-// kernels (lattice pitches up to 141) leave the code out.
+// third time, which pays where most units are such pairs: an apply (with,
+// without) 462 and 432 us at 97^2, 1277 and 1294 at 128^2, 1682 and 1723 at 136^2,
+// 3365 and 3531 at 160^2, 9763 and 10195 at 200^2.  A kernel has the code or not, and
+// the kernel of lattice pitch 141 serves 98 to 129, so the line is the next pitch's
+// first grid.  (Grids of 228 and 229 have units marked so, but a run-time pitch: their
+// kernel takes them as two tiles.)
 __host__ __device__ constexpr bool disp_stacked(int n, int R) { return R == 12 && n >= 130; }
 constexpr int kStackedPitch = 173;  // the least pitch of those grids
 __host__ __device__ constexpr int disp_depth(int n) { return n >= 96 ? 12 : 8; }
@@ -129,8 +132,9 @@ __host__ __device__ constexpr int group_stride(int R, int lg) { return lg == 1 ?
 // lattice or its last ones: each window's units run as a launch of their own
 // with the window in shared memory, the rest (tiles that span more: at 256^2 a
 // tenth of the units, 17 % of the march) reads the lattice through L1, with a
-// transposed copy for the runs along x.  An apply at 256^2 with every unit
-// through L1 took 28.3 ms, with windows 25.1.
+// transposed copy for the runs along x.  An apply at 243^2 with every unit
+// through L1 took 28.3 ms, with windows 25.1 (24.3 with stacked blocks; 30.7 at
+// 256^2, 38.4 with one tile a unit and every unit through L1).
 constexpr int kGlobalMaxN = 258;
 constexpr int kGlobalPitch = 271;  // disp_pitch(kGlobalMaxN, 12)
 // rows of a window, and the first row of the second one (a multiple of 4: its

@@ -10,7 +10,9 @@
 // and the step is integrated exactly:
 //   Phi += e^{-tau} Q~ (1 - e^{-sigma~ D}) / sigma~,  tau += sigma~ D.
 //
-// What bounds it is instruction issue, so the step is kept short:
+// What bounds it is the L1 data path (85 % of its wavefronts at 32^3, 65 % of the
+// issue slots): the corners of a warp's points lie in several rows of cells, and a
+// step reads eight of them.  So the loads are few and the step is short:
 //  * sigma_t and Q sit side by side in one lattice with a ghost layer (edge
 //    copies), so that no coordinate needs clamping, a corner is one 8-byte load
 //    for both, and the two interpolations run as packed FP32 pairs; floors are
